@@ -213,29 +213,6 @@ __device__ __forceinline__ void micro_slope(const Prim<T>& s, T K, const T* b, T
     a[0] = b[0] - s.u * a[1] - s.v * a[2] - s.w * a[3] - T(0.5) * a4 * e;
 }
 
-// Slopes a_x, a_y, a_z and A of a Maxwellian with conservative gradients
-// g[i][q] (Eq. co): <a_i psi> = g_i / rho, <(A + sum_i a_i u_i) psi> = 0.
-// r (may be NULL) receives <A psi> = -sum_i <(a_i . psi) u_i psi>, which
-// the flux needs again (rho <A psi> is the W-rate of the equilibrium part).
-template <typename T>
-__device__ __forceinline__ void state_slopes(const Prim<T>& s, const Tab<T>& full, T K,
-                                             const T (*g)[5], T (*a)[5], T* A, T* r_out = nullptr) {
-    const T ir = T(1) / s.rho;
-#pragma unroll
-    for (int i = 0; i < 3; ++i) {
-        T b[5];
-#pragma unroll
-        for (int k = 0; k < 5; ++k) b[k] = g[i][k] * ir;
-        micro_slope(s, K, b, a[i]);
-    }
-    T r[5] = {T(0), T(0), T(0), T(0), T(0)};
-    acc_grad<0>(full, a, T(-1), r);
-    micro_slope(s, K, r, A);
-    if (r_out)
-#pragma unroll
-        for (int k = 0; k < 5; ++k) r_out[k] = r[k];
-}
-
 // Directional derivative of the Euler flux along x_dir (face frame) of the
 // state W (primitives s): out = (d F_dir / d W) dW, with
 // F_dir = (m_dir, m_j u_dir + p delta_j,dir, (E + p) u_dir) and
@@ -350,143 +327,6 @@ __device__ __forceinline__ void kinetic_side(const Phys<T>& ph, const Prim<T>& S
         make_tab(t, S, ph.K, half);
     }
 }
-
-// Time-dependent kinetic solution at one Gauss point, face frame.
-//   Wl, Wr: states; gl[i][q], gr[i][q]: gradients (direction i, comp q)
-// Outputs, each 5 long:
-//   Fh = int_0^{dt/2} F dt,  D = int_0^dt F dt - 2 Fh   (second-order part)
-//   W0 = W(0),               dW = W(dt) - W(0)
-// D and dW are formed from differences of the time coefficients, in which
-// the leading terms cancel exactly, instead of by subtracting the rounded
-// integrals (which loses about three digits in FP32).
-template <typename T>
-__device__ __forceinline__ void gks_point(const Phys<T>& ph, const T* Wl, const T (*gl)[5],
-                                          const T* Wr, const T (*gr)[5], T dt, T* Fh, T* D,
-                                          T* W0, T* dW) {
-    const Prim<T> P[2] = {to_prim(Wl, ph.gm1), to_prim(Wr, ph.gm1)};
-#pragma unroll
-    for (int k = 0; k < 5; ++k) {
-        Fh[k] = T(0);
-        D[k] = T(0);
-        W0[k] = T(0);
-        dW[k] = T(0);
-    }
-    // W^c from the half-space moments of both sides (Eq. new-equ-part)
-    T Wc[5] = {T(0), T(0), T(0), T(0), T(0)};
-    {
-        Tab<T> t;
-        make_tab(t, P[0], ph.K, +1);
-        acc_psi<0, 0, 0>(t, P[0].rho, Wc);
-        make_tab(t, P[1], ph.K, -1);
-        acc_psi<0, 0, 0>(t, P[1].rho, Wc);
-    }
-    const Prim<T> C = to_prim(Wc, ph.gm1);
-    const TimeCoef<T> tc = time_coefs(ph, P[0].p, P[1].p, C.p, dt);
-    const T tau = tc.tau;
-    // state integrals over [0, dt/2] and their "dt minus twice" differences,
-    // for the Pr fix only
-    const bool prfix = ph.prf != T(0);
-    T IWh[5], IWd[5];
-#pragma unroll
-    for (int k = 0; k < 5; ++k) IWh[k] = IWd[k] = T(0);
-    T dWc[3][5];
-#pragma unroll
-    for (int i = 0; i < 3; ++i)
-#pragma unroll
-        for (int k = 0; k < 5; ++k) dWc[i][k] = T(0);
-#pragma unroll 1
-    for (int side = 0; side < 2; ++side) {
-        const Prim<T> S = P[side];
-        Tab<T> t;
-        T a[3][5], A[5];
-        kinetic_side(ph, S, side == 0 ? gl : gr, side == 0 ? +1 : -1, t, a, A);
-#pragma unroll
-        for (int i = 0; i < 3; ++i) acc_apsi<0, 0, 0>(t, a[i], S.rho, dWc[i]);
-        if (ph.smooth) continue;
-        T mf0[5] = {0}, mf1[5] = {0}, mw0[5] = {0}, mw1[5] = {0};
-        acc_psi<1, 0, 0>(t, S.rho, mf0);
-        acc_grad<1>(t, a, S.rho, mf1);
-        acc_psi<0, 0, 0>(t, S.rho, mw0);
-        acc_grad<0>(t, a, S.rho, mw1);
-        axpy5(tc.k0, mf0, Fh);
-        axpy5(-(tau * tc.k0 + tc.k1), mf1, Fh);
-        axpy5(tc.dk0, mf0, D);
-        axpy5(-(tau * tc.dk0 + tc.dk1), mf1, D);
-        axpy5(T(1), mw0, W0);
-        axpy5(-tau, mw1, W0);
-        axpy5(tau - (tau + dt) * tc.E, mw1, dW);
-        if (prfix) {
-            axpy5(tc.k0, mw0, IWh);
-            axpy5(-(tau * tc.k0 + tc.k1), mw1, IWh);
-            axpy5(tc.dk0, mw0, IWd);
-            axpy5(-(tau * tc.dk0 + tc.dk1), mw1, IWd);
-        }
-        if (ph.viscous) {
-            T mf2[5] = {0}, mw2[5] = {0};
-            acc_apsi<1, 0, 0>(t, A, S.rho, mf2);
-            acc_apsi<0, 0, 0>(t, A, S.rho, mw2);
-            axpy5(-tau * tc.k0, mf2, Fh);
-            axpy5(-tau * tc.dk0, mf2, D);
-            axpy5(-tau, mw2, W0);
-            axpy5(tau * (T(1) - tc.E), mw2, dW);
-            if (prfix) {
-                axpy5(-tau * tc.k0, mw2, IWh);
-                axpy5(-tau * tc.dk0, mw2, IWd);
-            }
-        }
-    }
-    // hydrodynamic (equilibrium) part: C1 g^c + C2 a^c.u g^c + C3 A^c g^c
-    Tab<T> t;
-    make_tab(t, C, ph.K, 0);
-    T ac[3][5], Ac[5], rA[5];
-    state_slopes(C, t, ph.K, dWc, ac, Ac, rA);
-    T mf0[5] = {0}, mf1[5] = {0}, mf2[5] = {0}, mw1[5];
-    acc_psi<1, 0, 0>(t, C.rho, mf0);
-    acc_grad<1>(t, ac, C.rho, mf1);
-    acc_apsi<1, 0, 0>(t, Ac, C.rho, mf2);
-#pragma unroll
-    for (int k = 0; k < 5; ++k) mw1[k] = -C.rho * rA[k];  // rho sum_i <(a_i . psi) u_i psi> (Eq. co)
-    if (ph.smooth) {
-        // f = g^c - tau (a^c.u + A^c) g^c + A^c g^c t, Eq. 2nd-smooth-flux
-        const T hd = T(0.5) * dt;
-        axpy5(hd, mf0, Fh);
-        axpy5(-tau * hd, mf1, Fh);
-        axpy5(T(0.5) * hd * hd - tau * hd, mf2, Fh);
-        axpy5(T(0.25) * dt * dt, mf2, D);
-#pragma unroll
-        for (int k = 0; k < 5; ++k) W0[k] = Wc[k];  // tau terms cancel: <(a.u + A) psi> = 0
-        axpy5(-dt, mw1, dW);
-        if (prfix) {
-            // int psi f over [0, dt/2] = hd W^c - hd^2/2 rho <(a^c.u) psi> (the
-            // A^c moments are minus the a^c.u ones); the difference -dt^2/4 of it
-            axpy5(hd, Wc, IWh);
-            axpy5(-T(0.5) * hd * hd, mw1, IWh);
-            axpy5(-T(0.25) * dt * dt, mw1, IWd);
-        }
-    } else {
-        axpy5(tc.q1, mf0, Fh);
-        axpy5(tc.q2, mf1, Fh);
-        axpy5(tc.q3, mf2, Fh);
-        axpy5(tc.dq1, mf0, D);
-        axpy5(tc.dq2, mf1, D);
-        axpy5(tc.dq3, mf2, D);
-        // t = dt: C2, C3 (C1 cancelled against the kinetic W0 terms)
-        const T C2 = (dt + tau) * tc.E - tau, C3 = dt - tau + tau * tc.E;
-        axpy5(C2 - C3, mw1, dW);
-        if (prfix) {
-            axpy5(tc.q1, Wc, IWh);
-            axpy5(tc.q2 - tc.q3, mw1, IWh);
-            axpy5(tc.dq1, Wc, IWd);
-            axpy5(tc.dq2 - tc.dq3, mw1, IWd);
-        }
-    }
-    if (prfix) {
-        const T U[3] = {C.u, C.v, C.w};
-        prandtl_fix(ph.prf, U, IWh, Fh);
-        prandtl_fix(ph.prf, U, IWd, D);
-    }
-}
-
 
 // --------------------------------------------- half differences --
 // A quantity known on the two sides of a face: its values l, r and,

@@ -4,6 +4,7 @@
 // the ghost states of boundary faces (Sec. 4.4).
 #pragma once
 
+#include "gks_device.cuh"
 #include "gks_kernels.h"
 
 namespace gks {
@@ -42,8 +43,12 @@ __device__ __forceinline__ void eval_poly(const T* __restrict__ P, const T* X, T
 #pragma unroll
     for (int q = 0; q < 5; ++q) {
         const T* cq = c + q * 10;
-        const T v = cq[0] + cq[1] * x + cq[2] * y + cq[3] * z + cq[4] * x * x + cq[5] * x * y + cq[6] * x * z +
-                    cq[7] * y * y + cq[8] * y * z + cq[9] * z * z;
+        // nested form: s_i = c_i + (row i of the upper triangle) . X, so that
+        // v = c0 + X . s and d v / d x_i = s_i + (column i) . X
+        const T sx = cq[1] + cq[4] * x + cq[5] * y + cq[6] * z;
+        const T sy = cq[2] + cq[7] * y + cq[8] * z;
+        const T sz = cq[3] + cq[9] * z;
+        const T v = cq[0] + x * sx + y * sy + z * sz;
         if constexpr (sizeof(T) == 4) {
             val[q] = c[PHI + q] + v;
             if (dev) dev[q] = v;
@@ -52,9 +57,9 @@ __device__ __forceinline__ void eval_poly(const T* __restrict__ P, const T* X, T
         } else {
             val[q] = v;
         }
-        g[0][q] = cq[1] + T(2) * cq[4] * x + cq[5] * y + cq[6] * z;
-        g[1][q] = cq[2] + cq[5] * x + T(2) * cq[7] * y + cq[8] * z;
-        g[2][q] = cq[3] + cq[6] * x + cq[8] * y + T(2) * cq[9] * z;
+        g[0][q] = sx + cq[4] * x;
+        g[1][q] = sy + cq[5] * x + cq[7] * y;
+        g[2][q] = sz + cq[6] * x + cq[8] * y + cq[9] * z;
     }
 }
 
@@ -235,6 +240,48 @@ __device__ __forceinline__ void fixed_ghost(const T* __restrict__ x0, const T* X
             v += g[i][q] * X[i];
         }
         W[q] = v;
+    }
+}
+
+// One side's state and gradients at Gauss point k of a face, face frame: the
+// side's cell reconstruction there, or the boundary face's ghost (side 0:
+// left, 1: right; a missing side carries its kind).  XW: isothermal and
+// moving walls are compiled in.
+template <typename T, bool XW>
+__device__ __forceinline__ void side_state(const DevMesh<T>& m, const Phys<T>& ph, const T* __restrict__ Wavg,
+                                           const T* __restrict__ poly, const T* __restrict__ geo,
+                                           const T (*Rm)[3], int L, int Rc, int side, int k, T* tW, T (*tg)[5]) {
+    const int mine = side == 0 ? L : Rc, other = side == 0 ? Rc : L;
+    T Ws[5], gs[3][5];
+    if (mine == FLR_OPEN) {
+        // open boundary: the interior cell's average with zero gradient
+        // (zeroth-order extrapolation; the paper leaves outflow boundaries
+        // open, and copying the interior Gauss-point state is not stable)
+#pragma unroll
+        for (int q = 0; q < 5; ++q) {
+            Ws[q] = Wavg[(int64_t)other * Stride<T>::xs + q];
+            gs[0][q] = gs[1][q] = gs[2][q] = T(0);
+        }
+    } else {
+        // a wall or fixed side starts from the interior cell at the point
+        const int src = mine >= 0 ? side : 1 - side;
+        const int64_t c = mine >= 0 ? mine : other;
+        const T X[3] = {geo[4 + 9 * src + 3 * k], geo[5 + 9 * src + 3 * k], geo[6 + 9 * src + 3 * k]};
+        if (mine == FLR_FIXED)
+            fixed_ghost(m.fixed + c * Stride<T>::xs, X, Ws, gs);
+        else
+            eval_poly(poly + c * Stride<T>::poly, X, Ws, gs);
+    }
+    to_local(Rm, Ws, gs, tW, tg);
+    if (mine == FLR_SLIP_WALL) slip_wall_ghost(tW, tg);
+    if (mine == FLR_NOSLIP_WALL) noslip_wall_ghost(tW, tg);
+    if constexpr (XW) {
+        if (mine == FLR_ISOTHERMAL_WALL) isothermal_wall_ghost(tW, tg, ph.gm1, ph.twall);
+        if (mine == FLR_MOVING_WALL) {
+            T Uw[3];
+            rotate_vec(Rm, ph.uwall, Uw);
+            moving_wall_ghost(tW, tg, ph.gm1, Uw);
+        }
     }
 }
 

@@ -13,6 +13,7 @@
 #include <cuda_runtime.h>
 
 #include "gks_flux.cuh"
+#include "gks_kinetic.cuh"
 
 namespace gks {
 
@@ -21,15 +22,21 @@ namespace gks {
 // --------------------------------------------------------------------------
 
 
-// 3 threads per face, one Gauss point each (used for FP64, whose register
-// footprint leaves no room for the lane-pair split)
-template <typename T, int NR>
-__global__ void __launch_bounds__(3 * FLUX_FACES) k_flux_single(DevMesh<T> m, Phys<T> ph,
-                                                                 const T* __restrict__ Wavg,
-                                                                 const T* __restrict__ poly,
-                                                                 T* __restrict__ rec,
-                                                                 const double* __restrict__ ctrl,
-                                                                 double dt_override) {
+// 3 threads per face, one Gauss point each (FP64).  The kinetic solution's
+// sums over the two sides are accumulated in one loop body, so only one
+// side's state and moments are live at a time.  VISC: the time slopes of
+// viscous flow.
+//
+// Bound by the FP64 pipe (2 lanes an SM: 16 cycles a warp instruction), so
+// what counts is the number of FP64 instructions: 1,601 a Gauss point here
+// against about 3,000 with the moment tables, 896 -> 484 us on 49,280 faces
+// (stage 1, inviscid; pipe 86 % busy).  Occupancy does not matter: 2 blocks
+// an SM (232 registers, no spills) take 494 us, 5 blocks (128 registers)
+// 497 us.
+template <typename T, int NR, bool VISC>
+__global__ void __launch_bounds__(3 * FLUX_FACES, 2)
+    k_flux_single(DevMesh<T> m, Phys<T> ph, const T* __restrict__ Wavg, const T* __restrict__ poly,
+                  T* __restrict__ rec, const double* __restrict__ ctrl, double dt_override) {
     __shared__ T red[FLUX_FACES * 3 * NR];
     const int lf = threadIdx.x / 3;
     const int k = threadIdx.x - 3 * lf;
@@ -41,56 +48,25 @@ __global__ void __launch_bounds__(3 * FLUX_FACES) k_flux_single(DevMesh<T> m, Ph
         const T dt = dtc > 0.0 ? (T)dtc : T(1);
         const T* geo = m.fgeo + f * FGEO;
         const T n[3] = {geo[0], geo[1], geo[2]};
-        const T w = geo[3];
-        T WL[5], gL[3][5], WR[5], gR[3][5];
-        for (int side = 0; side < 2; ++side) {
-            const int cell = side == 0 ? L : Rc;
-            T* Wv = side == 0 ? WL : WR;
-            T (*g)[5] = side == 0 ? gL : gR;
-            if (cell >= 0 || cell == FLR_SLIP_WALL || cell == FLR_NOSLIP_WALL || cell == FLR_ISOTHERMAL_WALL ||
-                cell == FLR_MOVING_WALL) {
-                // a wall side starts from the interior cell's value at the point
-                const int src = cell >= 0 ? side : 1 - side;
-                const int64_t c = cell >= 0 ? cell : (side == 0 ? Rc : L);
-                const T X[3] = {geo[4 + 9 * src + 3 * k], geo[5 + 9 * src + 3 * k], geo[6 + 9 * src + 3 * k]};
-                eval_poly(poly + c * Stride<T>::poly, X, Wv, g);
-            } else if (cell == FLR_FIXED) {
-                const int64_t in = side == 0 ? Rc : L;
-                const int src = 1 - side;
-                const T X[3] = {geo[4 + 9 * src + 3 * k], geo[5 + 9 * src + 3 * k], geo[6 + 9 * src + 3 * k]};
-                fixed_ghost(m.fixed + in * Stride<T>::xs, X, Wv, g);
-            } else {
-                // open boundary: interior cell average, zero gradient
-                const int64_t in = side == 0 ? Rc : L;
-                for (int q = 0; q < 5; ++q) {
-                    Wv[q] = Wavg[in * Stride<T>::xs + q];
-                    g[0][q] = g[1][q] = g[2][q] = T(0);
-                }
-            }
-        }
         T Rm[3][3];
         face_frame(n, Rm);
-        T tWL[5], tgL[3][5], tWR[5], tgR[3][5];
-        to_local(Rm, WL, gL, tWL, tgL);
-        to_local(Rm, WR, gR, tWR, tgR);
-        if (L == FLR_SLIP_WALL) slip_wall_ghost(tWL, tgL);
-        if (Rc == FLR_SLIP_WALL) slip_wall_ghost(tWR, tgR);
-        if (L == FLR_NOSLIP_WALL) noslip_wall_ghost(tWL, tgL);
-        if (Rc == FLR_NOSLIP_WALL) noslip_wall_ghost(tWR, tgR);
-        if (L == FLR_ISOTHERMAL_WALL) isothermal_wall_ghost(tWL, tgL, ph.gm1, ph.twall);
-        if (Rc == FLR_ISOTHERMAL_WALL) isothermal_wall_ghost(tWR, tgR, ph.gm1, ph.twall);
-        if (L == FLR_MOVING_WALL || Rc == FLR_MOVING_WALL) {
-            T Uw[3];
-            rotate_vec(Rm, ph.uwall, Uw);
-            if (L == FLR_MOVING_WALL) moving_wall_ghost(tWL, tgL, ph.gm1, Uw);
-            if (Rc == FLR_MOVING_WALL) moving_wall_ghost(tWR, tgR, ph.gm1, Uw);
+        KSums<T> S;
+        S.init();
+        T pl = T(0), pr = T(0);
+#pragma unroll 1
+        for (int side = 0; side < 2; ++side) {
+            T tW[5], tg[3][5];
+            side_state<T, true>(m, ph, Wavg, poly, geo, Rm, L, Rc, side, k, tW, tg);
+            pl = pr;
+            pr = kin_side<VISC>(ph, tW, tg, side == 0 ? +1 : -1, S);
         }
-        T Fh[5], D[5], W0[5], dWt[5];
-        gks_point(ph, tWL, tgL, tWR, tgR, dt, Fh, D, W0, dWt);
+        T Wc[5], Fh[5], D[5], W0[5], dWt[5];
+        finish_point<VISC, false>(ph, S, pl, pr, dt, Wc, Fh, D, W0, dWt);
         to_global(Rm, Fh);
         to_global(Rm, D);
         to_global(Rm, W0);
         to_global(Rm, dWt);
+        const T w = geo[3];
 #pragma unroll
         for (int q = 0; q < 5; ++q) {
             if (NR == 40) {
@@ -155,10 +131,11 @@ cudaError_t Launch<T>::flux(const DevMesh<T>& m, const HostPhys& p, const T* W, 
                 prf ? go(k_flux<T, 20, 2, true, false>) : go(k_flux<T, 20, 2, false, false>);
         }
     } else {
+        auto go = [&](auto kernel) { kernel<<<grid, 3 * FLUX_FACES, 0, s>>>(m, ph, W, poly, rec, ctrl, dt_override); };
         if (stage == 1)
-            k_flux_single<T, 40><<<grid, 3 * FLUX_FACES, 0, s>>>(m, ph, W, poly, rec, ctrl, dt_override);
+            p.viscous ? go(k_flux_single<T, 40, true>) : go(k_flux_single<T, 40, false>);
         else
-            k_flux_single<T, 20><<<grid, 3 * FLUX_FACES, 0, s>>>(m, ph, W, poly, rec, ctrl, dt_override);
+            p.viscous ? go(k_flux_single<T, 20, true>) : go(k_flux_single<T, 20, false>);
     }
     return cudaGetLastError();
 }
