@@ -423,8 +423,8 @@ gks_status gks_adjoint_step_staged(gks_state* state, double dt, const double* d_
 
 /* Execution variant of a state (the same arithmetic, only speed differs):
  *   face_order   0 = faces in canonical order, 1 = grouped by left cell
- *   flux_blocks  resident flux blocks per SM, 3 (more warps, fewer registers)
- *                or 2 (no register spills); FP32 only, ignored in FP64
+ *   flux_blocks  occupancy of the flux: 3 (more warps, fewer registers) or 2
+ *                (fewer warps, more registers); FP32 only, ignored in FP64
  *   slopes_pass  0 = reconstruction step 1 (the P1 slopes, Sec. 4.3) is
  *                recomputed inside step 2 for each neighbour, 1 = a separate
  *                pass stores every cell's slopes first (WENO only)

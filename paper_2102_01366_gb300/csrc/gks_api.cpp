@@ -337,7 +337,7 @@ Layout layout_workspace(int64_t nc, int64_t nf, int64_t ncase, bool fp32, bool f
     L.G = L.add(T * 15 * nc);
     L.slopes = L.add(T * 15 * nc);
     L.poly = L.add(T * (fp32 ? Stride<float>::poly : Stride<double>::poly) * nc);
-    L.rec = L.add(T * (fp32 ? REC1_F32 : 40) * nf);
+    L.rec = L.add(T * (fp32 ? rec_stride<float, 40>() : rec_stride<double, 40>()) * nf);
     L.ctrl = L.add(8 * CTRL_N);
     L.case_t = L.add(8 * ncase);
     L.case_dt = L.add(8 * ncase);

@@ -213,40 +213,6 @@ __device__ __forceinline__ void micro_slope(const Prim<T>& s, T K, const T* b, T
     a[0] = b[0] - s.u * a[1] - s.v * a[2] - s.w * a[3] - T(0.5) * a4 * e;
 }
 
-// Directional derivative of the Euler flux along x_dir (face frame) of the
-// state W (primitives s): out = (d F_dir / d W) dW, with
-// F_dir = (m_dir, m_j u_dir + p delta_j,dir, (E + p) u_dir) and
-// p = (gamma - 1)(E - |m|^2 / (2 rho)).  For a Maxwellian g(W(x, t)), whose
-// derivatives are g (a . psi) with rho <a psi> = dW (Eq. co), the velocity
-// moments rho <u_dir (a . psi) psi> equal this product.
-template <typename T>
-__device__ __forceinline__ void euler_flux_jvp(const Prim<T>& s, const T* W, T gm1, int dir, const T* dW, T* out) {
-    const T u[3] = {s.u, s.v, s.w};
-    const T ud = u[dir];
-    const T dp = gm1 * (dW[4] - (u[0] * dW[1] + u[1] * dW[2] + u[2] * dW[3]) +
-                        T(0.5) * (u[0] * u[0] + u[1] * u[1] + u[2] * u[2]) * dW[0]);
-    const T dud = (dW[1 + dir] - ud * dW[0]) / s.rho;
-    out[0] = dW[1 + dir];
-#pragma unroll
-    for (int j = 0; j < 3; ++j) out[1 + j] = dW[1 + j] * ud + W[1 + j] * dud + (j == dir ? dp : T(0));
-    out[4] = (dW[4] + dp) * ud + (W[4] + s.p) * dud;
-}
-
-// sum_i (d F_i / d W) g_i: the divergence of the Euler flux for the
-// conservative gradients g[i][q] (face frame)
-template <typename T>
-__device__ __forceinline__ void euler_divergence(const Prim<T>& s, const T* W, T gm1, const T (*g)[5], T* out) {
-#pragma unroll
-    for (int q = 0; q < 5; ++q) out[q] = T(0);
-#pragma unroll
-    for (int i = 0; i < 3; ++i) {
-        T d[5];
-        euler_flux_jvp(s, W, gm1, i, g[i], d);
-#pragma unroll
-        for (int q = 0; q < 5; ++q) out[q] += d[q];
-    }
-}
-
 // Time coefficients of Eq. 2nd-flux over [0, dt/2] (k0, k1 for the kinetic
 // factors e and t e; q1..q3 for C1..C3) and their "dt minus twice dt/2"
 // differences (dk*, dq*), with E = exp(-dt/tau_n) = Eh^2.
@@ -298,34 +264,6 @@ __device__ __forceinline__ void prandtl_fix(T prf, const T* U, const T* IW, T* F
     const T qf = F[4] - (U[0] * F[1] + U[1] * F[2] + U[2] * F[3]) + uu * F[0];
     const T qw = IW[4] - (U[0] * IW[1] + U[1] * IW[2] + U[2] * IW[3]) + uu * IW[0];
     F[4] += prf * (qf - U[0] * qw);
-}
-
-// One side's initial-state (kinetic) part of Eq. 2nd-flux,
-//   e^{-t/tau_n} g [1 - (tau + t) a.u - tau A] H(+-u1),
-// added to Fh, D, W0, dW.  Each velocity moment is formed once and scaled by
-// the time coefficients of all four outputs; the A terms carry a factor tau
-// and are skipped for inviscid flow.  Also returns this side's contributions
-// rho <psi> to W^c and rho <a_i psi> to its slopes (half space).
-template <typename T>
-__device__ __forceinline__ void kinetic_side(const Phys<T>& ph, const Prim<T>& S, const T (*g)[5], int half,
-                                             Tab<T>& t, T (*a)[5], T* A) {
-    const T ir = T(1) / S.rho;
-#pragma unroll
-    for (int i = 0; i < 3; ++i) {
-        T b[5];
-#pragma unroll
-        for (int k = 0; k < 5; ++k) b[k] = g[i][k] * ir;
-        micro_slope(S, ph.K, b, a[i]);
-    }
-    if (ph.viscous) {
-        make_tab(t, S, ph.K, 0);
-        T r[5] = {T(0), T(0), T(0), T(0), T(0)};
-        acc_grad<0>(t, a, T(-1), r);
-        micro_slope(S, ph.K, r, A);
-        make_half_u(t, S, half);
-    } else {
-        make_tab(t, S, ph.K, half);
-    }
 }
 
 // --------------------------------------------- half differences --
@@ -438,33 +376,32 @@ __device__ __forceinline__ void psi_half_difference(const float* Wl, const float
     out[4] = hd_mul(E, e0).h + 0.5f * hd_mul(m1, g).h;
 }
 
-// Normal Euler flux F_n(W) = (m.n, m u_n + p n, (E + p) u_n), u_n = m.n / rho,
-// of a global-frame state.
-__device__ __forceinline__ void normal_flux(const float* W, const float* n, float gm1, float* out) {
-    const float mn = W[1] * n[0] + W[2] * n[1] + W[3] * n[2];
-    const float un = mn / W[0];
+// Euler flux along x1 of a face-frame state: (m1, m1 u + p, m2 u, m3 u,
+// (E + p) u), u = m1 / rho.
+__device__ __forceinline__ void euler_flux1(const float* W, float gm1, float* out) {
+    const float u = W[1] / W[0];
     const float p = gm1 * (W[4] - 0.5f * (W[1] * W[1] + W[2] * W[2] + W[3] * W[3]) / W[0]);
-    out[0] = mn;
-#pragma unroll
-    for (int j = 0; j < 3; ++j) out[1 + j] = W[1 + j] * un + p * n[j];
-    out[4] = (W[4] + p) * un;
+    out[0] = W[1];
+    out[1] = W[1] * u + p;
+    out[2] = W[2] * u;
+    out[3] = W[3] * u;
+    out[4] = (W[4] + p) * u;
 }
 
-// (F_n(Wl) - F_n(Wr)) / 2 of the normal Euler flux by the half-difference
-// rules, given the half-difference h of the two global-frame states: exact
-// to the rounding of the result itself, however close the two states.
-__device__ __forceinline__ void normal_flux_half_difference(const float* Wl, const float* Wr, const float* h,
-                                                            const float* n, float gm1, float* out) {
+// (F_1(Wl) - F_1(Wr)) / 2 by the half-difference rules, given the
+// half-difference h of the two face-frame states: exact to the rounding of
+// the result itself, however close the two states.
+__device__ __forceinline__ void flux1_half_difference(const float* Wl, const float* Wr, const float* h, float gm1,
+                                                      float* out) {
     const HDiff<float> rho{Wl[0], Wr[0], h[0]}, E{Wl[4], Wr[4], h[4]};
     const HDiff<float> m[3] = {{Wl[1], Wr[1], h[1]}, {Wl[2], Wr[2], h[2]}, {Wl[3], Wr[3], h[3]}};
-    const HDiff<float> mn = hd_add(hd_add(hd_scale(n[0], m[0]), hd_scale(n[1], m[1])), hd_scale(n[2], m[2]));
-    const HDiff<float> un = hd_div(mn, rho);
+    const HDiff<float> u = hd_div(m[0], rho);
     const HDiff<float> mm = hd_add(hd_add(hd_mul(m[0], m[0]), hd_mul(m[1], m[1])), hd_mul(m[2], m[2]));
     const HDiff<float> p = hd_scale(gm1, hd_add(E, hd_scale(-0.5f, hd_div(mm, rho))));
-    out[0] = mn.h;
+    out[0] = h[1];
 #pragma unroll
-    for (int j = 0; j < 3; ++j) out[1 + j] = hd_mul(m[j], un).h + n[j] * p.h;
-    out[4] = hd_mul(hd_add(E, p), un).h;
+    for (int j = 0; j < 3; ++j) out[1 + j] = hd_mul(m[j], u).h + (j == 0 ? p.h : 0.0f);
+    out[4] = hd_mul(hd_add(E, p), u).h;
 }
 
 // ------------------------------------------------- FP32 pair numbers --

@@ -12,13 +12,13 @@ namespace gks {
 // R and its gradient at X (relative to the centroid) from a cell's
 // reconstruction record.  FP64 records hold R in centroid-monomial form; FP32
 // records hold R minus the cell average and the average's hi / lo parts, and
-// val = hi + (R - average).  dev, ahi, alo (FP32, each may be NULL) receive
-// R - average at X and the average's parts.
+// val = hi + (R - average).  dev (FP32, may be NULL) receives R - average at X.
 template <typename T>
 __device__ __forceinline__ void eval_poly(const T* __restrict__ P, const T* X, T* val, T (*g)[5],
-                                          T* dev = nullptr, T* ahi = nullptr, T* alo = nullptr) {
-    // the record is 16-byte aligned: load it in vectors
-    constexpr int PS = Stride<T>::poly;
+                                          T* dev = nullptr) {
+    // the record is 16-byte aligned: load it in vectors (FP32: without the
+    // lo parts at its end)
+    constexpr int PS = sizeof(T) == 4 ? PLO + 1 : Stride<T>::poly;
     T c[PS];
     if constexpr (sizeof(T) == 4) {
         const float4* p4 = reinterpret_cast<const float4*>(P);
@@ -52,8 +52,6 @@ __device__ __forceinline__ void eval_poly(const T* __restrict__ P, const T* X, T
         if constexpr (sizeof(T) == 4) {
             val[q] = c[PHI + q] + v;
             if (dev) dev[q] = v;
-            if (ahi) ahi[q] = c[PHI + q];
-            if (alo) alo[q] = c[PLO + q];
         } else {
             val[q] = v;
         }
@@ -246,13 +244,19 @@ __device__ __forceinline__ void fixed_ghost(const T* __restrict__ x0, const T* X
 // One side's state and gradients at Gauss point k of a face, face frame: the
 // side's cell reconstruction there, or the boundary face's ghost (side 0:
 // left, 1: right; a missing side carries its kind).  XW: isothermal and
-// moving walls are compiled in.
+// moving walls are compiled in.  dev (FP32, may be NULL) receives the
+// evaluated reconstruction minus its cell's average, global frame (0 for an
+// open or fixed side).
 template <typename T, bool XW>
 __device__ __forceinline__ void side_state(const DevMesh<T>& m, const Phys<T>& ph, const T* __restrict__ Wavg,
                                            const T* __restrict__ poly, const T* __restrict__ geo,
-                                           const T (*Rm)[3], int L, int Rc, int side, int k, T* tW, T (*tg)[5]) {
+                                           const T (*Rm)[3], int L, int Rc, int side, int k, T* tW, T (*tg)[5],
+                                           T* dev = nullptr) {
     const int mine = side == 0 ? L : Rc, other = side == 0 ? Rc : L;
     T Ws[5], gs[3][5];
+    if (dev)
+#pragma unroll
+        for (int q = 0; q < 5; ++q) dev[q] = T(0);
     if (mine == FLR_OPEN) {
         // open boundary: the interior cell's average with zero gradient
         // (zeroth-order extrapolation; the paper leaves outflow boundaries
@@ -270,7 +274,7 @@ __device__ __forceinline__ void side_state(const DevMesh<T>& m, const Phys<T>& p
         if (mine == FLR_FIXED)
             fixed_ghost(m.fixed + c * Stride<T>::xs, X, Ws, gs);
         else
-            eval_poly(poly + c * Stride<T>::poly, X, Ws, gs);
+            eval_poly(poly + c * Stride<T>::poly, X, Ws, gs, dev);
     }
     to_local(Rm, Ws, gs, tW, tg);
     if (mine == FLR_SLIP_WALL) slip_wall_ghost(tW, tg);

@@ -170,10 +170,13 @@ __global__ void k_rec_out(const T* __restrict__ rec, const int32_t* __restrict__
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nf * nr; i += (int64_t)gridDim.x * blockDim.x) {
         const int64_t d = i / nr;
         const int j = (int)(i - d * nr);
-        // FP32 stage-1 records: device stride 50 (reference flux at 40..49)
-        const int rs = (sizeof(T) == 4 && nr == 40) ? REC1_F32 : nr;
-        const T* r = rec + d * rs;
-        double v = (double)r[j];
+        // the public record has the interface-state entries times the normal
+        const int nflux = nr == 40 ? 10 : 5;
+        const T* r = rec + d * (nr == 40 ? rec_stride<T, 40>() : rec_stride<T, 20>());
+        const int je = j - nflux;
+        double v = j < nflux ? (double)r[j]
+                             : (double)r[nflux + (je / 15) * 5 + (je % 15) / 3] *
+                                   (double)m.fgeo[d * FGEO + (je % 15) % 3];
         if (sizeof(T) == 4 && nr == 40 && j < 10) {
             // the reference flux (dt / 2) A F_n(W_m), twice in the S entries
             const double ref = (double)r[REC1_REF + j % 5] + (double)r[REC1_REF + 5 + j % 5];

@@ -28,11 +28,22 @@ constexpr int XS = 20;               // reals per cell working-state record, FP6
 //   minus the average and the 9 slopes/curvatures (50), the average's hi (5)
 //   and lo (5) parts
 constexpr int XS32 = 28;
-// FP32 stage-1 face records: the 40 entries of the definition (the flux and
-// interface-state entries relative to the mean W_m of the face's two cell
-// averages), then the reference flux (dt / 2) A F_n(W_m) as FP32 hi (5) and
-// lo (5) parts
-constexpr int REC1_F32 = 50, REC1_REF = 40;
+// Face records, sums over the face's Gauss points with their weights w:
+//   stage 1  sum w Fh (5), sum w (2 Fh - D / 3) (5), sum w W(t*) (5),
+//            sum w W(0) (5); FP32: the flux and interface-state entries are
+//            relative to the mean W_m of the face's two cell averages, and the
+//            reference flux (dt / 2) A F_n(W_m) follows as hi (5) and lo (5)
+//            parts (one aligned 128-byte record)
+//   stage 2  sum w 4/3 D (5), sum w dW (5)
+// The interface states enter a cell times the face's normal, which the
+// update multiplies in: a third of the words that (sum w W n) would take.
+// NR (40, 20) names the stage: the length of its record with the normal
+// multiplied in, as gks_debug_face_records gives it.
+constexpr int REC1_REF = 20;
+template <typename T, int NR>
+constexpr int rec_stride() {
+    return NR == 20 ? 10 : sizeof(T) == 4 ? 32 : 20;
+}
 constexpr int XLO = 20;              // offset of the lo parts in an FP32 working-state record
 constexpr int POLY_STRIDE32 = 60;
 constexpr int PHI = 50, PLO = 55;    // offsets of the average's hi / lo parts in an FP32 record
@@ -88,7 +99,7 @@ struct DevState {
     T* G;         // [15][nc] saved stage-1 gradient term
     T* slopes;    // [nc][15]
     T* poly;      // [nc][Stride<T>::poly]
-    T* rec;       // [nf][40]
+    T* rec;       // [nf][rec_stride]
     double* ctrl; // [CTRL_N] global controls (dt_fixed, t_end)
     double* case_t;   // [ncase] time of each case
     double* case_dt;  // [ncase] step of each case for the current step
@@ -129,7 +140,7 @@ struct Launch {
                              T* slopes_out, T* poly, int32_t* fallback, const Finalize* fin,
                              int32_t* err, cudaStream_t s);
     // case_dt: per-case step (NULL: dt_override for every face)
-    // variant: 1 = 3 blocks per SM (FP32), 0 = 2 blocks per SM; ignored in FP64
+    // variant (FP32): 1 = more resident warps, 0 = more registers; ignored in FP64
     static cudaError_t flux(const DevMesh<T>& m, const HostPhys& p, const T* X, const T* poly, T* rec,
                             const double* case_dt, double dt_override, int stage, cudaStream_t s,
                             int variant = 1);

@@ -3,7 +3,7 @@
 //
 // One block of 384 threads per SM runs the stage's three phases over the
 // whole (batched) mesh: the reconstruction as three groups of 128 threads
-// on blocks of 24 cells, the face flux as two groups of 192 threads on
+// on blocks of 24 cells, the face flux as four groups of 96 threads on
 // blocks of 32 faces, the cell update as three groups of 128 threads, each
 // group striding over its blocks; the phases are separated by grid-wide
 // barriers.  It is the same per-block source as the standalone kernels (the
@@ -20,12 +20,12 @@
 
 namespace gks {
 
-constexpr int STAGE_THREADS = 384;  // 3 cell groups of 128 = 2 flux groups of 192
-constexpr int CELL_GROUPS = STAGE_THREADS / CELL_THREADS, FLUX_GROUPS = STAGE_THREADS / (2 * FP_GP);
-static_assert(CELL_GROUPS * CELL_THREADS == STAGE_THREADS && FLUX_GROUPS * 2 * FP_GP == STAGE_THREADS,
+constexpr int STAGE_THREADS = 384;  // 3 cell groups of 128 = 4 flux groups of 96
+constexpr int CELL_GROUPS = STAGE_THREADS / CELL_THREADS, FLUX_GROUPS = STAGE_THREADS / FLUX_THREADS;
+static_assert(CELL_GROUPS * CELL_THREADS == STAGE_THREADS && FLUX_GROUPS * FLUX_THREADS == STAGE_THREADS,
               "the stage block holds whole cell and flux groups");
-// named barriers: flux side pairs 1-6, flux groups 7-8, cell groups 9-11
-constexpr int BAR_FLUX_PAIRS = 1, BAR_FLUX_GROUP = 7, BAR_CELL_GROUP = 9;
+// named barriers: flux groups 1-4, cell groups 5-7
+constexpr int BAR_FLUX_GROUP = 1, BAR_CELL_GROUP = 5;
 // bounded grid-barrier wait: polls with a short sleep, about a second in all
 constexpr int GRID_TRIES = 1 << 23;
 
@@ -87,7 +87,7 @@ constexpr size_t stage_smem_bytes() {
     return recon > flux ? (recon > upd ? recon : upd) : (flux > upd ? flux : upd);
 }
 
-template <int STAGE, bool PRF>
+template <int STAGE, bool VISC>
 __global__ void __launch_bounds__(STAGE_THREADS, 1)
     k_stage(DevMesh<float> m, Phys<float> ph, HostPhys hp, ReconConst<float> rc, DevState<float> st,
             FinArg<float> fin, unsigned* gbar) {
@@ -119,12 +119,12 @@ __global__ void __launch_bounds__(STAGE_THREADS, 1)
 
     // ---- face flux and records (Sec. 2.2, 3, 4.4, 4.5)
     {
-        const int grp = threadIdx.x / (2 * FP_GP), tid = threadIdx.x % (2 * FP_GP);
+        const int grp = threadIdx.x / FLUX_THREADS, tid = threadIdx.x % FLUX_THREADS;
         FluxSmem<float, NR>* fs = reinterpret_cast<FluxSmem<float, NR>*>(smem);
         for (int64_t fb = (int64_t)blockIdx.x * FLUX_GROUPS + grp; fb < nfb; fb += (int64_t)gridDim.x * FLUX_GROUPS) {
-            flux_faces<float, NR, PRF>(m, ph, X, st.poly, st.rec, st.case_dt, 0.0, fb, tid, fs[grp],
-                                       BAR_FLUX_PAIRS + 3 * grp, BAR_FLUX_GROUP + grp);
-            group_barrier(BAR_FLUX_GROUP + grp, 2 * FP_GP);  // shared memory free for the next block
+            flux_faces<float, NR, VISC, true>(m, ph, X, st.poly, st.rec, st.case_dt, 0.0, fb, tid, fs[grp],
+                                              BAR_FLUX_GROUP + grp);
+            group_barrier(BAR_FLUX_GROUP + grp, FLUX_THREADS);  // shared memory free for the next block
         }
     }
     grid_barrier(gbar, gbar + 1, st.err);
@@ -146,12 +146,12 @@ __global__ void __launch_bounds__(STAGE_THREADS, 1)
     }
 }
 
-template <int STAGE, bool PRF>
+template <int STAGE, bool VISC>
 static cudaError_t launch_stage_kernel(const DevMesh<float>& m, const Phys<float>& ph, const HostPhys& hp,
                                        const ReconConst<float>& rc, const DevState<float>& st,
                                        const FinArg<float>& fin, unsigned* gbar, cudaStream_t s) {
     constexpr size_t smem = stage_smem_bytes<STAGE == 1 ? 40 : 20>();
-    auto kern = k_stage<STAGE, PRF>;
+    auto kern = k_stage<STAGE, VISC>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     int dev = 0, nsm = 0, per_sm = 0;
@@ -182,19 +182,7 @@ static cudaError_t launch_stage_kernel(const DevMesh<float>& m, const Phys<float
 cudaError_t launch_stage(const DevMesh<float>& m, const HostPhys& p, const DevState<float>& st, int stage,
                          const Launch<float>::Finalize* fin, unsigned* gbar, cudaStream_t s) {
     if (m.nc == 0) return cudaSuccess;
-    Phys<float> ph;
-    ph.gamma = (float)p.gamma;
-    ph.gm1 = (float)(p.gamma - 1.0);
-    ph.K = (float)((5.0 - 3.0 * p.gamma) / (p.gamma - 1.0));
-    ph.tau_eps = (float)p.tau_eps;
-    ph.tau_c = (float)p.tau_c;
-    ph.mu = (float)p.mu;
-    ph.eps_w = (float)p.eps_weno;
-    ph.viscous = p.viscous;
-    ph.smooth = p.smooth;
-    ph.prf = (float)p.prf;
-    ph.twall = (float)p.twall;
-    for (int i = 0; i < 3; ++i) ph.uwall[i] = (float)p.uwall[i];
+    const Phys<float> ph = make_phys<float>(p);
     ReconConst<float> rc;
     rc.gm1 = (float)(p.gamma - 1.0);
     rc.eps = (float)p.eps_weno;
@@ -209,12 +197,11 @@ cudaError_t launch_stage(const DevMesh<float>& m, const HostPhys& p, const DevSt
         fa.cfl = fin->cfl;
         fa.ctrl = fin->ctrl;
     }
-    const bool prf = p.prf != 0.0;
     if (stage == 1)
-        return prf ? launch_stage_kernel<1, true>(m, ph, p, rc, st, fa, gbar, s)
-                   : launch_stage_kernel<1, false>(m, ph, p, rc, st, fa, gbar, s);
-    return prf ? launch_stage_kernel<2, true>(m, ph, p, rc, st, fa, gbar, s)
-               : launch_stage_kernel<2, false>(m, ph, p, rc, st, fa, gbar, s);
+        return p.viscous ? launch_stage_kernel<1, true>(m, ph, p, rc, st, fa, gbar, s)
+                         : launch_stage_kernel<1, false>(m, ph, p, rc, st, fa, gbar, s);
+    return p.viscous ? launch_stage_kernel<2, true>(m, ph, p, rc, st, fa, gbar, s)
+                     : launch_stage_kernel<2, false>(m, ph, p, rc, st, fa, gbar, s);
 }
 
 }  // namespace gks

@@ -62,11 +62,13 @@ __device__ __forceinline__ void update1_cells(const DevMesh<T>& m, const HostPhy
     fh.init();
     s1.init();
     T gs[3] = {T(0), T(0), T(0)}, g0[3] = {T(0), T(0), T(0)};
-    constexpr int RS = sizeof(T) == 4 ? REC1_F32 : 40;
+    constexpr int RS = rec_stride<T, 40>();
+#pragma unroll
     for (int f = 0; f < 4; ++f) {
         const int e = m.cface[f * nc + c];
         const T s = (e & 1) ? T(-1) : T(1);
         const T* r = st.rec + (int64_t)(e >> 1) * RS;
+        const T* n = m.fgeo + (int64_t)(e >> 1) * FGEO;
         fh.add(s * r[q]);
         s1.add(s * r[5 + q]);
         if constexpr (sizeof(T) == 4) {
@@ -77,10 +79,11 @@ __device__ __forceinline__ void update1_cells(const DevMesh<T>& m, const HostPhy
             s1.add(T(2) * s * r[REC1_REF + q]);
             s1.add(T(2) * s * r[REC1_REF + 5 + q]);
         }
+        const T ws = s * r[10 + q], w0 = s * r[15 + q];
 #pragma unroll
         for (int i = 0; i < 3; ++i) {
-            gs[i] += s * r[10 + 3 * q + i];
-            g0[i] += s * r[25 + 3 * q + i];
+            gs[i] += ws * n[i];
+            g0[i] += w0 * n[i];
         }
     }
     const double iv = m.inv_vol[c];
@@ -175,10 +178,12 @@ __device__ __forceinline__ void update2_cells(const DevMesh<T>& m, const HostPhy
     for (int f = 0; f < 4; ++f) {
         const int e = m.cface[f * nc + c];
         const T s = (e & 1) ? T(-1) : T(1);
-        const T* r = st.rec + (int64_t)(e >> 1) * 20;
+        const T* r = st.rec + (int64_t)(e >> 1) * rec_stride<T, 20>();
+        const T* n = m.fgeo + (int64_t)(e >> 1) * FGEO;
         f2.add(s * r[q]);
+        const T dw = s * r[5 + q];
 #pragma unroll
-        for (int i = 0; i < 3; ++i) dg[i] += s * r[5 + 3 * q + i];
+        for (int i = 0; i < 3; ++i) dg[i] += dw * n[i];
     }
     const double iv = m.inv_vol[c];
     // W^{n+1} |Omega| = W^n |Omega| - [dt F + dt^2/6 F_t](W^n) - [dt^2/3 F_t](W*)
