@@ -188,8 +188,7 @@ __device__ __forceinline__ void adj_point_setup(const DevMesh<double>& m, const 
             // a real side, or a wall side from the interior cell at the point
             const int src_side = cell >= 0 ? side : 1 - side;
             const int64_t c = cell >= 0 ? cell : in;
-            const double X[3] = {geo[4 + 9 * src_side + 3 * k], geo[5 + 9 * src_side + 3 * k],
-                                 geo[6 + 9 * src_side + 3 * k]};
+            const double X[3] = {geo[4 + 9 * src_side + 3 * k], geo[5 + 9 * src_side + 3 * k], geo[6 + 9 * src_side + 3 * k]};
             eval_poly(poly + c * POLY_STRIDE, X, Wv, g);
             to_local(Rm, Wv, g, xs, gs);
             if (cell == FLR_SLIP_WALL) slip_wall_ghost(xs, gs);
@@ -308,8 +307,7 @@ __global__ void k_adj_face_back(DevMesh<double> m, const double* __restrict__ lx
                 // the interior state at the point, face frame, then the ghost's transpose
                 const int src_side = 1 - side;
                 const int64_t c = side == 0 ? R : L;
-                const double X[3] = {geo[4 + 9 * src_side + 3 * k], geo[5 + 9 * src_side + 3 * k],
-                                     geo[6 + 9 * src_side + 3 * k]};
+                const double X[3] = {geo[4 + 9 * src_side + 3 * k], geo[5 + 9 * src_side + 3 * k], geo[6 + 9 * src_side + 3 * k]};
                 double Wv[5], g[3][5], x[20];
                 eval_poly(poly + c * POLY_STRIDE, X, Wv, g);
                 to_local(Rm, Wv, g, x, reinterpret_cast<double (*)[5]>(x + 5));

@@ -283,7 +283,7 @@ struct Layout {
     size_t total = 0;
     int64_t nwall = 0;  // slots of wall-constrained operators
     // mesh
-    size_t nbr, cface, inv_vol, dr, M1, tile, flr, fgeo, fan, cell_case, perm;
+    size_t nbr, cface, inv_vol, dr, M1, tile, flr, fgeo, fnw, fan, cell_case, perm;
     // state
     size_t Wd, X, Xs, X0, S, G, slopes, poly, rec, ctrl, case_t, case_dt, case_dtmin, part, err, stage, cperm, cinv,
         gbar, wslot, wop;
@@ -325,6 +325,7 @@ Layout layout_workspace(int64_t nc, int64_t nf, int64_t ncase, bool fp32, bool f
     L.tile = L.add(TO * TILE_ROWS * CELLS_PER_BLOCK * nblk);
     L.flr = L.add(4 * 2 * nf);
     L.fgeo = L.add(T * FGEO * nf);
+    L.fnw = L.add(T * 4 * nf);
     L.fan = fp32 ? L.add(4 * 6 * nf) : 0;  // FP32 bulk: face area vectors A n as FP32 hi / lo pairs
     L.cell_case = L.add(4 * nc);
     L.perm = L.add(4 * nf);
@@ -528,6 +529,7 @@ static void make_views(gks_state* s, DevMesh<T>& m, DevState<T>& st) {
     }
     m.flr = at<int32_t>(s, L.flr);
     m.fgeo = at<T>(s, L.fgeo);
+    m.fnw = at<T>(s, L.fnw);
     m.fan = L.fan ? at<float>(s, L.fan) : nullptr;
     m.fixed = L.X0 ? at<T>(s, L.X0) : nullptr;
     m.wslot = L.wslot ? at<int32_t>(s, L.wslot) : nullptr;
@@ -578,7 +580,7 @@ static gks_status upload_faces(gks_state* s) {
     std::vector<int32_t> inv((size_t)nf);
     for (int64_t d = 0; d < nf; ++d) inv[perm[d]] = (int32_t)d;
     std::vector<int32_t> cface(4 * nc), flr(2 * nf);
-    std::vector<T> fgeo(FGEO * nf, T(0));
+    std::vector<T> fgeo(FGEO * nf, T(0)), fnw(4 * nf);
     std::vector<float> fan(s->L.fan ? 6 * nf : 0, 0.0f);
     for (int64_t d = 0; d < nc; ++d) {
         const int64_t c = s->pub(d);
@@ -597,6 +599,7 @@ static gks_status upload_faces(gks_state* s) {
         T* r = &fgeo[d * FGEO];
         for (int a = 0; a < 3; ++a) r[a] = (T)g.fnorm[f * 3 + a];
         r[3] = (T)(g.farea[f] / 3.0);
+        for (int a = 0; a < 4; ++a) fnw[d * 4 + a] = r[a];
         for (int k = 0; k < 9; ++k) {
             r[4 + k] = (T)g.gp_l[f * 9 + k];
             r[13 + k] = (T)g.gp_r[f * 9 + k];
@@ -614,6 +617,7 @@ static gks_status upload_faces(gks_state* s) {
     GKS_CHECK_CUDA(put(L.cface, cface.data(), 4 * cface.size()));
     GKS_CHECK_CUDA(put(L.flr, flr.data(), 4 * flr.size()));
     GKS_CHECK_CUDA(put(L.fgeo, fgeo.data(), sizeof(T) * fgeo.size()));
+    GKS_CHECK_CUDA(put(L.fnw, fnw.data(), sizeof(T) * fnw.size()));
     if (!fan.empty()) GKS_CHECK_CUDA(put(L.fan, fan.data(), 4 * fan.size()));
     GKS_CHECK_CUDA(put(L.perm, perm.data(), 4 * perm.size()));
     GKS_CHECK_CUDA(cudaStreamSynchronize(s->stream));  // host vectors die here

@@ -16,19 +16,41 @@ __device__ __forceinline__ void group_barrier(int id, int count) {
         asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(count) : "memory");
 }
 
-// A group of CELL_THREADS threads on one block of cells: the block index
-// vb, the thread's index tid in the group, the group's barrier (named id,
-// 0 the whole thread block) and its slice of shared memory for the block
-// reductions.
-struct CellGroup {
-    int64_t vb;
-    int tid;
-    int bar_id;
-    double* sv;   // [CELLS_PER_BLOCK]
-    int32_t* sc;  // [CELLS_PER_BLOCK]
-    double* red;  // [CELL_THREADS / 32][6]
-    __device__ __forceinline__ void sync() const { group_barrier(bar_id, CELL_THREADS); }
-};
+// N values (N a multiple of the vector's length) from 16-byte aligned memory
+template <int N, typename T>
+__device__ __forceinline__ void load_vec(const T* __restrict__ p, T* v) {
+    if constexpr (sizeof(T) == 4) {
+        static_assert(N % 4 == 0, "whole vectors");
+#pragma unroll
+        for (int i = 0; i < N / 4; ++i) {
+            const float4 x = reinterpret_cast<const float4*>(p)[i];
+            v[4 * i] = x.x;
+            v[4 * i + 1] = x.y;
+            v[4 * i + 2] = x.z;
+            v[4 * i + 3] = x.w;
+        }
+    } else {
+        static_assert(N % 2 == 0, "whole vectors");
+#pragma unroll
+        for (int i = 0; i < N / 2; ++i) {
+            const double2 x = reinterpret_cast<const double2*>(p)[i];
+            v[2 * i] = x.x;
+            v[2 * i + 1] = x.y;
+        }
+    }
+}
+
+template <int N, typename T>
+__device__ __forceinline__ void store_vec(T* __restrict__ p, const T* v) {
+    if constexpr (sizeof(T) == 4) {
+#pragma unroll
+        for (int i = 0; i < N / 4; ++i)
+            reinterpret_cast<float4*>(p)[i] = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
+    } else {
+#pragma unroll
+        for (int i = 0; i < N / 2; ++i) reinterpret_cast<double2*>(p)[i] = make_double2(v[2 * i], v[2 * i + 1]);
+    }
+}
 
 // 5 lanes per cell (one per conservative component), 6 cells per warp (lanes
 // 30, 31 idle), CELLS_PER_BLOCK cells per 128-thread block

@@ -35,6 +35,52 @@ __device__ __forceinline__ float d_cbrt(float x) { return cbrtf(x); }
 template <typename T>
 __device__ __forceinline__ T pow43(T x) { return x * d_cbrt(x); }
 
+// FP32 <-> FP64 conversions on the integer pipe.  The FP64 unit (which also
+// takes the conversion instructions) issues a warp instruction in 16 cycles,
+// the integer unit in half a cycle, and the cell updates convert more than
+// they add.  Same values as the conversions: widening is exact, narrowing
+// rounds to nearest even; numbers outside the range the bit forms cover
+// (zeros apart) take the conversion instruction.
+// The conversion instructions stand in functions of their own: inlined, the
+// compiler would compute both forms and select.
+__device__ __noinline__ static double widen_any(float x) { return (double)x; }
+__device__ __noinline__ static float narrow_any(double x) { return (float)x; }
+
+__device__ __forceinline__ double widen(float x) {
+    const uint32_t b = __float_as_uint(x), m = b & 0x7fffffffu;
+    if (m - 0x00800000u >= 0x7f000000u && m != 0u) return widen_any(x);  // denormal, infinite, NaN
+    const uint32_t hi = m != 0u ? (m >> 3) + (896u << 20) : 0u;
+    return __hiloint2double((int)((b & 0x80000000u) | hi), (int)(m << 29));
+}
+__device__ __forceinline__ double widen(double x) { return x; }
+
+// x = hi + lo + (below half an ulp of lo): hi = x and lo = x - hi, each
+// rounded to nearest
+__device__ __forceinline__ void split_pair(double x, float& hi, float& lo) {
+    const uint64_t b = (uint64_t)__double_as_longlong(x);
+    const uint32_t e = (uint32_t)(b >> 52) & 0x7ffu;
+    if (e - 963u > 120u && (b << 1) != 0u) {  // not within 2^-60 .. 2^61
+        hi = narrow_any(x);
+        lo = narrow_any(x - widen_any(hi));
+        return;
+    }
+    const uint64_t m = b & 0x7fffffffffffffffull;
+    const uint64_t r = (m + 0x0fffffffull + ((m >> 29) & 1u)) >> 29;  // rounded to 23 fraction bits
+    const uint32_t sign = (uint32_t)(b >> 32) & 0x80000000u;
+    const int32_t rest = (int32_t)((uint32_t)m - (uint32_t)(r << 29));  // |rest| <= 2^28 units of 2^(e - 1075)
+    const bool zero = m == 0u;
+    hi = __uint_as_float(zero ? sign : sign | ((uint32_t)r - (896u << 23)));
+    const float scale = __uint_as_float(sign | ((e - 948u) << 23));
+    lo = zero ? 0.0f : (float)rest * scale;
+}
+__device__ __forceinline__ float narrow(double x) {
+    const uint64_t b = (uint64_t)__double_as_longlong(x), m = b & 0x7fffffffffffffffull;
+    const uint32_t e = (uint32_t)(m >> 52), sign = (uint32_t)(b >> 32) & 0x80000000u;
+    if (e - 897u > 252u && m != 0u) return narrow_any(x);  // not within 2^-126 .. 2^127
+    const uint64_t r = (m + 0x0fffffffull + ((m >> 29) & 1u)) >> 29;
+    return __uint_as_float(m == 0u ? sign : sign | ((uint32_t)r - (896u << 23)));
+}
+
 // Error-free transformation of a sum (Knuth's TwoSum): a + b = s + e exactly.
 template <typename T>
 __device__ __forceinline__ void two_sum(T a, T b, T& s, T& e) {
@@ -54,7 +100,7 @@ struct CSum {
         hi = s;
         lo += e;
     }
-    __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
+    __device__ __forceinline__ double value() const { return widen(hi) + widen(lo); }
 };
 
 // ------------------------------------------------------------ params --

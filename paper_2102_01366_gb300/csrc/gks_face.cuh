@@ -234,7 +234,7 @@ __device__ __forceinline__ void fixed_ghost(const T* __restrict__ x0, const T* X
         T v = x0[q];
 #pragma unroll
         for (int i = 0; i < 3; ++i) {
-            g[i][q] = x0[5 + 3 * q + i];
+            g[i][q] = x0[Stride<T>::xg + 3 * q + i];
             v += g[i][q] * X[i];
         }
         W[q] = v;

@@ -236,7 +236,6 @@ __device__ __forceinline__ void flux_faces(const DevMesh<T>& m, const Phys<T>& p
     if (f >= m.nf) return;
     constexpr int RS = rec_stride<T, NR>();
     T* r = rec + f * RS;
-    const T* geo = m.fgeo + f * FGEO;
     if (job == 2) {
         if constexpr (REL) {
             const int L = m.flr[f], Rc = m.flr[m.nf + f];
@@ -245,14 +244,15 @@ __device__ __forceinline__ void flux_faces(const DevMesh<T>& m, const Phys<T>& p
         }
         return;
     }
-    T Rm[3][3];
+    T Rm[3][3], n[4];
+    load_vec<4>(m.fgeo + f * FGEO, n);
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
-        Rm[0][i] = geo[i];
+        Rm[0][i] = n[i];
         Rm[1][i] = sm.frame[lf][i];
         Rm[2][i] = sm.frame[lf][3 + i];
     }
-    const T w = geo[3];
+    const T w = n[3];
     auto sum = [&](int at, T* v) {
 #pragma unroll
         for (int q = 0; q < 5; ++q)

@@ -21,57 +21,50 @@
 
 namespace gks {
 
+constexpr int DT_THREADS = 128;    // threads (cells) a block of k_init_dtmin
+constexpr int PACK_THREADS = 128;  // threads (cells) a block of k_pack, k_unpack_grad
 
 template <typename T>
-__global__ void __launch_bounds__(CELL_THREADS) k_update1(DevMesh<T> m, HostPhys p, DevState<T> st) {
-    update1_cells<T>(m, p, st, blockIdx.x, threadIdx.x);
-}
-
-// the block's own slice of shared memory for a whole-block cell group
-#define GKS_BLOCK_GROUP(name)                                        \
-    __shared__ double name##_sv[CELLS_PER_BLOCK];                    \
-    __shared__ int32_t name##_sc[CELLS_PER_BLOCK];                   \
-    __shared__ double name##_red[CELL_THREADS / 32 * 6];             \
-    const CellGroup name{(int64_t)blockIdx.x, (int)threadIdx.x, 0, name##_sv, name##_sc, name##_red}
-
-template <typename T>
-__global__ void __launch_bounds__(CELL_THREADS) k_update2(DevMesh<T> m, HostPhys p, DevState<T> st) {
-    GKS_BLOCK_GROUP(grp);
-    update2_cells<T>(m, p, st, grp);
+__global__ void __launch_bounds__(CELL_THREADS) k_update1(DevMesh<T> m, DevState<T> st) {
+    update1_cells<T>(m, st, blockIdx.x, threadIdx.x);
 }
 
 template <typename T>
-__global__ void __launch_bounds__(CELL_THREADS) k_dt_partials(DevMesh<T> m, HostPhys p,
-                                                               const T* __restrict__ X,
-                                                               double* __restrict__ part) {
-    const CellLane cl = cell_lane(m.nc);
+__global__ void __launch_bounds__(CELL_THREADS) k_update2(DevMesh<T> m, DtPhys<T> p, DevState<T> st) {
+    __shared__ T red[CELL_THREADS / 32][5];
+    update2_cells<T>(m, p, st, blockIdx.x, threadIdx.x, 0, red);
+}
+
+// local limit of one cell from the averages in X, one thread per cell
+template <typename T>
+__device__ __forceinline__ T cell_dt(const DevMesh<T>& m, const DtPhys<T>& p, const T* __restrict__ X, int64_t c) {
+    T Wv[5];
+#pragma unroll
+    for (int q = 0; q < 5; ++q) Wv[q] = X[c * Stride<T>::xs + q];
+    return local_dt(Wv, m.dr[c], p);
+}
+
+// block b: the minimum over its CELLS_PER_BLOCK cells (one warp of the block
+// size that update_blocks counts)
+template <typename T>
+__global__ void __launch_bounds__(32) k_dt_partials(DevMesh<T> m, DtPhys<T> p, const T* __restrict__ X,
+                                                    double* __restrict__ part) {
+    const int64_t c = (int64_t)blockIdx.x * CELLS_PER_BLOCK + threadIdx.x;
     T mn = T(INFINITY);
-    T zero[5] = {T(0), T(0), T(0), T(0), T(0)};
-    if (cl.active && cl.q == 0) {
-        T Wv[5];
-#pragma unroll
-        for (int q = 0; q < 5; ++q) Wv[q] = X[cl.c * Stride<T>::xs + q];
-        mn = local_dt(Wv, m.dr[cl.c], p);
-    }
-    GKS_BLOCK_GROUP(grp);
-    block_reduce_part<T>(mn, zero, part + (int64_t)blockIdx.x * PART_N, grp);
+    if (threadIdx.x < CELLS_PER_BLOCK && c < m.nc) mn = cell_dt(m, p, X, c);
+    if (!(mn < T(INFINITY))) mn = T(INFINITY);
+    mn = warp_min(mn);
+    if (threadIdx.x == 0) part[(int64_t)blockIdx.x * PART_N + PART_DTMIN] = (double)mn;
 }
 
 template <typename T>
-__global__ void __launch_bounds__(CELL_THREADS) k_init_dtmin(DevMesh<T> m, HostPhys p, const T* __restrict__ X,
-                                                              unsigned long long* __restrict__ dtmin) {
-    const CellLane cl = cell_lane(m.nc);
-    const bool lead = cl.active && cl.q == 0;
-    double mn = INFINITY;
-    if (lead) {
-        T Wv[5];
-#pragma unroll
-        for (int q = 0; q < 5; ++q) Wv[q] = X[cl.c * Stride<T>::xs + q];
-        mn = (double)local_dt(Wv, m.dr[cl.c], p);
-    }
-    const int lc = (int)(cl.c - (int64_t)blockIdx.x * CELLS_PER_BLOCK);
-    GKS_BLOCK_GROUP(grp);
-    block_case_min(mn, m.cell_case[cl.c], lead && lc >= 0 && lc < CELLS_PER_BLOCK && mn < INFINITY, lc, dtmin, grp);
+__global__ void __launch_bounds__(DT_THREADS) k_init_dtmin(DevMesh<T> m, DtPhys<T> p, const T* __restrict__ X,
+                                                           unsigned long long* __restrict__ dtmin) {
+    const int64_t c0 = (int64_t)blockIdx.x * DT_THREADS + threadIdx.x;
+    const int64_t c = c0 < m.nc ? c0 : m.nc - 1;
+    T mn = T(INFINITY);
+    if (c0 < m.nc) mn = cell_dt(m, p, X, c);
+    warp_case_min(mn, m.cell_case[c], dtmin);
 }
 
 __global__ void k_set_control(double* ctrl, double* case_t, double* case_dt, unsigned long long* dtmin,
@@ -94,35 +87,52 @@ __global__ void k_convert(const A* __restrict__ in, B* __restrict__ out, int64_t
         out[i] = (B)in[i];
 }
 
-// cperm (may be NULL): device cell -> the caller's cell of W, dW
+// One thread per cell: rows of the caller's [component][cell] arrays are read
+// (written) in full lines, records as 16-byte vectors.  cperm (may be NULL):
+// device cell -> the caller's cell of W, dW.  Bound by memory: with one thread
+// per word of the record, each reading another row, an initialisation and a
+// read-back of 1.57 M cells in FP32 took about 1.17 ms, now 0.40 ms.
 template <typename T>
-__global__ void k_pack(const double* __restrict__ W, const double* __restrict__ dW, T* __restrict__ X, int64_t nc,
-                       const int32_t* __restrict__ cperm) {
+__global__ void __launch_bounds__(PACK_THREADS) k_pack(const double* __restrict__ W, const double* __restrict__ dW,
+                                                       T* __restrict__ X, int64_t nc,
+                                                       const int32_t* __restrict__ cperm) {
     constexpr int XSR = Stride<T>::xs;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nc * XSR; i += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t d = i / XSR;
-        const int64_t c = cperm ? (int64_t)cperm[d] : d;
-        const int j = (int)(i - d * XSR);
-        T v = T(0);
-        if (j < 5) {
-            v = (T)W[j * nc + c];
-        } else if (j < 20) {
-            v = (T)dW[(j - 5) * nc + c];
-        } else if (sizeof(T) == 4 && j < XLO + 5) {
-            const double w = W[(j - XLO) * nc + c];
-            v = (T)(w - (double)(T)w);  // lo part of the FP32 pair
-        }
-        X[i] = v;
+    const int64_t d = (int64_t)blockIdx.x * PACK_THREADS + threadIdx.x;
+    if (d >= nc) return;
+    const int64_t c = cperm ? (int64_t)cperm[d] : d;
+    T x[XSR];
+#pragma unroll
+    for (int j = 0; j < XSR; ++j) x[j] = T(0);
+#pragma unroll
+    for (int q = 0; q < 5; ++q) {
+        const double w = W[q * nc + c];
+        if constexpr (sizeof(T) == 4)
+            split_pair(w, x[q], x[XLO + q]);
+        else
+            x[q] = w;
     }
+#pragma unroll
+    for (int j = 0; j < 15; ++j) {
+        if constexpr (sizeof(T) == 4)
+            x[Stride<T>::xg + j] = narrow(dW[j * nc + c]);
+        else
+            x[Stride<T>::xg + j] = dW[j * nc + c];
+    }
+    store_vec<XSR>(X + d * XSR, x);
 }
 
 template <typename T>
-__global__ void k_unpack_grad(const T* __restrict__ X, double* __restrict__ dW, int64_t nc,
-                              const int32_t* __restrict__ cperm) {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nc * 15; i += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t j = i / nc, d = i - j * nc;
-        dW[j * nc + (cperm ? (int64_t)cperm[d] : d)] = (double)X[d * Stride<T>::xs + 5 + j];
-    }
+__global__ void __launch_bounds__(PACK_THREADS) k_unpack_grad(const T* __restrict__ X, double* __restrict__ dW,
+                                                              int64_t nc, const int32_t* __restrict__ cperm) {
+    constexpr int XSR = Stride<T>::xs;
+    const int64_t d = (int64_t)blockIdx.x * PACK_THREADS + threadIdx.x;
+    if (d >= nc) return;
+    const int64_t c = cperm ? (int64_t)cperm[d] : d;
+    constexpr int A = sizeof(T) == 4 ? 12 : 4;  // the aligned start of the gradients' vectors
+    T x[XSR - A];
+    load_vec<XSR - A>(X + d * XSR + A, x);
+#pragma unroll
+    for (int j = 0; j < 15; ++j) dW[j * nc + c] = widen(x[Stride<T>::xg - A + j]);
 }
 
 // the averages of an FP64 working state [nc][XS] to W [5][nc]
@@ -176,7 +186,7 @@ __global__ void k_rec_out(const T* __restrict__ rec, const int32_t* __restrict__
         const int je = j - nflux;
         double v = j < nflux ? (double)r[j]
                              : (double)r[nflux + (je / 15) * 5 + (je % 15) / 3] *
-                                   (double)m.fgeo[d * FGEO + (je % 15) % 3];
+                                   (double)m.fnw[d * 4 + (je % 15) % 3];
         if (sizeof(T) == 4 && nr == 40 && j < 10) {
             // the reference flux (dt / 2) A F_n(W_m), twice in the S entries
             const double ref = (double)r[REC1_REF + j % 5] + (double)r[REC1_REF + 5 + j % 5];
@@ -189,8 +199,8 @@ __global__ void k_rec_out(const T* __restrict__ rec, const int32_t* __restrict__
             const int L = m.flr[d], R = m.flr[m.nf + d];
             auto avg = [&](int c) { return (double)X[(int64_t)c * XSR + q] + (double)X[(int64_t)c * XSR + XLO + q]; };
             const double wm = (L >= 0 && R >= 0) ? 0.5 * (avg(L) + avg(R)) : avg(L >= 0 ? L : R);
-            const T* geo = m.fgeo + d * FGEO;
-            v += wm * 3.0 * (double)geo[3] * (double)geo[dir];
+            const T* nw = m.fnw + d * 4;
+            v += wm * 3.0 * (double)nw[3] * (double)nw[dir];
         }
         out[(int64_t)perm[d] * nr + j] = v;
     }
@@ -222,7 +232,7 @@ int update_blocks(int64_t nc) { return (int)cell_grid(nc); }
 template <typename T>
 cudaError_t Launch<T>::update1(const DevMesh<T>& m, const HostPhys& p, const DevState<T>& st, cudaStream_t s) {
     if (m.nc == 0) return cudaSuccess;
-    k_update1<T><<<cell_grid(m.nc), CELL_THREADS, 0, s>>>(m, p, st);
+    k_update1<T><<<cell_grid(m.nc), CELL_THREADS, 0, s>>>(m, st);
     return cudaGetLastError();
 }
 
@@ -230,7 +240,7 @@ template <typename T>
 cudaError_t Launch<T>::update2(const DevMesh<T>& m, const HostPhys& p, const DevState<T>& st,
                                cudaStream_t s) {
     if (m.nc == 0) return cudaSuccess;
-    k_update2<T><<<cell_grid(m.nc), CELL_THREADS, 0, s>>>(m, p, st);
+    k_update2<T><<<cell_grid(m.nc), CELL_THREADS, 0, s>>>(m, DtPhys<T>(p), st);
     return cudaGetLastError();
 }
 
@@ -238,7 +248,7 @@ template <typename T>
 cudaError_t Launch<T>::dt_partials(const DevMesh<T>& m, const HostPhys& p, const T* X,
                                    double* part, cudaStream_t s) {
     if (m.nc == 0) return cudaSuccess;
-    k_dt_partials<T><<<cell_grid(m.nc), CELL_THREADS, 0, s>>>(m, p, X, part);
+    k_dt_partials<T><<<cell_grid(m.nc), 32, 0, s>>>(m, DtPhys<T>(p), X, part);
     return cudaGetLastError();
 }
 
@@ -246,9 +256,11 @@ template <typename T>
 cudaError_t Launch<T>::init_dtmin(const DevMesh<T>& m, const HostPhys& p, const T* X,
                                   unsigned long long* case_dtmin, cudaStream_t s) {
     if (m.nc == 0) return cudaSuccess;
-    k_init_dtmin<T><<<cell_grid(m.nc), CELL_THREADS, 0, s>>>(m, p, X, case_dtmin);
+    k_init_dtmin<T><<<(unsigned)((m.nc + DT_THREADS - 1) / DT_THREADS), DT_THREADS, 0, s>>>(m, DtPhys<T>(p), X, case_dtmin);
     return cudaGetLastError();
 }
+
+static inline unsigned pack_grid(int64_t nc) { return (unsigned)((nc + PACK_THREADS - 1) / PACK_THREADS); }
 
 static inline unsigned ew_grid(int64_t n) { return (unsigned)((n + 255) / 256 < 8192 ? (n + 255) / 256 : 8192); }
 
@@ -256,14 +268,14 @@ template <typename T>
 cudaError_t Launch<T>::pack(const double* W, const double* dW, T* X, int64_t nc, cudaStream_t s,
                             const int32_t* cperm) {
     if (nc == 0) return cudaSuccess;
-    k_pack<T><<<ew_grid(nc * Stride<T>::xs), 256, 0, s>>>(W, dW, X, nc, cperm);
+    k_pack<T><<<pack_grid(nc), PACK_THREADS, 0, s>>>(W, dW, X, nc, cperm);
     return cudaGetLastError();
 }
 
 template <typename T>
 cudaError_t Launch<T>::unpack_grad(const T* X, double* dW, int64_t nc, cudaStream_t s, const int32_t* cperm) {
     if (nc == 0) return cudaSuccess;
-    k_unpack_grad<T><<<ew_grid(nc * 15), 256, 0, s>>>(X, dW, nc, cperm);
+    k_unpack_grad<T><<<pack_grid(nc), PACK_THREADS, 0, s>>>(X, dW, nc, cperm);
     return cudaGetLastError();
 }
 

@@ -23,11 +23,14 @@ constexpr int XS = 20;               // reals per cell working-state record, FP6
 // FP32 bulk keeps each cell average as an unevaluated pair hi + lo of FP32
 // numbers (the FP64 average to ~48 bits), so that differences between
 // neighbouring averages stay exact to FP32 rounding of the difference:
-//   working state [nc][28]: W hi (5), grad W (15), W lo (5), pad (3)
+//   working state [nc][28]: W hi (5), W lo (5), pad (2), grad W (15), pad (1):
+//   the averages, which most gathers of a neighbour want alone, are three
+//   16-byte vectors, the gradients four
 //   reconstruction record [nc][60]: per component the constant R(centroid)
 //   minus the average and the 9 slopes/curvatures (50), the average's hi (5)
 //   and lo (5) parts
 constexpr int XS32 = 28;
+constexpr int XLO = 5;               // offset of the lo parts in an FP32 working-state record
 // Face records, sums over the face's Gauss points with their weights w:
 //   stage 1  sum w Fh (5), sum w (2 Fh - D / 3) (5), sum w W(t*) (5),
 //            sum w W(0) (5); FP32: the flux and interface-state entries are
@@ -44,12 +47,12 @@ template <typename T, int NR>
 constexpr int rec_stride() {
     return NR == 20 ? 10 : sizeof(T) == 4 ? 32 : 20;
 }
-constexpr int XLO = 20;              // offset of the lo parts in an FP32 working-state record
 constexpr int POLY_STRIDE32 = 60;
 constexpr int PHI = 50, PLO = 55;    // offsets of the average's hi / lo parts in an FP32 record
 template <typename T>
 struct Stride {
     static constexpr int xs = sizeof(T) == 4 ? XS32 : XS;
+    static constexpr int xg = sizeof(T) == 4 ? 12 : 5;  // offset of grad W (row 3 q + i) in it
     static constexpr int poly = sizeof(T) == 4 ? POLY_STRIDE32 : POLY_STRIDE;
 };
 // Per-block tile of the reconstruction's static cell data, one contiguous
@@ -79,6 +82,7 @@ struct DevMesh {
     const double* tiled;
     const int32_t* flr;    // [2][nf]
     const T* fgeo;         // [nf][FGEO]: n(3), w, XL(9), XR(9), pad
+    const T* fnw;          // [nf][4]: n(3), w once more, apart from the rest for the updates
     const float* fan;      // FP32 bulk: [nf][6] face area vectors A n as FP32 hi / lo pairs (NULL in FP64)
     const T* fixed;        // [nc][Stride<T>::xs] state held by fixed boundary faces (NULL: none)
     // Sec. 4.4 wall-constrained momentum stencils (NULL: none): slot of each
@@ -95,8 +99,8 @@ struct DevState {
     double* Wd;   // [5][nc] master cell averages (FP64)
     T* X;         // [nc][Stride<T>::xs] working state W^n, grad W^n (cell-major for neighbour gathers)
     T* Xs;        // [nc][Stride<T>::xs] stage state W*, grad W*
-    double* S;    // [5][nc] saved stage-1 flux term
-    T* G;         // [15][nc] saved stage-1 gradient term
+    double* S;    // [nc][5] saved stage-1 flux term
+    T* G;         // [nc][15] saved stage-1 gradient term
     T* slopes;    // [nc][15]
     T* poly;      // [nc][Stride<T>::poly]
     T* rec;       // [nf][rec_stride]
@@ -178,18 +182,25 @@ struct Launch {
 
 // Local time-step limit of one cell (Sec. 5, Eq. time-step, without C_CFL):
 // dr / (|U| + a), and dr^2 / (3 nu) if viscous, from its averages Wv[5],
-// in the working precision T.
+// in the working precision T.  The constants are rounded to T on the host:
+// done in the kernel, each costs every warp FP64 instructions.
+template <typename T>
+struct DtPhys {
+    T gamma, gm1, mu3;  // mu3 = 3 mu (0: inviscid)
+    explicit DtPhys(const HostPhys& p)
+        : gamma((T)p.gamma), gm1((T)(p.gamma - 1.0)), mu3((T)(p.viscous && p.mu > 0.0 ? 3.0 * p.mu : 0.0)) {}
+};
 #ifdef __CUDACC__
 template <typename T>
-__device__ __forceinline__ T local_dt(const T* Wv, T dr, const HostPhys& p) {
+__device__ __forceinline__ T local_dt(const T* Wv, T dr, const DtPhys<T>& p) {
     const T ir = T(1) / Wv[0];
     const T u = Wv[1] * ir, v = Wv[2] * ir, w = Wv[3] * ir;
     const T q = u * u + v * v + w * w;
-    const T pr = T(p.gamma - 1.0) * (Wv[4] - T(0.5) * Wv[0] * q);
-    const T a = sqrt(T(p.gamma) * pr * ir);
+    const T pr = p.gm1 * (Wv[4] - T(0.5) * Wv[0] * q);
+    const T a = sqrt(p.gamma * pr * ir);
     T d = dr / (sqrt(q) + a);
-    if (p.viscous && p.mu > 0.0) {
-        const T dv = dr * dr * Wv[0] / (T(3.0 * p.mu));
+    if (p.mu3 > T(0)) {
+        const T dv = dr * dr * Wv[0] / p.mu3;
         d = d < dv ? d : dv;
     }
     return d;
@@ -244,6 +255,6 @@ cudaError_t adjoint_reverse(const DevMesh<double>& m, const HostPhys& p, double 
 cudaError_t launch_set_control(double* ctrl, double* case_t, double* case_dt,
                                unsigned long long* case_dtmin, int32_t ncase, double dt_fixed,
                                double t_end, int reset_time, cudaStream_t s);
-int update_blocks(int64_t nc);
+int update_blocks(int64_t nc);  // blocks of CELLS_PER_BLOCK cells
 
 }  // namespace gks

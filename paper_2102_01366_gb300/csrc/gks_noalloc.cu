@@ -37,7 +37,7 @@ __device__ __align__(256) double g_dt_partials[NA_MAX_BLOCKS];
 // the same local limit and reduction order as the workspace version
 __global__ void __launch_bounds__(NA_THREADS) k_na_partials(const double* __restrict__ W,
                                                            const double* __restrict__ dr, int64_t nc,
-                                                           HostPhys p, double* __restrict__ part) {
+                                                           DtPhys<double> p, double* __restrict__ part) {
     __shared__ double smin[NA_THREADS];
     const int64_t c = (int64_t)blockIdx.x * NA_THREADS + threadIdx.x;
     double mn = INFINITY;
@@ -123,7 +123,7 @@ extern "C" gks_status gks_timestep_noalloc(const gks_params* p, const double* d_
                 p->weno, p->order, p->smooth_flux, p->viscous};
     const int nblk = (int)((n_cell + NA_THREADS - 1) / NA_THREADS);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    k_na_partials<<<nblk, NA_THREADS, 0, s>>>(d_W, d_dr, n_cell, hp, part);
+    k_na_partials<<<nblk, NA_THREADS, 0, s>>>(d_W, d_dr, n_cell, DtPhys<double>(hp), part);
     k_na_finish<<<1, NA_THREADS, 0, s>>>(part, nblk, p->cfl, d_dt);
     e = cudaGetLastError();
     if (e != cudaSuccess) {

@@ -229,7 +229,7 @@ __device__ __forceinline__ void recon_cells(const DevMesh<T>& m, const ReconCons
         else
             d[f] = ok ? xn[q] - Q0 : T(0);
 #pragma unroll
-        for (int l = 0; l < 3; ++l) d[4 + 3 * f + l] = ok ? (TO)xn[5 + 3 * q + l] : TO(0);
+        for (int l = 0; l < 3; ++l) d[4 + 3 * f + l] = ok ? (TO)xn[Stride<T>::xg + 3 * q + l] : TO(0);
     }
     // the tile has landed (all threads wait; a give-up is reported, and the
     // values computed from an incomplete tile are never trusted by the host)

@@ -83,13 +83,13 @@ template <int NR>
 constexpr size_t stage_smem_bytes() {
     const size_t recon = CELL_GROUPS * sizeof(Tile<float>) + CELL_GROUPS * sizeof(unsigned long long);
     const size_t flux = FLUX_GROUPS * sizeof(FluxSmem<float, NR>);
-    const size_t upd = CELL_GROUPS * (2 * CELLS_PER_BLOCK + CELL_THREADS / 32 * 6) * sizeof(double);
+    const size_t upd = STAGE_THREADS / 32 * 5 * sizeof(float);
     return recon > flux ? (recon > upd ? recon : upd) : (flux > upd ? flux : upd);
 }
 
 template <int STAGE, bool VISC>
 __global__ void __launch_bounds__(STAGE_THREADS, 1)
-    k_stage(DevMesh<float> m, Phys<float> ph, HostPhys hp, ReconConst<float> rc, DevState<float> st,
+    k_stage(DevMesh<float> m, Phys<float> ph, DtPhys<float> hp, ReconConst<float> rc, DevState<float> st,
             FinArg<float> fin, unsigned* gbar) {
     constexpr int NR = STAGE == 1 ? 40 : 20;
     extern __shared__ __align__(128) unsigned char smem[];
@@ -132,22 +132,19 @@ __global__ void __launch_bounds__(STAGE_THREADS, 1)
     // ---- cell update (Sec. 3, Eq. s2o4)
     {
         const int grp = threadIdx.x / CELL_THREADS, tid = threadIdx.x % CELL_THREADS;
-        double* base = reinterpret_cast<double*>(smem) + grp * (2 * CELLS_PER_BLOCK + CELL_THREADS / 32 * 6);
+        float (*red)[5] = reinterpret_cast<float (*)[5]>(smem) + grp * (CELL_THREADS / 32);
         for (int64_t vb = (int64_t)blockIdx.x * CELL_GROUPS + grp; vb < ncb; vb += (int64_t)gridDim.x * CELL_GROUPS) {
-            if (STAGE == 1) {
-                update1_cells<float>(m, hp, st, vb, tid);
-            } else {
-                const CellGroup cg{vb, tid, BAR_CELL_GROUP + grp, base, reinterpret_cast<int32_t*>(base + CELLS_PER_BLOCK),
-                                   base + 2 * CELLS_PER_BLOCK};
-                update2_cells<float>(m, hp, st, cg);
-            }
+            if (STAGE == 1)
+                update1_cells<float>(m, st, vb, tid);
+            else
+                update2_cells<float>(m, hp, st, vb, tid, BAR_CELL_GROUP + grp, red);
             group_barrier(BAR_CELL_GROUP + grp, CELL_THREADS);
         }
     }
 }
 
 template <int STAGE, bool VISC>
-static cudaError_t launch_stage_kernel(const DevMesh<float>& m, const Phys<float>& ph, const HostPhys& hp,
+static cudaError_t launch_stage_kernel(const DevMesh<float>& m, const Phys<float>& ph, const DtPhys<float>& hp,
                                        const ReconConst<float>& rc, const DevState<float>& st,
                                        const FinArg<float>& fin, unsigned* gbar, cudaStream_t s) {
     constexpr size_t smem = stage_smem_bytes<STAGE == 1 ? 40 : 20>();
@@ -198,10 +195,10 @@ cudaError_t launch_stage(const DevMesh<float>& m, const HostPhys& p, const DevSt
         fa.ctrl = fin->ctrl;
     }
     if (stage == 1)
-        return p.viscous ? launch_stage_kernel<1, true>(m, ph, p, rc, st, fa, gbar, s)
-                         : launch_stage_kernel<1, false>(m, ph, p, rc, st, fa, gbar, s);
-    return p.viscous ? launch_stage_kernel<2, true>(m, ph, p, rc, st, fa, gbar, s)
-                     : launch_stage_kernel<2, false>(m, ph, p, rc, st, fa, gbar, s);
+        return p.viscous ? launch_stage_kernel<1, true>(m, ph, DtPhys<float>(p), rc, st, fa, gbar, s)
+                         : launch_stage_kernel<1, false>(m, ph, DtPhys<float>(p), rc, st, fa, gbar, s);
+    return p.viscous ? launch_stage_kernel<2, true>(m, ph, DtPhys<float>(p), rc, st, fa, gbar, s)
+                     : launch_stage_kernel<2, false>(m, ph, DtPhys<float>(p), rc, st, fa, gbar, s);
 }
 
 }  // namespace gks
