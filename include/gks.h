@@ -427,7 +427,8 @@ gks_status gks_adjoint_step_staged(gks_state* state, double dt, const double* d_
  *                (fewer warps, more registers); FP32 only, ignored in FP64
  *   slopes_pass  0 = reconstruction step 1 (the P1 slopes, Sec. 4.3) is
  *                recomputed inside step 2 for each neighbour, 1 = a separate
- *                pass stores every cell's slopes first (WENO only)
+ *                pass stores what step 2 takes of every cell's slopes first
+ *                (WENO only; the default, as 0, 3, 1 is for the three)
  * Returns GKS_E_ARG for any other value.  Re-uploads the face arrays when the
  * order changes; the next gks_step captures a new graph. */
 gks_status gks_state_set_variant(gks_state* state, int32_t face_order, int32_t flux_blocks,

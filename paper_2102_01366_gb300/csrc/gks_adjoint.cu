@@ -378,8 +378,9 @@ __global__ void k_adj_recon_local(DevMesh<double> m, const double* __restrict__ 
         fallback_back(lp, c, q, ld, nullptr, own);
         return;
     }
-    const double* tile = m.tile + (c / CELLS_PER_BLOCK) * TILE_ROWS * CELLS_PER_BLOCK + c % CELLS_PER_BLOCK;
-    auto T_ = [&](int row) { return tile[(int64_t)row * CELLS_PER_BLOCK]; };
+    const double* tile = m.tile + (c / CELLS_PER_BLOCK) * TILE_ROWS * CELLS_PER_BLOCK;
+    const int lc = (int)(c % CELLS_PER_BLOCK);
+    auto T_ = [&](int row) { return tile[tile_at<double>(row, lc)]; };
     const double* l = lp + c * 50 + q * 10;
     const double lc0 = l[0];
     double la[9];
@@ -500,8 +501,9 @@ __global__ void k_adj_recon_weno(DevMesh<double> m, double eps, const double* __
         fallback_back(lp, c, q, ld, lbn, own);
         return;
     }
-    const double* tile = m.tile + (c / CELLS_PER_BLOCK) * TILE_ROWS * CELLS_PER_BLOCK + c % CELLS_PER_BLOCK;
-    auto T_ = [&](int row) { return tile[(int64_t)row * CELLS_PER_BLOCK]; };
+    const double* tile = m.tile + (c / CELLS_PER_BLOCK) * TILE_ROWS * CELLS_PER_BLOCK;
+    const int lc = (int)(c % CELLS_PER_BLOCK);
+    auto T_ = [&](int row) { return tile[tile_at<double>(row, lc)]; };
     int nb[4];
     for (int f = 0; f < 4; ++f) nb[f] = m.nbr[f * nc + c];
     const double Q0 = X[c * XS + q];
@@ -640,8 +642,9 @@ __global__ void k_adj_recon_weno2(DevMesh<double> m, double eps, const double* _
         fallback_back(lp, c, q, ld, lbn, own);
         return;
     }
-    const double* tile = m.tile + (c / CELLS_PER_BLOCK) * TILE_ROWS * CELLS_PER_BLOCK + c % CELLS_PER_BLOCK;
-    auto T_ = [&](int row) { return tile[(int64_t)row * CELLS_PER_BLOCK]; };
+    const double* tile = m.tile + (c / CELLS_PER_BLOCK) * TILE_ROWS * CELLS_PER_BLOCK;
+    const int lc = (int)(c % CELLS_PER_BLOCK);
+    auto T_ = [&](int row) { return tile[tile_at<double>(row, lc)]; };
     int nb[4];
     for (int f = 0; f < 4; ++f) nb[f] = m.nbr[f * nc + c];
     const double Q0 = X[c * XS + q];
@@ -718,14 +721,15 @@ __global__ void k_adj_recon_p1(DevMesh<double> m, const double* __restrict__ lp,
         fallback_back(lp, c, q, ld, nullptr, own);
         return;
     }
-    const double* tile = m.tile + (c / CELLS_PER_BLOCK) * TILE_ROWS * CELLS_PER_BLOCK + c % CELLS_PER_BLOCK;
+    const double* tile = m.tile + (c / CELLS_PER_BLOCK) * TILE_ROWS * CELLS_PER_BLOCK;
+    const int lc = (int)(c % CELLS_PER_BLOCK);
     const double* l = lp + c * 50 + q * 10;
     double* o = ld + (c * 5 + q) * 16;
     double s = 0.0;
     for (int j = 0; j < 16; ++j) o[j] = 0.0;
     for (int j = 0; j < 4; ++j) {
         if (m.nbr[j * m.nc + c] < 0) continue;
-        for (int i = 0; i < 3; ++i) o[j] += tile[(int64_t)(TILE_M1 + i * 4 + j) * CELLS_PER_BLOCK] * l[1 + i];
+        for (int i = 0; i < 3; ++i) o[j] += tile[tile_at<double>(TILE_M1 + i * 4 + j, lc)] * l[1 + i];
         s += o[j];
     }
     own[c * 5 + q] = l[0] - s;

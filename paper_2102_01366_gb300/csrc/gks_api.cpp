@@ -383,7 +383,11 @@ struct gks_state {
     bool fixed_pinned = false;  // gks_set_fixed_state was called: initialisations keep the fixed state
     int face_order = 0;    // 0: canonical face order, 1: grouped by left cell
     int flux_variant = 1;  // 1: 3 blocks/SM, 0: 2 blocks/SM (FP32 flux)
-    int slopes_pass = 0;   // 1: reconstruction step 1 as its own pass
+    // 1: reconstruction step 1 as its own pass (WENO only).  The default, as
+    // the faster one at every size measured, from 1,536 cells (a step 37.2 ->
+    // 33.1 us) over 24,576 (81 -> 76; FP64 1,163 -> 1,140) and 409,644 (996 ->
+    // 869) to 580,320 (1,556 -> 1,284 us); 0 forms each neighbour's slopes anew.
+    int slopes_pass = 1;
     int fused = 0;         // 1: each stage as one persistent launch (precision 1 only)
     // cell ordering of the device arrays (FP32 bulk): 0 the caller's, 1
     // reverse Cuthill-McKee, 2 Morton, each within each case; cperm maps a
@@ -635,7 +639,7 @@ static gks_status upload_cells(gks_state* s) {
     const int64_t nblk = update_blocks(nc);
     std::vector<T> dr(nc);
     std::vector<TO> M1(12 * nc);
-    // per-block tile [blk][TILE_ROWS][CELLS_PER_BLOCK], zero past the last cell
+    // per-block tile of TILE_ROWS values a cell (tile_at), zero past the last cell
     std::vector<TO> tile((size_t)nblk * TILE_ROWS * CELLS_PER_BLOCK, TO(0));
     // Sec. 4.4: with linear weights a boundary cell's third-order step is the
     // least-squares first-order fit to its P2 stencil
@@ -649,16 +653,22 @@ static gks_status upload_cells(gks_state* s) {
     for (int64_t d = 0; d < nc; ++d) {
         const int64_t c = s->pub(d);
         cell_case[d] = g.cell_case[c];
-        TO* tc = &tile[(size_t)(d / CELLS_PER_BLOCK) * TILE_ROWS * CELLS_PER_BLOCK + d % CELLS_PER_BLOCK];
-        auto put_row = [&](int row, double v) { tc[(size_t)row * CELLS_PER_BLOCK] = (TO)v; };
+        TO* tc = &tile[(size_t)(d / CELLS_PER_BLOCK) * TILE_ROWS * CELLS_PER_BLOCK];
+        const int lc = (int)(d % CELLS_PER_BLOCK);
+        auto put_row = [&](int row, double v) { tc[tile_at<TO>(row, lc)] = (TO)v; };
+        double far[3] = {0.0, 0.0, 0.0};
         for (int f = 0; f < 4; ++f) {
             nbr[f * nc + d] = g.nbr[c * 4 + f] >= 0 ? (int32_t)s->dev(g.nbr[c * 4 + f]) : -1;
             const int64_t fi = g.csr_face[c * 4 + f];
             const bool left = g.csr_sign[c * 4 + f] > 0;
             const double* gp = left ? &g.gp_l[fi * 9] : &g.gp_r[fi * 9];
-            for (int k = 0; k < 9; ++k) put_row(TILE_G + f * 9 + k, gp[k]);
+            for (int k = 0; k < 9; ++k) {
+                put_row(TILE_G + f * 9 + k, gp[k]);
+                far[k % 3] = std::max(far[k % 3], std::abs(gp[k]));
+            }
         }
         inv_vol[d] = 1.0 / g.vol[c];
+        for (int k = 0; k < 3; ++k) put_row(TILE_BND + k, far[k]);
         put_row(TILE_V23, std::pow(g.vol[c], 2.0 / 3.0));
         put_row(TILE_V43, std::pow(g.vol[c], 4.0 / 3.0));
         dr[d] = (T)g.dr[c];

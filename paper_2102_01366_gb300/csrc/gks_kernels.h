@@ -56,11 +56,24 @@ struct Stride {
     static constexpr int poly = sizeof(T) == 4 ? POLY_STRIDE32 : POLY_STRIDE;
 };
 // Per-block tile of the reconstruction's static cell data, one contiguous
-// [TILE_ROWS][CELLS_PER_BLOCK] record per block of cells, loaded into shared
-// memory by one bulk copy: M2 (144 rows), the cell's 12 face Gauss points
-// about its centroid (36), M1 (12), central second moments (6), |Omega|^(2/3),
-// |Omega|^(4/3).
-enum { TILE_M2 = 0, TILE_G = 144, TILE_M1 = 180, TILE_MOM = 192, TILE_V23 = 198, TILE_V43 = 199, TILE_ROWS = 200 };
+// record of TILE_ROWS values for each of the block's CELLS_PER_BLOCK cells: M2
+// (144), M1 (12), central second moments (6), |Omega|^(2/3), |Omega|^(4/3),
+// the largest |x|, |y|, |z| of the cell's 12 face Gauss points about its
+// centroid (3, pad 1); these first TILE_COPY rows come into shared memory by
+// one bulk copy.  The Gauss points themselves (36) stay in global memory:
+// only cells that the bound from the largest offsets cannot clear read them.
+// Consecutive rows of a cell lie together in 16-byte groups, so that a lane
+// reads four (FP64: two) in one shared-memory access.
+enum { TILE_M2 = 0, TILE_M1 = 144, TILE_MOM = 156, TILE_V23 = 162, TILE_V43 = 163, TILE_BND = 164, TILE_COPY = 168,
+       TILE_G = 168, TILE_ROWS = 204 };
+template <typename TO>
+#ifdef __CUDACC__
+__host__ __device__
+#endif
+constexpr int64_t tile_at(int row, int cell) {
+    constexpr int V = 16 / (int)sizeof(TO);
+    return ((int64_t)(row / V) * CELLS_PER_BLOCK + cell) * V + row % V;
+}
 // a wall-constrained operator slot: W2 [9][17] (P2 from [data (16); Q0])
 // then W1 [3][5] (P1 slopes from [dQ_f (4); Q0])
 enum { WOP_W1 = 153, WOP_STRIDE = 168 };
@@ -75,7 +88,7 @@ struct DevMesh {
     const double* inv_vol; // [nc]
     const T* dr;           // [nc]
     const T* M1;           // [12][nc]
-    const T* tile;         // [blocks][TILE_ROWS][CELLS_PER_BLOCK] reconstruction data
+    const T* tile;         // [blocks][TILE_ROWS * CELLS_PER_BLOCK] reconstruction data (tile_at)
     // FP32 bulk with FP64 stencil operators (precision 2): the same two in
     // FP64, M1 and tile NULL (else these are NULL)
     const double* M1d;
@@ -101,7 +114,7 @@ struct DevState {
     T* Xs;        // [nc][Stride<T>::xs] stage state W*, grad W*
     double* S;    // [nc][5] saved stage-1 flux term
     T* G;         // [nc][15] saved stage-1 gradient term
-    T* slopes;    // [nc][15]
+    T* slopes;    // [nc][5] |b|^2 of the P1 slopes (slopes pass), or [nc][15] the slopes (diagnostics)
     T* poly;      // [nc][Stride<T>::poly]
     T* rec;       // [nf][rec_stride]
     double* ctrl; // [CTRL_N] global controls (dt_fixed, t_end)
@@ -133,14 +146,15 @@ struct Launch {
         double cfl;
         const double* ctrl;
     };
-    static cudaError_t slopes(const DevMesh<T>& m, const T* X, T* slopes, const Finalize* fin,
+    // step 1 of the reconstruction: |b|^2 of every cell's P1 slopes, s2[nc][5]
+    static cudaError_t slopes(const DevMesh<T>& m, const T* X, T* s2, const Finalize* fin,
                               cudaStream_t s);
-    // slopes_in (may be NULL): the step-1 slopes of every cell from a slopes
-    // pass; without it the kernel computes its own and its neighbours' slopes.
+    // s2_in (may be NULL): the slopes pass's result; without it the kernel
+    // computes its neighbours' slopes itself.
     // slopes_out (may be NULL) receives the cell's own step-1 slopes.
     // err: ERR_TIMEOUT is or-ed in if a block's bounded wait for its tile
     // gave up
-    static cudaError_t recon(const DevMesh<T>& m, const HostPhys& p, const T* X, const T* slopes_in,
+    static cudaError_t recon(const DevMesh<T>& m, const HostPhys& p, const T* X, const T* s2_in,
                              T* slopes_out, T* poly, int32_t* fallback, const Finalize* fin,
                              int32_t* err, cudaStream_t s);
     // case_dt: per-case step (NULL: dt_override for every face)

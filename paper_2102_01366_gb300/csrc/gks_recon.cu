@@ -1,7 +1,7 @@
 // gks_recon.cu -- reconstruction kernels (Sec. 4.1-4.3), sm_103a, FP64 and
 // FP32-bulk instantiations.
 //
-//   k_slopes   reconstruction step 1: P1 slopes per cell (Sec. 4.3)
+//   k_slopes   reconstruction step 1: |b|^2 of the P1 slopes (Sec. 4.3)
 //   k_recon    reconstruction step 2: P2 by the 9x16 operator, smoothness
 //              indicators, two-step beta_0, nonlinear weights, positivity
 //              (Sec. 4.1-4.3); R written about the centroid in monomial form
@@ -14,38 +14,34 @@
 
 namespace gks {
 
-// reconstruction step 1: P1 slopes b = M1 (Q_nb - Q_0), Sec. 4.3, the
-// products in the operator precision TO
+// reconstruction step 1: |b|^2 of the P1 slopes b = M1 (Q_nb - Q_0), Sec.
+// 4.3, the products in the operator precision TO; beta_0 of the cells around
+// (Eq. p0-non-linear-weight) takes the slopes in this form only
 template <typename T, typename TO>
 __global__ void __launch_bounds__(CELL_THREADS) k_slopes(DevMesh<T> m, const T* __restrict__ X,
-                                                          T* __restrict__ slopes, FinArg<T> fin) {
+                                                          T* __restrict__ s2, FinArg<T> fin) {
     if (fin.dtmin && blockIdx.x == 0) finalize_cases(fin.dtmin, fin.case_t, fin.case_dt, fin.ncase, fin.cfl, fin.ctrl);
     const CellLane cl = cell_lane(m.nc);
     if (!cl.active) return;
-    const int64_t nc = m.nc, c = cl.c;
-    const int q = cl.q;
     T b[3];
-    p1_slope<T, TO>(m, X, c, q, b);  // with the wall-constrained slopes of Sec. 4.4
-    T* out = slopes + c * 15 + 3 * q;
-    out[0] = b[0];
-    out[1] = b[1];
-    out[2] = b[2];
+    p1_slope<T, TO>(m, X, cl.c, cl.q, b);  // with the wall-constrained slopes of Sec. 4.4
+    s2[cl.c * 5 + cl.q] = slope_sq(b);
 }
 
 template <typename T, typename TO, bool WALL>
 __global__ void __launch_bounds__(CELL_THREADS) k_recon(DevMesh<T> m, ReconConst<T> rc,
                                                          const T* __restrict__ X,
-                                                         const T* __restrict__ slopes_in,
+                                                         const T* __restrict__ s2_in,
                                                          T* __restrict__ slopes_out,
                                                          T* __restrict__ poly,
                                                          int32_t* __restrict__ fallback,
                                                          FinArg<T> fin, int32_t* __restrict__ err) {
-    __shared__ alignas(128) TO sT[TILE_ROWS][CELLS_PER_BLOCK];
+    __shared__ alignas(128) Tile<TO> sT;
     __shared__ alignas(8) unsigned long long bar;
     if (threadIdx.x == 0) mbar_init(&bar, 1);
     __syncthreads();  // the barrier exists before anyone waits on it
     if (fin.dtmin && blockIdx.x == 0) finalize_cases(fin.dtmin, fin.case_t, fin.case_dt, fin.ncase, fin.cfl, fin.ctrl);
-    recon_cells<T, TO, WALL>(m, rc, X, slopes_in, slopes_out, poly, fallback, err, blockIdx.x, threadIdx.x, sT, &bar,
+    recon_cells<T, TO, WALL>(m, rc, X, s2_in, slopes_out, poly, fallback, err, blockIdx.x, threadIdx.x, sT, &bar,
                              0);
 }
 
@@ -65,18 +61,18 @@ static FinArg<T> fin_arg(const typename Launch<T>::Finalize* fin) {
 }
 
 template <typename T>
-cudaError_t Launch<T>::slopes(const DevMesh<T>& m, const T* X, T* slopes, const Finalize* fin,
+cudaError_t Launch<T>::slopes(const DevMesh<T>& m, const T* X, T* s2, const Finalize* fin,
                               cudaStream_t s) {
     if (m.nc == 0) return cudaSuccess;
     if (m.M1d && sizeof(T) == 4)
-        k_slopes<T, double><<<cell_grid(m.nc), CELL_THREADS, 0, s>>>(m, X, slopes, fin_arg<T>(fin));
+        k_slopes<T, double><<<cell_grid(m.nc), CELL_THREADS, 0, s>>>(m, X, s2, fin_arg<T>(fin));
     else
-        k_slopes<T, T><<<cell_grid(m.nc), CELL_THREADS, 0, s>>>(m, X, slopes, fin_arg<T>(fin));
+        k_slopes<T, T><<<cell_grid(m.nc), CELL_THREADS, 0, s>>>(m, X, s2, fin_arg<T>(fin));
     return cudaGetLastError();
 }
 
 template <typename T>
-cudaError_t Launch<T>::recon(const DevMesh<T>& m, const HostPhys& p, const T* X, const T* slopes_in,
+cudaError_t Launch<T>::recon(const DevMesh<T>& m, const HostPhys& p, const T* X, const T* s2_in,
                              T* slopes, T* poly, int32_t* fallback, const Finalize* fin, int32_t* err,
                              cudaStream_t s) {
     if (m.nc == 0) return cudaSuccess;
@@ -87,7 +83,7 @@ cudaError_t Launch<T>::recon(const DevMesh<T>& m, const HostPhys& p, const T* X,
     rc.order = p.order;
     // the wall-constrained instances only where the mesh has such cells
     auto go = [&](auto kernel) {
-        kernel<<<cell_grid(m.nc), CELL_THREADS, 0, s>>>(m, rc, X, slopes_in, slopes, poly, fallback, fin_arg<T>(fin),
+        kernel<<<cell_grid(m.nc), CELL_THREADS, 0, s>>>(m, rc, X, s2_in, slopes, poly, fallback, fin_arg<T>(fin),
                                                          err);
     };
     if (m.tiled && sizeof(T) == 4)

@@ -226,7 +226,7 @@ class State:
         self.torch = torch
         self.mesh = mesh
         self.params = p
-        self.variant = (0, 3, 0)  # the library default: canonical faces, 3 flux blocks per SM, fused slopes
+        self.variant = (0, 3, 1)  # the library default: canonical faces, more flux warps, separate slopes pass
         self.cell_order = 0  # the caller's cell order
         self.device = torch.device(device)
         nbytes = lib().gks_workspace_bytes(mesh._h, C.byref(p))
