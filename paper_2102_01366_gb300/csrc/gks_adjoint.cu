@@ -38,7 +38,7 @@
 namespace gks {
 
 constexpr int ADJ_IN = 40;       // inputs of the point solution: WL, gL, WR, gR (face frame)
-constexpr int ADJ_THREADS = 64;  // threads per block of k_adj_point_rev
+constexpr int ADJ_THREADS = 64;  // threads per block of the face kernels
 
 // stage 2 records: [sum w 4/3 D (5) | sum w dW n (15)]; the cell sums enter
 // W^{n+1} = W^n - (S + sum s rec[0:5]) / |Omega| and
@@ -78,19 +78,21 @@ __global__ void k_adj_src1(DevMesh<double> m, const double* __restrict__ lW, con
 __device__ __forceinline__ void eval_poly_adj(const double* X, const double* lv, const double (*lg)[5],
                                               double* lc) {
     const double x = X[0], y = X[1], z = X[2];
+#pragma unroll
     for (int q = 0; q < 5; ++q) {
         double* c = lc + q * 10;
         const double v = lv[q], g0 = lg[0][q], g1 = lg[1][q], g2 = lg[2][q];
+        const double sx = v * x + g0, sy = v * y + g1, sz = v * z + g2;
         c[0] += v;
-        c[1] += v * x + g0;
-        c[2] += v * y + g1;
-        c[3] += v * z + g2;
-        c[4] += v * x * x + 2.0 * x * g0;
-        c[5] += v * x * y + y * g0 + x * g1;
-        c[6] += v * x * z + z * g0 + x * g2;
-        c[7] += v * y * y + 2.0 * y * g1;
-        c[8] += v * y * z + z * g1 + y * g2;
-        c[9] += v * z * z + 2.0 * z * g2;
+        c[1] += sx;
+        c[2] += sy;
+        c[3] += sz;
+        c[4] += x * (sx + g0);
+        c[5] += y * sx + x * g1;
+        c[6] += z * sx + x * g2;
+        c[7] += y * (sy + g1);
+        c[8] += z * sy + y * g2;
+        c[9] += z * (sz + g2);
     }
 }
 
@@ -118,28 +120,32 @@ __device__ __forceinline__ void rotate_in(const double (*Rm)[3], double* v) {
     for (int j = 0; j < 3; ++j) v[1 + j] = Rm[j][0] * a + Rm[j][1] * b + Rm[j][2] * c;
 }
 
-// The point's inputs in the face frame (WL, gL, WR, gR: 40 values) from the
-// stored reconstruction, and the output adjoints of the point (face frame)
-// from the record adjoints (the transposed record formulas of the stage).
+// The point's inputs in the face frame (per side W, g: 20 values) from the
+// stored reconstruction, as the forward flux forms them, and the output
+// adjoints of the point (face frame) from the record adjoints (the transposed
+// record formulas of the stage).
 template <int NR>
-__device__ __forceinline__ void adj_point_setup(const DevMesh<double>& m, const double* __restrict__ poly,
-                                                const double* __restrict__ Xavg, const double* __restrict__ src,
-                                                int64_t f, int k, double (*Rm)[3], double* x, double* lFh,
-                                                double* lD, double* lW0, double* ldWt,
-                                                const Phys<double>* ph = nullptr) {
+__device__ __forceinline__ void adj_point_setup(const DevMesh<double>& m, const Phys<double>& ph,
+                                                const double* __restrict__ poly, const double* __restrict__ Xavg,
+                                                const double* __restrict__ src, int64_t f, int k, double (*x)[20],
+                                                double* lFh, double* lD, double* lW0, double* ldWt) {
     const int L = m.flr[f], R = m.flr[m.nf + f];
     const double* geo = m.fgeo + f * FGEO;
     const double n[3] = {geo[0], geo[1], geo[2]};
     const double w = geo[3];
+    double Rm[3][3];
     face_frame(n, Rm);
     // record adjoints: the left cell adds the record, the right one subtracts it
     // (a boundary face has one cell)
     double lr[NR];
+#pragma unroll
     for (int j = 0; j < NR; ++j)
         lr[j] = (L >= 0 ? src[(int64_t)L * NR + j] : 0.0) - (R >= 0 ? src[(int64_t)R * NR + j] : 0.0);
+#pragma unroll
     for (int q = 0; q < 5; ++q) {
         double sn0 = 0.0, sn1 = 0.0;
         if (NR == 40) {
+#pragma unroll
             for (int i = 0; i < 3; ++i) {
                 sn0 += n[i] * lr[10 + 3 * q + i];
                 sn1 += n[i] * lr[25 + 3 * q + i];
@@ -149,6 +155,7 @@ __device__ __forceinline__ void adj_point_setup(const DevMesh<double>& m, const 
             lW0[q] = w * (sn0 + sn1);
             ldWt[q] = 0.5 * w * sn0;
         } else {
+#pragma unroll
             for (int i = 0; i < 3; ++i) sn0 += n[i] * lr[5 + 3 * q + i];
             lFh[q] = 0.0;
             lD[q] = w * (4.0 / 3.0) * lr[q];
@@ -156,51 +163,16 @@ __device__ __forceinline__ void adj_point_setup(const DevMesh<double>& m, const 
             ldWt[q] = w * sn0;
         }
     }
-    rotate_in(Rm, lFh);
-    rotate_in(Rm, lD);
-    rotate_in(Rm, lW0);
-    rotate_in(Rm, ldWt);
-    if (x) {
-        // each side's state in the face frame, as the forward flux forms it
-        for (int side = 0; side < 2; ++side) {
-            const int cell = side == 0 ? L : R;
-            const int in = side == 0 ? R : L;
-            double* xs = x + 20 * side;
-            double (*gs)[5] = reinterpret_cast<double (*)[5]>(xs + 5);
-            double Wv[5], g[3][5];
-            if (cell == FLR_OPEN) {
-                // open: the interior cell's average, zero gradient
-                for (int q = 0; q < 5; ++q) {
-                    Wv[q] = Xavg[(int64_t)in * XS + q];
-                    g[0][q] = g[1][q] = g[2][q] = 0.0;
-                }
-                to_local(Rm, Wv, g, xs, gs);
-                continue;
-            }
-            if (cell == FLR_FIXED) {
-                // fixed: the interior cell's fixed state carried to the point
-                const int si = 1 - side;
-                const double X[3] = {geo[4 + 9 * si + 3 * k], geo[5 + 9 * si + 3 * k], geo[6 + 9 * si + 3 * k]};
-                fixed_ghost(m.fixed + (int64_t)in * XS, X, Wv, g);
-                to_local(Rm, Wv, g, xs, gs);
-                continue;
-            }
-            // a real side, or a wall side from the interior cell at the point
-            const int src_side = cell >= 0 ? side : 1 - side;
-            const int64_t c = cell >= 0 ? cell : in;
-            const double X[3] = {geo[4 + 9 * src_side + 3 * k], geo[5 + 9 * src_side + 3 * k], geo[6 + 9 * src_side + 3 * k]};
-            eval_poly(poly + c * POLY_STRIDE, X, Wv, g);
-            to_local(Rm, Wv, g, xs, gs);
-            if (cell == FLR_SLIP_WALL) slip_wall_ghost(xs, gs);
-            if (cell == FLR_NOSLIP_WALL) noslip_wall_ghost(xs, gs);
-            if (cell == FLR_ISOTHERMAL_WALL) isothermal_wall_ghost(xs, gs, ph->gm1, ph->twall);
-            if (cell == FLR_MOVING_WALL) {
-                double Uw[3];
-                rotate_vec(Rm, ph->uwall, Uw);
-                moving_wall_ghost(xs, gs, ph->gm1, Uw);
-            }
-        }
+    if (NR == 40) {
+        rotate_in(Rm, lFh);
+        rotate_in(Rm, lW0);
     }
+    rotate_in(Rm, lD);
+    rotate_in(Rm, ldWt);
+#pragma unroll 1
+    for (int side = 0; side < 2; ++side)
+        side_state<double, true>(m, ph, Xavg, poly, geo, Rm, L, R, side, k, x[side],
+                                 reinterpret_cast<double (*)[5]>(x[side] + 5));
 }
 
 // A forward-mode number (value and one derivative) for the Jacobian of the
@@ -244,110 +216,116 @@ __device__ void wall_ghost_adj(int kind, const double* x, const double* ls, doub
     }
 }
 
-// One thread per (face, Gauss point) of interior faces: the point
-// solution's adjoint in reverse mode (gks_point_adj), lx[f][k][0:40].
+// One thread per (face, Gauss point): the point solution's adjoint in reverse
+// mode (gks_point_adj), lx[i][f][k] for the 40 inputs i (input-major, so that
+// a warp writes and the face kernel reads full lines).
 template <int NR, bool VISC>
 __global__ void __launch_bounds__(ADJ_THREADS) k_adj_point_rev(DevMesh<double> m, Phys<double> ph,
                                                                const double* __restrict__ poly,
                                                                const double* __restrict__ Xavg,
                                                                const double* __restrict__ src, double dt,
                                                                double* __restrict__ lx) {
-    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= m.nf * 3) return;
+    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, nt = m.nf * 3;
+    if (t >= nt) return;
     const int64_t f = t / 3;
     const int k = (int)(t - f * 3);
-    double Rm[3][3], x[ADJ_IN], lFh[5], lD[5], lW0[5], ldWt[5];
-    adj_point_setup<NR>(m, poly, Xavg, src, f, k, Rm, x, lFh, lD, lW0, ldWt, &ph);
-    double* l = lx + t * ADJ_IN;
-    double lin[ADJ_IN];
-    for (int i = 0; i < ADJ_IN; ++i) lin[i] = 0.0;
-    gks_point_adj<VISC>(ph, x, reinterpret_cast<const double (*)[5]>(x + 5), x + 20,
-                  reinterpret_cast<const double (*)[5]>(x + 25), dt, lFh, lD, lW0, ldWt, lin,
-                  reinterpret_cast<double (*)[5]>(lin + 5), lin + 20, reinterpret_cast<double (*)[5]>(lin + 25));
-    for (int i = 0; i < ADJ_IN; ++i) l[i] = lin[i];
+    double x[2][20], lFh[5], lD[5], lW0[5], ldWt[5], lin[2][20];
+    adj_point_setup<NR>(m, ph, poly, Xavg, src, f, k, x, lFh, lD, lW0, ldWt);
+    gks_point_adj<VISC, NR == 40>(ph, x, dt, lFh, lD, lW0, ldWt, lin);
+#pragma unroll
+    for (int s = 0; s < 2; ++s)
+#pragma unroll
+        for (int i = 0; i < 20; ++i) lx[(20 * s + i) * nt + t] = lin[s][i];
 }
 
-// One thread per face: the input adjoints of its three points carried back
-// through the rotations and the evaluation at the points into
-// lpf[f][side][5][10].
+// One thread per (side, face) with a cell: the input adjoints of the face's
+// three points carried back through the rotations and the evaluation at the
+// points into lpf[f][side][5][10].
 // A wall side's adjoint joins the interior side's at the same point (a
 // mirror is its own transpose; the isothermal and moving walls' ghost
-// Jacobians are transposed at the interior state); an open side's goes to the interior cell's average,
-// lwo[f][5] (zero on every other face).
+// Jacobians are transposed at the interior state); an open side's goes to the
+// interior cell's average, lwo[f][5] (zero on every other boundary face, not
+// read on interior ones).
 // XW: the mesh has isothermal or moving wall faces, whose ghosts' Jacobians
-// (and the local frame they need) only those instances carry
+// (and the local frame they need) only those instances carry.
+// One thread for both sides of a face held 100 sums and spilled: 291 us on
+// 96,000 faces, 210 us with a thread a side and input-major lx.
 template <bool XW>
-__global__ void k_adj_face_back(DevMesh<double> m, const double* __restrict__ lx, double* __restrict__ lpf,
-                                double* __restrict__ lwo, const double* __restrict__ poly, Phys<double> ph) {
-    const int64_t f = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (f >= m.nf) return;
-    const int L = m.flr[f], R = m.flr[m.nf + f];
+__global__ void __launch_bounds__(ADJ_THREADS) k_adj_face_back(DevMesh<double> m, const double* __restrict__ lx,
+                                                               double* __restrict__ lpf, double* __restrict__ lwo,
+                                                               const double* __restrict__ poly, Phys<double> ph) {
+    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, nt = m.nf * 3;
+    if (t >= m.nf * 2) return;
+    const int side = t >= m.nf ? 1 : 0;
+    const int64_t f = t - side * m.nf;
+    const int64_t cell = m.flr[side * m.nf + f];
+    if (cell < 0) return;
+    const int other = m.flr[(1 - side) * m.nf + f];
     const double* geo = m.fgeo + f * FGEO;
     const double n[3] = {geo[0], geo[1], geo[2]};
     double Rm[3][3];
     face_frame(n, Rm);
-    double lp[2][50], lw[5] = {0, 0, 0, 0, 0};
-    for (int j = 0; j < 50; ++j) lp[0][j] = lp[1][j] = 0.0;
+    double lp[50], lw[5] = {0, 0, 0, 0, 0};
+#pragma unroll
+    for (int j = 0; j < 50; ++j) lp[j] = 0.0;
+#pragma unroll 1
     for (int k = 0; k < 3; ++k) {
-        double l[ADJ_IN];
-        for (int i = 0; i < ADJ_IN; ++i) l[i] = lx[(f * 3 + k) * ADJ_IN + i];
-        for (int side = 0; side < 2; ++side) {
-            const int cell = side == 0 ? L : R;
-            if (cell >= 0) continue;
-            double* ls = l + 20 * side;
+        const double X[3] = {geo[4 + 9 * side + 3 * k], geo[5 + 9 * side + 3 * k], geo[6 + 9 * side + 3 * k]};
+        const double* lk = lx + f * 3 + k;
+        double l[20];
+#pragma unroll
+        for (int i = 0; i < 20; ++i) l[i] = lk[(20 * side + i) * nt];
+        // a set fixed state is a constant of the step: nothing flows back
+        if (other < 0 && other != FLR_FIXED) {
+            double ls[20];
             double (*lg)[5] = reinterpret_cast<double (*)[5]>(ls + 5);
-            double* li = l + 20 * (1 - side);
-            if (cell == FLR_OPEN) {
+#pragma unroll
+            for (int i = 0; i < 20; ++i) ls[i] = lk[(20 * (1 - side) + i) * nt];
+            if (other == FLR_OPEN) {
                 double lW[5], lgg[3][5];
                 to_local_adj(Rm, ls, lg, lW, lgg);
                 for (int q = 0; q < 5; ++q) lw[q] += lW[q];
-            } else if (cell == FLR_FIXED) {
-                // a set fixed state is a constant of the step: nothing flows back
-            } else if (XW && (cell == FLR_ISOTHERMAL_WALL || cell == FLR_MOVING_WALL)) {
+            } else if (XW && (other == FLR_ISOTHERMAL_WALL || other == FLR_MOVING_WALL)) {
                 // the interior state at the point, face frame, then the ghost's transpose
-                const int src_side = 1 - side;
-                const int64_t c = side == 0 ? R : L;
-                const double X[3] = {geo[4 + 9 * src_side + 3 * k], geo[5 + 9 * src_side + 3 * k], geo[6 + 9 * src_side + 3 * k]};
                 double Wv[5], g[3][5], x[20];
-                eval_poly(poly + c * POLY_STRIDE, X, Wv, g);
+                eval_poly(poly + cell * POLY_STRIDE, X, Wv, g);
                 to_local(Rm, Wv, g, x, reinterpret_cast<double (*)[5]>(x + 5));
                 double Uw[3];
                 rotate_vec(Rm, ph.uwall, Uw);
-                wall_ghost_adj(cell, x, ls, ph.gm1, ph.twall, Uw, li);
+                wall_ghost_adj(other, x, ls, ph.gm1, ph.twall, Uw, l);
             } else {
-                if (cell == FLR_SLIP_WALL) slip_wall_ghost(ls, lg);
-                if (cell == FLR_NOSLIP_WALL) noslip_wall_ghost(ls, lg);
-                for (int i = 0; i < 20; ++i) li[i] += ls[i];
+                if (other == FLR_SLIP_WALL) slip_wall_ghost(ls, lg);
+                if (other == FLR_NOSLIP_WALL) noslip_wall_ghost(ls, lg);
+#pragma unroll
+                for (int i = 0; i < 20; ++i) l[i] += ls[i];
             }
         }
-        for (int side = 0; side < 2; ++side) {
-            if ((side == 0 ? L : R) < 0) continue;
-            const double X[3] = {geo[4 + 9 * side + 3 * k], geo[5 + 9 * side + 3 * k], geo[6 + 9 * side + 3 * k]};
-            double lW[5], lg[3][5];
-            to_local_adj(Rm, l + 20 * side, reinterpret_cast<const double (*)[5]>(l + 20 * side + 5), lW, lg);
-            eval_poly_adj(X, lW, lg, lp[side]);
-        }
+        double lW[5], lg[3][5];
+        to_local_adj(Rm, l, reinterpret_cast<const double (*)[5]>(l + 5), lW, lg);
+        eval_poly_adj(X, lW, lg, lp);
     }
-    double* o = lpf + f * 100;
-    for (int j = 0; j < 50; ++j) {
-        o[j] = lp[0][j];
-        o[50 + j] = lp[1][j];
-    }
-    for (int q = 0; q < 5; ++q) lwo[f * 5 + q] = lw[q];
+    double2* o = reinterpret_cast<double2*>(lpf + f * 100 + side * 50);
+#pragma unroll
+    for (int j = 0; j < 25; ++j) o[j] = make_double2(lp[2 * j], lp[2 * j + 1]);
+    if (other < 0)
+        for (int q = 0; q < 5; ++q) lwo[f * 5 + q] = lw[q];
 }
 
-// adjoint of a cell's reconstruction coefficients: the sum over its faces
+// adjoint of a cell's reconstruction coefficients: the sum over its faces,
+// one thread per (cell, coefficient) so that a warp reads whole records
+// (48,000 cells: 42 us with a thread a cell, 22 us)
 __global__ void k_adj_gather_poly(DevMesh<double> m, const double* __restrict__ lpf, double* __restrict__ lp) {
-    const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= m.nc) return;
-    double acc[50];
-    for (int j = 0; j < 50; ++j) acc[j] = 0.0;
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= m.nc * 50) return;
+    const int64_t c = i / 50;
+    const int j = (int)(i - c * 50);
+    double acc = 0.0;
+#pragma unroll
     for (int f = 0; f < 4; ++f) {
         const int e = m.cface[f * m.nc + c];
-        const double* src = lpf + (int64_t)(e >> 1) * 100 + (e & 1) * 50;
-        for (int j = 0; j < 50; ++j) acc[j] += src[j];
+        acc += lpf[(int64_t)(e >> 1) * 100 + (e & 1) * 50 + j];
     }
-    for (int j = 0; j < 50; ++j) lp[c * 50 + j] = acc[j];
+    lp[i] = acc;
 }
 
 // A cell whose reconstruction fell back to its average (the positivity
@@ -861,10 +839,10 @@ static void flux_back(const DevMesh<double>& m, const Phys<double>& ph, const Ad
         k_adj_point_rev<NR, false><<<grid_of(m.nf * 3, ADJ_THREADS), ADJ_THREADS, 0, s>>>(m, ph, poly, X, b.src, dt,
                                                                                         b.lx);
     if (m.xwalls)
-        k_adj_face_back<true><<<grid_of(m.nf, B), B, 0, s>>>(m, b.lx, b.lpf, b.lwo, poly, ph);
+        k_adj_face_back<true><<<grid_of(m.nf * 2, ADJ_THREADS), ADJ_THREADS, 0, s>>>(m, b.lx, b.lpf, b.lwo, poly, ph);
     else
-        k_adj_face_back<false><<<grid_of(m.nf, B), B, 0, s>>>(m, b.lx, b.lpf, b.lwo, poly, ph);
-    k_adj_gather_poly<<<grid_of(m.nc, B), B, 0, s>>>(m, b.lpf, b.lp);
+        k_adj_face_back<false><<<grid_of(m.nf * 2, ADJ_THREADS), ADJ_THREADS, 0, s>>>(m, b.lx, b.lpf, b.lwo, poly, ph);
+    k_adj_gather_poly<<<grid_of(m.nc * 50, B), B, 0, s>>>(m, b.lpf, b.lp);
 }
 
 // The reverse sweep proper; the forward intermediates (the two stages'
