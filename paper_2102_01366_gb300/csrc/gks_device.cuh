@@ -313,113 +313,105 @@ __device__ __forceinline__ void prandtl_fix(T prf, const T* U, const T* IW, T* F
 }
 
 // --------------------------------------------- half differences --
-// A quantity known on the two sides of a face: its values l, r and,
-// accurate to the rounding of itself, its half-difference h = (l - r) / 2.
-// The rules below are exact identities for finite differences (not
-// linearisations), so h keeps its relative accuracy however small it is,
-// where (l - r) / 2 formed from the rounded values would carry the rounding
-// of l and r.  FP32 bulk uses them to form the interface state W^c
-// (Eq. new-equ-part) relative to the mean of the two sides.
+// A quantity known on the two sides of a face: its values l, r and, accurate
+// to the rounding of itself, its half-difference h = (l - r) / 2.  The rules
+// below are exact identities for finite differences (not linearisations), so
+// h keeps its relative accuracy however small it is, where (l - r) / 2 formed
+// from the rounded values would carry the rounding of l and r:
+//   product   (l_a l_b - r_a r_b) / 2 = h_a mid_b + mid_a h_b
+//   quotient  (l_a / l_b - r_a / r_b) / 2 = (h_a mid_b - mid_a h_b) / (l_b r_b)
+//   root      (sqrt l - sqrt r) / 2 = h / (sqrt l + sqrt r)
+// FP32 bulk uses them to form the interface state W^c (Eq. new-equ-part)
+// relative to the mean of the two sides.
+
+// What the deviation below takes of a side's half-space moments: <u^0>,
+// sqrt(lambda) and e^{-s^2}, s = sqrt(lambda) U
 template <typename T>
-struct HDiff {
-    T l, r, h;
-    __device__ __forceinline__ T mid() const { return T(0.5) * (l + r); }
+struct HalfSpace {
+    T m0, rl, ex;
 };
-
-template <typename T>
-__device__ __forceinline__ HDiff<T> hd_add(const HDiff<T>& a, const HDiff<T>& b) {
-    return {a.l + b.l, a.r + b.r, a.h + b.h};
-}
-
-template <typename T>
-__device__ __forceinline__ HDiff<T> hd_scale(T c, const HDiff<T>& a) {
-    return {c * a.l, c * a.r, c * a.h};
-}
-
-// (l_a l_b - r_a r_b) / 2 = h_a mid_b + mid_a h_b
-template <typename T>
-__device__ __forceinline__ HDiff<T> hd_mul(const HDiff<T>& a, const HDiff<T>& b) {
-    return {a.l * b.l, a.r * b.r, a.h * b.mid() + a.mid() * b.h};
-}
-
-// (l_a / l_b - r_a / r_b) / 2 = (h_a mid_b - mid_a h_b) / (l_b r_b)
-template <typename T>
-__device__ __forceinline__ HDiff<T> hd_div(const HDiff<T>& a, const HDiff<T>& b) {
-    return {a.l / b.l, a.r / b.r, (a.h * b.mid() - a.mid() * b.h) / (b.l * b.r)};
-}
-
-// (sqrt l - sqrt r) / 2 = h / (sqrt l + sqrt r)
-template <typename T>
-__device__ __forceinline__ HDiff<T> hd_sqrt(const HDiff<T>& a) {
-    const T sl = d_sqrt(a.l), sr = d_sqrt(a.r);
-    return {sl, sr, a.h / (sl + sr)};
-}
-
-// (e^{-l} - e^{-r}) / 2, factored on the larger exponential so that expm1
-// stays within (-1, 0] (the other factoring overflows times underflows for
-// far-apart arguments): -e^{-l} expm1(2 h) / 2 for h <= 0, e^{-r}
-// expm1(-2 h) / 2 otherwise
-__device__ __forceinline__ HDiff<float> hd_expneg(const HDiff<float>& a) {
-    const float el = expf(-a.l), er = expf(-a.r);
-    const float h = a.h <= 0.0f ? -0.5f * el * expm1f(2.0f * a.h) : 0.5f * er * expm1f(-2.0f * a.h);
-    return {el, er, h};
-}
-
-// (erf l - erf r) / 2 = (1 / sqrt pi) int_r^l e^{-t^2} dt, given erf l and
-// erf r (el, er).  For |l - r| <= 0.1 the integral is taken by 3-point and
-// up to |l - r| <= 1 by 5-point Gauss-Legendre quadrature on [r, l] (errors
-// below 1e-9 and 2e-8 of the integral at those lengths, far less for
-// shorter intervals); for longer intervals the difference of the two
-// complementary error functions of the tails, which does not cancel there.
-__device__ __forceinline__ HDiff<float> hd_erf(const HDiff<float>& a, float el, float er) {
-    float h;
-    if (fabsf(a.h) <= 0.05f) {
-        // nodes and weights of the 3-point Gauss-Legendre rule on [-1, 1]
-        const float x1 = 0.77459666924148338f, w0 = 0.88888888888888889f, w1 = 0.55555555555555556f;
-        const float m = a.mid(), d = a.h;
-        auto g = [](float t) { return expf(-t * t); };
-        h = 0.56418958354775628695f * d * (w0 * g(m) + w1 * (g(m + x1 * d) + g(m - x1 * d)));
-    } else if (fabsf(a.h) <= 0.5f) {
-        // nodes and weights of the 5-point Gauss-Legendre rule on [-1, 1]
-        const float x1 = 0.53846931010568309f, x2 = 0.90617984593866399f;
-        const float w0 = 0.56888888888888889f, w1 = 0.47862867049936647f, w2 = 0.23692688505618909f;
-        const float m = a.mid(), d = a.h;
-        auto g = [](float t) { return expf(-t * t); };
-        const float sum = w0 * g(m) + w1 * (g(m + x1 * d) + g(m - x1 * d)) + w2 * (g(m + x2 * d) + g(m - x2 * d));
-        h = 0.56418958354775628695f * d * sum;  // 1 / sqrt(pi)
-    } else if (a.mid() > 0.0f) {
-        h = 0.5f * (erfcf(a.r) - erfcf(a.l));
-    } else {
-        h = 0.5f * (erfcf(-a.l) - erfcf(-a.r));
-    }
-    return {el, er, h};
-}
 
 // Half-difference of psi(W) = rho <psi>_{u1>0} - rho <psi>_{u1<0} between
 // the two states Wl, Wr (face frame, x1 along the normal), given the
-// half-difference h of the states themselves and erf of each state's s
-// (below).  With s = sqrt(lambda) U1 =
-// W1 / sqrt(2 p rho), e0 = erf(s) and g = e^{-s^2} / sqrt(pi lambda) =
-// e^{-s^2} sqrt(2 p / (pi rho)), the half-space moments of Sec. 2.2 give
-//   psi(W) = (rho e0, W1 e0 + rho g, W2 e0, W3 e0, W4 e0 + W1 g / 2),
+// half-difference h of the states themselves.  With e0 = erf(s) and
+// G = rho e^{-s^2} / sqrt(pi lambda), the half-space moments of Sec. 2.2 give
+//   psi(W) = (rho e0, W1 e0 + G, W2 e0, W3 e0, W4 e0 + U1 G / 2),
 // and W^c = rho_l <psi>_{u1>0} + rho_r <psi>_{u1<0} = (Wl + Wr) / 2 +
 // (psi(Wl) - psi(Wr)) / 2, so W^c minus the mean of the two states is h_psi.
+//
+// (erf l - erf r) / 2 and (e^{-l^2} - e^{-r^2}) / 2 are the integrals of
+// e^{-t^2} / sqrt(pi) and -t e^{-t^2} over [s_r, s_l] by one Gauss-Legendre
+// rule on the same nodes: 3 points for |s_l - s_r| <= 0.1, 5 points up to 1
+// (errors below 1e-9 and 2e-7 of the integrands' scale at those lengths, far
+// less for shorter intervals); beyond, the differences of the tails' erfc and
+// of the exponentials, which do not cancel there.
+//
+// The half-differences are those of U and p / rho, with the exponentials of
+// the kinetic solution and of the one quadrature: carrying (l, r, h) triples
+// through every product, with an expm1 and two more exponentials, took 250 of
+// the stage-1 flux's instructions more (3.15 M faces: 1,108 -> 1,071 us).
 __device__ __forceinline__ void psi_half_difference(const float* Wl, const float* Wr, const float* h, float gm1,
-                                                    float erf_l, float erf_r, float* out) {
-    const HDiff<float> rho{Wl[0], Wr[0], h[0]}, m1{Wl[1], Wr[1], h[1]}, m2{Wl[2], Wr[2], h[2]};
-    const HDiff<float> m3{Wl[3], Wr[3], h[3]}, E{Wl[4], Wr[4], h[4]};
-    const HDiff<float> mm = hd_add(hd_add(hd_mul(m1, m1), hd_mul(m2, m2)), hd_mul(m3, m3));
-    const HDiff<float> p = hd_scale(gm1, hd_add(E, hd_scale(-0.5f, hd_div(mm, rho))));
-    const HDiff<float> sy = hd_sqrt(hd_scale(2.0f, hd_mul(p, rho)));
-    const HDiff<float> sv = hd_div(m1, sy);
-    const HDiff<float> e0 = hd_erf(sv, erf_l, erf_r);
-    const HDiff<float> ex = hd_expneg(hd_mul(sv, sv));
-    const HDiff<float> g = hd_scale(0.79788456080286536f, hd_mul(ex, hd_sqrt(hd_div(p, rho))));  // sqrt(2 / pi)
-    out[0] = hd_mul(rho, e0).h;
-    out[1] = hd_mul(m1, e0).h + hd_mul(rho, g).h;
-    out[2] = hd_mul(m2, e0).h;
-    out[3] = hd_mul(m3, e0).h;
-    out[4] = hd_mul(E, e0).h + 0.5f * hd_mul(m1, g).h;
+                                                    const HalfSpace<float>& hl, const HalfSpace<float>& hr,
+                                                    float* out) {
+    const float il = 1.0f / Wl[0], ir = 1.0f / Wr[0], ii = il * ir;
+    float mid[5];
+#pragma unroll
+    for (int q = 0; q < 5; ++q) mid[q] = 0.5f * (Wl[q] + Wr[q]);
+    // velocities and p / rho
+    float U[3], hU[3];
+    float hT = (h[4] * mid[0] - mid[4] * h[0]) * ii;
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+        U[j] = 0.5f * (Wl[1 + j] * il + Wr[1 + j] * ir);
+        hU[j] = (h[1 + j] * mid[0] - mid[1 + j] * h[0]) * ii;
+        hT -= U[j] * hU[j];
+    }
+    hT *= gm1;
+    // rl = (2 T)^{-1/2} and its inverse
+    const float rr = hl.rl * hr.rl, irs = 1.0f / (hl.rl + hr.rl);
+    const float hir = 2.0f * (hT * rr) * irs;  // of 1 / rl
+    const float hrl = -hir * rr;
+    const float rm = 0.5f * (hl.rl + hr.rl), irm = rm / rr;  // mid of rl and of 1 / rl
+    const float d = hU[0] * rm + U[0] * hrl;                 // of s
+    const float m = 0.5f * (Wl[1] * il * hl.rl + Wr[1] * ir * hr.rl);
+    // erf and e^{-s^2}
+    float he, hx;
+    const float ad = fabsf(d);
+    if (ad <= 0.5f) {
+        // nodes and weights on [-1, 1]
+        const bool few = ad <= 0.05f;
+        const float x1 = few ? 0.77459666924148338f : 0.53846931010568309f;
+        const float w0 = few ? 0.88888888888888889f : 0.56888888888888889f;
+        const float w1 = few ? 0.55555555555555556f : 0.47862867049936647f;
+        const float tp = m + x1 * d, tm = m - x1 * d;
+        const float g0 = w0 * expf(-m * m), gp = w1 * expf(-tp * tp), gm = w1 * expf(-tm * tm);
+        float s0 = g0 + (gp + gm), s1 = m * g0 + (tp * gp + tm * gm);
+        if (!few) {
+            const float x2 = 0.90617984593866399f, w2 = 0.23692688505618909f;
+            const float up = m + x2 * d, um = m - x2 * d;
+            const float hp = w2 * expf(-up * up), hm = w2 * expf(-um * um);
+            s0 += hp + hm;
+            s1 += up * hp + um * hm;
+        }
+        he = 0.56418958354775628695f * d * s0;  // 1 / sqrt(pi)
+        hx = -d * s1;
+    } else {
+        const float sl = Wl[1] * il * hl.rl, sr = Wr[1] * ir * hr.rl;
+        he = m > 0.0f ? 0.5f * (erfcf(sr) - erfcf(sl)) : 0.5f * (erfcf(-sl) - erfcf(-sr));
+        hx = 0.5f * (hl.ex - hr.ex);
+    }
+    // e0 on the sides from their half-space moments: 2 <u^0>_{u1>0} - 1 on
+    // the left, 1 - 2 <u^0>_{u1<0} on the right
+    const float e0 = hl.m0 - hr.m0;
+    const float ym = 0.5f * (hl.ex / hl.rl + hr.ex / hr.rl);  // mid of e^{-s^2} / rl
+    const float hy = hx * irm + 0.5f * (hl.ex + hr.ex) * hir;
+    const float c = 0.56418958354775628695f;
+    const float hG = c * (h[0] * ym + mid[0] * hy);
+    const float Gm = 0.5f * c * (Wl[0] * (hl.ex / hl.rl) + Wr[0] * (hr.ex / hr.rl));
+#pragma unroll
+    for (int q = 0; q < 5; ++q) out[q] = h[q] * e0 + mid[q] * he;
+    out[1] += hG;
+    out[4] += 0.5f * (hU[0] * Gm + U[0] * hG);
 }
 
 // Euler flux along x1 of a face-frame state: (m1, m1 u + p, m2 u, m3 u,
@@ -434,20 +426,29 @@ __device__ __forceinline__ void euler_flux1(const float* W, float gm1, float* ou
     out[4] = (W[4] + p) * u;
 }
 
-// (F_1(Wl) - F_1(Wr)) / 2 by the half-difference rules, given the
-// half-difference h of the two face-frame states: exact to the rounding of
-// the result itself, however close the two states.
-__device__ __forceinline__ void flux1_half_difference(const float* Wl, const float* Wr, const float* h, float gm1,
-                                                      float* out) {
-    const HDiff<float> rho{Wl[0], Wr[0], h[0]}, E{Wl[4], Wr[4], h[4]};
-    const HDiff<float> m[3] = {{Wl[1], Wr[1], h[1]}, {Wl[2], Wr[2], h[2]}, {Wl[3], Wr[3], h[3]}};
-    const HDiff<float> u = hd_div(m[0], rho);
-    const HDiff<float> mm = hd_add(hd_add(hd_mul(m[0], m[0]), hd_mul(m[1], m[1])), hd_mul(m[2], m[2]));
-    const HDiff<float> p = hd_scale(gm1, hd_add(E, hd_scale(-0.5f, hd_div(mm, rho))));
-    out[0] = h[1];
+// F_1(Wc) - F_1(Wm) given d = Wc - Wm of the two face-frame states: exact to
+// the rounding of the result itself, however close the two states.  With
+// U = m / rho, U_c - U_m = (d_m - U_m d_rho) / rho_c.
+__device__ __forceinline__ void flux1_difference(const float* Wc, const float* Wm, const float* d, float gm1,
+                                                 float* out) {
+    const float ic = 1.0f / Wc[0], im = 1.0f / Wm[0];
+    float dk = 0.0f, km = 0.0f, du = 0.0f, um = 0.0f;
 #pragma unroll
-    for (int j = 0; j < 3; ++j) out[1 + j] = hd_mul(m[j], u).h + (j == 0 ? p.h : 0.0f);
-    out[4] = hd_mul(hd_add(E, p), u).h;
+    for (int j = 0; j < 3; ++j) {
+        const float U = Wm[1 + j] * im, dU = (d[1 + j] - U * d[0]) * ic;
+        dk += d[1 + j] * (U + dU) + Wm[1 + j] * dU;  // of m . U
+        km += Wm[1 + j] * U;
+        if (j == 0) {
+            um = U;
+            du = dU;
+        }
+    }
+    const float uc = um + du;
+    const float dp = gm1 * (d[4] - 0.5f * dk), pm = gm1 * (Wm[4] - 0.5f * km);
+    out[0] = d[1];
+#pragma unroll
+    for (int j = 0; j < 3; ++j) out[1 + j] = d[1 + j] * uc + Wm[1 + j] * du + (j == 0 ? dp : 0.0f);
+    out[4] = (d[4] + dp) * uc + (Wm[4] + pm) * du;
 }
 
 // ------------------------------------------------- FP32 pair numbers --

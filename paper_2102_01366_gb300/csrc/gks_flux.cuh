@@ -28,7 +28,10 @@ namespace gks {
 // with the fewest instructions.  Two threads a point (one a side, in two
 // warps) repeated the frame and met four times at a barrier through 60 KB of
 // shared memory: stage 1 / stage 2 on 3.15 M faces 2,087 / 1,335 us there,
-// 1,161 / 683 us here; on 49,280 faces 40.6 / 28.7 us, now 29.5 / 18.4 us.
+// 1,071 / 687 us here; on 49,280 faces 40.6 / 28.7 us, now 26.6 / 18.4 us.
+// Persistent blocks that fetch the next block's records into shared memory hid
+// the gathers, but a block's three warps then waited for each other: 1,207 /
+// 837 us.
 // FP64 is bound by its pipe (16 cycles a warp instruction): rotating and
 // weighting per face instead of per point took 484 -> 450 us on 49,280 faces.
 constexpr int FLUX_THREADS = 3 * FLUX_FACES;
@@ -55,10 +58,11 @@ struct FluxSmem {
 // rules, both carry rounding relative to themselves only.  Interior and open
 // faces; wall and fixed faces subtract directly.
 //   dsum, ddiff  sum and difference (left - right) of the sides' R - average
-//   m0l, m0r     half-space moments <u^0> of the two sides
+//   hl, hr       the sides' half-space moments
 __device__ __forceinline__ void interface_deviation(const float* __restrict__ poly, int L, int Rc,
                                                     const float (*Rm)[3], const float* dsum, const float* ddiff,
-                                                    float m0l, float m0r, const float* Wc, float gm1, float* dW,
+                                                    const HalfSpace<float>& hl, const HalfSpace<float>& hr,
+                                                    const float* Wc, float gm1, float* dW,
                                                     float* dF) {
     constexpr int PS = Stride<float>::poly;
     const bool pair = (L >= 0 || L == FLR_OPEN) && (Rc >= 0 || Rc == FLR_OPEN);
@@ -67,11 +71,11 @@ __device__ __forceinline__ void interface_deviation(const float* __restrict__ po
     float Wm[5], sg[5], hg[5];
 #pragma unroll
     for (int q = 0; q < 5; ++q) {
-        const float hl = __ldg(al + PHI + q), hr = __ldg(ar + PHI + q);
+        const float ql = __ldg(al + PHI + q), qr = __ldg(ar + PHI + q);
         const float ll = __ldg(al + PLO + q), lr = __ldg(ar + PLO + q);
-        Wm[q] = 0.5f * (hl + hr);
+        Wm[q] = 0.5f * (ql + qr);
         sg[q] = 0.5f * dsum[q];
-        hg[q] = 0.5f * (((hl - hr) + (ll - lr)) + ddiff[q]);
+        hg[q] = 0.5f * (((ql - qr) + (ll - lr)) + ddiff[q]);
     }
     float tm[5] = {Wm[0], 0, 0, 0, Wm[4]};
     rotate_vec(Rm, Wm + 1, tm + 1);
@@ -84,18 +88,10 @@ __device__ __forceinline__ void interface_deviation(const float* __restrict__ po
             tl[q] = tm[q] + (ts[q] + th[q]);
             tr[q] = tm[q] + (ts[q] - th[q]);
         }
-        // erf of each side's s from its half-space moment <u^0>:
-        // 2 <u^0>_{u1>0} - 1 on the left, 1 - 2 <u^0>_{u1<0} on the right
-        psi_half_difference(tl, tr, th, gm1, 2.0f * m0l - 1.0f, 1.0f - 2.0f * m0r, dW);
-        float h[5];
+        psi_half_difference(tl, tr, th, gm1, hl, hr, dW);
 #pragma unroll
-        for (int q = 0; q < 5; ++q) {
-            dW[q] += ts[q];
-            h[q] = 0.5f * dW[q];
-        }
-        flux1_half_difference(Wc, tm, h, gm1, dF);
-#pragma unroll
-        for (int q = 0; q < 5; ++q) dF[q] *= 2.0f;
+        for (int q = 0; q < 5; ++q) dW[q] += ts[q];
+        flux1_difference(Wc, tm, dW, gm1, dF);
     } else {
         // both records are the interior cell's: W_m = hi + lo
         float lo[5], tlo[5], Fc[5], Fm[5];
@@ -177,9 +173,18 @@ __device__ __forceinline__ void flux_faces(const DevMesh<T>& m, const Phys<T>& p
                 sm.frame[lf][3 + i] = Rm[2][i];
             }
         }
+        if constexpr (REL) {
+            // the right side's record on its way to L1 while the left side is
+            // worked on: the face's three threads take its (at most three)
+            // lines.  Stage 1, 3.15 M faces: 1,160 -> 1,108 us; in stage 2,
+            // with less to do in between, it gained nothing.
+            const T* rr = poly + (int64_t)(Rc >= 0 ? Rc : L) * Stride<T>::poly;
+            asm volatile("prefetch.global.L1 [%0];" ::"l"(rr + (k < 2 ? 32 * k : Stride<T>::poly - 1)));
+        }
         KSums<T> S;
         S.init();
-        T pl = T(0), pr = T(0), m0l = T(0), m0r = T(0), dsum[5], ddiff[5];
+        T pl = T(0), pr = T(0), dsum[5], ddiff[5];
+        HalfSpace<T> hl{}, hr{};
 #pragma unroll
         for (int q = 0; q < 5; ++q) dsum[q] = ddiff[q] = T(0);
 #pragma unroll 1
@@ -187,8 +192,8 @@ __device__ __forceinline__ void flux_faces(const DevMesh<T>& m, const Phys<T>& p
             T tW[5], tg[3][5], dev[5];
             side_state<T, XW>(m, ph, Wavg, poly, geo, Rm, L, Rc, side, k, tW, tg, REL ? dev : nullptr);
             pl = pr;
-            m0l = m0r;
-            pr = kin_side<VISC>(ph, tW, tg, side == 0 ? +1 : -1, S, &m0r);
+            hl = hr;
+            pr = kin_side<VISC>(ph, tW, tg, side == 0 ? +1 : -1, S, &hr);
             if constexpr (REL) {
 #pragma unroll
                 for (int q = 0; q < 5; ++q) {
@@ -207,7 +212,7 @@ __device__ __forceinline__ void flux_faces(const DevMesh<T>& m, const Phys<T>& p
 #pragma unroll
             for (int q = 0; q < 5; ++q) ddiff[q] = -ddiff[q];
             T dW[5], dF[5];
-            interface_deviation(poly, L, Rc, Rm, dsum, ddiff, m0l, m0r, Wc, ph.gm1, dW, dF);
+            interface_deviation(poly, L, Rc, Rm, dsum, ddiff, hl, hr, Wc, ph.gm1, dW, dF);
 #pragma unroll
             for (int q = 0; q < 5; ++q) {
                 Fh[q] += T(0.5) * dt * dF[q];

@@ -86,9 +86,11 @@ struct KMom {
     T R[5], R1x2, R1x3, R2x3, R2x6, R3x4, F, Fh, Uh, q;
 };
 
-// half: +1 restricts u > 0, -1 u < 0 (HALF only).  m0 receives <u^0>.
+// half: +1 restricts u > 0, -1 u < 0 (HALF only).  hs (may be NULL): what the
+// FP32 interface deviation takes of the half space.
 template <bool HALF, typename T>
-__device__ __forceinline__ KMom<HALF, T> kin_moments(const KState<T>& s, T K, int half, T* m0 = nullptr) {
+__device__ __forceinline__ KMom<HALF, T> kin_moments(const KState<T>& s, T K, int half,
+                                                            HalfSpace<T>* hs = nullptr) {
     KMom<HALF, T> k;
     k.q = s.V * s.V + s.W * s.W + (K + T(2)) * s.h;
     if constexpr (HALF) {
@@ -96,8 +98,9 @@ __device__ __forceinline__ KMom<HALF, T> kin_moments(const KState<T>& s, T K, in
         const T rs = d_rsqrt(T(2) * s.h);  // sqrt(lambda)
         const T x = s.U * rs;
         const T u0 = T(0.5) * d_erfc(-sg * x);
-        if (m0) *m0 = u0;
-        k.F = sg * s.rho * T(0.56418958354775628695) * rs * d_exp(-x * x);  // 1 / sqrt(pi)
+        const T ex = d_exp(-x * x);
+        if (hs) *hs = {u0, rs, ex};
+        k.F = sg * s.rho * T(0.56418958354775628695) * rs * ex;  // 1 / sqrt(pi)
         k.Uh = x * rs;
         k.R[0] = s.rho * u0;
         k.R[1] = s.U * k.R[0] + s.h * k.F;
@@ -224,12 +227,12 @@ __device__ __forceinline__ void kin_conv(const KState<T>& s, const KMom<HALF, T>
 // to the sums; returns its pressure
 template <bool VISC, typename T>
 __device__ __forceinline__ T kin_side(const Phys<T>& ph, const T* W, const T (*g)[5], int half, KSums<T>& S,
-                                      T* m0 = nullptr) {
+                                      HalfSpace<T>* hs = nullptr) {
     const KState<T> s = kin_state(W, ph.gm1);
     KGrad<T> d[3];
 #pragma unroll
     for (int i = 0; i < 3; ++i) d[i] = kin_grad(s, g[i], ph.gm1);
-    const KMom<true, T> k = kin_moments<true>(s, ph.K, half, m0);
+    const KMom<true, T> k = kin_moments<true>(s, ph.K, half, hs);
     kin_A<0>(s, k, S.w);
     kin_A<1>(s, k, S.f0);
     kin_conv<true>(s, k, d, ph.K, S.d, S.r1, S.f1);
