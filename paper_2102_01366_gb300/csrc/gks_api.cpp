@@ -586,35 +586,39 @@ static gks_status upload_faces(gks_state* s) {
     std::vector<int32_t> cface(4 * nc), flr(2 * nf);
     std::vector<T> fgeo(FGEO * nf, T(0)), fnw(4 * nf);
     std::vector<float> fan(s->L.fan ? 6 * nf : 0, 0.0f);
-    for (int64_t d = 0; d < nc; ++d) {
-        const int64_t c = s->pub(d);
-        for (int f = 0; f < 4; ++f) {
-            const int64_t fi = g.csr_face[c * 4 + f];
-            const bool left = g.csr_sign[c * 4 + f] > 0;
-            cface[f * nc + d] = (int32_t)((int64_t)inv[fi] * 2 + (left ? 0 : 1));
-        }
-    }
-    for (int64_t d = 0; d < nf; ++d) {
-        const int64_t f = perm[d];
-        // a boundary face's missing side carries its kind: -1 - GKS_BC_*
-        const int32_t miss = -1 - (int32_t)g.bkind[f];
-        flr[d] = g.face_lr[f * 2] >= 0 ? (int32_t)s->dev(g.face_lr[f * 2]) : miss;
-        flr[nf + d] = g.face_lr[f * 2 + 1] >= 0 ? (int32_t)s->dev(g.face_lr[f * 2 + 1]) : miss;
-        T* r = &fgeo[d * FGEO];
-        for (int a = 0; a < 3; ++a) r[a] = (T)g.fnorm[f * 3 + a];
-        r[3] = (T)(g.farea[f] / 3.0);
-        for (int a = 0; a < 4; ++a) fnw[d * 4 + a] = r[a];
-        for (int k = 0; k < 9; ++k) {
-            r[4 + k] = (T)g.gp_l[f * 9 + k];
-            r[13 + k] = (T)g.gp_r[f * 9 + k];
-        }
-        if (!fan.empty())
-            for (int a = 0; a < 3; ++a) {
-                const double v = g.farea[f] * g.fnorm[f * 3 + a];
-                fan[d * 6 + 2 * a] = (float)v;
-                fan[d * 6 + 2 * a + 1] = (float)(v - (double)(float)v);
+    run_ranges(nc, host_threads(nc), [&](int64_t, int64_t lo, int64_t hi) {
+        for (int64_t d = lo; d < hi; ++d) {
+            const int64_t c = s->pub(d);
+            for (int f = 0; f < 4; ++f) {
+                const int64_t fi = g.csr_face[c * 4 + f];
+                const bool left = g.csr_sign[c * 4 + f] > 0;
+                cface[f * nc + d] = (int32_t)((int64_t)inv[fi] * 2 + (left ? 0 : 1));
             }
-    }
+        }
+    });
+    run_ranges(nf, host_threads(nf), [&](int64_t, int64_t lo, int64_t hi) {
+        for (int64_t d = lo; d < hi; ++d) {
+            const int64_t f = perm[d];
+            // a boundary face's missing side carries its kind: -1 - GKS_BC_*
+            const int32_t miss = -1 - (int32_t)g.bkind[f];
+            flr[d] = g.face_lr[f * 2] >= 0 ? (int32_t)s->dev(g.face_lr[f * 2]) : miss;
+            flr[nf + d] = g.face_lr[f * 2 + 1] >= 0 ? (int32_t)s->dev(g.face_lr[f * 2 + 1]) : miss;
+            T* r = &fgeo[d * FGEO];
+            for (int a = 0; a < 3; ++a) r[a] = (T)g.fnorm[f * 3 + a];
+            r[3] = (T)(g.farea[f] / 3.0);
+            for (int a = 0; a < 4; ++a) fnw[d * 4 + a] = r[a];
+            for (int k = 0; k < 9; ++k) {
+                r[4 + k] = (T)g.gp_l[f * 9 + k];
+                r[13 + k] = (T)g.gp_r[f * 9 + k];
+            }
+            if (!fan.empty())
+                for (int a = 0; a < 3; ++a) {
+                    const double v = g.farea[f] * g.fnorm[f * 3 + a];
+                    fan[d * 6 + 2 * a] = (float)v;
+                    fan[d * 6 + 2 * a + 1] = (float)(v - (double)(float)v);
+                }
+        }
+    });
     auto put = [&](size_t off, const void* src, size_t bytes) -> cudaError_t {
         return cudaMemcpyAsync(s->ws + off, src, bytes, cudaMemcpyHostToDevice, s->stream);
     };
@@ -650,50 +654,53 @@ static gks_status upload_cells(gks_state* s) {
     std::vector<TO> wop((size_t)L.nwall * WOP_STRIDE, TO(0));
     int64_t nwop = 0;
     // d: device cell; c: the caller's cell it holds
-    for (int64_t d = 0; d < nc; ++d) {
+    for (int64_t d = 0; L.wslot && d < nc; ++d) {
         const int64_t c = s->pub(d);
-        cell_case[d] = g.cell_case[c];
-        TO* tc = &tile[(size_t)(d / CELLS_PER_BLOCK) * TILE_ROWS * CELLS_PER_BLOCK];
-        const int lc = (int)(d % CELLS_PER_BLOCK);
-        auto put_row = [&](int row, double v) { tc[tile_at<TO>(row, lc)] = (TO)v; };
-        double far[3] = {0.0, 0.0, 0.0};
-        for (int f = 0; f < 4; ++f) {
-            nbr[f * nc + d] = g.nbr[c * 4 + f] >= 0 ? (int32_t)s->dev(g.nbr[c * 4 + f]) : -1;
-            const int64_t fi = g.csr_face[c * 4 + f];
-            const bool left = g.csr_sign[c * 4 + f] > 0;
-            const double* gp = left ? &g.gp_l[fi * 9] : &g.gp_r[fi * 9];
-            for (int k = 0; k < 9; ++k) {
-                put_row(TILE_G + f * 9 + k, gp[k]);
-                far[k % 3] = std::max(far[k % 3], std::abs(gp[k]));
-            }
+        double w2[153], w1[15];
+        if (has_wall_face(g, c) && cell_wall_stencil(g, c, w2, w1)) {
+            wslot[d] = (int32_t)(nwop++);
+            TO* o = &wop[(size_t)wslot[d] * WOP_STRIDE];
+            for (int k = 0; k < 153; ++k) o[k] = (TO)w2[k];
+            for (int k = 0; k < 15; ++k) o[WOP_W1 + k] = (TO)w1[k];
         }
-        inv_vol[d] = 1.0 / g.vol[c];
-        for (int k = 0; k < 3; ++k) put_row(TILE_BND + k, far[k]);
-        put_row(TILE_V23, std::pow(g.vol[c], 2.0 / 3.0));
-        put_row(TILE_V43, std::pow(g.vol[c], 4.0 / 3.0));
-        dr[d] = (T)g.dr[c];
-        for (int q = 0; q < 6; ++q) put_row(TILE_MOM + q, g.mom2[c * 6 + q]);
-        for (int k = 0; k < 12; ++k) {
-            M1[k * nc + d] = (TO)g.M1[c * 12 + k];
-            put_row(TILE_M1 + k, g.M1[c * 12 + k]);
-        }
-        if (L.wslot) {
-            double w2[153], w1[15];
-            if (has_wall_face(g, c) && cell_wall_stencil(g, c, w2, w1)) {
-                wslot[d] = (int32_t)(nwop++);
-                TO* o = &wop[(size_t)wslot[d] * WOP_STRIDE];
-                for (int k = 0; k < 153; ++k) o[k] = (TO)w2[k];
-                for (int k = 0; k < 15; ++k) o[WOP_W1 + k] = (TO)w1[k];
-            }
-        }
-        const double* M2c = &g.M2[c * 144];
-        double M2lin[144];
-        if (linear_boundary && !g.singular[c] &&
-            (g.nbr[c * 4] < 0 || g.nbr[c * 4 + 1] < 0 || g.nbr[c * 4 + 2] < 0 || g.nbr[c * 4 + 3] < 0) &&
-            cell_linear_fit(g, c, M2lin))
-            M2c = M2lin;
-        for (int k = 0; k < 144; ++k) put_row(TILE_M2 + k, M2c[k]);
     }
+    run_ranges(nc, host_threads(nc), [&](int64_t, int64_t lo, int64_t hi) {
+        for (int64_t d = lo; d < hi; ++d) {
+            const int64_t c = s->pub(d);
+            cell_case[d] = g.cell_case[c];
+            TO* tc = &tile[(size_t)(d / CELLS_PER_BLOCK) * TILE_ROWS * CELLS_PER_BLOCK];
+            const int lc = (int)(d % CELLS_PER_BLOCK);
+            auto put_row = [&](int row, double v) { tc[tile_at<TO>(row, lc)] = (TO)v; };
+            double far[3] = {0.0, 0.0, 0.0};
+            for (int f = 0; f < 4; ++f) {
+                nbr[f * nc + d] = g.nbr[c * 4 + f] >= 0 ? (int32_t)s->dev(g.nbr[c * 4 + f]) : -1;
+                const int64_t fi = g.csr_face[c * 4 + f];
+                const bool left = g.csr_sign[c * 4 + f] > 0;
+                const double* gp = left ? &g.gp_l[fi * 9] : &g.gp_r[fi * 9];
+                for (int k = 0; k < 9; ++k) {
+                    put_row(TILE_G + f * 9 + k, gp[k]);
+                    far[k % 3] = std::max(far[k % 3], std::abs(gp[k]));
+                }
+            }
+            inv_vol[d] = 1.0 / g.vol[c];
+            for (int k = 0; k < 3; ++k) put_row(TILE_BND + k, far[k]);
+            put_row(TILE_V23, std::pow(g.vol[c], 2.0 / 3.0));
+            put_row(TILE_V43, std::pow(g.vol[c], 4.0 / 3.0));
+            dr[d] = (T)g.dr[c];
+            for (int q = 0; q < 6; ++q) put_row(TILE_MOM + q, g.mom2[c * 6 + q]);
+            for (int k = 0; k < 12; ++k) {
+                M1[k * nc + d] = (TO)g.M1[c * 12 + k];
+                put_row(TILE_M1 + k, g.M1[c * 12 + k]);
+            }
+            const double* M2c = &g.M2[c * 144];
+            double M2lin[144];
+            if (linear_boundary && !g.singular[c] &&
+                (g.nbr[c * 4] < 0 || g.nbr[c * 4 + 1] < 0 || g.nbr[c * 4 + 2] < 0 || g.nbr[c * 4 + 3] < 0) &&
+                cell_linear_fit(g, c, M2lin))
+                M2c = M2lin;
+            for (int k = 0; k < 144; ++k) put_row(TILE_M2 + k, M2c[k]);
+        }
+    });
     auto put = [&](size_t off, const void* src, size_t bytes) -> cudaError_t {
         return cudaMemcpyAsync(s->ws + off, src, bytes, cudaMemcpyHostToDevice, s->stream);
     };
@@ -781,12 +788,17 @@ extern "C" gks_status gks_state_create(const gks_mesh* mesh, const gks_params* p
         s->own_stream = true;
     }
     gks_status st;
-    if (fp32) {
-        make_views<float>(s, s->m32, s->s32);
-        st = upload_mesh<float>(s);
-    } else {
-        make_views<double>(s, s->m64, s->s64);
-        st = upload_mesh<double>(s);
+    try {
+        if (fp32) {
+            make_views<float>(s, s->m32, s->s32);
+            st = upload_mesh<float>(s);
+        } else {
+            make_views<double>(s, s->m64, s->s64);
+            st = upload_mesh<double>(s);
+        }
+    } catch (const std::bad_alloc&) {
+        set_error("gks_state_create: out of memory");
+        st = GKS_E_NOMEM;
     }
     if (st != GKS_OK) {
         if (s->own_stream) cudaStreamDestroy(s->stream);

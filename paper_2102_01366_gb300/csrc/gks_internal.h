@@ -2,9 +2,12 @@
 // libgks (mesh setup, stencil construction, device state).
 #pragma once
 
+#include <algorithm>
 #include <cstddef>
 #include <cstdint>
 #include <string>
+#include <system_error>
+#include <thread>
 #include <vector>
 
 #include "../../include/gks.h"
@@ -45,4 +48,30 @@ bool cell_linear_fit(const gks_mesh& m, int64_t c, double* M2);  // boundary cel
 // faces (see gks_stencil.cpp); false when it has none or they cannot be built
 bool cell_wall_stencil(const gks_mesh& m, int64_t c, double* W2, double* W1);
 bool has_wall_face(const gks_mesh& m, int64_t c);
+
+// threads for a loop over n cells or faces
+inline int64_t host_threads(int64_t n) {
+    const unsigned hw = std::max(1u, std::thread::hardware_concurrency());
+    return std::min<int64_t>((int64_t)hw, std::max<int64_t>(1, n / 16384));
+}
+
+// fn(t, lo, hi) over nthr contiguous ranges of [0, n); range 0 on the calling
+// thread, and any range whose thread cannot be started runs inline too
+template <typename Fn>
+void run_ranges(int64_t n, int64_t nthr, Fn fn) {
+    const int64_t chunk = (n + nthr - 1) / nthr;
+    std::vector<std::thread> pool;
+    pool.reserve((size_t)nthr);
+    for (int64_t t = 1; t < nthr; ++t) {
+        const int64_t lo = std::min(n, t * chunk), hi = std::min(n, (t + 1) * chunk);
+        try {
+            pool.emplace_back(fn, t, lo, hi);
+        } catch (const std::system_error&) {
+            fn(t, lo, hi);
+        }
+    }
+    fn((int64_t)0, (int64_t)0, std::min(n, chunk));
+    for (auto& th : pool) th.join();
+}
+
 }  // namespace gks

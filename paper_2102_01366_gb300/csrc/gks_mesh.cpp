@@ -87,30 +87,6 @@ struct HalfFace {
     Side side;
 };
 
-int64_t host_threads(int64_t n) {
-    const unsigned hw = std::max(1u, std::thread::hardware_concurrency());
-    return std::min<int64_t>((int64_t)hw, std::max<int64_t>(1, n / 16384));
-}
-
-// fn(t, lo, hi) over nthr contiguous ranges of [0, n); range 0 on the calling
-// thread, and any range whose thread cannot be started runs inline too
-template <typename Fn>
-void run_ranges(int64_t n, int64_t nthr, Fn fn) {
-    const int64_t chunk = (n + nthr - 1) / nthr;
-    std::vector<std::thread> pool;
-    pool.reserve((size_t)nthr);
-    for (int64_t t = 1; t < nthr; ++t) {
-        const int64_t lo = std::min(n, t * chunk), hi = std::min(n, (t + 1) * chunk);
-        try {
-            pool.emplace_back(fn, t, lo, hi);
-        } catch (const std::system_error&) {
-            fn(t, lo, hi);
-        }
-    }
-    fn((int64_t)0, (int64_t)0, std::min(n, chunk));
-    for (auto& th : pool) th.join();
-}
-
 // The first failure of a parallel loop: the smallest index at which one was
 // found, and its message (set_error is per thread, so workers only record).
 struct FirstError {
