@@ -829,17 +829,12 @@ static gks_status init_impl(gks_state* s, DevMesh<T>& m, DevState<T>& st, const 
                             const double* d_dW) {
     s->stage_valid = false;
     const int64_t nc = m.nc;
-    if (s->dperm())
-        GKS_CHECK_CUDA(launch_cells_perm(d_W, st.Wd, nc, 5, s->dperm(), 0, s->stream));
-    else
-        GKS_CHECK_CUDA(cudaMemcpyAsync(st.Wd, d_W, 8 * 5 * nc, cudaMemcpyDeviceToDevice, s->stream));
-    GKS_CHECK_CUDA(Launch<T>::pack(d_W, d_dW, st.X, nc, s->stream, s->dperm()));
+    GKS_CHECK_CUDA(launch_set_control(st.ctrl, st.case_t, st.case_dt, st.case_dtmin, m.ncase, 0.0, 0.0, 1, st.err,
+                                      s->stream));
+    GKS_CHECK_CUDA(Launch<T>::pack(m, s->phys, d_W, d_dW, st.X, st.Wd, st.case_dtmin, s->stream, s->dperm()));
     if (m.fixed && !s->fixed_pinned)  // fixed boundaries hold the initial state
         GKS_CHECK_CUDA(cudaMemcpyAsync((void*)m.fixed, st.X, sizeof(T) * Stride<T>::xs * nc, cudaMemcpyDeviceToDevice,
                                        s->stream));
-    GKS_CHECK_CUDA(launch_set_control(st.ctrl, st.case_t, st.case_dt, st.case_dtmin, m.ncase, 0.0, 0.0, 1, s->stream));
-    GKS_CHECK_CUDA(cudaMemsetAsync(st.err, 0, 4, s->stream));
-    GKS_CHECK_CUDA(Launch<T>::init_dtmin(m, s->phys, st.X, st.case_dtmin, s->stream));
     return GKS_OK;
 }
 
@@ -849,9 +844,11 @@ extern "C" gks_status gks_set_fixed_state(gks_state* s, const double* d_W, const
     order_after_caller(s);
     const int64_t nc = s->mesh->nc;
     if (s->fp32)
-        GKS_CHECK_CUDA(Launch<float>::pack(d_W, d_dW, const_cast<float*>(s->m32.fixed), nc, s->stream, s->dperm()));
+        GKS_CHECK_CUDA(Launch<float>::pack(s->m32, s->phys, d_W, d_dW, const_cast<float*>(s->m32.fixed), nullptr, nullptr,
+                                           s->stream, s->dperm()));
     else
-        GKS_CHECK_CUDA(Launch<double>::pack(d_W, d_dW, const_cast<double*>(s->m64.fixed), nc, s->stream));
+        GKS_CHECK_CUDA(Launch<double>::pack(s->m64, s->phys, d_W, d_dW, const_cast<double*>(s->m64.fixed), nullptr, nullptr,
+                                            s->stream));
     s->fixed_pinned = true;
     GKS_CHECK_CUDA(cudaStreamSynchronize(s->stream));
     return GKS_OK;
@@ -912,9 +909,9 @@ static cudaError_t enqueue_step(gks_state* s, DevMesh<T>& m, DevState<T>& st) {
 static cudaError_t set_control(gks_state* s, double dt_fixed, double t_end, int reset) {
     if (s->fp32)
         return launch_set_control(s->s32.ctrl, s->s32.case_t, s->s32.case_dt, s->s32.case_dtmin, s->mesh->ncase,
-                                  dt_fixed, t_end, reset, s->stream);
+                                  dt_fixed, t_end, reset, nullptr, s->stream);
     return launch_set_control(s->s64.ctrl, s->s64.case_t, s->s64.case_dt, s->s64.case_dtmin, s->mesh->ncase,
-                              dt_fixed, t_end, reset, s->stream);
+                              dt_fixed, t_end, reset, nullptr, s->stream);
 }
 
 static gks_status build_graph(gks_state* s) {
@@ -1051,13 +1048,7 @@ extern "C" gks_status gks_sync(gks_state* s) {
 
 template <typename T>
 static gks_status get_impl(gks_state* s, DevState<T>& st, int64_t nc, double* d_W, double* d_dW) {
-    if (d_W) {
-        if (s->dperm())
-            GKS_CHECK_CUDA(launch_cells_perm(st.Wd, d_W, nc, 5, s->dperm(), 1, s->stream));
-        else
-            GKS_CHECK_CUDA(cudaMemcpyAsync(d_W, st.Wd, 8 * 5 * nc, cudaMemcpyDeviceToDevice, s->stream));
-    }
-    if (d_dW) GKS_CHECK_CUDA(Launch<T>::unpack_grad(st.X, d_dW, nc, s->stream, s->dperm()));
+    if (d_W || d_dW) GKS_CHECK_CUDA(Launch<T>::unpack(st.Wd, st.X, d_W, d_dW, nc, s->stream, s->dperm()));
     return GKS_OK;
 }
 
@@ -1101,32 +1092,21 @@ static gks_status step_host_impl(gks_state* s, DevMesh<T>& m, DevState<T>& st, c
                                  double* h_dW_out) {
     const int64_t nc = m.nc;
     double* stage = at<double>(s, s->L.stage);
-    if (s->dperm()) {
-        // the caller's order in the staging buffer, then into device order
-        GKS_CHECK_CUDA(cudaMemcpyAsync(stage + 15 * nc, h_W, 8 * 5 * nc, cudaMemcpyHostToDevice, s->stream));
-        GKS_CHECK_CUDA(launch_cells_perm(stage + 15 * nc, st.Wd, nc, 5, s->dperm(), 0, s->stream));
-        GKS_CHECK_CUDA(cudaMemcpyAsync(stage, h_dW, 8 * 15 * nc, cudaMemcpyHostToDevice, s->stream));
-        GKS_CHECK_CUDA(Launch<T>::pack(stage + 15 * nc, stage, st.X, nc, s->stream, s->dperm()));
-    } else {
-        GKS_CHECK_CUDA(cudaMemcpyAsync(st.Wd, h_W, 8 * 5 * nc, cudaMemcpyHostToDevice, s->stream));
-        GKS_CHECK_CUDA(cudaMemcpyAsync(stage, h_dW, 8 * 15 * nc, cudaMemcpyHostToDevice, s->stream));
-        GKS_CHECK_CUDA(Launch<T>::pack(st.Wd, stage, st.X, nc, s->stream));
-    }
+    // averages: with a cell ordering through the staging buffer, else in place
+    double* in = s->dperm() ? stage + 15 * nc : st.Wd;
+    GKS_CHECK_CUDA(cudaMemcpyAsync(in, h_W, 8 * 5 * nc, cudaMemcpyHostToDevice, s->stream));
+    GKS_CHECK_CUDA(cudaMemcpyAsync(stage, h_dW, 8 * 15 * nc, cudaMemcpyHostToDevice, s->stream));
+    GKS_CHECK_CUDA(set_control(s, 0.0, 0.0, 1));
+    GKS_CHECK_CUDA(Launch<T>::pack(m, s->phys, in, stage, st.X, s->dperm() ? st.Wd : nullptr, st.case_dtmin, s->stream,
+                                   s->dperm()));
     if (m.fixed && !s->fixed_pinned)
         GKS_CHECK_CUDA(cudaMemcpyAsync((void*)m.fixed, st.X, sizeof(T) * Stride<T>::xs * nc, cudaMemcpyDeviceToDevice,
                                        s->stream));
-    GKS_CHECK_CUDA(set_control(s, 0.0, 0.0, 1));
-    GKS_CHECK_CUDA(Launch<T>::init_dtmin(m, s->phys, st.X, st.case_dtmin, s->stream));
     s->initialised = true;
     gks_status r = gks_step(s, nsteps, dt_fixed, 0.0);
     if (r != GKS_OK) return r;
-    if (s->dperm()) {
-        GKS_CHECK_CUDA(launch_cells_perm(st.Wd, stage + 15 * nc, nc, 5, s->dperm(), 1, s->stream));
-        GKS_CHECK_CUDA(cudaMemcpyAsync(h_W_out, stage + 15 * nc, 8 * 5 * nc, cudaMemcpyDeviceToHost, s->stream));
-    } else {
-        GKS_CHECK_CUDA(cudaMemcpyAsync(h_W_out, st.Wd, 8 * 5 * nc, cudaMemcpyDeviceToHost, s->stream));
-    }
-    GKS_CHECK_CUDA(Launch<T>::unpack_grad(st.X, stage, nc, s->stream, s->dperm()));
+    GKS_CHECK_CUDA(Launch<T>::unpack(st.Wd, st.X, s->dperm() ? in : nullptr, stage, nc, s->stream, s->dperm()));
+    GKS_CHECK_CUDA(cudaMemcpyAsync(h_W_out, in, 8 * 5 * nc, cudaMemcpyDeviceToHost, s->stream));
     GKS_CHECK_CUDA(cudaMemcpyAsync(h_dW_out, stage, 8 * 15 * nc, cudaMemcpyDeviceToHost, s->stream));
     return gks_sync(s);
 }
@@ -1270,7 +1250,7 @@ static gks_status adjoint_impl(gks_state* s, double dt, const double* d_W, const
     GKS_CHECK_CUDA(cudaMemcpyAsync(poly1, st.poly, 8 * POLY_STRIDE * nc, cudaMemcpyDeviceToDevice, s->stream));
     if (d_Ws) {
         // the caller's stage state in place of the stage-1 flux and update
-        GKS_CHECK_CUDA(Launch<double>::pack(d_Ws, d_dWs, st.Xs, nc, s->stream));
+        GKS_CHECK_CUDA(Launch<double>::pack(m, s->phys, d_Ws, d_dWs, st.Xs, nullptr, nullptr, s->stream));
     } else {
         GKS_CHECK_CUDA(Launch<double>::flux(m, s->phys, st.X, st.poly, st.rec, st.case_dt, 0.0, 1, s->stream,
                                             s->flux_variant));
@@ -1319,8 +1299,7 @@ extern "C" gks_status gks_get_stage_state(gks_state* s, double* d_Ws, double* d_
     if (!s || !d_Ws || !d_dWs) { set_error("gks_get_stage_state: NULL argument"); return GKS_E_ARG; }
     if (s->fp32) { set_error("gks_get_stage_state: FP64 states only"); return GKS_E_UNSUPPORTED; }
     if (!s->stage_valid) { set_error("gks_get_stage_state: no step since the initialisation"); return GKS_E_STATE; }
-    GKS_CHECK_CUDA(launch_unpack_avg(s->s64.Xs, d_Ws, s->mesh->nc, s->stream));
-    GKS_CHECK_CUDA(Launch<double>::unpack_grad(s->s64.Xs, d_dWs, s->mesh->nc, s->stream));
+    GKS_CHECK_CUDA(Launch<double>::unpack(nullptr, s->s64.Xs, d_Ws, d_dWs, s->mesh->nc, s->stream));
     return gks_sync(s);
 }
 

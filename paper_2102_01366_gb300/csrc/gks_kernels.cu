@@ -7,7 +7,7 @@
 //   k_update2  W^{n+1}, grad W^{n+1}; per-case minima of the next step's
 //              local time-step limits (Sec. 5) and residual sums
 //   k_dt_*     time-step rule of Sec. 5 (deterministic per-block minima)
-//   k_pack / k_unpack_grad   public [component][cell] FP64 state <-> the
+//   k_pack / k_unpack   public [component][cell] FP64 state <-> the
 //              cell-major working state
 //
 // No atomics on data: every sum has a fixed order, so results are
@@ -21,8 +21,7 @@
 
 namespace gks {
 
-constexpr int DT_THREADS = 128;    // threads (cells) a block of k_init_dtmin
-constexpr int PACK_THREADS = 128;  // threads (cells) a block of k_pack, k_unpack_grad
+constexpr int PACK_THREADS = 128;  // threads (cells) a block of k_pack, k_unpack
 
 template <typename T>
 __global__ void __launch_bounds__(CELL_THREADS) k_update1(DevMesh<T> m, DevState<T> st) {
@@ -57,21 +56,12 @@ __global__ void __launch_bounds__(32) k_dt_partials(DevMesh<T> m, DtPhys<T> p, c
     if (threadIdx.x == 0) part[(int64_t)blockIdx.x * PART_N + PART_DTMIN] = (double)mn;
 }
 
-template <typename T>
-__global__ void __launch_bounds__(DT_THREADS) k_init_dtmin(DevMesh<T> m, DtPhys<T> p, const T* __restrict__ X,
-                                                           unsigned long long* __restrict__ dtmin) {
-    const int64_t c0 = (int64_t)blockIdx.x * DT_THREADS + threadIdx.x;
-    const int64_t c = c0 < m.nc ? c0 : m.nc - 1;
-    T mn = T(INFINITY);
-    if (c0 < m.nc) mn = cell_dt(m, p, X, c);
-    warp_case_min(mn, m.cell_case[c], dtmin);
-}
-
 __global__ void k_set_control(double* ctrl, double* case_t, double* case_dt, unsigned long long* dtmin,
-                              int32_t ncase, double dt_fixed, double t_end, int reset) {
+                              int32_t ncase, double dt_fixed, double t_end, int reset, int32_t* err) {
     if (threadIdx.x == 0 && blockIdx.x == 0) {
         ctrl[CTRL_DT_FIXED] = dt_fixed;
         ctrl[CTRL_T_END] = t_end;
+        if (err) *err = 0;
     }
     if (reset)
         for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < ncase; k += gridDim.x * blockDim.x) {
@@ -91,14 +81,23 @@ __global__ void k_convert(const A* __restrict__ in, B* __restrict__ out, int64_t
 // (written) in full lines, records as 16-byte vectors.  cperm (may be NULL):
 // device cell -> the caller's cell of W, dW.  Bound by memory: with one thread
 // per word of the record, each reading another row, an initialisation and a
-// read-back of 1.57 M cells in FP32 took about 1.17 ms, now 0.40 ms.
+// read-back of 1.57 M cells in FP32 took about 1.17 ms, 0.40 ms this way.
+//
+// k_pack also writes (where not NULL) the FP64 master averages Wd and each
+// case's minimum of the local time-step limits into dtmin; k_unpack takes the
+// averages from Wd (NULL: from the FP64 working state): one launch each, where
+// copies, conversions, a memset and a kernel for the minima were five and two
+// (a run of two steps on 24,576 cells in FP32, start to end: 277 -> 261 us).
 template <typename T>
-__global__ void __launch_bounds__(PACK_THREADS) k_pack(const double* __restrict__ W, const double* __restrict__ dW,
-                                                       T* __restrict__ X, int64_t nc,
+__global__ void __launch_bounds__(PACK_THREADS) k_pack(DevMesh<T> m, DtPhys<T> p, const double* __restrict__ W,
+                                                       const double* __restrict__ dW, T* __restrict__ X,
+                                                       double* __restrict__ Wd,
+                                                       unsigned long long* __restrict__ dtmin,
                                                        const int32_t* __restrict__ cperm) {
     constexpr int XSR = Stride<T>::xs;
-    const int64_t d = (int64_t)blockIdx.x * PACK_THREADS + threadIdx.x;
-    if (d >= nc) return;
+    const int64_t nc = m.nc, d0 = (int64_t)blockIdx.x * PACK_THREADS + threadIdx.x;
+    const bool active = d0 < nc;
+    const int64_t d = active ? d0 : nc - 1;
     const int64_t c = cperm ? (int64_t)cperm[d] : d;
     T x[XSR];
 #pragma unroll
@@ -106,6 +105,7 @@ __global__ void __launch_bounds__(PACK_THREADS) k_pack(const double* __restrict_
 #pragma unroll
     for (int q = 0; q < 5; ++q) {
         const double w = W[q * nc + c];
+        if (Wd && active) Wd[q * nc + d] = w;
         if constexpr (sizeof(T) == 4)
             split_pair(w, x[q], x[XLO + q]);
         else
@@ -118,36 +118,26 @@ __global__ void __launch_bounds__(PACK_THREADS) k_pack(const double* __restrict_
         else
             x[Stride<T>::xg + j] = dW[j * nc + c];
     }
-    store_vec<XSR>(X + d * XSR, x);
+    if (active) store_vec<XSR>(X + d * XSR, x);
+    if (dtmin) warp_case_min(active ? local_dt(x, m.dr[d], p) : T(INFINITY), m.cell_case[d], dtmin);
 }
 
 template <typename T>
-__global__ void __launch_bounds__(PACK_THREADS) k_unpack_grad(const T* __restrict__ X, double* __restrict__ dW,
-                                                              int64_t nc, const int32_t* __restrict__ cperm) {
+__global__ void __launch_bounds__(PACK_THREADS) k_unpack(const double* __restrict__ Wd, const T* __restrict__ X,
+                                                         double* __restrict__ W, double* __restrict__ dW,
+                                                         int64_t nc, const int32_t* __restrict__ cperm) {
     constexpr int XSR = Stride<T>::xs;
     const int64_t d = (int64_t)blockIdx.x * PACK_THREADS + threadIdx.x;
     if (d >= nc) return;
     const int64_t c = cperm ? (int64_t)cperm[d] : d;
-    constexpr int A = sizeof(T) == 4 ? 12 : 4;  // the aligned start of the gradients' vectors
-    T x[XSR - A];
-    load_vec<XSR - A>(X + d * XSR + A, x);
+    T x[XSR];
+    if (dW || !Wd) load_vec<XSR>(X + d * XSR, x);
+    if (W)
 #pragma unroll
-    for (int j = 0; j < 15; ++j) dW[j * nc + c] = widen(x[Stride<T>::xg - A + j]);
-}
-
-// the averages of an FP64 working state [nc][XS] to W [5][nc]
-__global__ void k_unpack_avg(const double* __restrict__ X, double* __restrict__ W, int64_t nc) {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nc * 5; i += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t q = i / nc, c = i - q * nc;
-        W[q * nc + c] = X[c * Stride<double>::xs + q];
-    }
-}
-
-cudaError_t launch_unpack_avg(const double* X, double* W, int64_t nc, cudaStream_t s) {
-    if (nc == 0) return cudaSuccess;
-    const int64_t blocks = std::min<int64_t>((5 * nc + 255) / 256, 65535);
-    k_unpack_avg<<<(unsigned)blocks, 256, 0, s>>>(X, W, nc);
-    return cudaGetLastError();
+        for (int q = 0; q < 5; ++q) W[q * nc + c] = Wd ? Wd[q * nc + d] : widen(x[q]);
+    if (dW)
+#pragma unroll
+        for (int j = 0; j < 15; ++j) dW[j * nc + c] = widen(x[Stride<T>::xg + j]);
 }
 
 // component-major [ncomp][nc] arrays between the device cell order and the
@@ -252,30 +242,23 @@ cudaError_t Launch<T>::dt_partials(const DevMesh<T>& m, const HostPhys& p, const
     return cudaGetLastError();
 }
 
-template <typename T>
-cudaError_t Launch<T>::init_dtmin(const DevMesh<T>& m, const HostPhys& p, const T* X,
-                                  unsigned long long* case_dtmin, cudaStream_t s) {
-    if (m.nc == 0) return cudaSuccess;
-    k_init_dtmin<T><<<(unsigned)((m.nc + DT_THREADS - 1) / DT_THREADS), DT_THREADS, 0, s>>>(m, DtPhys<T>(p), X, case_dtmin);
-    return cudaGetLastError();
-}
-
 static inline unsigned pack_grid(int64_t nc) { return (unsigned)((nc + PACK_THREADS - 1) / PACK_THREADS); }
 
 static inline unsigned ew_grid(int64_t n) { return (unsigned)((n + 255) / 256 < 8192 ? (n + 255) / 256 : 8192); }
 
 template <typename T>
-cudaError_t Launch<T>::pack(const double* W, const double* dW, T* X, int64_t nc, cudaStream_t s,
-                            const int32_t* cperm) {
-    if (nc == 0) return cudaSuccess;
-    k_pack<T><<<pack_grid(nc), PACK_THREADS, 0, s>>>(W, dW, X, nc, cperm);
+cudaError_t Launch<T>::pack(const DevMesh<T>& m, const HostPhys& p, const double* W, const double* dW, T* X,
+                            double* Wd, unsigned long long* dtmin, cudaStream_t s, const int32_t* cperm) {
+    if (m.nc == 0) return cudaSuccess;
+    k_pack<T><<<pack_grid(m.nc), PACK_THREADS, 0, s>>>(m, DtPhys<T>(p), W, dW, X, Wd, dtmin, cperm);
     return cudaGetLastError();
 }
 
 template <typename T>
-cudaError_t Launch<T>::unpack_grad(const T* X, double* dW, int64_t nc, cudaStream_t s, const int32_t* cperm) {
+cudaError_t Launch<T>::unpack(const double* Wd, const T* X, double* W, double* dW, int64_t nc, cudaStream_t s,
+                              const int32_t* cperm) {
     if (nc == 0) return cudaSuccess;
-    k_unpack_grad<T><<<pack_grid(nc), PACK_THREADS, 0, s>>>(X, dW, nc, cperm);
+    k_unpack<T><<<pack_grid(nc), PACK_THREADS, 0, s>>>(Wd, X, W, dW, nc, cperm);
     return cudaGetLastError();
 }
 
@@ -330,10 +313,11 @@ cudaError_t Launch<T>::poly_to_double(const T* in, double* out, int64_t nc, cuda
 }
 
 cudaError_t launch_set_control(double* ctrl, double* case_t, double* case_dt, unsigned long long* case_dtmin,
-                               int32_t ncase, double dt_fixed, double t_end, int reset_time, cudaStream_t s) {
+                               int32_t ncase, double dt_fixed, double t_end, int reset_time, int32_t* err,
+                               cudaStream_t s) {
     const int grid = reset_time ? (int)((ncase + 255) / 256 < 1024 ? (ncase + 255) / 256 : 1024) : 1;
     k_set_control<<<grid < 1 ? 1 : grid, 256, 0, s>>>(ctrl, case_t, case_dt, case_dtmin, ncase, dt_fixed,
-                                                      t_end, reset_time);
+                                                      t_end, reset_time, err);
     return cudaGetLastError();
 }
 
@@ -345,11 +329,10 @@ cudaError_t launch_set_control(double* ctrl, double* case_t, double* case_dt, un
                                             cudaStream_t);                                                  \
     template cudaError_t Launch<T>::dt_partials(const DevMesh<T>&, const HostPhys&, const T*, double*,      \
                                                 cudaStream_t);                                              \
-    template cudaError_t Launch<T>::init_dtmin(const DevMesh<T>&, const HostPhys&, const T*,                \
-                                               unsigned long long*, cudaStream_t);                          \
-    template cudaError_t Launch<T>::pack(const double*, const double*, T*, int64_t, cudaStream_t,           \
-                                         const int32_t*);                                                   \
-    template cudaError_t Launch<T>::unpack_grad(const T*, double*, int64_t, cudaStream_t, const int32_t*);  \
+    template cudaError_t Launch<T>::pack(const DevMesh<T>&, const HostPhys&, const double*, const double*, T*, \
+                                         double*, unsigned long long*, cudaStream_t, const int32_t*);       \
+    template cudaError_t Launch<T>::unpack(const double*, const T*, double*, double*, int64_t, cudaStream_t, \
+                                           const int32_t*);                                                 \
     template cudaError_t Launch<T>::to_double(const T*, double*, int64_t, cudaStream_t);                    \
     template cudaError_t Launch<T>::from_double(const double*, T*, int64_t, cudaStream_t);                  \
     template cudaError_t Launch<T>::rec_to_double(const T*, const int32_t*, double*, int64_t, int,          \

@@ -167,16 +167,16 @@ struct Launch {
                                cudaStream_t s);
     static cudaError_t dt_partials(const DevMesh<T>& m, const HostPhys& p, const T* X,
                                    double* part, cudaStream_t s);
-    // per-case minima of the local limits of X into case_dtmin (reset first)
-    static cudaError_t init_dtmin(const DevMesh<T>& m, const HostPhys& p, const T* X,
-                                  unsigned long long* case_dtmin, cudaStream_t s);
-    // X = [W | grad W] per cell from FP64 component-major W[5][nc], dW[15][nc]
-    // (cperm, may be NULL: device cell -> cell of W, dW)
-    static cudaError_t pack(const double* W, const double* dW, T* X, int64_t nc, cudaStream_t s,
-                            const int32_t* cperm = nullptr);
-    // FP64 component-major dW[15][nc] from X (in the order of cperm's cells)
-    static cudaError_t unpack_grad(const T* X, double* dW, int64_t nc, cudaStream_t s,
-                                   const int32_t* cperm = nullptr);
+    // X (and, where not NULL, the master averages Wd and the per-case minima of
+    // the local time-step limits dtmin, reset before) from FP64
+    // component-major W[5][nc], dW[15][nc] (cperm, may be NULL: device cell ->
+    // cell of W, dW)
+    static cudaError_t pack(const DevMesh<T>& m, const HostPhys& p, const double* W, const double* dW, T* X,
+                            double* Wd, unsigned long long* dtmin, cudaStream_t s, const int32_t* cperm = nullptr);
+    // FP64 component-major W[5][nc] from Wd (NULL: from the FP64 state X) and
+    // dW[15][nc] from X, in the order of cperm's cells; W, dW may be NULL
+    static cudaError_t unpack(const double* Wd, const T* X, double* W, double* dW, int64_t nc, cudaStream_t s,
+                              const int32_t* cperm = nullptr);
     // conversions for diagnostics
     static cudaError_t to_double(const T* in, double* out, int64_t n, cudaStream_t s);
     static cudaError_t from_double(const double* in, T* out, int64_t n, cudaStream_t s);
@@ -247,8 +247,6 @@ cudaError_t launch_rows_gather(const void* in, void* out, int64_t nrows, int wid
 // the one-launch stage's grid barrier on a barrier nothing completes: each
 // of two blocks polls `limit` times, gives up and sets ERR_TIMEOUT
 cudaError_t launch_grid_barrier_probe(unsigned* gbar, int32_t* err, int limit, cudaStream_t s);
-// the averages W [5][nc] of an FP64 working state X [nc][XS]
-cudaError_t launch_unpack_avg(const double* X, double* W, int64_t nc, cudaStream_t s);
 // one stage of the FP32-bulk step (reconstruction with the neighbours'
 // slopes recomputed, face flux, cell update) as one persistent launch with
 // grid-wide barriers; gbar: 2 unsigned words of device scratch (reset by the
@@ -265,10 +263,10 @@ cudaError_t adjoint_reverse(const DevMesh<double>& m, const HostPhys& p, double 
                             double* odW, cudaStream_t s);
 
 // sets dt_fixed and t_end; with reset_time also zeroes the case times and
-// steps and sets the case minima to +inf
+// steps and sets the case minima to +inf; err (may be NULL) is cleared
 cudaError_t launch_set_control(double* ctrl, double* case_t, double* case_dt,
                                unsigned long long* case_dtmin, int32_t ncase, double dt_fixed,
-                               double t_end, int reset_time, cudaStream_t s);
+                               double t_end, int reset_time, int32_t* err, cudaStream_t s);
 int update_blocks(int64_t nc);  // blocks of CELLS_PER_BLOCK cells
 
 }  // namespace gks
