@@ -586,7 +586,7 @@ static gks_status upload_faces(gks_state* s) {
     std::vector<int32_t> cface(4 * nc), flr(2 * nf);
     std::vector<T> fgeo(FGEO * nf, T(0)), fnw(4 * nf);
     std::vector<float> fan(s->L.fan ? 6 * nf : 0, 0.0f);
-    run_ranges(nc, host_threads(nc), [&](int64_t, int64_t lo, int64_t hi) {
+    run_ranges(nc, host_threads(nc, 2048), [&](int64_t, int64_t lo, int64_t hi) {
         for (int64_t d = lo; d < hi; ++d) {
             const int64_t c = s->pub(d);
             for (int f = 0; f < 4; ++f) {
@@ -596,7 +596,7 @@ static gks_status upload_faces(gks_state* s) {
             }
         }
     });
-    run_ranges(nf, host_threads(nf), [&](int64_t, int64_t lo, int64_t hi) {
+    run_ranges(nf, host_threads(nf, 4096), [&](int64_t, int64_t lo, int64_t hi) {
         for (int64_t d = lo; d < hi; ++d) {
             const int64_t f = perm[d];
             // a boundary face's missing side carries its kind: -1 - GKS_BC_*
@@ -664,33 +664,31 @@ static gks_status upload_cells(gks_state* s) {
             for (int k = 0; k < 15; ++k) o[WOP_W1 + k] = (TO)w1[k];
         }
     }
-    run_ranges(nc, host_threads(nc), [&](int64_t, int64_t lo, int64_t hi) {
+    run_ranges(nc, host_threads(nc, 2048), [&](int64_t, int64_t lo, int64_t hi) {
         for (int64_t d = lo; d < hi; ++d) {
             const int64_t c = s->pub(d);
             cell_case[d] = g.cell_case[c];
-            TO* tc = &tile[(size_t)(d / CELLS_PER_BLOCK) * TILE_ROWS * CELLS_PER_BLOCK];
-            const int lc = (int)(d % CELLS_PER_BLOCK);
-            auto put_row = [&](int row, double v) { tc[tile_at<TO>(row, lc)] = (TO)v; };
-            double far[3] = {0.0, 0.0, 0.0};
+            double row[TILE_ROWS], far[3] = {0.0, 0.0, 0.0};
             for (int f = 0; f < 4; ++f) {
                 nbr[f * nc + d] = g.nbr[c * 4 + f] >= 0 ? (int32_t)s->dev(g.nbr[c * 4 + f]) : -1;
                 const int64_t fi = g.csr_face[c * 4 + f];
                 const bool left = g.csr_sign[c * 4 + f] > 0;
                 const double* gp = left ? &g.gp_l[fi * 9] : &g.gp_r[fi * 9];
                 for (int k = 0; k < 9; ++k) {
-                    put_row(TILE_G + f * 9 + k, gp[k]);
+                    row[TILE_G + f * 9 + k] = gp[k];
                     far[k % 3] = std::max(far[k % 3], std::abs(gp[k]));
                 }
             }
             inv_vol[d] = 1.0 / g.vol[c];
-            for (int k = 0; k < 3; ++k) put_row(TILE_BND + k, far[k]);
-            put_row(TILE_V23, std::pow(g.vol[c], 2.0 / 3.0));
-            put_row(TILE_V43, std::pow(g.vol[c], 4.0 / 3.0));
+            for (int k = 0; k < 3; ++k) row[TILE_BND + k] = far[k];
+            row[TILE_BND + 3] = 0.0;
+            row[TILE_V23] = std::pow(g.vol[c], 2.0 / 3.0);
+            row[TILE_V43] = std::pow(g.vol[c], 4.0 / 3.0);
             dr[d] = (T)g.dr[c];
-            for (int q = 0; q < 6; ++q) put_row(TILE_MOM + q, g.mom2[c * 6 + q]);
+            for (int q = 0; q < 6; ++q) row[TILE_MOM + q] = g.mom2[c * 6 + q];
             for (int k = 0; k < 12; ++k) {
                 M1[k * nc + d] = (TO)g.M1[c * 12 + k];
-                put_row(TILE_M1 + k, g.M1[c * 12 + k]);
+                row[TILE_M1 + k] = g.M1[c * 12 + k];
             }
             const double* M2c = &g.M2[c * 144];
             double M2lin[144];
@@ -698,7 +696,13 @@ static gks_status upload_cells(gks_state* s) {
                 (g.nbr[c * 4] < 0 || g.nbr[c * 4 + 1] < 0 || g.nbr[c * 4 + 2] < 0 || g.nbr[c * 4 + 3] < 0) &&
                 cell_linear_fit(g, c, M2lin))
                 M2c = M2lin;
-            for (int k = 0; k < 144; ++k) put_row(TILE_M2 + k, M2c[k]);
+            for (int k = 0; k < 144; ++k) row[TILE_M2 + k] = M2c[k];
+            // the cell's rows in their 16-byte groups (tile_at)
+            constexpr int V = 16 / (int)sizeof(TO);
+            TO* to = &tile[(size_t)(d / CELLS_PER_BLOCK) * TILE_ROWS * CELLS_PER_BLOCK +
+                           (size_t)tile_at<TO>(0, (int)(d % CELLS_PER_BLOCK))];
+            for (int k = 0; k < TILE_ROWS / V; ++k, to += CELLS_PER_BLOCK * V)
+                for (int v = 0; v < V; ++v) to[v] = (TO)row[k * V + v];
         }
     });
     auto put = [&](size_t off, const void* src, size_t bytes) -> cudaError_t {

@@ -49,10 +49,10 @@ bool cell_linear_fit(const gks_mesh& m, int64_t c, double* M2);  // boundary cel
 bool cell_wall_stencil(const gks_mesh& m, int64_t c, double* W2, double* W1);
 bool has_wall_face(const gks_mesh& m, int64_t c);
 
-// threads for a loop over n cells or faces
-inline int64_t host_threads(int64_t n) {
+// threads for a loop over n cells or faces, with at least `grain` of them each
+inline int64_t host_threads(int64_t n, int64_t grain = 16384) {
     const unsigned hw = std::max(1u, std::thread::hardware_concurrency());
-    return std::min<int64_t>((int64_t)hw, std::max<int64_t>(1, n / 16384));
+    return std::min<int64_t>((int64_t)hw, std::max<int64_t>(1, n / grain));
 }
 
 // fn(t, lo, hi) over nthr contiguous ranges of [0, n); range 0 on the calling
