@@ -22,8 +22,8 @@
 //   k_adj_gather_poly        per cell: sum over its four faces
 //   k_adj_recon_local        per cell: transpose of a = M2 d and of the
 //                            monomial constant (linear weights)
-//   k_adj_recon_weno         the same with the nonlinear WENO weights, and
-//   k_adj_slopes             the neighbours' P1 slopes those weights use
+//   k_adj_recon_weno         the same with the nonlinear WENO weights, after
+//   k_adj_p1, k_adj_slopes   and the neighbours' P1 slopes those weights use
 //   k_adj_recon_gather       per cell: adjoint of its working state from its
 //                            own and its neighbours' stencil adjoints
 //   k_adj_final              the three paths into (W^n, grad W^n)
@@ -34,6 +34,7 @@
 #include "gks_face.cuh"
 #include "gks_kernels.h"
 #include "gks_point_adj.cuh"
+#include "gks_recon.cuh"
 
 namespace gks {
 
@@ -376,19 +377,25 @@ __global__ void k_adj_recon_local(DevMesh<double> m, const double* __restrict__ 
     own[c * 5 + q] = lc0 - s;
 }
 
-// P1 slope of cell x for component q from the working state X (the
-// reconstruction's step 1, Sec. 4.3)
-__device__ __forceinline__ void adj_p1_slope(const DevMesh<double>& m, const double* __restrict__ X, int64_t x,
-                                             int q, double* b) {
-    const int64_t nc = m.nc;
-    const double Qx = X[x * XS + q];
-    b[0] = b[1] = b[2] = 0.0;
+// P1 slopes of every cell and component from the working state X (the
+// reconstruction's step 1, Sec. 4.3), slopes[c][q][3]
+__global__ void k_adj_p1(DevMesh<double> m, const double* __restrict__ X, double* __restrict__ slopes) {
+    const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, nc = m.nc;
+    if (idx >= nc * 5) return;
+    const int64_t c = idx / 5;
+    const int q = (int)(idx - c * 5);
+    const double Q0 = X[c * XS + q];
+    double b[3] = {0.0, 0.0, 0.0};
+#pragma unroll
     for (int f = 0; f < 4; ++f) {
-        const int nb = m.nbr[f * nc + x];
+        const int nb = m.nbr[f * nc + c];
         if (nb < 0) continue;
-        const double dq = X[(int64_t)nb * XS + q] - Qx;
-        for (int i = 0; i < 3; ++i) b[i] += m.M1[(i * 4 + f) * nc + x] * dq;
+        const double dq = X[(int64_t)nb * XS + q] - Q0;
+#pragma unroll
+        for (int i = 0; i < 3; ++i) b[i] += m.M1[(i * 4 + f) * nc + c] * dq;
     }
+#pragma unroll
+    for (int i = 0; i < 3; ++i) slopes[idx * 3 + i] = b[i];
 }
 
 __device__ __forceinline__ double sgn(double x) { return x > 0.0 ? 1.0 : (x < 0.0 ? -1.0 : 0.0); }
@@ -398,66 +405,80 @@ __device__ __forceinline__ double sgn(double x) { return x > 0.0 ? 1.0 : (x < 0.
 // w1j = 1 + s1 / (eps + beta_0j) with s1 the 4/3 power of the mean pairwise
 // |beta_0j - beta_0k|, beta_0 = sum w1j beta_0j / sum w1j; kept for the reverse.
 struct Beta0 {
-    double bj[4][3], b0j[4], w1j[4];
-    double s1, ws, accb, sum, beta;
-    int slot[4], nn, npair;
+    // per local face: the neighbour's slopes, beta_0j, 1 / (eps + beta_0j), w1j
+    // (zero without a neighbour)
+    double bj[4][3], b0j[4], ie[4], w1j[4];
+    double s1, iws, mean, ipair, beta;
+    bool on[4];
 };
 
-__device__ __forceinline__ void beta0_forward(const DevMesh<double>& m, const double* __restrict__ X,
-                                              const int* nb, int q, double v23, double eps, Beta0& B) {
-    B.nn = 0;
+// slopes: [nc][5][3] P1 slopes of the stage's state
+__device__ __forceinline__ void beta0_forward(const double* __restrict__ slopes, const int* nb, int q, double v23,
+                                              double eps, Beta0& B) {
+    int nn = 0;
+#pragma unroll
     for (int f = 0; f < 4; ++f) {
-        if (nb[f] < 0) continue;
-        adj_p1_slope(m, X, nb[f], q, B.bj[B.nn]);
-        const double* bj = B.bj[B.nn];
-        B.b0j[B.nn] = v23 * (bj[0] * bj[0] + bj[1] * bj[1] + bj[2] * bj[2]);
-        B.slot[B.nn++] = f;
+        B.on[f] = nb[f] >= 0;
+        nn += B.on[f];
+#pragma unroll
+        for (int i = 0; i < 3; ++i) B.bj[f][i] = B.on[f] ? slopes[((int64_t)nb[f] * 5 + q) * 3 + i] : 0.0;
+        const double* bj = B.bj[f];
+        B.b0j[f] = v23 * (bj[0] * bj[0] + bj[1] * bj[1] + bj[2] * bj[2]);
+        B.w1j[f] = 0.0;
     }
-    B.beta = B.s1 = B.ws = B.accb = B.sum = 0.0;
-    B.npair = 0;
-    if (B.nn > 0) {
-        for (int j = 0; j < B.nn; ++j)
-            for (int k = 0; k < j; ++k) {
-                B.sum += fabs(B.b0j[j] - B.b0j[k]);
-                ++B.npair;
-            }
-        B.s1 = B.npair ? pow43(B.sum / B.npair) : 0.0;
-        for (int j = 0; j < B.nn; ++j) {
-            B.w1j[j] = 1.0 + B.s1 / (eps + B.b0j[j]);
-            B.ws += B.w1j[j];
-            B.accb += B.w1j[j] * B.b0j[j];
-        }
-        B.beta = B.accb / B.ws;
+    B.beta = B.s1 = B.iws = B.mean = B.ipair = 0.0;
+    if (nn == 0) return;
+    double sum = 0.0, ws = 0.0, acc = 0.0;
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+#pragma unroll
+        for (int k = 0; k < j; ++k)
+            if (B.on[j] && B.on[k]) sum += fabs(B.b0j[j] - B.b0j[k]);
+    B.ipair = nn == 4 ? 1.0 / 6.0 : nn == 3 ? 1.0 / 3.0 : nn == 2 ? 1.0 : 0.0;
+    B.mean = sum * B.ipair;
+    B.s1 = pow43(B.mean);
+    recip2(eps + B.b0j[0], eps + B.b0j[1], B.ie[0], B.ie[1]);
+    recip2(eps + B.b0j[2], eps + B.b0j[3], B.ie[2], B.ie[3]);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        if (!B.on[j]) continue;
+        B.w1j[j] = 1.0 + B.s1 * B.ie[j];
+        ws += B.w1j[j];
+        acc += B.w1j[j] * B.b0j[j];
     }
+    B.iws = 1.0 / ws;
+    B.beta = acc * B.iws;
 }
 
-// adjoint of beta_0 into the adjoints of the neighbours' slopes lbj[j][3]
-__device__ __forceinline__ void beta0_backward(const Beta0& B, double lbeta0, double v23, double eps,
-                                               double (*lbj)[3]) {
-    for (int j = 0; j < 4; ++j) lbj[j][0] = lbj[j][1] = lbj[j][2] = 0.0;
-    if (B.nn == 0) return;
-    const double lacc = lbeta0 / B.ws, lws = -lbeta0 * B.accb / (B.ws * B.ws);
-    double lb0[4], ls1 = 0.0;
-    for (int j = 0; j < B.nn; ++j) {
-        const double lwj = lacc * B.b0j[j] + lws;
-        lb0[j] = lacc * B.w1j[j] - lwj * B.s1 / ((eps + B.b0j[j]) * (eps + B.b0j[j]));
-        ls1 += lwj / (eps + B.b0j[j]);
+// adjoint of beta_0 into the adjoints of the neighbours' slopes lbj[f][3]
+__device__ __forceinline__ void beta0_backward(const Beta0& B, double lbeta0, double v23, double (*lbj)[3]) {
+    const double lacc = lbeta0 * B.iws, lws = -lacc * B.beta;
+    double lb0[4] = {0.0, 0.0, 0.0, 0.0}, ls1 = 0.0;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        if (!B.on[j]) continue;
+        const double lwe = (lacc * B.b0j[j] + lws) * B.ie[j];
+        lb0[j] = lacc * B.w1j[j] - lwe * B.s1 * B.ie[j];
+        ls1 += lwe;
     }
-    if (B.npair) {
-        const double lsum = ls1 * (4.0 / 3.0) * cbrt(B.sum / B.npair) / B.npair;
-        for (int j = 0; j < B.nn; ++j)
-            for (int k = 0; k < B.nn; ++k)
-                if (k != j) lb0[j] += lsum * sgn(B.b0j[j] - B.b0j[k]);
-    }
-    for (int j = 0; j < B.nn; ++j)
+    const double lsum = ls1 * (4.0 / 3.0) * cbrt(B.mean) * B.ipair;
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            if (k != j && B.on[j] && B.on[k]) lb0[j] += lsum * sgn(B.b0j[j] - B.b0j[k]);
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+#pragma unroll
         for (int i = 0; i < 3; ++i) lbj[j][i] = 2.0 * v23 * B.bj[j][i] * lb0[j];
 }
 
 // the neighbours' slope adjoints into lbn[f][3] (zero for missing neighbours)
-__device__ __forceinline__ void store_lbn(const Beta0& B, const double (*lbj)[3], double* __restrict__ ob) {
-    for (int j = 0; j < 12; ++j) ob[j] = 0.0;
-    for (int j = 0; j < B.nn; ++j)
-        for (int i = 0; i < 3; ++i) ob[3 * B.slot[j] + i] = lbj[j][i];
+__device__ __forceinline__ void store_lbn(const double (*lbj)[3], double* __restrict__ ob) {
+#pragma unroll
+    for (int f = 0; f < 4; ++f)
+#pragma unroll
+        for (int i = 0; i < 3; ++i) ob[3 * f + i] = lbj[f][i];
 }
 
 // Transpose of the third-order multi-resolution WENO reconstruction of one
@@ -469,6 +490,7 @@ __device__ __forceinline__ void store_lbn(const Beta0& B, const double (*lbj)[3]
 // the neighbours' slopes as this cell uses them) and own[c][q] (of Q0 through
 // c0 and the differences d[0:4]).
 __global__ void k_adj_recon_weno(DevMesh<double> m, double eps, const double* __restrict__ X,
+                                 const double* __restrict__ slopes,
                                  const double* __restrict__ lp, const int32_t* __restrict__ fb,
                                  double* __restrict__ ld, double* __restrict__ lbn, double* __restrict__ own) {
     const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -510,7 +532,7 @@ __global__ void k_adj_recon_weno(DevMesh<double> m, double eps, const double* __
     // forward: beta_1, beta_0 (two-step), beta_2, sigma, weights
     const double beta1 = v23 * (b[0] * b[0] + b[1] * b[1] + b[2] * b[2]);
     Beta0 B0;
-    beta0_forward(m, X, nb, q, v23, eps, B0);
+    beta0_forward(slopes, nb, q, v23, eps, B0);
     const double beta0 = B0.beta;
     const double H[3][3] = {{2.0 * a[3], a[4], a[5]}, {a[4], 2.0 * a[6], a[7]}, {a[5], a[7], 2.0 * a[8]}};
     const double MM[3][3] = {{Mm[0], Mm[1], Mm[2]}, {Mm[1], Mm[3], Mm[4]}, {Mm[2], Mm[4], Mm[5]}};
@@ -525,14 +547,18 @@ __global__ void k_adj_recon_weno(DevMesh<double> m, double eps, const double* __
     const double z = 0.5 * (fabs(beta2 - beta1) + fabs(beta2 - beta0));
     const double sigma = pow43(z);
     const double bet[3] = {beta0, beta1, beta2}, gam[3] = {g02, g12, g22};
-    double r[3], w[3];
+    const double i22 = 111.0 / 100.0, i11 = 11.0 / 10.0;  // 1 / g22, 1 / g11
+    double r[3], w[3], ib[3];
+    recip2(eps + bet[0], eps + bet[1], ib[0], ib[1]);
+    ib[2] = 1.0 / (eps + bet[2]);
+#pragma unroll
     for (int k = 0; k < 3; ++k) {
-        r[k] = sigma / (eps + bet[k]);
+        r[k] = sigma * ib[k];
         w[k] = gam[k] * (1.0 + r[k] * r[k]);
     }
     const double iw = 1.0 / (w[0] + w[1] + w[2]);
-    const double c2 = (w[2] * iw) / g22;
-    const double cb = (w[1] * iw) / g11 - c2 * g12 / g11;
+    const double c2 = (w[2] * iw) * i22;
+    const double cb = (w[1] * iw) * i11 - c2 * (g12 * i11);
 
     // reverse
     const double* l = lp + c * 50 + q * 10;
@@ -550,16 +576,17 @@ __global__ void k_adj_recon_weno(DevMesh<double> m, double eps, const double* __
         lcb += lR[i] * b[i];
     }
     // c2 = w2 iw / g22, cb = w1 iw / g11 - c2 g12 / g11
-    const double lc2t = lc2 - lcb * g12 / g11;
-    double lw[3] = {0.0, lcb * iw / g11, lc2t * iw / g22};
-    const double liw = lc2t * w[2] / g22 + lcb * w[1] / g11;
-    const double lS = -liw * iw * iw;
+    const double lc2t = lc2 - lcb * (g12 * i11);
+    const double l1 = lcb * i11, l2t = lc2t * i22;
+    double lw[3] = {0.0, l1 * iw, l2t * iw};
+    const double lS = -(l2t * w[2] + l1 * w[1]) * iw * iw;
     double lbet[3] = {0.0, 0.0, 0.0}, lsig = 0.0;
+#pragma unroll
     for (int k = 0; k < 3; ++k) {
         lw[k] += lS;
-        const double lr = lw[k] * gam[k] * 2.0 * r[k];
-        lsig += lr / (eps + bet[k]);
-        lbet[k] += -lr * sigma / ((eps + bet[k]) * (eps + bet[k]));
+        const double lri = lw[k] * gam[k] * 2.0 * r[k] * ib[k];
+        lsig += lri;
+        lbet[k] -= lri * r[k];
     }
     // sigma = z^{4/3}, z = (|b2 - b1| + |b2 - b0|) / 2
     const double lz = lsig * (4.0 / 3.0) * cbrt(z);
@@ -589,7 +616,7 @@ __global__ void k_adj_recon_weno(DevMesh<double> m, double eps, const double* __
     // beta_1 = v23 |b|^2
     for (int i = 0; i < 3; ++i) lb[i] += 2.0 * v23 * b[i] * lbet[1];
     double lbj[4][3];
-    beta0_backward(B0, lbet[0], v23, eps, lbj);
+    beta0_backward(B0, lbet[0], v23, lbj);
     // a = M2 d, b = M1 d[0:4]
     double* o = ld + (c * 5 + q) * 16;
     double s = 0.0;
@@ -602,7 +629,7 @@ __global__ void k_adj_recon_weno(DevMesh<double> m, double eps, const double* __
         if (j < 4 && nb[j] >= 0) s += acc;
     }
     own[c * 5 + q] = lc0 - s;
-    store_lbn(B0, lbj, lbn + (c * 5 + q) * 12);
+    store_lbn(lbj, lbn + (c * 5 + q) * 12);
 }
 
 // Transpose of the second-order WENO reconstruction R^2nd (Eq.
@@ -610,6 +637,7 @@ __global__ void k_adj_recon_weno(DevMesh<double> m, double eps, const double* __
 // cb = (w1 / (w0 + w1)) / g11, w0, w1 from beta_0 (two-step) and beta_1,
 // sigma = |beta_1 - beta_0|^{4/3}.  Same outputs as k_adj_recon_weno.
 __global__ void k_adj_recon_weno2(DevMesh<double> m, double eps, const double* __restrict__ X,
+                                 const double* __restrict__ slopes,
                                   const double* __restrict__ lp, const int32_t* __restrict__ fb,
                                   double* __restrict__ ld, double* __restrict__ lbn, double* __restrict__ own) {
     const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -637,18 +665,21 @@ __global__ void k_adj_recon_weno2(DevMesh<double> m, double eps, const double* _
     const double g01 = 1.0 / 11.0, g11 = 10.0 / 11.0;
     const double beta1 = v23 * (b[0] * b[0] + b[1] * b[1] + b[2] * b[2]);
     Beta0 B0;
-    beta0_forward(m, X, nb, q, v23, eps, B0);
+    beta0_forward(slopes, nb, q, v23, eps, B0);
     const double beta0 = B0.beta;
     const double z = fabs(beta1 - beta0);
     const double sigma = pow43(z);
     const double bet[2] = {beta0, beta1}, gam[2] = {g01, g11};
-    double r[2], w[2];
+    const double i11 = 11.0 / 10.0;  // 1 / g11
+    double r[2], w[2], ib[2];
+    recip2(eps + bet[0], eps + bet[1], ib[0], ib[1]);
+#pragma unroll
     for (int k = 0; k < 2; ++k) {
-        r[k] = sigma / (eps + bet[k]);
+        r[k] = sigma * ib[k];
         w[k] = gam[k] * (1.0 + r[k] * r[k]);
     }
-    const double wsum = w[0] + w[1];
-    const double cb = w[1] / (wsum * g11);
+    const double iwsum = 1.0 / (w[0] + w[1]);
+    const double cb = w[1] * iwsum * i11;
 
     // reverse: only the constant and the linear coefficients of R are nonzero
     const double* l = lp + c * 50 + q * 10;
@@ -659,14 +690,15 @@ __global__ void k_adj_recon_weno2(DevMesh<double> m, double eps, const double* _
         lcb += l[1 + i] * b[i];
     }
     double lw[2];
-    const double lwsum = -lcb * w[1] / (wsum * wsum * g11);
+    const double lwsum = -lcb * cb * iwsum;
     lw[0] = lwsum;
-    lw[1] = lwsum + lcb / (wsum * g11);
+    lw[1] = lwsum + lcb * iwsum * i11;
     double lbet[2] = {0.0, 0.0}, lsig = 0.0;
+#pragma unroll
     for (int k = 0; k < 2; ++k) {
-        const double lr = lw[k] * gam[k] * 2.0 * r[k];
-        lsig += lr / (eps + bet[k]);
-        lbet[k] += -lr * sigma / ((eps + bet[k]) * (eps + bet[k]));
+        const double lri = lw[k] * gam[k] * 2.0 * r[k] * ib[k];
+        lsig += lri;
+        lbet[k] -= lri * r[k];
     }
     const double lz = lsig * (4.0 / 3.0) * cbrt(z);
     const double s10 = sgn(beta1 - beta0);
@@ -674,7 +706,7 @@ __global__ void k_adj_recon_weno2(DevMesh<double> m, double eps, const double* _
     lbet[0] -= lz * s10;
     for (int i = 0; i < 3; ++i) lb[i] += 2.0 * v23 * b[i] * lbet[1];
     double lbj[4][3];
-    beta0_backward(B0, lbet[0], v23, eps, lbj);
+    beta0_backward(B0, lbet[0], v23, lbj);
     double* o = ld + (c * 5 + q) * 16;
     double s = 0.0;
     for (int j = 0; j < 16; ++j) o[j] = 0.0;
@@ -684,7 +716,7 @@ __global__ void k_adj_recon_weno2(DevMesh<double> m, double eps, const double* _
         s += o[j];
     }
     own[c * 5 + q] = lc0 - s;
-    store_lbn(B0, lbj, lbn + (c * 5 + q) * 12);
+    store_lbn(lbj, lbn + (c * 5 + q) * 12);
 }
 
 // Transpose of the second-order reconstruction with linear weights: R = P1,
@@ -711,6 +743,21 @@ __global__ void k_adj_recon_p1(DevMesh<double> m, const double* __restrict__ lp,
         s += o[j];
     }
     own[c * 5 + q] = l[0] - s;
+}
+
+// Reverse face slots: rev[f][c] = the local face of neighbour n = nbr(c, f)
+// that is the same face.  Found here on each call (microseconds), where the
+// host's table was copied over from pageable memory.
+__global__ void k_adj_rev(DevMesh<double> m, int8_t* __restrict__ rev) {
+    const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, nc = m.nc;
+    if (idx >= nc * 4) return;
+    const int64_t f = idx / nc, c = idx - f * nc;
+    const int n = m.nbr[idx], face = m.cface[f * nc + c] >> 1;
+    int8_t r = 0;
+    if (n >= 0)
+        for (int k = 0; k < 4; ++k)
+            if ((m.cface[k * nc + n] >> 1) == face) r = (int8_t)k;
+    rev[idx] = r;
 }
 
 // Adjoint of the neighbours' P1 slopes, per cell n and component: the slope
@@ -811,10 +858,12 @@ static void recon_back(const DevMesh<double>& m, const HostPhys& p, const AdjBuf
                        double* lX, cudaStream_t s) {
     const int B = 128;
     if (p.weno) {
+        // the slopes lie in lds until k_adj_slopes writes it
+        k_adj_p1<<<grid_of(m.nc * 5, B), B, 0, s>>>(m, X, b.lds);
         if (p.order == 2)
-            k_adj_recon_weno2<<<grid_of(m.nc * 5, B), B, 0, s>>>(m, p.eps_weno, X, b.lp, fb, b.ld, b.lbn, b.own);
+            k_adj_recon_weno2<<<grid_of(m.nc * 5, B), B, 0, s>>>(m, p.eps_weno, X, b.lds, b.lp, fb, b.ld, b.lbn, b.own);
         else
-            k_adj_recon_weno<<<grid_of(m.nc * 5, B), B, 0, s>>>(m, p.eps_weno, X, b.lp, fb, b.ld, b.lbn, b.own);
+            k_adj_recon_weno<<<grid_of(m.nc * 5, B), B, 0, s>>>(m, p.eps_weno, X, b.lds, b.lp, fb, b.ld, b.lbn, b.own);
         k_adj_slopes<<<grid_of(m.nc * 5, B), B, 0, s>>>(m, b.rev, b.lbn, b.lds);
         k_adj_recon_gather<<<grid_of(m.nc * 5, B), B, 0, s>>>(m, b.rev, b.ld, b.lds, b.own, b.lwo, lX);
     } else {
@@ -854,6 +903,7 @@ cudaError_t adjoint_reverse(const DevMesh<double>& m, const HostPhys& p, double 
     const Phys<double> ph = phys64(p);
     const int B = 128;
     cudaError_t e;
+    k_adj_rev<<<grid_of(m.nc * 4, B), B, 0, s>>>(m, b.rev);
     // stage 2
     k_adj_src2<<<grid_of(m.nc, B), B, 0, s>>>(m, lW, ldW, b.src);
     flux_back<20>(m, ph, b, b.poly2, X2, dt, s);

@@ -394,7 +394,6 @@ struct gks_state {
     // device cell to the caller's cell, cinv back (empty: identity)
     int cell_order = 0;
     std::vector<int32_t> cperm, cinv;
-    std::vector<int8_t> adj_rev;  // reverse face slots of the adjoint (built on first use)
     // device copy of cperm, or NULL for the caller's order
     const int32_t* dperm() const { return cperm.empty() ? nullptr : reinterpret_cast<const int32_t*>(ws + L.cperm); }
     const int32_t* dinv() const { return cinv.empty() ? nullptr : reinterpret_cast<const int32_t*>(ws + L.cinv); }
@@ -1226,21 +1225,6 @@ static gks_status adjoint_impl(gks_state* s, double dt, const double* d_W, const
     DevState<double>& st = s->s64;
     const int64_t nc = g.nc;
     char* base = static_cast<char*>(d_scratch);
-    // reverse face slots: rev[f][c] = the local face of neighbour n = nbr(c, f)
-    // that is the same face
-    std::vector<int8_t>& rev = s->adj_rev;
-    if (rev.size() != (size_t)4 * nc) {
-        rev.assign((size_t)4 * nc, 0);
-        for (int64_t c = 0; c < nc; ++c)
-            for (int f = 0; f < 4; ++f) {
-                const int64_t n = g.nbr[c * 4 + f];
-                if (n < 0) continue;
-                const int64_t fi = g.csr_face[c * 4 + f];
-                for (int r = 0; r < 4; ++r)
-                    if (g.csr_face[n * 4 + r] == fi) rev[(size_t)f * nc + c] = (int8_t)r;
-            }
-    }
-    GKS_CHECK_CUDA(cudaMemcpyAsync(base + A.rev, rev.data(), rev.size(), cudaMemcpyHostToDevice, s->stream));
     // forward recomputation of the step's two reconstructions with the frozen dt
     gks_status r = init_impl<double>(s, m, st, d_W, d_dW);
     if (r != GKS_OK) return r;
@@ -1249,8 +1233,10 @@ static gks_status adjoint_impl(gks_state* s, double dt, const double* d_W, const
     GKS_CHECK_CUDA(cudaMemcpyAsync(st.case_dt, &dth, 8, cudaMemcpyHostToDevice, s->stream));
     int32_t* fb = reinterpret_cast<int32_t*>(base + A.fallback);
     double* poly1 = reinterpret_cast<double*>(base + A.poly1);
-    GKS_CHECK_CUDA(Launch<double>::recon(m, s->phys, st.X, nullptr, nullptr, st.poly, fb, nullptr, st.err,
-                                         s->stream));
+    // (with the slopes pass: st.slopes is free until the next step)
+    double* s2 = s->phys.weno ? st.slopes : nullptr;
+    if (s2) GKS_CHECK_CUDA(Launch<double>::slopes(m, st.X, s2, nullptr, s->stream));
+    GKS_CHECK_CUDA(Launch<double>::recon(m, s->phys, st.X, s2, nullptr, st.poly, fb, nullptr, st.err, s->stream));
     GKS_CHECK_CUDA(cudaMemcpyAsync(poly1, st.poly, 8 * POLY_STRIDE * nc, cudaMemcpyDeviceToDevice, s->stream));
     if (d_Ws) {
         // the caller's stage state in place of the stage-1 flux and update
@@ -1260,8 +1246,8 @@ static gks_status adjoint_impl(gks_state* s, double dt, const double* d_W, const
                                             s->flux_variant));
         GKS_CHECK_CUDA(Launch<double>::update1(m, s->phys, st, s->stream));
     }
-    GKS_CHECK_CUDA(Launch<double>::recon(m, s->phys, st.Xs, nullptr, nullptr, st.poly, fb + nc, nullptr, st.err,
-                                         s->stream));
+    if (s2) GKS_CHECK_CUDA(Launch<double>::slopes(m, st.Xs, s2, nullptr, s->stream));
+    GKS_CHECK_CUDA(Launch<double>::recon(m, s->phys, st.Xs, s2, nullptr, st.poly, fb + nc, nullptr, st.err, s->stream));
     AdjBuffers b;
     b.poly1 = poly1;
     b.poly2 = st.poly;
@@ -1276,7 +1262,7 @@ static gks_status adjoint_impl(gks_state* s, double dt, const double* d_W, const
     b.lbn = reinterpret_cast<double*>(base + A.lbn);
     b.lds = reinterpret_cast<double*>(base + A.lds);
     b.lwo = reinterpret_cast<double*>(base + A.lwo);
-    b.rev = reinterpret_cast<const int8_t*>(base + A.rev);
+    b.rev = reinterpret_cast<int8_t*>(base + A.rev);
     b.fallback = fb;
     GKS_CHECK_CUDA(adjoint_reverse(m, s->phys, dt, b, st.X, st.Xs, d_lamW, d_lamdW, d_lamW_out, d_lamdW_out,
                                    s->stream));
