@@ -41,10 +41,10 @@ constexpr int FLUX_THREADS = 3 * FLUX_FACES;
 template <int NR>
 constexpr int flux_vals() { return NR == 40 ? 20 : 10; }
 
-template <typename T, int NR>
+template <typename T, int NR, int TH = FLUX_THREADS>
 struct FluxSmem {
-    T out[FLUX_THREADS][flux_vals<NR>() + 1];
-    T frame[FLUX_FACES][7];  // tangents of the face frame
+    T out[TH][flux_vals<NR>() + 1];
+    T frame[(TH + 2) / 3][7];  // tangents of the face frame
 };
 
 // Stage 1, FP32: the interface state W^c of Eq. new-equ-part relative to W_m,
@@ -146,20 +146,22 @@ __device__ __forceinline__ void reference_flux(const float* __restrict__ poly, c
     }
 }
 
-// One block of FLUX_FACES faces (block index fb) by FLUX_THREADS threads
-// (tid): sm its shared memory, bar_id the barrier of its threads (0: the
+// One block of TH / 3 faces (block index fb) by TH threads (tid; one may be
+// left over, which computes and stores nothing): sm its shared memory, bar_id the barrier of its threads (0: the
 // whole thread block).  VISC: viscous flow (time slopes, Pr fix).  XW: the
 // mesh may have isothermal or moving wall faces (their ghosts are compiled
 // only into those instances).
-template <typename T, int NR, bool VISC, bool XW>
+template <typename T, int NR, bool VISC, bool XW, int TH = FLUX_THREADS>
 __device__ __forceinline__ void flux_faces(const DevMesh<T>& m, const Phys<T>& ph, const T* __restrict__ Wavg,
                                            const T* __restrict__ poly, T* __restrict__ rec,
                                            const double* __restrict__ ctrl, double dt_override, int64_t fb, int tid,
-                                           FluxSmem<T, NR>& sm, int bar_id) {
+                                           FluxSmem<T, NR, TH>& sm, int bar_id) {
     constexpr bool REL = sizeof(T) == 4 && NR == 40;
+    constexpr int FACES = TH / 3;
+    static_assert(REL ? FACES == 32 : 2 * FACES <= TH, "a thread per face and job");
     {
         const int lf = tid / 3, k = tid - 3 * lf;
-        const int64_t f0 = fb * FLUX_FACES + lf;
+        const int64_t f0 = fb * FACES + lf;
         const int64_t f = f0 < m.nf ? f0 : m.nf - 1;  // idle points compute a valid face, store nothing
         const int L = m.flr[f], Rc = m.flr[m.nf + f];
         const T* geo = m.fgeo + f * FGEO;
@@ -233,21 +235,21 @@ __device__ __forceinline__ void flux_faces(const DevMesh<T>& m, const Phys<T>& p
             }
         }
     }
-    group_barrier(bar_id, FLUX_THREADS);
-    // per face, one warp each: the flux entries, the interface-state entries
-    // and (FP32 stage 1) the reference flux
-    const int job = tid >> 5, lf = tid & 31;
-    const int64_t f = fb * FLUX_FACES + lf;
-    if (f >= m.nf) return;
+    group_barrier(bar_id, TH);
+    // per face, a thread each (with 32 faces a warp each): the flux entries,
+    // the interface-state entries and (FP32 stage 1) the reference flux
+    const int job = tid / FACES, lf = tid - FACES * job;
+    const int64_t f = fb * FACES + lf;
+    if (f >= m.nf || job > (REL ? 2 : 1)) return;
     constexpr int RS = rec_stride<T, NR>();
     T* r = rec + f * RS;
-    if (job == 2) {
-        if constexpr (REL) {
+    if constexpr (REL) {
+        if (job == 2) {
             const int L = m.flr[f], Rc = m.flr[m.nf + f];
             const double dtc = ctrl ? ctrl[m.cell_case[L >= 0 ? L : Rc]] : dt_override;
             reference_flux(poly, m.fan + 6 * f, L, Rc, ph.gm1, dtc > 0.0 ? (T)dtc : T(1), r + REC1_REF);
+            return;
         }
-        return;
     }
     T Rm[3][3], n[4];
     load_vec<4>(m.fgeo + f * FGEO, n);
@@ -308,43 +310,59 @@ inline Phys<T> make_phys(const HostPhys& p) {
 }
 
 
-// the flux kernel: one block of FLUX_FACES faces per thread block; MINB
-// resident blocks an SM
-template <typename T, int NR, int MINB, bool VISC, bool XW>
-__global__ void __launch_bounds__(FLUX_THREADS, MINB) k_flux(DevMesh<T> m, Phys<T> ph, const T* __restrict__ Wavg,
-                                                             const T* __restrict__ poly, T* __restrict__ rec,
-                                                             const double* __restrict__ ctrl, double dt_override) {
-    __shared__ FluxSmem<T, NR> sm;
-    flux_faces<T, NR, VISC, XW>(m, ph, Wavg, poly, rec, ctrl, dt_override, blockIdx.x, threadIdx.x, sm, 0);
+// the flux kernel: one block of TH / 3 faces per thread block; MINB resident
+// blocks an SM
+template <typename T, int NR, int TH, int MINB, bool VISC, bool XW>
+__global__ void __launch_bounds__(TH, MINB) k_flux(DevMesh<T> m, Phys<T> ph, const T* __restrict__ Wavg,
+                                                   const T* __restrict__ poly, T* __restrict__ rec,
+                                                   const double* __restrict__ ctrl, double dt_override) {
+    __shared__ FluxSmem<T, NR, TH> sm;
+    flux_faces<T, NR, VISC, XW, TH>(m, ph, Wavg, poly, rec, ctrl, dt_override, blockIdx.x, threadIdx.x, sm, 0);
 }
 
-// Resident blocks an SM, hence registers: FP64 is bound by its pipe whatever
-// the occupancy (2 blocks, 218-238 registers, no spills).  FP32 variant 1:
-// 15 warps at 128 registers, no spills (stage 1, 3.15 M faces: 1,161 us,
+// Threads a block and resident blocks an SM, hence registers.  FP32 variant
+// 1: 15 warps at 128 registers, no spills (stage 1, 3.15 M faces: 1,161 us,
 // against 1,273 us with 6 blocks and 1,419 us with 8, which spill); variant
 // 0: 12 warps with more registers, the faster one in some viscous and small
 // launches.
-constexpr int FLUX_BLOCKS_FP64 = 2, FLUX_BLOCKS_V1 = 5, FLUX_BLOCKS_V0 = 4;
+constexpr int FLUX_BLOCKS_V1 = 5, FLUX_BLOCKS_V0 = 4;
+// FP64 is bound by its pipe whatever the occupancy (218-238 registers, no
+// spills), so a launch lasts as long as the SM with the most warps: blocks of
+// 96 threads (32 faces, no lane idle) or of 64 (21 faces, one lane idle),
+// whichever leaves the fullest SM with fewer warps.  6,144 faces: 6 warps with
+// blocks of 96, 4 with 64, a step of both fluxes 215 and 153 us; 49,280 faces:
+// 33 and 32 warps, 1,242 and 1,188 us; from about 10^6 faces the blocks of 96
+// win by their full lanes.
+constexpr int FLUX_THREADS_FP64 = 64, SMS = 152;
+
+inline int64_t fullest_sm_warps(int64_t nf, int threads) {
+    const int64_t blocks = (nf + threads / 3 - 1) / (threads / 3);
+    return (blocks + SMS - 1) / SMS * (threads / 32);
+}
 
 template <typename T, bool XW>
 static cudaError_t launch_flux(const DevMesh<T>& m, const HostPhys& p, const T* W, const T* poly, T* rec,
                                const double* ctrl, double dt_override, int stage, cudaStream_t s, int variant) {
-    const unsigned grid = (unsigned)((m.nf + FLUX_FACES - 1) / FLUX_FACES);
     const Phys<T> ph = make_phys<T>(p);
-    auto go = [&](auto kernel) { kernel<<<grid, FLUX_THREADS, 0, s>>>(m, ph, W, poly, rec, ctrl, dt_override); };
-    auto blocks = [&](auto minb) {
-        constexpr int B = decltype(minb)::value;
+    auto blocks = [&](auto threads, auto minb) {
+        constexpr int TH = decltype(threads)::value, B = decltype(minb)::value;
+        const unsigned grid = (unsigned)((m.nf + TH / 3 - 1) / (TH / 3));
+        auto go = [&](auto kernel) { kernel<<<grid, TH, 0, s>>>(m, ph, W, poly, rec, ctrl, dt_override); };
         if (stage == 1)
-            p.viscous ? go(k_flux<T, 40, B, true, XW>) : go(k_flux<T, 40, B, false, XW>);
+            p.viscous ? go(k_flux<T, 40, TH, B, true, XW>) : go(k_flux<T, 40, TH, B, false, XW>);
         else
-            p.viscous ? go(k_flux<T, 20, B, true, XW>) : go(k_flux<T, 20, B, false, XW>);
+            p.viscous ? go(k_flux<T, 20, TH, B, true, XW>) : go(k_flux<T, 20, TH, B, false, XW>);
     };
-    if constexpr (sizeof(T) == 8)
-        blocks(std::integral_constant<int, FLUX_BLOCKS_FP64>{});
-    else if (variant == 1)
-        blocks(std::integral_constant<int, FLUX_BLOCKS_V1>{});
+    using std::integral_constant;
+    if constexpr (sizeof(T) == 8) {
+        if (fullest_sm_warps(m.nf, FLUX_THREADS_FP64) < fullest_sm_warps(m.nf, FLUX_THREADS))
+            blocks(integral_constant<int, FLUX_THREADS_FP64>{}, integral_constant<int, 4>{});
+        else
+            blocks(integral_constant<int, FLUX_THREADS>{}, integral_constant<int, 2>{});
+    } else if (variant == 1)
+        blocks(integral_constant<int, FLUX_THREADS>{}, integral_constant<int, FLUX_BLOCKS_V1>{});
     else
-        blocks(std::integral_constant<int, FLUX_BLOCKS_V0>{});
+        blocks(integral_constant<int, FLUX_THREADS>{}, integral_constant<int, FLUX_BLOCKS_V0>{});
     return cudaGetLastError();
 }
 
