@@ -22,8 +22,6 @@ __device__ __forceinline__ double d_exp(double x) { return exp(x); }
 __device__ __forceinline__ float d_exp(float x) { return expf(x); }
 __device__ __forceinline__ double d_erfc(double x) { return erfc(x); }
 __device__ __forceinline__ float d_erfc(float x) { return erfcf(x); }
-__device__ __forceinline__ double d_sqrt(double x) { return sqrt(x); }
-__device__ __forceinline__ float d_sqrt(float x) { return sqrtf(x); }
 __device__ __forceinline__ double d_rsqrt(double x) { return rsqrt(x); }
 __device__ __forceinline__ float d_rsqrt(float x) { return rsqrtf(x); }
 __device__ __forceinline__ double d_abs(double x) { return fabs(x); }
@@ -115,158 +113,15 @@ struct Phys {
     int viscous, smooth;
 };
 
-// ------------------------------------------------------- Maxwellian --
-template <typename T>
-struct Prim {
-    T rho, u, v, w, lam, p;
-};
-
-template <typename T>
-__device__ __forceinline__ Prim<T> to_prim(const T* W, T gm1) {
-    Prim<T> s;
-    s.rho = W[0];
-    T ir = T(1) / W[0];
-    s.u = W[1] * ir;
-    s.v = W[2] * ir;
-    s.w = W[3] * ir;
-    s.p = gm1 * (W[4] - T(0.5) * (W[1] * s.u + W[2] * s.v + W[3] * s.w));
-    s.lam = T(0.5) * s.rho / s.p;
-    return s;
-}
-
-// normalised moments <u^k> (k < 7) for u (full or half space), v, w and
-// <xi^2>, <xi^4>
-template <typename T>
-struct Tab {
-    T u[7], v[7], w[7];
-    T xi2, xi4;
-};
-
-template <typename T>
-__device__ __forceinline__ void mom_recur(T* m, T U, T h) {
-    // h = 1 / (2 lambda); <u^(k+2)> = U <u^(k+1)> + (k+1) h <u^k>
-#pragma unroll
-    for (int k = 0; k < 5; ++k) m[k + 2] = U * m[k + 1] + T(k + 1) * h * m[k];
-}
-
-// half: +1 restricts u > 0, -1 restricts u < 0, 0 is the whole space
-template <typename T>
-__device__ __forceinline__ void make_tab(Tab<T>& t, const Prim<T>& s, T K, int half) {
-    const T h = T(0.5) / s.lam;
-    if (half == 0) {
-        t.u[0] = T(1);
-        t.u[1] = s.u;
-    } else {
-        const T sg = half > 0 ? T(1) : T(-1);
-        const T sl = d_sqrt(s.lam);
-        t.u[0] = T(0.5) * d_erfc(-sg * sl * s.u);
-        // Gaussian tail term exp(-lam U^2) / (2 sqrt(pi lam))
-        const T inv_sqrt_pi = T(0.56418958354775628695);
-        t.u[1] = s.u * t.u[0] + sg * T(0.5) * inv_sqrt_pi * d_exp(-s.lam * s.u * s.u) / sl;
-    }
-    mom_recur(t.u, s.u, h);
-    t.v[0] = T(1);
-    t.v[1] = s.v;
-    mom_recur(t.v, s.v, h);
-    t.w[0] = T(1);
-    t.w[1] = s.w;
-    mom_recur(t.w, s.w, h);
-    t.xi2 = K * h;
-    t.xi4 = (K * K + T(2) * K) * h * h;
-}
-
-// only the u-moments change between the full space and a half space
-template <typename T>
-__device__ __forceinline__ void make_half_u(Tab<T>& t, const Prim<T>& s, int half) {
-    const T h = T(0.5) / s.lam;
-    const T sg = half > 0 ? T(1) : T(-1);
-    const T sl = d_sqrt(s.lam);
-    t.u[0] = T(0.5) * d_erfc(-sg * sl * s.u);
-    const T inv_sqrt_pi = T(0.56418958354775628695);
-    t.u[1] = s.u * t.u[0] + sg * T(0.5) * inv_sqrt_pi * d_exp(-s.lam * s.u * s.u) / sl;
-    mom_recur(t.u, s.u, h);
-}
-
-template <int P, int Q, int R, typename T>
-__device__ __forceinline__ T Gm(const Tab<T>& t) {
-    return t.u[P] * t.v[Q] * t.w[R];
-}
-
-// <eps u^P v^Q w^R>, eps = (u^2 + v^2 + w^2 + xi^2) / 2
-template <int P, int Q, int R, typename T>
-__device__ __forceinline__ T Em(const Tab<T>& t) {
-    return T(0.5) * (Gm<P + 2, Q, R>(t) + Gm<P, Q + 2, R>(t) + Gm<P, Q, R + 2>(t) + t.xi2 * Gm<P, Q, R>(t));
-}
-
-// <eps^2 u^P v^Q w^R>
-template <int P, int Q, int R, typename T>
-__device__ __forceinline__ T E2m(const Tab<T>& t) {
-    return T(0.25) * (Gm<P + 4, Q, R>(t) + Gm<P, Q + 4, R>(t) + Gm<P, Q, R + 4>(t) + t.xi4 * Gm<P, Q, R>(t) +
-                      T(2) * (Gm<P + 2, Q + 2, R>(t) + Gm<P + 2, Q, R + 2>(t) + Gm<P, Q + 2, R + 2>(t)) +
-                      T(2) * t.xi2 * (Gm<P + 2, Q, R>(t) + Gm<P, Q + 2, R>(t) + Gm<P, Q, R + 2>(t)));
-}
-
-// out_alpha += c * <psi_alpha u^P v^Q w^R>
-template <int P, int Q, int R, typename T>
-__device__ __forceinline__ void acc_psi(const Tab<T>& t, T c, T* out) {
-    out[0] += c * Gm<P, Q, R>(t);
-    out[1] += c * Gm<P + 1, Q, R>(t);
-    out[2] += c * Gm<P, Q + 1, R>(t);
-    out[3] += c * Gm<P, Q, R + 1>(t);
-    out[4] += c * Em<P, Q, R>(t);
-}
-
-// out_alpha += c * <psi_alpha (a.psi) u^P v^Q w^R>
-template <int P, int Q, int R, typename T>
-__device__ __forceinline__ void acc_apsi(const Tab<T>& t, const T* a, T c, T* out) {
-    const T a0 = c * a[0], a1 = c * a[1], a2 = c * a[2], a3 = c * a[3], a4 = c * a[4];
-    out[0] += a0 * Gm<P, Q, R>(t) + a1 * Gm<P + 1, Q, R>(t) + a2 * Gm<P, Q + 1, R>(t) +
-              a3 * Gm<P, Q, R + 1>(t) + a4 * Em<P, Q, R>(t);
-    out[1] += a0 * Gm<P + 1, Q, R>(t) + a1 * Gm<P + 2, Q, R>(t) + a2 * Gm<P + 1, Q + 1, R>(t) +
-              a3 * Gm<P + 1, Q, R + 1>(t) + a4 * Em<P + 1, Q, R>(t);
-    out[2] += a0 * Gm<P, Q + 1, R>(t) + a1 * Gm<P + 1, Q + 1, R>(t) + a2 * Gm<P, Q + 2, R>(t) +
-              a3 * Gm<P, Q + 1, R + 1>(t) + a4 * Em<P, Q + 1, R>(t);
-    out[3] += a0 * Gm<P, Q, R + 1>(t) + a1 * Gm<P + 1, Q, R + 1>(t) + a2 * Gm<P, Q + 1, R + 1>(t) +
-              a3 * Gm<P, Q, R + 2>(t) + a4 * Em<P, Q, R + 1>(t);
-    out[4] += a0 * Em<P, Q, R>(t) + a1 * Em<P + 1, Q, R>(t) + a2 * Em<P, Q + 1, R>(t) +
-              a3 * Em<P, Q, R + 1>(t) + a4 * E2m<P, Q, R>(t);
-}
-
-// out += c * sum_i <psi (a_i . psi) u_i u^P>   (P = 0 or 1 extra powers of u)
-template <int P, typename T>
-__device__ __forceinline__ void acc_grad(const Tab<T>& t, const T (*a)[5], T c, T* out) {
-    acc_apsi<P + 1, 0, 0>(t, a[0], c, out);
-    acc_apsi<P, 1, 0>(t, a[1], c, out);
-    acc_apsi<P, 0, 1>(t, a[2], c, out);
-}
-
-// Micro-slope of a Maxwellian: solves <a psi> = b (full space) for a, with
-// the closed-form inverse of the moment matrix.
-template <typename T>
-__device__ __forceinline__ void micro_slope(const Prim<T>& s, T K, const T* b, T* a) {
-    const T q = s.u * s.u + s.v * s.v + s.w * s.w;
-    const T e = q + (K + T(3)) * T(0.5) / s.lam;  // 2 <eps>
-    const T r1 = b[1] - s.u * b[0];
-    const T r2 = b[2] - s.v * b[0];
-    const T r3 = b[3] - s.w * b[0];
-    const T r4 = T(2) * b[4] - e * b[0];
-    const T a4 = T(4) * s.lam * s.lam / (K + T(3)) * (r4 - T(2) * (s.u * r1 + s.v * r2 + s.w * r3));
-    const T tl = T(2) * s.lam;
-    a[1] = tl * r1 - s.u * a4;
-    a[2] = tl * r2 - s.v * a4;
-    a[3] = tl * r3 - s.w * a4;
-    a[4] = a4;
-    a[0] = b[0] - s.u * a[1] - s.v * a[2] - s.w * a[3] - T(0.5) * a4 * e;
-}
-
+// ------------------------------------------------- time integration --
 // Time coefficients of Eq. 2nd-flux over [0, dt/2] (k0, k1 for the kinetic
-// factors e and t e; q1..q3 for C1..C3) and their "dt minus twice dt/2"
+// factors e and t e; q2, q3 for C2, C3) and their "dt minus twice dt/2"
 // differences (dk*, dq*), with E = exp(-dt/tau_n) = Eh^2.
 template <typename T>
 struct TimeCoef {
     T tau, tau_n, E;
-    T k0, k1, q1, q2, q3;
-    T dk0, dk1, dq1, dq2, dq3;
+    T k0, k1, q2, q3;
+    T dk0, dk1, dq2, dq3;
 };
 
 template <typename T>
@@ -282,21 +137,13 @@ __device__ __forceinline__ TimeCoef<T> time_coefs(const Phys<T>& ph, T pl, T pr,
     const T tn = c.tau_n, tau = c.tau;
     c.k0 = tn * omh;
     c.k1 = tn * (tn * omh - hd * Eh);
-    c.q1 = hd - c.k0;
     c.q2 = c.k1 + tau * c.k0 - tau * hd;
     c.q3 = T(0.5) * hd * hd - tau * hd + tau * c.k0;
     c.dk0 = -tn * omh * omh;
     c.dk1 = -tn * tn * omh * omh + tn * dt * Eh * omh;
-    c.dq1 = tn * omh * omh;
     c.dq2 = c.dk1 + tau * c.dk0;
     c.dq3 = T(0.25) * dt * dt + tau * c.dk0;
     return c;
-}
-
-template <typename T>
-__device__ __forceinline__ void axpy5(T a, const T* x, T* y) {
-#pragma unroll
-    for (int k = 0; k < 5; ++k) y[k] += a * x[k];
 }
 
 // Pr fix of the energy flux over one time interval: F_E += (1/Pr - 1) q with
@@ -496,6 +343,5 @@ __device__ __forceinline__ F2 f2_div(F2 a, F2 b) {
     return f2_norm(q, r.hi / b.hi);
 }
 
-__device__ __forceinline__ double f2_value(F2 a) { return (double)a.hi + (double)a.lo; }
 
 }  // namespace gks

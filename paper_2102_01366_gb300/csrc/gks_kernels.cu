@@ -140,19 +140,6 @@ __global__ void __launch_bounds__(PACK_THREADS) k_unpack(const double* __restric
         for (int j = 0; j < 15; ++j) dW[j * nc + c] = widen(x[Stride<T>::xg + j]);
 }
 
-// component-major [ncomp][nc] arrays between the device cell order and the
-// caller's (cperm: device cell -> caller's cell)
-__global__ void k_cells_perm(const double* __restrict__ in, double* __restrict__ out, int64_t nc, int ncomp,
-                             const int32_t* __restrict__ cperm, int to_public) {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nc * ncomp; i += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t k = i / nc, d = i - k * nc, c = cperm[d];
-        if (to_public)
-            out[k * nc + c] = in[i];
-        else
-            out[i] = in[k * nc + c];
-    }
-}
-
 // out row r = in row map[r], rows of `width` words of 4 bytes
 __global__ void k_rows_gather(const uint32_t* __restrict__ in, uint32_t* __restrict__ out, int64_t nrows, int width,
                               const int32_t* __restrict__ map) {
@@ -259,13 +246,6 @@ cudaError_t Launch<T>::unpack(const double* Wd, const T* X, double* W, double* d
                               const int32_t* cperm) {
     if (nc == 0) return cudaSuccess;
     k_unpack<T><<<pack_grid(nc), PACK_THREADS, 0, s>>>(Wd, X, W, dW, nc, cperm);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_cells_perm(const double* in, double* out, int64_t nc, int ncomp, const int32_t* cperm,
-                              int to_public, cudaStream_t s) {
-    if (nc == 0) return cudaSuccess;
-    k_cells_perm<<<ew_grid(nc * ncomp), 256, 0, s>>>(in, out, nc, ncomp, cperm, to_public);
     return cudaGetLastError();
 }
 

@@ -237,10 +237,6 @@ struct AdjBuffers {
     int8_t* rev;
     int32_t* fallback;
 };
-// [ncomp][nc] FP64 arrays between device cell order and the caller's
-// (cperm: device cell -> caller's cell; to_public 1: out[cperm[d]] = in[d])
-cudaError_t launch_cells_perm(const double* in, double* out, int64_t nc, int ncomp, const int32_t* cperm,
-                              int to_public, cudaStream_t s);
 // out row r = in row map[r] for rows of width_words 4-byte words
 cudaError_t launch_rows_gather(const void* in, void* out, int64_t nrows, int width_words, const int32_t* map,
                                cudaStream_t s);

@@ -305,7 +305,7 @@ __device__ __forceinline__ void finish_point(const Phys<T>& ph, const KSums<T>& 
 #pragma unroll
         for (int q = 0; q < 5; ++q) {
             // kinetic minus equilibrium moments under the kinetic factors
-            // (q1 = dt/2 - k0, q2 = k1 + tau k0 - tau dt/2)
+            // (C1's is dt/2 - k0, C2's k1 + tau k0 - tau dt/2)
             const T e0 = S.f0[q] - f0[q], e1 = S.f1[q] - f1[q];
             Fh[q] = tc.k0 * e0 - c1 * e1 + tc.q3 * f2[q];
             if (!REL) Fh[q] += hd * f0[q];
@@ -346,18 +346,6 @@ __device__ __forceinline__ void finish_point(const Phys<T>& ph, const KSums<T>& 
             prandtl_fix(ph.prf, U, IWd, D);
         }
     }
-}
-
-// The whole point from both sides' states and gradients (face frame).
-template <bool VISC, typename T>
-__device__ __forceinline__ void kin_point(const Phys<T>& ph, const T* Wl, const T (*gl)[5], const T* Wr,
-                                          const T (*gr)[5], T dt, T* Fh, T* D, T* W0, T* dW) {
-    KSums<T> S;
-    S.init();
-    const T pl = kin_side<VISC>(ph, Wl, gl, +1, S);
-    const T pr = kin_side<VISC>(ph, Wr, gr, -1, S);
-    T Wc[5];
-    finish_point<VISC, false>(ph, S, pl, pr, dt, Wc, Fh, D, W0, dW);
 }
 
 }  // namespace gks
