@@ -9,6 +9,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <memory>
 #include <new>
 #include <string>
 #include <vector>
@@ -595,7 +596,7 @@ static gks_status upload_faces(gks_state* s) {
             }
         }
     });
-    run_ranges(nf, host_threads(nf, 4096), [&](int64_t, int64_t lo, int64_t hi) {
+    run_ranges(nf, host_threads(nf, 2048), [&](int64_t, int64_t lo, int64_t hi) {
         for (int64_t d = lo; d < hi; ++d) {
             const int64_t f = perm[d];
             // a boundary face's missing side carries its kind: -1 - GKS_BC_*
@@ -642,8 +643,12 @@ static gks_status upload_cells(gks_state* s) {
     const int64_t nblk = update_blocks(nc);
     std::vector<T> dr(nc);
     std::vector<TO> M1(12 * nc);
-    // per-block tile of TILE_ROWS values a cell (tile_at), zero past the last cell
-    std::vector<TO> tile((size_t)nblk * TILE_ROWS * CELLS_PER_BLOCK, TO(0));
+    // per-block tile of TILE_ROWS values a cell (tile_at), zero past the last
+    // cell; not cleared as a whole, so that its pages are first touched by the
+    // threads that fill them
+    constexpr size_t TILE = (size_t)TILE_ROWS * CELLS_PER_BLOCK;
+    const std::unique_ptr<TO[]> tile(new TO[(size_t)nblk * TILE]);
+    if (nc % CELLS_PER_BLOCK) std::fill_n(&tile[(size_t)(nblk - 1) * TILE], TILE, TO(0));
     // Sec. 4.4: with linear weights a boundary cell's third-order step is the
     // least-squares first-order fit to its P2 stencil
     const bool linear_boundary = !s->params.weno && s->params.order == 3;
@@ -663,7 +668,7 @@ static gks_status upload_cells(gks_state* s) {
             for (int k = 0; k < 15; ++k) o[WOP_W1 + k] = (TO)w1[k];
         }
     }
-    run_ranges(nc, host_threads(nc, 2048), [&](int64_t, int64_t lo, int64_t hi) {
+    run_ranges(nc, host_threads(nc, 768), [&](int64_t, int64_t lo, int64_t hi) {
         for (int64_t d = lo; d < hi; ++d) {
             const int64_t c = s->pub(d);
             cell_case[d] = g.cell_case[c];
@@ -698,8 +703,7 @@ static gks_status upload_cells(gks_state* s) {
             for (int k = 0; k < 144; ++k) row[TILE_M2 + k] = M2c[k];
             // the cell's rows in their 16-byte groups (tile_at)
             constexpr int V = 16 / (int)sizeof(TO);
-            TO* to = &tile[(size_t)(d / CELLS_PER_BLOCK) * TILE_ROWS * CELLS_PER_BLOCK +
-                           (size_t)tile_at<TO>(0, (int)(d % CELLS_PER_BLOCK))];
+            TO* to = &tile[(size_t)(d / CELLS_PER_BLOCK) * TILE + (size_t)tile_at<TO>(0, (int)(d % CELLS_PER_BLOCK))];
             for (int k = 0; k < TILE_ROWS / V; ++k, to += CELLS_PER_BLOCK * V)
                 for (int v = 0; v < V; ++v) to[v] = (TO)row[k * V + v];
         }
@@ -711,7 +715,7 @@ static gks_status upload_cells(gks_state* s) {
     GKS_CHECK_CUDA(put(L.inv_vol, inv_vol.data(), 8 * inv_vol.size()));
     GKS_CHECK_CUDA(put(L.dr, dr.data(), sizeof(T) * dr.size()));
     GKS_CHECK_CUDA(put(L.M1, M1.data(), sizeof(TO) * M1.size()));
-    GKS_CHECK_CUDA(put(L.tile, tile.data(), sizeof(TO) * tile.size()));
+    GKS_CHECK_CUDA(put(L.tile, tile.get(), sizeof(TO) * (size_t)nblk * TILE));
     GKS_CHECK_CUDA(put(L.cell_case, cell_case.data(), 4 * cell_case.size()));
     if (L.wslot) {
         GKS_CHECK_CUDA(put(L.wslot, wslot.data(), 4 * wslot.size()));
