@@ -44,8 +44,22 @@ constexpr int flux_vals() { return NR == 40 ? 20 : 10; }
 template <typename T, int NR, int TH = FLUX_THREADS>
 struct FluxSmem {
     T out[TH][flux_vals<NR>() + 1];
-    T frame[(TH + 2) / 3][7];  // tangents of the face frame
+    T frame[(TH + 2) / 3][7];                                 // tangents of the face frame
+    T ref[sizeof(T) == 4 && NR == 40 ? (TH + 2) / 3 : 1][11];  // reference flux (FP32 stage 1)
 };
+
+// hi (5) and lo (5) parts of a record's cell average, in whole vectors: ten
+// single loads each went to as many lines as the warp has faces
+__device__ __forceinline__ void load_average(const float* __restrict__ P, float* hi, float* lo) {
+    static_assert(PHI == 50 && PLO == 55 && POLY_STRIDE32 == 60, "the averages end the record");
+    float v[12];
+    load_vec<12>(P + 48, v);
+#pragma unroll
+    for (int q = 0; q < 5; ++q) {
+        hi[q] = v[2 + q];
+        lo[q] = v[7 + q];
+    }
+}
 
 // Stage 1, FP32: the interface state W^c of Eq. new-equ-part relative to W_m,
 // the mean of the two cells' averages (the interior cell's average on a
@@ -68,14 +82,14 @@ __device__ __forceinline__ void interface_deviation(const float* __restrict__ po
     const bool pair = (L >= 0 || L == FLR_OPEN) && (Rc >= 0 || Rc == FLR_OPEN);
     const float* al = poly + (int64_t)(L >= 0 ? L : Rc) * PS;
     const float* ar = poly + (int64_t)(Rc >= 0 ? Rc : L) * PS;
-    float Wm[5], sg[5], hg[5];
+    float Wm[5], sg[5], hg[5], ql[5], ll[5], qr[5], lr[5];
+    load_average(al, ql, ll);
+    load_average(ar, qr, lr);
 #pragma unroll
     for (int q = 0; q < 5; ++q) {
-        const float ql = __ldg(al + PHI + q), qr = __ldg(ar + PHI + q);
-        const float ll = __ldg(al + PLO + q), lr = __ldg(ar + PLO + q);
-        Wm[q] = 0.5f * (ql + qr);
+        Wm[q] = 0.5f * (ql[q] + qr[q]);
         sg[q] = 0.5f * dsum[q];
-        hg[q] = 0.5f * (((ql - qr) + (ll - lr)) + ddiff[q]);
+        hg[q] = 0.5f * (((ql[q] - qr[q]) + (ll[q] - lr[q])) + ddiff[q]);
     }
     float tm[5] = {Wm[0], 0, 0, 0, Wm[4]};
     rotate_vec(Rm, Wm + 1, tm + 1);
@@ -94,12 +108,10 @@ __device__ __forceinline__ void interface_deviation(const float* __restrict__ po
         flux1_difference(Wc, tm, dW, gm1, dF);
     } else {
         // both records are the interior cell's: W_m = hi + lo
-        float lo[5], tlo[5], Fc[5], Fm[5];
-#pragma unroll
-        for (int q = 0; q < 5; ++q) lo[q] = __ldg(al + PLO + q);
-        tlo[0] = lo[0];
-        tlo[4] = lo[4];
-        rotate_vec(Rm, lo + 1, tlo + 1);
+        float tlo[5], Fc[5], Fm[5];
+        tlo[0] = ll[0];
+        tlo[4] = ll[4];
+        rotate_vec(Rm, ll + 1, tlo + 1);
 #pragma unroll
         for (int q = 0; q < 5; ++q) {
             dW[q] = (Wc[q] - tm[q]) - tlo[q];
@@ -123,9 +135,12 @@ __device__ __forceinline__ void reference_flux(const float* __restrict__ poly, c
     const float* al = poly + (int64_t)(L >= 0 ? L : Rc) * PS;
     const float* ar = poly + (int64_t)(Rc >= 0 ? Rc : L) * PS;
     F2 Wm[5], ref[5];
+    float ql[5], ll[5], qr[5], lr[5];
+    load_average(al, ql, ll);
+    load_average(ar, qr, lr);
 #pragma unroll
     for (int q = 0; q < 5; ++q) {
-        const F2 a = f2_add({__ldg(al + PHI + q), __ldg(al + PLO + q)}, {__ldg(ar + PHI + q), __ldg(ar + PLO + q)});
+        const F2 a = f2_add({ql[q], ll[q]}, {qr[q], lr[q]});
         Wm[q] = {0.5f * a.hi, 0.5f * a.lo};
     }
     const F2 A[3] = {{an[0], an[1]}, {an[2], an[3]}, {an[4], an[5]}};
@@ -240,54 +255,65 @@ __device__ __forceinline__ void flux_faces(const DevMesh<T>& m, const Phys<T>& p
     // the interface-state entries and (FP32 stage 1) the reference flux
     const int job = tid / FACES, lf = tid - FACES * job;
     const int64_t f = fb * FACES + lf;
-    if (f >= m.nf || job > (REL ? 2 : 1)) return;
-    constexpr int RS = rec_stride<T, NR>();
-    T* r = rec + f * RS;
+    constexpr int VALS = flux_vals<NR>(), RS = rec_stride<T, NR>();
+    if (f < m.nf && job < 2) {
+        T Rm[3][3], n[4];
+        load_vec<4>(m.fgeo + f * FGEO, n);
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            Rm[0][i] = n[i];
+            Rm[1][i] = sm.frame[lf][i];
+            Rm[2][i] = sm.frame[lf][3 + i];
+        }
+        const T w = n[3];
+        auto sum = [&](int at, T* v) {
+#pragma unroll
+            for (int q = 0; q < 5; ++q)
+                v[q] = w * ((sm.out[3 * lf][at + q] + sm.out[3 * lf + 1][at + q]) + sm.out[3 * lf + 2][at + q]);
+            to_global(Rm, v);
+        };
+        // FP32 stage 1: into the columns that only this thread has read
+        T* r = (REL ? sm.out[3 * lf] : rec + f * RS) + (VALS / 2) * job;
+        T a[5], b[5];
+        sum((VALS / 2) * job, a);
+        if constexpr (NR == 40) {
+            sum(10 * job + 5, b);
+#pragma unroll
+            for (int q = 0; q < 5; ++q) {
+                // dt L + dt^2/6 L_t = 8/3 Fh - 1/3 F = 2 Fh - D / 3 (Eqs. linear-system, s2o4)
+                // f* = f^n + dt/2 f_t^n
+                r[q] = job == 0 ? a[q] : a[q] + T(0.5) * b[q];
+                r[5 + q] = job == 0 ? T(2) * a[q] - b[q] * T(1.0 / 3.0) : a[q];
+            }
+        } else {
+#pragma unroll
+            for (int q = 0; q < 5; ++q)
+                // dt^2/3 L_t(W*) = 4/3 (F* - 2 Fh*); f^{n+1} = f^n + dt f_t^*
+                r[q] = job == 0 ? T(4.0 / 3.0) * a[q] : a[q];
+        }
+    }
     if constexpr (REL) {
-        if (job == 2) {
+        if (f < m.nf && job == 2) {
             const int L = m.flr[f], Rc = m.flr[m.nf + f];
             const double dtc = ctrl ? ctrl[m.cell_case[L >= 0 ? L : Rc]] : dt_override;
-            reference_flux(poly, m.fan + 6 * f, L, Rc, ph.gm1, dtc > 0.0 ? (T)dtc : T(1), r + REC1_REF);
-            return;
+            reference_flux(poly, m.fan + 6 * f, L, Rc, ph.gm1, dtc > 0.0 ? (T)dtc : T(1), sm.ref[lf]);
         }
-    }
-    T Rm[3][3], n[4];
-    load_vec<4>(m.fgeo + f * FGEO, n);
+        group_barrier(bar_id, TH);
+        // the block's records are one stretch of memory: whole vectors by all
+        // threads, where a thread per face wrote each of its 10 words to a line
+        // of its own (L1's data pipe 67 % busy).  Stage 1, 3.15 M faces: 1,071
+        // -> 973 us.  Stage 2's short records lost more by the second barrier
+        // (687 -> 733 us) and FP64 has its pipe as bound: these write directly.
+        const int64_t left = m.nf - fb * FACES;
+        const int words = (int)(left < FACES ? left : FACES) * (RS / 4);
+        for (int i = tid; i < words; i += TH) {
+            const int face = i / (RS / 4), e = 4 * (i - face * (RS / 4));
+            T v[4];
 #pragma unroll
-    for (int i = 0; i < 3; ++i) {
-        Rm[0][i] = n[i];
-        Rm[1][i] = sm.frame[lf][i];
-        Rm[2][i] = sm.frame[lf][3 + i];
-    }
-    const T w = n[3];
-    auto sum = [&](int at, T* v) {
-#pragma unroll
-        for (int q = 0; q < 5; ++q)
-            v[q] = w * ((sm.out[3 * lf][at + q] + sm.out[3 * lf + 1][at + q]) + sm.out[3 * lf + 2][at + q]);
-        to_global(Rm, v);
-    };
-    if constexpr (NR == 40) {
-        T a[5], b[5];
-        sum(10 * job, a);
-        sum(10 * job + 5, b);
-#pragma unroll
-        for (int q = 0; q < 5; ++q) {
-            if (job == 0) {
-                // dt L + dt^2/6 L_t = 8/3 Fh - 1/3 F = 2 Fh - D / 3 (Eqs. linear-system, s2o4)
-                r[q] = a[q];
-                r[5 + q] = T(2) * a[q] - b[q] * T(1.0 / 3.0);
-            } else {
-                r[10 + q] = a[q] + T(0.5) * b[q];  // f* = f^n + dt/2 f_t^n
-                r[15 + q] = a[q];
-            }
+            for (int k = 0; k < 4; ++k)
+                v[k] = e < VALS ? sm.out[3 * face][e + k] : e + k < VALS + 10 ? sm.ref[face][e + k - VALS] : T(0);
+            store_vec<4>(rec + fb * FACES * RS + 4 * (int64_t)i, v);
         }
-    } else {
-        T a[5];
-        sum(5 * job, a);
-#pragma unroll
-        for (int q = 0; q < 5; ++q)
-            // dt^2/3 L_t(W*) = 4/3 (F* - 2 Fh*); f^{n+1} = f^n + dt f_t^*
-            r[5 * job + q] = job == 0 ? T(4.0 / 3.0) * a[q] : a[q];
     }
 }
 
