@@ -172,8 +172,8 @@ __device__ __forceinline__ void adj_point_setup(const DevMesh<double>& m, const 
     rotate_in(Rm, ldWt);
 #pragma unroll 1
     for (int side = 0; side < 2; ++side)
-        side_state<double, true>(m, ph, Xavg, poly, geo, Rm, L, R, side, k, x[side],
-                                 reinterpret_cast<double (*)[5]>(x[side] + 5));
+        side_state<double, true>(m, ph, Xavg, poly + side_cell(L, R, side) * POLY_STRIDE, geo, Rm, L, R, side, k,
+                                 x[side], reinterpret_cast<double (*)[5]>(x[side] + 5));
 }
 
 // A forward-mode number (value and one derivative) for the Jacobian of the

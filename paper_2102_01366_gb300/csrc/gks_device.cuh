@@ -1,16 +1,12 @@
 // gks_device.cuh -- device-side building blocks of libgks, templated on the
 // working precision T (double: FP64 path; float: FP32-bulk path).
 //
-//   * Maxwellian moments <u^p v^q w^r> over the full space or a half space
-//     (Sec. 2.2; the half-space zeroth and first moments come from erfc and
-//     the Gaussian tail, higher ones from the standard recursion);
-//   * micro-slopes a = a_1 + a_2 u + a_3 v + a_4 w + a_5 (u^2+xi^2)/2 solving
-//     <a psi> = dW / rho (Eq. co) in closed form (the inverse of the 5x5
-//     moment matrix of a Maxwellian);
-//   * the time-dependent kinetic solution at one Gauss point in the face
-//     frame (Eq. 2nd-flux / Eq. 2nd-smooth-flux with the equilibrium state
-//     of Eq. new-equ-part): time integrals of the flux over [0, dt/2] and
-//     [0, dt], and the interface states at t = 0 and t = dt.
+//   * conversions between FP64 and FP32 off the FP64 pipe, compensated sums
+//     and FP32 pairs;
+//   * the time coefficients of Eq. 2nd-flux over [0, dt/2] and [0, dt];
+//   * the Pr fix, the wall-independent parts of the FP32 interface deviation
+//     (half-differences) and the Euler flux.
+// The kinetic solution itself is in gks_kinetic.cuh.
 #pragma once
 
 #include <cstdint>

@@ -24,7 +24,7 @@ __device__ __forceinline__ void eval_poly(const T* __restrict__ P, const T* X, T
         const float4* p4 = reinterpret_cast<const float4*>(P);
 #pragma unroll
         for (int i = 0; i < PS / 4; ++i) {
-            const float4 v = __ldg(p4 + i);
+            const float4 v = p4[i];
             c[4 * i] = v.x;
             c[4 * i + 1] = v.y;
             c[4 * i + 2] = v.z;
@@ -241,15 +241,22 @@ __device__ __forceinline__ void fixed_ghost(const T* __restrict__ x0, const T* X
     }
 }
 
+// the cell whose record a side is evaluated from: its own, or the interior
+// one for a boundary face's missing side
+__device__ __forceinline__ int64_t side_cell(int L, int Rc, int side) {
+    const int mine = side == 0 ? L : Rc;
+    return mine >= 0 ? mine : side == 0 ? Rc : L;
+}
+
 // One side's state and gradients at Gauss point k of a face, face frame: the
-// side's cell reconstruction there, or the boundary face's ghost (side 0:
+// reconstruction P of side_cell there, or the boundary face's ghost (side 0:
 // left, 1: right; a missing side carries its kind).  XW: isothermal and
 // moving walls are compiled in.  dev (FP32, may be NULL) receives the
 // evaluated reconstruction minus its cell's average, global frame (0 for an
 // open or fixed side).
 template <typename T, bool XW>
 __device__ __forceinline__ void side_state(const DevMesh<T>& m, const Phys<T>& ph, const T* __restrict__ Wavg,
-                                           const T* __restrict__ poly, const T* __restrict__ geo,
+                                           const T* __restrict__ P, const T* __restrict__ geo,
                                            const T (*Rm)[3], int L, int Rc, int side, int k, T* tW, T (*tg)[5],
                                            T* dev = nullptr) {
     const int mine = side == 0 ? L : Rc, other = side == 0 ? Rc : L;
@@ -274,7 +281,7 @@ __device__ __forceinline__ void side_state(const DevMesh<T>& m, const Phys<T>& p
         if (mine == FLR_FIXED)
             fixed_ghost(m.fixed + c * Stride<T>::xs, X, Ws, gs);
         else
-            eval_poly(poly + c * Stride<T>::poly, X, Ws, gs, dev);
+            eval_poly(P, X, Ws, gs, dev);
     }
     to_local(Rm, Ws, gs, tW, tg);
     if (mine == FLR_SLIP_WALL) slip_wall_ghost(tW, tg);

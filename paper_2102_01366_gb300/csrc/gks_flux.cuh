@@ -41,8 +41,19 @@ constexpr int FLUX_THREADS = 3 * FLUX_FACES;
 template <int NR>
 constexpr int flux_vals() { return NR == 40 ? 20 : 10; }
 
+// FP32 stage 2 has its faces' records and geometry copied to shared memory
+// while it forms the face frames: one barrier, but no wait for a gather in
+// either side's turn (stage 2 on 3.15 M faces 679 -> 631 us, viscous on 1.16 M
+// 287 -> 255 us).  In stage 1, whose longer output leaves the L1 less room and
+// which prefetches the right side, it cost 975 -> 1,018 us.
+template <typename T, int NR>
+constexpr bool flux_copies() { return sizeof(T) == 4 && NR == 20; }
+
 template <typename T, int NR, int TH = FLUX_THREADS>
 struct FluxSmem {
+    // FP32 stage 2: both sides' reconstruction records and the geometry of each face
+    alignas(16) T poly[flux_copies<T, NR>() ? (TH + 2) / 3 : 1][2][flux_copies<T, NR>() ? Stride<T>::poly : 4];
+    alignas(16) T geo[flux_copies<T, NR>() ? (TH + 2) / 3 : 1][flux_copies<T, NR>() ? FGEO : 4];
     T out[TH][flux_vals<NR>() + 1];
     T frame[(TH + 2) / 3][7];                                 // tangents of the face frame
     T ref[sizeof(T) == 4 && NR == 40 ? (TH + 2) / 3 : 1][11];  // reference flux (FP32 stage 1)
@@ -50,7 +61,7 @@ struct FluxSmem {
 
 // hi (5) and lo (5) parts of a record's cell average, in whole vectors: ten
 // single loads each went to as many lines as the warp has faces
-__device__ __forceinline__ void load_average(const float* __restrict__ P, float* hi, float* lo) {
+__device__ __forceinline__ void load_average(const float* P, float* hi, float* lo) {
     static_assert(PHI == 50 && PLO == 55 && POLY_STRIDE32 == 60, "the averages end the record");
     float v[12];
     load_vec<12>(P + 48, v);
@@ -71,17 +82,15 @@ __device__ __forceinline__ void load_average(const float* __restrict__ P, float*
 // (exact differences of the hi / lo averages) and by the half-difference
 // rules, both carry rounding relative to themselves only.  Interior and open
 // faces; wall and fixed faces subtract directly.
+//   al, ar       the sides' records (a missing side's: the interior cell's)
 //   dsum, ddiff  sum and difference (left - right) of the sides' R - average
 //   hl, hr       the sides' half-space moments
-__device__ __forceinline__ void interface_deviation(const float* __restrict__ poly, int L, int Rc,
+__device__ __forceinline__ void interface_deviation(const float* al, const float* ar, int L, int Rc,
                                                     const float (*Rm)[3], const float* dsum, const float* ddiff,
                                                     const HalfSpace<float>& hl, const HalfSpace<float>& hr,
                                                     const float* Wc, float gm1, float* dW,
                                                     float* dF) {
-    constexpr int PS = Stride<float>::poly;
     const bool pair = (L >= 0 || L == FLR_OPEN) && (Rc >= 0 || Rc == FLR_OPEN);
-    const float* al = poly + (int64_t)(L >= 0 ? L : Rc) * PS;
-    const float* ar = poly + (int64_t)(Rc >= 0 ? Rc : L) * PS;
     float Wm[5], sg[5], hg[5], ql[5], ll[5], qr[5], lr[5];
     load_average(al, ql, ll);
     load_average(ar, qr, lr);
@@ -129,11 +138,8 @@ __device__ __forceinline__ void interface_deviation(const float* __restrict__ po
 // over a closed cell vanishes to FP64 rounding, where the FP32 weights and
 // normals leave eps A), in FP32 pairs, stored as hi and lo parts; entering
 // both cells with opposite signs, it keeps the update exactly conservative.
-__device__ __forceinline__ void reference_flux(const float* __restrict__ poly, const float* __restrict__ an, int L,
-                                               int Rc, float gm1, float dt, float* __restrict__ out) {
-    constexpr int PS = Stride<float>::poly;
-    const float* al = poly + (int64_t)(L >= 0 ? L : Rc) * PS;
-    const float* ar = poly + (int64_t)(Rc >= 0 ? Rc : L) * PS;
+__device__ __forceinline__ void reference_flux(const float* al, const float* ar, const float* __restrict__ an,
+                                               float gm1, float dt, float* __restrict__ out) {
     F2 Wm[5], ref[5];
     float ql[5], ll[5], qr[5], lr[5];
     load_average(al, ql, ll);
@@ -161,6 +167,12 @@ __device__ __forceinline__ void reference_flux(const float* __restrict__ poly, c
     }
 }
 
+// asynchronous copy of 16 bytes to shared memory
+__device__ __forceinline__ void copy16(float* to, const float* from) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(to)), "l"(from)
+                 : "memory");
+}
+
 // One block of TH / 3 faces (block index fb) by TH threads (tid; one may be
 // left over, which computes and stores nothing): sm its shared memory, bar_id the barrier of its threads (0: the
 // whole thread block).  VISC: viscous flow (time slopes, Pr fix).  XW: the
@@ -171,7 +183,7 @@ __device__ __forceinline__ void flux_faces(const DevMesh<T>& m, const Phys<T>& p
                                            const T* __restrict__ poly, T* __restrict__ rec,
                                            const double* __restrict__ ctrl, double dt_override, int64_t fb, int tid,
                                            FluxSmem<T, NR, TH>& sm, int bar_id) {
-    constexpr bool REL = sizeof(T) == 4 && NR == 40;
+    constexpr bool REL = sizeof(T) == 4 && NR == 40, COPY = flux_copies<T, NR>();
     constexpr int FACES = TH / 3;
     static_assert(REL ? FACES == 32 : 2 * FACES <= TH, "a thread per face and job");
     {
@@ -181,6 +193,18 @@ __device__ __forceinline__ void flux_faces(const DevMesh<T>& m, const Phys<T>& p
         const int L = m.flr[f], Rc = m.flr[m.nf + f];
         const T* geo = m.fgeo + f * FGEO;
         const T n[3] = {geo[0], geo[1], geo[2]};
+        if constexpr (COPY) {
+            // both sides' records on their way to shared memory, 16 bytes a
+            // copy, a third of each by each of the face's threads
+#pragma unroll
+            for (int side = 0; side < 2; ++side) {
+                const T* p = poly + side_cell(L, Rc, side) * Stride<T>::poly;
+#pragma unroll
+                for (int j = 4 * k; j < Stride<T>::poly; j += 12) copy16(&sm.poly[lf][side][j], p + j);
+            }
+#pragma unroll
+            for (int j = 4 * k; j < FGEO; j += 12) copy16(&sm.geo[lf][j], geo + j);
+        }
         T Rm[3][3];
         face_frame(n, Rm);
         if (k == 0) {
@@ -193,10 +217,13 @@ __device__ __forceinline__ void flux_faces(const DevMesh<T>& m, const Phys<T>& p
         if constexpr (REL) {
             // the right side's record on its way to L1 while the left side is
             // worked on: the face's three threads take its (at most three)
-            // lines.  Stage 1, 3.15 M faces: 1,160 -> 1,108 us; in stage 2,
-            // with less to do in between, it gained nothing.
-            const T* rr = poly + (int64_t)(Rc >= 0 ? Rc : L) * Stride<T>::poly;
+            // lines.  Stage 1, 3.15 M faces: 1,160 -> 1,108 us.
+            const T* rr = poly + side_cell(L, Rc, 1) * Stride<T>::poly;
             asm volatile("prefetch.global.L1 [%0];" ::"l"(rr + (k < 2 ? 32 * k : Stride<T>::poly - 1)));
+        }
+        if constexpr (COPY) {
+            asm volatile("cp.async.wait_all;" ::: "memory");
+            group_barrier(bar_id, TH);
         }
         KSums<T> S;
         S.init();
@@ -207,7 +234,9 @@ __device__ __forceinline__ void flux_faces(const DevMesh<T>& m, const Phys<T>& p
 #pragma unroll 1
         for (int side = 0; side < 2; ++side) {
             T tW[5], tg[3][5], dev[5];
-            side_state<T, XW>(m, ph, Wavg, poly, geo, Rm, L, Rc, side, k, tW, tg, REL ? dev : nullptr);
+            const T* P = COPY ? &sm.poly[lf][side][0] : poly + side_cell(L, Rc, side) * Stride<T>::poly;
+            const T* G = COPY ? &sm.geo[lf][0] : geo;
+            side_state<T, XW>(m, ph, Wavg, P, G, Rm, L, Rc, side, k, tW, tg, REL ? dev : nullptr);
             pl = pr;
             hl = hr;
             pr = kin_side<VISC>(ph, tW, tg, side == 0 ? +1 : -1, S, &hr);
@@ -229,7 +258,8 @@ __device__ __forceinline__ void flux_faces(const DevMesh<T>& m, const Phys<T>& p
 #pragma unroll
             for (int q = 0; q < 5; ++q) ddiff[q] = -ddiff[q];
             T dW[5], dF[5];
-            interface_deviation(poly, L, Rc, Rm, dsum, ddiff, hl, hr, Wc, ph.gm1, dW, dF);
+            interface_deviation(poly + side_cell(L, Rc, 0) * Stride<T>::poly,
+                                poly + side_cell(L, Rc, 1) * Stride<T>::poly, L, Rc, Rm, dsum, ddiff, hl, hr, Wc, ph.gm1, dW, dF);
 #pragma unroll
             for (int q = 0; q < 5; ++q) {
                 Fh[q] += T(0.5) * dt * dF[q];
@@ -258,7 +288,7 @@ __device__ __forceinline__ void flux_faces(const DevMesh<T>& m, const Phys<T>& p
     constexpr int VALS = flux_vals<NR>(), RS = rec_stride<T, NR>();
     if (f < m.nf && job < 2) {
         T Rm[3][3], n[4];
-        load_vec<4>(m.fgeo + f * FGEO, n);
+        load_vec<4>(COPY ? &sm.geo[lf][0] : m.fgeo + f * FGEO, n);
 #pragma unroll
         for (int i = 0; i < 3; ++i) {
             Rm[0][i] = n[i];
@@ -296,7 +326,8 @@ __device__ __forceinline__ void flux_faces(const DevMesh<T>& m, const Phys<T>& p
         if (f < m.nf && job == 2) {
             const int L = m.flr[f], Rc = m.flr[m.nf + f];
             const double dtc = ctrl ? ctrl[m.cell_case[L >= 0 ? L : Rc]] : dt_override;
-            reference_flux(poly, m.fan + 6 * f, L, Rc, ph.gm1, dtc > 0.0 ? (T)dtc : T(1), sm.ref[lf]);
+            reference_flux(poly + side_cell(L, Rc, 0) * Stride<T>::poly, poly + side_cell(L, Rc, 1) * Stride<T>::poly,
+                           m.fan + 6 * f, ph.gm1, dtc > 0.0 ? (T)dtc : T(1), sm.ref[lf]);
         }
         group_barrier(bar_id, TH);
         // the block's records are one stretch of memory: whole vectors by all
@@ -350,8 +381,9 @@ __global__ void __launch_bounds__(TH, MINB) k_flux(DevMesh<T> m, Phys<T> ph, con
 // 1: 15 warps at 128 registers, no spills (stage 1, 3.15 M faces: 1,161 us,
 // against 1,273 us with 6 blocks and 1,419 us with 8, which spill); variant
 // 0: 12 warps with more registers, the faster one in some viscous and small
-// launches.
-constexpr int FLUX_BLOCKS_V1 = 5, FLUX_BLOCKS_V0 = 4;
+// launches.  Inviscid stage 2 fits 96 registers without spills: 6 blocks (3.15
+// M faces 631 -> 595 us; the viscous one would spill, 255 -> 260 us on 1.16 M).
+constexpr int FLUX_BLOCKS_V1 = 5, FLUX_BLOCKS_V1_STAGE2 = 6, FLUX_BLOCKS_V0 = 4;
 // FP64 is bound by its pipe whatever the occupancy (218-238 registers, no
 // spills), so a launch lasts as long as the SM with the most warps: blocks of
 // 96 threads (32 faces, no lane idle) or of 64 (21 faces, one lane idle),
@@ -377,7 +409,8 @@ static cudaError_t launch_flux(const DevMesh<T>& m, const HostPhys& p, const T* 
         if (stage == 1)
             p.viscous ? go(k_flux<T, 40, TH, B, true, XW>) : go(k_flux<T, 40, TH, B, false, XW>);
         else
-            p.viscous ? go(k_flux<T, 20, TH, B, true, XW>) : go(k_flux<T, 20, TH, B, false, XW>);
+            p.viscous ? go(k_flux<T, 20, TH, B, true, XW>)
+                      : go(k_flux<T, 20, TH, B == FLUX_BLOCKS_V1 ? FLUX_BLOCKS_V1_STAGE2 : B, false, XW>);
     };
     using std::integral_constant;
     if constexpr (sizeof(T) == 8) {
