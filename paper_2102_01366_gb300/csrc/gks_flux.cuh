@@ -28,7 +28,8 @@ namespace gks {
 // with the fewest instructions.  Two threads a point (one a side, in two
 // warps) repeated the frame and met four times at a barrier through 60 KB of
 // shared memory: stage 1 / stage 2 on 3.15 M faces 2,087 / 1,335 us there,
-// 1,071 / 687 us here; on 49,280 faces 40.6 / 28.7 us, now 26.6 / 18.4 us.
+// 1,071 / 687 us here at first, 907 / 594 us now; on 49,280 faces 40.6 / 28.7
+// us, now 22.5 / 18.4 us.
 // Persistent blocks that fetch the next block's records into shared memory hid
 // the gathers, but a block's three warps then waited for each other: 1,207 /
 // 837 us.
@@ -56,7 +57,7 @@ struct FluxSmem {
     alignas(16) T geo[flux_copies<T, NR>() ? (TH + 2) / 3 : 1][flux_copies<T, NR>() ? FGEO : 4];
     T out[TH][flux_vals<NR>() + 1];
     T frame[(TH + 2) / 3][7];                                 // tangents of the face frame
-    T ref[sizeof(T) == 4 && NR == 40 ? (TH + 2) / 3 : 1][11];  // reference flux (FP32 stage 1)
+    T rec[sizeof(T) == 4 && NR == 40 ? (TH + 2) / 3 : 1][33];  // the block's records (FP32 stage 1)
 };
 
 // hi (5) and lo (5) parts of a record's cell average, in whole vectors: ten
@@ -136,7 +137,7 @@ __device__ __forceinline__ void interface_deviation(const float* al, const float
 // The reference flux (dt / 2) A F_n(W_m) of a face (FP32 stage 1): W_m from
 // the hi / lo averages and the face's area vector A n taken exactly (its sum
 // over a closed cell vanishes to FP64 rounding, where the FP32 weights and
-// normals leave eps A), in FP32 pairs, stored as hi and lo parts; entering
+// normals leave eps A), in FP32 pairs, stored as the record's hi and lo parts; entering
 // both cells with opposite signs, it keeps the update exactly conservative.
 __device__ __forceinline__ void reference_flux(const float* al, const float* ar, const float* __restrict__ an,
                                                float gm1, float dt, float* __restrict__ out) {
@@ -162,9 +163,10 @@ __device__ __forceinline__ void reference_flux(const float* al, const float* ar,
     ref[4] = f2_scale(hd, f2_mul(f2_add(Wm[4], pm), un));
 #pragma unroll
     for (int q = 0; q < 5; ++q) {
-        out[q] = ref[q].hi;
-        out[5 + q] = ref[q].lo;
+        out[6 * q + 4] = ref[q].hi;
+        out[6 * q + 5] = ref[q].lo;
     }
+    out[30] = out[31] = 0.0f;
 }
 
 // asynchronous copy of 16 bytes to shared memory
@@ -285,7 +287,7 @@ __device__ __forceinline__ void flux_faces(const DevMesh<T>& m, const Phys<T>& p
     // the interface-state entries and (FP32 stage 1) the reference flux
     const int job = tid / FACES, lf = tid - FACES * job;
     const int64_t f = fb * FACES + lf;
-    constexpr int VALS = flux_vals<NR>(), RS = rec_stride<T, NR>();
+    constexpr int VALS = flux_vals<NR>(), RS = rec_stride<T, NR>(), J = rec_entries<T, NR>();
     if (f < m.nf && job < 2) {
         T Rm[3][3], n[4];
         load_vec<4>(COPY ? &sm.geo[lf][0] : m.fgeo + f * FGEO, n);
@@ -302,8 +304,8 @@ __device__ __forceinline__ void flux_faces(const DevMesh<T>& m, const Phys<T>& p
                 v[q] = w * ((sm.out[3 * lf][at + q] + sm.out[3 * lf + 1][at + q]) + sm.out[3 * lf + 2][at + q]);
             to_global(Rm, v);
         };
-        // FP32 stage 1: into the columns that only this thread has read
-        T* r = (REL ? sm.out[3 * lf] : rec + f * RS) + (VALS / 2) * job;
+        // FP32 stage 1: by way of shared memory
+        T* r = REL ? sm.rec[lf] : rec + f * RS;
         T a[5], b[5];
         sum((VALS / 2) * job, a);
         if constexpr (NR == 40) {
@@ -312,14 +314,14 @@ __device__ __forceinline__ void flux_faces(const DevMesh<T>& m, const Phys<T>& p
             for (int q = 0; q < 5; ++q) {
                 // dt L + dt^2/6 L_t = 8/3 Fh - 1/3 F = 2 Fh - D / 3 (Eqs. linear-system, s2o4)
                 // f* = f^n + dt/2 f_t^n
-                r[q] = job == 0 ? a[q] : a[q] + T(0.5) * b[q];
-                r[5 + q] = job == 0 ? T(2) * a[q] - b[q] * T(1.0 / 3.0) : a[q];
+                r[J * q + 2 * job] = job == 0 ? a[q] : a[q] + T(0.5) * b[q];
+                r[J * q + 2 * job + 1] = job == 0 ? T(2) * a[q] - b[q] * T(1.0 / 3.0) : a[q];
             }
         } else {
 #pragma unroll
             for (int q = 0; q < 5; ++q)
                 // dt^2/3 L_t(W*) = 4/3 (F* - 2 Fh*); f^{n+1} = f^n + dt f_t^*
-                r[q] = job == 0 ? T(4.0 / 3.0) * a[q] : a[q];
+                r[J * q + job] = job == 0 ? T(4.0 / 3.0) * a[q] : a[q];
         }
     }
     if constexpr (REL) {
@@ -327,13 +329,13 @@ __device__ __forceinline__ void flux_faces(const DevMesh<T>& m, const Phys<T>& p
             const int L = m.flr[f], Rc = m.flr[m.nf + f];
             const double dtc = ctrl ? ctrl[m.cell_case[L >= 0 ? L : Rc]] : dt_override;
             reference_flux(poly + side_cell(L, Rc, 0) * Stride<T>::poly, poly + side_cell(L, Rc, 1) * Stride<T>::poly,
-                           m.fan + 6 * f, ph.gm1, dtc > 0.0 ? (T)dtc : T(1), sm.ref[lf]);
+                           m.fan + 6 * f, ph.gm1, dtc > 0.0 ? (T)dtc : T(1), sm.rec[lf]);
         }
         group_barrier(bar_id, TH);
         // the block's records are one stretch of memory: whole vectors by all
         // threads, where a thread per face wrote each of its 10 words to a line
         // of its own (L1's data pipe 67 % busy).  Stage 1, 3.15 M faces: 1,071
-        // -> 973 us.  Stage 2's short records lost more by the second barrier
+        // -> 907 us.  Stage 2's short records lost more by the second barrier
         // (687 -> 733 us) and FP64 has its pipe as bound: these write directly.
         const int64_t left = m.nf - fb * FACES;
         const int words = (int)(left < FACES ? left : FACES) * (RS / 4);
@@ -341,8 +343,7 @@ __device__ __forceinline__ void flux_faces(const DevMesh<T>& m, const Phys<T>& p
             const int face = i / (RS / 4), e = 4 * (i - face * (RS / 4));
             T v[4];
 #pragma unroll
-            for (int k = 0; k < 4; ++k)
-                v[k] = e < VALS ? sm.out[3 * face][e + k] : e + k < VALS + 10 ? sm.ref[face][e + k - VALS] : T(0);
+            for (int k = 0; k < 4; ++k) v[k] = sm.rec[face][e + k];
             store_vec<4>(rec + fb * FACES * RS + 4 * (int64_t)i, v);
         }
     }

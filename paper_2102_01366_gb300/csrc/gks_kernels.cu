@@ -161,12 +161,13 @@ __global__ void k_rec_out(const T* __restrict__ rec, const int32_t* __restrict__
         const int nflux = nr == 40 ? 10 : 5;
         const T* r = rec + d * (nr == 40 ? rec_stride<T, 40>() : rec_stride<T, 20>());
         const int je = j - nflux;
-        double v = j < nflux ? (double)r[j]
-                             : (double)r[nflux + (je / 15) * 5 + (je % 15) / 3] *
+        const int J = nr == 40 ? rec_entries<T, 40>() : rec_entries<T, 20>();
+        double v = j < nflux ? (double)r[(j % 5) * J + j / 5]
+                             : (double)r[((je % 15) / 3) * J + nflux / 5 + je / 15] *
                                    (double)m.fnw[d * 4 + (je % 15) % 3];
         if (sizeof(T) == 4 && nr == 40 && j < 10) {
             // the reference flux (dt / 2) A F_n(W_m), twice in the S entries
-            const double ref = (double)r[REC1_REF + j % 5] + (double)r[REC1_REF + 5 + j % 5];
+            const double ref = (double)r[(j % 5) * J + 4] + (double)r[(j % 5) * J + 5];
             v += j < 5 ? ref : 2.0 * ref;
         }
         if (sizeof(T) == 4 && addback && j >= 10) {

@@ -32,17 +32,25 @@ constexpr int XS = 20;               // reals per cell working-state record, FP6
 constexpr int XS32 = 28;
 constexpr int XLO = 5;               // offset of the lo parts in an FP32 working-state record
 // Face records, sums over the face's Gauss points with their weights w:
-//   stage 1  sum w Fh (5), sum w (2 Fh - D / 3) (5), sum w W(t*) (5),
-//            sum w W(0) (5); FP32: the flux and interface-state entries are
+//   stage 1  per component: sum w Fh, sum w (2 Fh - D / 3), sum w W(t*),
+//            sum w W(0); FP32: the flux and interface-state entries are
 //            relative to the mean W_m of the face's two cell averages, and the
-//            reference flux (dt / 2) A F_n(W_m) follows as hi (5) and lo (5)
-//            parts (one aligned 128-byte record)
-//   stage 2  sum w 4/3 D (5), sum w dW (5)
+//            reference flux (dt / 2) A F_n(W_m) follows as hi and lo parts
+//            (one aligned 128-byte record)
+//   stage 2  per component: sum w 4/3 D, sum w dW
 // The interface states enter a cell times the face's normal, which the
 // update multiplies in: a third of the words that (sum w W n) would take.
 // NR (40, 20) names the stage: the length of its record with the normal
 // multiplied in, as gks_debug_face_records gives it.
-constexpr int REC1_REF = 20;
+// A component's entries (rec_entries of them) lie together, so that an update
+// lane reads them as vectors.
+template <typename T, int NR>
+#ifdef __CUDACC__
+__host__ __device__
+#endif
+constexpr int rec_entries() {
+    return NR == 20 ? 2 : sizeof(T) == 4 ? 6 : 4;
+}
 template <typename T, int NR>
 constexpr int rec_stride() {
     return NR == 20 ? 10 : sizeof(T) == 4 ? 32 : 20;

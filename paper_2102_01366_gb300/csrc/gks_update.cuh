@@ -5,6 +5,8 @@
 
 #include <cuda_runtime.h>
 
+#include <type_traits>
+
 #include "gks_cells.cuh"
 #include "gks_device.cuh"
 #include "gks_kernels.h"
@@ -59,10 +61,22 @@ __device__ __forceinline__ bool positive(double x) { return __double_as_longlong
 // the FP64 pipe, so FP32 <-> FP64 conversions go through the integer pipe
 // (widen, split_pair).  On 1.57 M cells, FP32, stage 1 / stage 2: 393 / 707 us
 // before, 306 / 303 with warp_case_min and cell-major S and G, 281 / 171 with
-// the integer conversions and the normals apart from the Gauss points.  One
-// thread per cell with 16-byte gathers took 349 / 236 us (too few warps in
+// the integer conversions and the normals apart from the Gauss points, 254 /
+// 171 with a component's record entries together.  One thread per cell with 16-byte gathers took 349 / 236 us (too few warps in
 // flight) and twice the time on 1,536 to 3,072 cells.
 // --------------------------------------------------------------------------
+
+// N values of a record (8- or 16-byte aligned) as vectors of two
+template <int N, typename T>
+__device__ __forceinline__ void load_pairs(const T* __restrict__ p, T* v) {
+    using T2 = std::conditional_t<sizeof(T) == 4, float2, double2>;
+#pragma unroll
+    for (int i = 0; i < N / 2; ++i) {
+        const T2 x = reinterpret_cast<const T2*>(p)[i];
+        v[2 * i] = x.x;
+        v[2 * i + 1] = x.y;
+    }
+}
 
 // the face's unit normal and w = area / 3, one 16-byte (FP64: two) load
 template <typename T>
@@ -76,7 +90,7 @@ __device__ __forceinline__ void update1_cells(const DevMesh<T>& m, const DevStat
     if (!cl.active) return;
     const int64_t nc = m.nc, c = cl.c;
     const int q = cl.q;
-    constexpr int RS = rec_stride<T, 40>(), XSR = Stride<T>::xs;
+    constexpr int RS = rec_stride<T, 40>(), J = rec_entries<T, 40>(), XSR = Stride<T>::xs;
     constexpr bool F32 = sizeof(T) == 4;
     int e[4], nb[4];
 #pragma unroll
@@ -86,16 +100,14 @@ __device__ __forceinline__ void update1_cells(const DevMesh<T>& m, const DevStat
     }
     const double dtd = st.case_dt[m.cell_case[c]];
     const double iv = m.inv_vol[c], w0d = st.Wd[q * nc + c];
-    T r[4][F32 ? 6 : 4], n[4][4], nx[4][2], own[2] = {T(0), T(0)};
+    T r[4][J], n[4][4], nx[4][2], own[2] = {T(0), T(0)};
     if constexpr (F32) {
         own[0] = st.X[c * XSR + q];
         own[1] = st.X[c * XSR + XLO + q];
     }
 #pragma unroll
     for (int f = 0; f < 4; ++f) {
-        const T* p = st.rec + (int64_t)(e[f] >> 1) * RS + q;
-#pragma unroll
-        for (int j = 0; j < (F32 ? 6 : 4); ++j) r[f][j] = p[5 * j];
+        load_pairs<J>(st.rec + (int64_t)(e[f] >> 1) * RS + q * J, r[f]);
         load_normal(m, e[f] >> 1, n[f]);
         if constexpr (F32) {
             // a missing neighbour reads the cell itself
@@ -178,9 +190,7 @@ __device__ __forceinline__ void update2_cells(const DevMesh<T>& m, const DtPhys<
     for (int i = 0; i < 3; ++i) g0[i] = st.G[c * 15 + 3 * q + i];
 #pragma unroll
     for (int f = 0; f < 4; ++f) {
-        const T* pr = st.rec + (int64_t)(e[f] >> 1) * RS + q;
-        r[f][0] = pr[0];
-        r[f][1] = pr[5];
+        load_pairs<2>(st.rec + (int64_t)(e[f] >> 1) * RS + q * 2, r[f]);
         load_normal(m, e[f] >> 1, n[f]);
     }
     const bool live = cl.active && positive(dtd);  // finished cases keep their state
