@@ -46,8 +46,8 @@ FLUSH_BYTES = 512 << 20  # > 129 MB L2
 # a launch), and its DRAM bytes (read + write) per launch, the mean of the
 # stage-1 and stage-2 launches, from the same capture (the flux kernel's
 # summary under profiles/)
-FLUX_FLOPS_PER_GP = {"fp32": (4546.7, 3874.2)}
-FLUX_DRAM_BYTES_PER_LAUNCH = 11827840.0
+FLUX_FLOPS_PER_GP = {"fp32": (2565.2, 1998.9)}
+FLUX_DRAM_BYTES_PER_LAUNCH = 11785984.0
 SM_COUNT, FP32_LANES, SM_MAX_MHZ = 152, 128, 2070.0
 # algorithmic HBM traffic of one cell-stage: the minimum of the four passes
 # the method's two global dependencies impose (neighbour slopes; both sides'
