@@ -62,6 +62,32 @@ def test_fp64_flux_blocks(cuda, oracle_mod, dims, warps, viscous):
             assert np.abs(got[:, a:b] - ref[:, a:b]).max() <= TOL[0] * np.abs(ref[:, a:b]).max(), (stage, a)
 
 
+# FP32: blocks of 32 faces, stage 1's records stored as one stretch, stage 2's
+# copied ahead; a box of a x b x c hexahedra open on all sides has 12 abc +
+# 2 (ab + bc + ca) faces, the last block here 18, 2, 30 and 16 of them.
+# Groups that nearly vanish are held to 1e-3 of the state, as the parity tests do
+@pytest.mark.parametrize("viscous", [0, 1])
+@pytest.mark.parametrize("flux_blocks", [2, 3])
+@pytest.mark.parametrize("dims, nf", [((1, 1, 1), 18), ((2, 1, 1), 34), ((3, 2, 1), 94), ((3, 2, 2), 176)])
+def test_fp32_flux_ragged_blocks(cuda, oracle_mod, dims, nf, flux_blocks, viscous):
+    mesh = I.box_mesh(dims, jitter=0.0, seed=0, periodic=(False, False, False))
+    W, dW = _rough_state(mesh, 0.05, 69)
+    kw = dict(weno=1, cfl=0.4, viscous=viscous, mu=1e-3 * viscous)
+    g, o, p = gks.Mesh(mesh), oracle_mod.Mesh(mesh), oracle_mod.params(**kw)
+    assert g.nf == nf
+    s = gks.State(g, gks.params(precision=1, **kw))
+    s.set_variant(0, flux_blocks, 1)
+    s.init(W, dW)
+    dt = o.timestep(p, W)
+    for stage, groups in ((1, (0, 5, 10, 25, 40)), (2, (0, 5, 20))):
+        got = s.debug_face_records(dt, stage).cpu().numpy()
+        ref = o.face_records(p, W, dW, dt, stage)
+        floor = 1e-3 * g.geometry()["farea"].max() / 3.0 * np.abs(W).max()
+        for a, b in zip(groups, groups[1:]):
+            scale = max(np.abs(ref[:, a:b]).max(), floor)
+            assert np.abs(got[:, a:b] - ref[:, a:b]).max() <= TOL[1] * scale, (stage, a)
+
+
 @pytest.mark.parametrize("precision", [0, 1])
 @pytest.mark.parametrize("shapes", [[(1, 1, 1)] * 7, [(2, 1, 1), (1, 1, 1), (3, 2, 1), (1, 1, 1), (1, 1, 1)],
                                     [(2, 1, 1), (1, 1, 1), (1, 1, 1), (2, 1, 1), (1, 1, 1)]])
