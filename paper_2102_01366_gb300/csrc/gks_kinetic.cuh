@@ -97,8 +97,8 @@ __device__ __forceinline__ KMom<HALF, T> kin_moments(const KState<T>& s, T K, in
         const T sg = half > 0 ? T(1) : T(-1);
         const T rs = d_rsqrt(T(2) * s.h);  // sqrt(lambda)
         const T x = s.U * rs;
-        const T u0 = T(0.5) * d_erfc(-sg * x);
         const T ex = d_exp(-x * x);
+        const T u0 = half_erfc(-sg * x, ex);
         if (hs) *hs = {u0, rs, ex};
         k.F = sg * s.rho * T(0.56418958354775628695) * rs * ex;  // 1 / sqrt(pi)
         k.Uh = x * rs;
