@@ -13,7 +13,8 @@ namespace gks {
 // reconstruction record.  FP64 records hold R in centroid-monomial form; FP32
 // records hold R minus the cell average and the average's hi / lo parts, and
 // val = hi + (R - average).  dev (FP32, may be NULL) receives R - average at X.
-template <typename T>
+// PLAIN: the value as the plain sum of its ten terms (the adjoint).
+template <bool PLAIN = false, typename T>
 __device__ __forceinline__ void eval_poly(const T* __restrict__ P, const T* X, T* val, T (*g)[5],
                                           T* dev = nullptr) {
     // the record is 16-byte aligned: load it in vectors (FP32: without the
@@ -48,7 +49,9 @@ __device__ __forceinline__ void eval_poly(const T* __restrict__ P, const T* X, T
         const T sx = cq[1] + cq[4] * x + cq[5] * y + cq[6] * z;
         const T sy = cq[2] + cq[7] * y + cq[8] * z;
         const T sz = cq[3] + cq[9] * z;
-        const T v = cq[0] + x * sx + y * sy + z * sz;
+        const T v = PLAIN ? cq[0] + cq[1] * x + cq[2] * y + cq[3] * z + cq[4] * x * x + cq[5] * x * y + cq[6] * x * z +
+                                cq[7] * y * y + cq[8] * y * z + cq[9] * z * z
+                          : cq[0] + x * sx + y * sy + z * sz;
         if constexpr (sizeof(T) == 4) {
             val[q] = c[PHI + q] + v;
             if (dev) dev[q] = v;
@@ -254,7 +257,7 @@ __device__ __forceinline__ int64_t side_cell(int L, int Rc, int side) {
 // moving walls are compiled in.  dev (FP32, may be NULL) receives the
 // evaluated reconstruction minus its cell's average, global frame (0 for an
 // open or fixed side).
-template <typename T, bool XW>
+template <typename T, bool XW, bool PLAIN = false>
 __device__ __forceinline__ void side_state(const DevMesh<T>& m, const Phys<T>& ph, const T* __restrict__ Wavg,
                                            const T* __restrict__ P, const T* __restrict__ geo,
                                            const T (*Rm)[3], int L, int Rc, int side, int k, T* tW, T (*tg)[5],
@@ -281,7 +284,7 @@ __device__ __forceinline__ void side_state(const DevMesh<T>& m, const Phys<T>& p
         if (mine == FLR_FIXED)
             fixed_ghost(m.fixed + c * Stride<T>::xs, X, Ws, gs);
         else
-            eval_poly(P, X, Ws, gs, dev);
+            eval_poly<PLAIN>(P, X, Ws, gs, dev);
     }
     to_local(Rm, Ws, gs, tW, tg);
     if (mine == FLR_SLIP_WALL) slip_wall_ghost(tW, tg);
