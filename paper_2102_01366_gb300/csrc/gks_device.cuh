@@ -17,8 +17,8 @@ namespace gks {
 __device__ __forceinline__ double d_exp(double x) { return exp(x); }
 __device__ __forceinline__ float d_exp(float x) { return expf(x); }
 // erfc(y) / 2, given ex = exp(-y^2).  FP64 by erfcx, which saves the second
-// exponential of a pipe-bound kernel (flux on 49,280 faces, a step of both 1,191
-// -> 1,169 us; reverse step of 48,000 cells 5,704 -> 5,648 us).  ex carries the
+// exponential of a pipe-bound kernel (a whole step with 49,280 faces 1,191 ->
+// 1,169 us; a reverse step of 48,000 cells 5,704 -> 5,648 us).  ex carries the
 // rounding of y^2, a relative error of at most y^2 half units: at most 0.2 half
 // units of 1, as erfc falls faster than y^2 grows, and the same error that
 // the Gaussian tail beside it has.

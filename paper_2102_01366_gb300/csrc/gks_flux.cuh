@@ -389,7 +389,7 @@ constexpr int FLUX_BLOCKS_V1 = 5, FLUX_BLOCKS_V1_STAGE2 = 6, FLUX_BLOCKS_V0 = 4;
 // spills), so a launch lasts as long as the SM with the most warps: blocks of
 // 96 threads (32 faces, no lane idle) or of 64 (21 faces, one lane idle),
 // whichever leaves the fullest SM with fewer warps.  6,144 faces: 6 warps with
-// blocks of 96, 4 with 64, a step of both fluxes 215 and 153 us; 49,280 faces:
+// blocks of 96, 4 with 64, a whole step 215 and 153 us; 49,280 faces:
 // 33 and 32 warps, 1,242 and 1,188 us; from about 10^6 faces the blocks of 96
 // win by their full lanes.
 constexpr int FLUX_THREADS_FP64 = 64, SMS = 152;
