@@ -196,12 +196,7 @@ __device__ __forceinline__ T slope_sq(const T* b) {
 }
 
 // 1 / a and 1 / b by one division where it can neither overflow nor
-// underflow (FP64, whose division is a dozen instructions of the bound pipe);
-// FP32 divides by the hardware reciprocal
-__device__ __forceinline__ void recip2(float a, float b, float& ia, float& ib) {
-    ia = 1.0f / a;
-    ib = 1.0f / b;
-}
+// underflow (FP64, whose division is a dozen instructions of the bound pipe)
 __device__ __forceinline__ void recip2(double a, double b, double& ia, double& ib) {
     const double p = a * b;
     if (p > 1e-290 && p < 1e290) {
@@ -211,6 +206,26 @@ __device__ __forceinline__ void recip2(double a, double b, double& ia, double& i
     } else {
         ia = 1.0 / a;
         ib = 1.0 / b;
+    }
+}
+
+// n / a and n / b: FP64 by one division for both where it can neither overflow
+// nor underflow, else by two, not by reciprocals (a uniform component has n = 0
+// over an epsilon that may be subnormal, whose reciprocal is infinite); FP32 by
+// the hardware reciprocal
+__device__ __forceinline__ void ratio2(float n, float a, float b, float& ra, float& rb) {
+    ra = n * (1.0f / a);
+    rb = n * (1.0f / b);
+}
+__device__ __forceinline__ void ratio2(double n, double a, double b, double& ra, double& rb) {
+    const double p = a * b;
+    if (p > 1e-290 && p < 1e290) {
+        const double ip = 1.0 / p;
+        ra = n * (ip * b);
+        rb = n * (ip * a);
+    } else {
+        ra = n / a;
+        rb = n / b;
     }
 }
 
@@ -428,13 +443,13 @@ __device__ __forceinline__ void recon_cells(const DevMesh<T>& m, const ReconCons
                     if (nb[j] >= 0 && nb[k] >= 0) sum += d_abs(b0j[j] - b0j[k]);
             const T inv_pairs = nn == 4 ? T(1.0 / 6.0) : nn == 3 ? T(1.0 / 3.0) : T(1);
             const T s1 = pow43(sum * inv_pairs);
-            T ie[4], ws = T(0), acc = T(0);
-            recip2(rc.eps + b0j[0], rc.eps + b0j[1], ie[0], ie[1]);
-            recip2(rc.eps + b0j[2], rc.eps + b0j[3], ie[2], ie[3]);
+            T r1[4], ws = T(0), acc = T(0);
+            ratio2(s1, rc.eps + b0j[0], rc.eps + b0j[1], r1[0], r1[1]);
+            ratio2(s1, rc.eps + b0j[2], rc.eps + b0j[3], r1[2], r1[3]);
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
                 if (nb[j] < 0) continue;
-                const T w1 = T(1) + s1 * ie[j];
+                const T w1 = T(1) + r1[j];
                 ws += w1;
                 acc += w1 * b0j[j];
             }
@@ -442,9 +457,8 @@ __device__ __forceinline__ void recon_cells(const DevMesh<T>& m, const ReconCons
         }
         if (rc.order == 2) {
             const T sigma = pow43(d_abs(beta1 - beta0));
-            T i0, i1;
-            recip2(rc.eps + beta0, rc.eps + beta1, i0, i1);
-            const T r0 = sigma * i0, r1 = sigma * i1;
+            T r0, r1;
+            ratio2(sigma, rc.eps + beta0, rc.eps + beta1, r0, r1);
             const T w0 = g01 * (T(1) + r0 * r0), w1 = g11 * (T(1) + r1 * r1);
             const T cl1 = (w1 / (w0 + w1)) * i11;
 #pragma unroll
@@ -467,9 +481,9 @@ __device__ __forceinline__ void recon_cells(const DevMesh<T>& m, const ReconCons
             const T beta2 = v23 * first + v43 * second;
             // global smoothness indicator and nonlinear weights, Eq. non-linear-weight
             const T sigma = pow43(T(0.5) * (d_abs(beta2 - beta1) + d_abs(beta2 - beta0)));
-            T i0, i1;
-            recip2(rc.eps + beta0, rc.eps + beta1, i0, i1);
-            const T r0 = sigma * i0, r1 = sigma * i1, r2 = sigma / (rc.eps + beta2);
+            T r0, r1;
+            ratio2(sigma, rc.eps + beta0, rc.eps + beta1, r0, r1);
+            const T r2 = sigma / (rc.eps + beta2);
             const T w0 = g02 * (T(1) + r0 * r0), w1 = g12 * (T(1) + r1 * r1), w2 = g22 * (T(1) + r2 * r2);
             const T iw = T(1) / (w0 + w1 + w2);
             const T c2 = (w2 * iw) * i22;
