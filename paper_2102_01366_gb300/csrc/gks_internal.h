@@ -5,8 +5,8 @@
 #include <algorithm>
 #include <cstddef>
 #include <cstdint>
+#include <exception>
 #include <string>
-#include <system_error>
 #include <thread>
 #include <vector>
 
@@ -56,22 +56,33 @@ inline int64_t host_threads(int64_t n, int64_t grain = 16384) {
 }
 
 // fn(t, lo, hi) over nthr contiguous ranges of [0, n); range 0 on the calling
-// thread, and any range whose thread cannot be started runs inline too
+// thread, and any range whose thread cannot be started runs there too.  An
+// exception of any range is thrown on to the caller once every thread has
+// ended.
 template <typename Fn>
-void run_ranges(int64_t n, int64_t nthr, Fn fn) {
+void run_ranges(int64_t n, int64_t nthr, const Fn& fn) {
     const int64_t chunk = (n + nthr - 1) / nthr;
+    std::vector<std::exception_ptr> thrown((size_t)nthr);
     std::vector<std::thread> pool;
     pool.reserve((size_t)nthr);
-    for (int64_t t = 1; t < nthr; ++t) {
-        const int64_t lo = std::min(n, t * chunk), hi = std::min(n, (t + 1) * chunk);
+    auto range = [&](int64_t t) noexcept {
         try {
-            pool.emplace_back(fn, t, lo, hi);
-        } catch (const std::system_error&) {
-            fn(t, lo, hi);
+            fn(t, std::min(n, t * chunk), std::min(n, (t + 1) * chunk));
+        } catch (...) {
+            thrown[(size_t)t] = std::current_exception();
+        }
+    };
+    for (int64_t t = 1; t < nthr; ++t) {
+        try {
+            pool.emplace_back(range, t);
+        } catch (...) {  // no thread or no memory for one
+            range(t);
         }
     }
-    fn((int64_t)0, (int64_t)0, std::min(n, chunk));
+    range(0);
     for (auto& th : pool) th.join();
+    for (const std::exception_ptr& e : thrown)
+        if (e) std::rethrow_exception(e);
 }
 
 }  // namespace gks

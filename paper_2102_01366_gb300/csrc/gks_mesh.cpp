@@ -23,8 +23,6 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
-#include <system_error>
-#include <thread>
 #include <unordered_map>
 
 #include "gks_internal.h"

@@ -16,7 +16,6 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
-#include <thread>
 
 #include "gks_internal.h"
 
@@ -262,9 +261,7 @@ gks_status build_stencils(gks_mesh& m) {
     m.M2.assign((size_t)m.nc * 144, 0.0);
     m.singular.assign((size_t)m.nc, 0);
     // independent per cell: split the cells over the host's hardware threads
-    const unsigned hw = std::max(1u, std::thread::hardware_concurrency());
-    const int64_t nthr = std::min<int64_t>((int64_t)hw, std::max<int64_t>(1, m.nc / 4096));
-    auto work = [&](int64_t lo, int64_t hi) {
+    run_ranges(m.nc, host_threads(m.nc, 4096), [&](int64_t, int64_t lo, int64_t hi) {
         for (int64_t c = lo; c < hi; ++c) {
             if (!cell_stencil(m, c, &m.M1[c * 12], &m.M2[c * 144])) {
                 m.singular[c] = 1;
@@ -272,13 +269,7 @@ gks_status build_stencils(gks_mesh& m) {
                 std::memset(&m.M2[c * 144], 0, sizeof(double) * 144);
             }
         }
-    };
-    std::vector<std::thread> pool;
-    const int64_t chunk = (m.nc + nthr - 1) / nthr;
-    for (int64_t t = 1; t < nthr; ++t)
-        pool.emplace_back(work, std::min(m.nc, t * chunk), std::min(m.nc, (t + 1) * chunk));
-    work(0, std::min(m.nc, chunk));
-    for (auto& th : pool) th.join();
+    });
     m.n_singular = 0;
     for (int64_t c = 0; c < m.nc; ++c) m.n_singular += m.singular[c];
     m.has_stencils = true;
