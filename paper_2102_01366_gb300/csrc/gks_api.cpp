@@ -35,6 +35,18 @@ using namespace gks;
         }                                                                           \
     } while (0)
 
+// fn(), with no exception past the C boundary: memory that cannot be had is
+// GKS_E_NOMEM (the message is short enough to be stored without any)
+template <typename Fn>
+static gks_status guarded(const Fn& fn) {
+    try {
+        return fn();
+    } catch (const std::bad_alloc&) {
+        set_error("out of memory");
+        return GKS_E_NOMEM;
+    }
+}
+
 extern "C" const char* gks_last_error(void) { return g_err.c_str(); }
 
 extern "C" void gks_params_default(gks_params* p) {
@@ -173,21 +185,23 @@ extern "C" gks_status gks_mesh_info(const gks_mesh* m, int64_t* n_cell, int64_t*
 
 extern "C" gks_status gks_mesh_set_boundary(gks_mesh* m, const int8_t* kind) {
     if (!m || !kind) { set_error("gks_mesh_set_boundary: NULL argument"); return GKS_E_ARG; }
-    std::vector<int8_t> bk((size_t)m->nf, 0);
-    for (int64_t c = 0; c < m->nc; ++c)
-        for (int f = 0; f < 4; ++f) {
-            if (m->nbr[c * 4 + f] >= 0) continue;
-            const int8_t k = kind[c * 4 + f];
-            if (k != GKS_BC_OPEN && k != GKS_BC_SLIP_WALL && k != GKS_BC_FIXED && k != GKS_BC_NOSLIP_WALL &&
-                k != GKS_BC_ISOTHERMAL_WALL && k != GKS_BC_MOVING_WALL) {
-                set_error("gks_mesh_set_boundary: unknown kind " + std::to_string((int)k) + " at cell " +
-                          std::to_string(c) + " face " + std::to_string(f));
-                return GKS_E_ARG;
+    return guarded([&]() -> gks_status {
+        std::vector<int8_t> bk((size_t)m->nf, 0);
+        for (int64_t c = 0; c < m->nc; ++c)
+            for (int f = 0; f < 4; ++f) {
+                if (m->nbr[c * 4 + f] >= 0) continue;
+                const int8_t k = kind[c * 4 + f];
+                if (k != GKS_BC_OPEN && k != GKS_BC_SLIP_WALL && k != GKS_BC_FIXED && k != GKS_BC_NOSLIP_WALL &&
+                    k != GKS_BC_ISOTHERMAL_WALL && k != GKS_BC_MOVING_WALL) {
+                    set_error("gks_mesh_set_boundary: unknown kind " + std::to_string((int)k) + " at cell " +
+                              std::to_string(c) + " face " + std::to_string(f));
+                    return GKS_E_ARG;
+                }
+                bk[(size_t)m->csr_face[c * 4 + f]] = k;
             }
-            bk[(size_t)m->csr_face[c * 4 + f]] = k;
-        }
-    m->bkind.swap(bk);
-    return GKS_OK;
+        m->bkind.swap(bk);
+        return GKS_OK;
+    });
 }
 
 extern "C" gks_status gks_mesh_cases(const gks_mesh* m, int32_t* n_case, int64_t* case_first_cell) {
@@ -575,59 +589,75 @@ static std::vector<int32_t> face_permutation(const gks_mesh& g, int order, const
     return perm;
 }
 
+// The device's face arrays, in a face order
 template <typename T>
-static gks_status upload_faces(gks_state* s) {
+struct FaceArrays {
+    std::vector<int32_t> perm, cface, flr;
+    std::vector<T> fgeo, fnw;
+    std::vector<float> fan;
+};
+
+template <typename T>
+static FaceArrays<T> build_faces(const gks_state* s, int face_order) {
     const gks_mesh& g = *s->mesh;
     const int64_t nc = g.nc, nf = g.nf;
-    const Layout& L = s->L;
-    const std::vector<int32_t> perm = face_permutation(g, s->face_order, s->cinv);
+    FaceArrays<T> a;
+    a.perm = face_permutation(g, face_order, s->cinv);
     std::vector<int32_t> inv((size_t)nf);
-    for (int64_t d = 0; d < nf; ++d) inv[perm[d]] = (int32_t)d;
-    std::vector<int32_t> cface(4 * nc), flr(2 * nf);
-    std::vector<T> fgeo(FGEO * nf, T(0)), fnw(4 * nf);
-    std::vector<float> fan(s->L.fan ? 6 * nf : 0, 0.0f);
+    for (int64_t d = 0; d < nf; ++d) inv[a.perm[d]] = (int32_t)d;
+    a.cface.resize(4 * nc);
+    a.flr.resize(2 * nf);
+    a.fgeo.resize(FGEO * nf);
+    a.fnw.resize(4 * nf);
+    a.fan.resize(s->L.fan ? 6 * nf : 0);
     run_ranges(nc, host_threads(nc, 2048), [&](int64_t, int64_t lo, int64_t hi) {
         for (int64_t d = lo; d < hi; ++d) {
             const int64_t c = s->pub(d);
             for (int f = 0; f < 4; ++f) {
                 const int64_t fi = g.csr_face[c * 4 + f];
                 const bool left = g.csr_sign[c * 4 + f] > 0;
-                cface[f * nc + d] = (int32_t)((int64_t)inv[fi] * 2 + (left ? 0 : 1));
+                a.cface[f * nc + d] = (int32_t)((int64_t)inv[fi] * 2 + (left ? 0 : 1));
             }
         }
     });
     run_ranges(nf, host_threads(nf, 2048), [&](int64_t, int64_t lo, int64_t hi) {
         for (int64_t d = lo; d < hi; ++d) {
-            const int64_t f = perm[d];
+            const int64_t f = a.perm[d];
             // a boundary face's missing side carries its kind: -1 - GKS_BC_*
             const int32_t miss = -1 - (int32_t)g.bkind[f];
-            flr[d] = g.face_lr[f * 2] >= 0 ? (int32_t)s->dev(g.face_lr[f * 2]) : miss;
-            flr[nf + d] = g.face_lr[f * 2 + 1] >= 0 ? (int32_t)s->dev(g.face_lr[f * 2 + 1]) : miss;
-            T* r = &fgeo[d * FGEO];
-            for (int a = 0; a < 3; ++a) r[a] = (T)g.fnorm[f * 3 + a];
+            a.flr[d] = g.face_lr[f * 2] >= 0 ? (int32_t)s->dev(g.face_lr[f * 2]) : miss;
+            a.flr[nf + d] = g.face_lr[f * 2 + 1] >= 0 ? (int32_t)s->dev(g.face_lr[f * 2 + 1]) : miss;
+            T* r = &a.fgeo[d * FGEO];
+            for (int i = 0; i < 3; ++i) r[i] = (T)g.fnorm[f * 3 + i];
             r[3] = (T)(g.farea[f] / 3.0);
-            for (int a = 0; a < 4; ++a) fnw[d * 4 + a] = r[a];
+            for (int i = 0; i < 4; ++i) a.fnw[d * 4 + i] = r[i];
             for (int k = 0; k < 9; ++k) {
                 r[4 + k] = (T)g.gp_l[f * 9 + k];
                 r[13 + k] = (T)g.gp_r[f * 9 + k];
             }
-            if (!fan.empty())
-                for (int a = 0; a < 3; ++a) {
-                    const double v = g.farea[f] * g.fnorm[f * 3 + a];
-                    fan[d * 6 + 2 * a] = (float)v;
-                    fan[d * 6 + 2 * a + 1] = (float)(v - (double)(float)v);
+            if (!a.fan.empty())
+                for (int i = 0; i < 3; ++i) {
+                    const double v = g.farea[f] * g.fnorm[f * 3 + i];
+                    a.fan[d * 6 + 2 * i] = (float)v;
+                    a.fan[d * 6 + 2 * i + 1] = (float)(v - (double)(float)v);
                 }
         }
     });
+    return a;
+}
+
+template <typename T>
+static gks_status put_faces(gks_state* s, const FaceArrays<T>& a) {
+    const Layout& L = s->L;
     auto put = [&](size_t off, const void* src, size_t bytes) -> cudaError_t {
         return cudaMemcpyAsync(s->ws + off, src, bytes, cudaMemcpyHostToDevice, s->stream);
     };
-    GKS_CHECK_CUDA(put(L.cface, cface.data(), 4 * cface.size()));
-    GKS_CHECK_CUDA(put(L.flr, flr.data(), 4 * flr.size()));
-    GKS_CHECK_CUDA(put(L.fgeo, fgeo.data(), sizeof(T) * fgeo.size()));
-    GKS_CHECK_CUDA(put(L.fnw, fnw.data(), sizeof(T) * fnw.size()));
-    if (!fan.empty()) GKS_CHECK_CUDA(put(L.fan, fan.data(), 4 * fan.size()));
-    GKS_CHECK_CUDA(put(L.perm, perm.data(), 4 * perm.size()));
+    GKS_CHECK_CUDA(put(L.cface, a.cface.data(), 4 * a.cface.size()));
+    GKS_CHECK_CUDA(put(L.flr, a.flr.data(), 4 * a.flr.size()));
+    GKS_CHECK_CUDA(put(L.fgeo, a.fgeo.data(), sizeof(T) * a.fgeo.size()));
+    GKS_CHECK_CUDA(put(L.fnw, a.fnw.data(), sizeof(T) * a.fnw.size()));
+    if (!a.fan.empty()) GKS_CHECK_CUDA(put(L.fan, a.fan.data(), 4 * a.fan.size()));
+    GKS_CHECK_CUDA(put(L.perm, a.perm.data(), 4 * a.perm.size()));
     GKS_CHECK_CUDA(cudaStreamSynchronize(s->stream));  // host vectors die here
     return GKS_OK;
 }
@@ -635,6 +665,9 @@ static gks_status upload_faces(gks_state* s) {
 // the reconstruction's static cell data in the operator precision TO
 template <typename T, typename TO>
 static gks_status upload_cells(gks_state* s) {
+    // everything that takes memory comes before the first upload: where it
+    // cannot be had, the device's arrays stay as they were
+    const FaceArrays<T> faces = build_faces<T>(s, s->face_order);
     const gks_mesh& g = *s->mesh;
     const int64_t nc = g.nc;
     const Layout& L = s->L;
@@ -728,7 +761,7 @@ static gks_status upload_cells(gks_state* s) {
     GKS_CHECK_CUDA(cudaMemsetAsync(s->ws + L.ctrl, 0, 8 * CTRL_N, s->stream));
     GKS_CHECK_CUDA(cudaMemsetAsync(s->ws + L.err, 0, 4, s->stream));
     GKS_CHECK_CUDA(cudaStreamSynchronize(s->stream));  // host vectors die here
-    return upload_faces<T>(s);
+    return put_faces<T>(s, faces);
 }
 
 template <typename T>
@@ -794,19 +827,14 @@ extern "C" gks_status gks_state_create(const gks_mesh* mesh, const gks_params* p
         }
         s->own_stream = true;
     }
-    gks_status st;
-    try {
+    const gks_status st = guarded([&]() -> gks_status {
         if (fp32) {
             make_views<float>(s, s->m32, s->s32);
-            st = upload_mesh<float>(s);
-        } else {
-            make_views<double>(s, s->m64, s->s64);
-            st = upload_mesh<double>(s);
+            return upload_mesh<float>(s);
         }
-    } catch (const std::bad_alloc&) {
-        set_error("gks_state_create: out of memory");
-        st = GKS_E_NOMEM;
-    }
+        make_views<double>(s, s->m64, s->s64);
+        return upload_mesh<double>(s);
+    });
     if (st != GKS_OK) {
         if (s->own_stream) cudaStreamDestroy(s->stream);
         delete s;
@@ -849,7 +877,6 @@ extern "C" gks_status gks_set_fixed_state(gks_state* s, const double* d_W, const
     if (!s || !d_W || !d_dW) { set_error("gks_set_fixed_state: NULL argument"); return GKS_E_ARG; }
     if (!has_fixed(*s->mesh)) { set_error("gks_set_fixed_state: the mesh has no fixed boundary faces"); return GKS_E_ARG; }
     order_after_caller(s);
-    const int64_t nc = s->mesh->nc;
     if (s->fp32)
         GKS_CHECK_CUDA(Launch<float>::pack(s->m32, s->phys, d_W, d_dW, const_cast<float*>(s->m32.fixed), nullptr, nullptr,
                                            s->stream, s->dperm()));
@@ -1145,22 +1172,26 @@ static gks_status timestep_impl(gks_state* s, DevMesh<T>& m, DevState<T>& st, do
 extern "C" gks_status gks_timestep(gks_state* s, double* dt) {
     if (!s || !dt) { set_error("gks_timestep: NULL argument"); return GKS_E_ARG; }
     if (!s->initialised) { set_error("gks_timestep: state not initialised"); return GKS_E_STATE; }
-    return s->fp32 ? timestep_impl<float>(s, s->m32, s->s32, dt) : timestep_impl<double>(s, s->m64, s->s64, dt);
+    return guarded([&]() -> gks_status {
+        return s->fp32 ? timestep_impl<float>(s, s->m32, s->s32, dt) : timestep_impl<double>(s, s->m64, s->s64, dt);
+    });
 }
 
 extern "C" gks_status gks_residual(gks_state* s, double* out_l2) {
     if (!s || !out_l2) { set_error("gks_residual: NULL argument"); return GKS_E_ARG; }
-    const int nblk = update_blocks(s->mesh->nc);
-    std::vector<double> part((size_t)nblk * PART_N);
-    GKS_CHECK_CUDA(cudaMemcpyAsync(part.data(), s->fp32 ? s->s32.part : s->s64.part, 8 * part.size(),
-                                   cudaMemcpyDeviceToHost, s->stream));
-    GKS_CHECK_CUDA(cudaStreamSynchronize(s->stream));
-    for (int q = 0; q < 5; ++q) {
-        double acc = 0.0;
-        for (int b = 0; b < nblk; ++b) acc += part[(size_t)b * PART_N + PART_RES + q];
-        out_l2[q] = std::sqrt(acc / (double)s->mesh->nc);
-    }
-    return GKS_OK;
+    return guarded([&]() -> gks_status {
+        const int nblk = update_blocks(s->mesh->nc);
+        std::vector<double> part((size_t)nblk * PART_N);
+        GKS_CHECK_CUDA(cudaMemcpyAsync(part.data(), s->fp32 ? s->s32.part : s->s64.part, 8 * part.size(),
+                                       cudaMemcpyDeviceToHost, s->stream));
+        GKS_CHECK_CUDA(cudaStreamSynchronize(s->stream));
+        for (int q = 0; q < 5; ++q) {
+            double acc = 0.0;
+            for (int b = 0; b < nblk; ++b) acc += part[(size_t)b * PART_N + PART_RES + q];
+            out_l2[q] = std::sqrt(acc / (double)s->mesh->nc);
+        }
+        return GKS_OK;
+    });
 }
 
 // --------------------------------------------------------------- adjoint --
@@ -1399,13 +1430,20 @@ extern "C" gks_status gks_state_set_variant(gks_state* s, int32_t face_order, in
         cudaGraphExecDestroy(s->graph);
         s->graph = nullptr;
     }
+    const gks_status st = guarded([&]() -> gks_status {
+        if (face_order == s->face_order) return GKS_OK;
+        if (s->fp32) {
+            const FaceArrays<float> a = build_faces<float>(s, face_order);
+            s->face_order = face_order;
+            return put_faces<float>(s, a);
+        }
+        const FaceArrays<double> a = build_faces<double>(s, face_order);
+        s->face_order = face_order;
+        return put_faces<double>(s, a);
+    });
+    if (st != GKS_OK) return st;
     s->flux_variant = flux_blocks == 3 ? 1 : 0;
     s->slopes_pass = slopes_pass;
-    if (face_order != s->face_order) {
-        s->face_order = face_order;
-        gks_status st = s->fp32 ? upload_faces<float>(s) : upload_faces<double>(s);
-        if (st != GKS_OK) return st;
-    }
     return GKS_OK;
 }
 
@@ -1440,6 +1478,9 @@ static gks_status reorder_impl(gks_state* s, DevMesh<T>& m, DevState<T>& st, int
     std::vector<int32_t> np = cell_permutation(g, order);  // new device cell -> caller's cell
     std::vector<int32_t> map((size_t)nc);                  // new device cell -> old device cell
     for (int64_t d = 0; d < nc; ++d) map[d] = (int32_t)s->dev(np[d]);
+    std::vector<int32_t> ninv(order ? (size_t)nc : 0);
+    for (int64_t d = 0; order && d < nc; ++d) ninv[np[d]] = (int32_t)d;
+    if (order == 0) np.clear();
     char* sb = s->ws + s->L.stage;
     const size_t wd_b = 8 * 5 * (size_t)nc, x_b = sizeof(T) * Stride<T>::xs * (size_t)nc;
     char* map_d = sb + wd_b + 2 * x_b;
@@ -1450,16 +1491,19 @@ static gks_status reorder_impl(gks_state* s, DevMesh<T>& m, DevState<T>& st, int
     if (m.fixed) GKS_CHECK_CUDA(cudaMemcpyAsync(sb + wd_b + x_b, m.fixed, x_b, cudaMemcpyDeviceToDevice, s->stream));
     GKS_CHECK_CUDA(cudaMemcpyAsync(map_d, map.data(), 4 * (size_t)nc, cudaMemcpyHostToDevice, s->stream));
     GKS_CHECK_CUDA(cudaStreamSynchronize(s->stream));  // map dies with this call
-    s->cell_order = order;
-    if (order == 0) {
-        s->cperm.clear();
-        s->cinv.clear();
-    } else {
-        s->cperm = np;
-        s->cinv.assign((size_t)nc, 0);
-        for (int64_t d = 0; d < nc; ++d) s->cinv[np[d]] = (int32_t)d;
+    auto exchange = [&] {
+        std::swap(s->cell_order, order);
+        s->cperm.swap(np);
+        s->cinv.swap(ninv);
+    };
+    exchange();
+    gks_status r = GKS_OK;
+    try {
+        r = upload_mesh<T>(s);
+    } catch (...) {  // nothing uploaded
+        exchange();
+        throw;
     }
-    gks_status r = upload_mesh<T>(s);
     if (r != GKS_OK) return r;
     const int32_t* mp = reinterpret_cast<const int32_t*>(map_d);
     if (s->initialised) {
@@ -1487,7 +1531,7 @@ extern "C" gks_status gks_state_set_cell_order(gks_state* s, int32_t order) {
         s->graph = nullptr;
     }
     order_after_caller(s);
-    return reorder_impl<float>(s, s->m32, s->s32, order);
+    return guarded([&]() -> gks_status { return reorder_impl<float>(s, s->m32, s->s32, order); });
 }
 
 extern "C" gks_status gks_state_get_cell_order(const gks_state* s, int32_t* order) {

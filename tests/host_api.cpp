@@ -1,0 +1,234 @@
+// The C ABI's host side without a GPU: the API's sources over a stand-in for
+// the CUDA runtime (device memory is host memory, copies are done at once)
+// and launches that only note what they were given.  Reads a mesh from the
+// file argv[2], runs the check argv[1], prints "ok" and counts.
+#include <atomic>
+#include <cstdio>
+#include <cstdlib>
+#include <new>
+#include <string>
+
+#include "gks_api.cpp"
+
+// ---- the n-th allocation from here on fails (-1: none)
+static std::atomic<long> fail_in{-1};
+void* operator new(std::size_t n) {
+    if (fail_in.load() >= 0 && fail_in.fetch_sub(1) == 0) throw std::bad_alloc();
+    if (void* p = std::malloc(n)) return p;
+    throw std::bad_alloc();
+}
+void operator delete(void* p) noexcept { std::free(p); }
+void operator delete(void* p, std::size_t) noexcept { std::free(p); }
+
+// ---- CUDA runtime
+extern "C" {
+cudaError_t cudaMemcpyAsync(void* d, const void* s, size_t n, cudaMemcpyKind, cudaStream_t) {
+    std::memmove(d, s, n);
+    return cudaSuccess;
+}
+cudaError_t cudaMemsetAsync(void* d, int v, size_t n, cudaStream_t) {
+    std::memset(d, v, n);
+    return cudaSuccess;
+}
+cudaError_t cudaPointerGetAttributes(cudaPointerAttributes* a, const void*) {
+    a->type = cudaMemoryTypeDevice;
+    return cudaSuccess;
+}
+cudaError_t cudaStreamCreateWithFlags(cudaStream_t* s, unsigned) { *s = nullptr; return cudaSuccess; }
+cudaError_t cudaStreamDestroy(cudaStream_t) { return cudaSuccess; }
+cudaError_t cudaStreamSynchronize(cudaStream_t) { return cudaSuccess; }
+cudaError_t cudaStreamBeginCapture(cudaStream_t, cudaStreamCaptureMode) { return cudaSuccess; }
+cudaError_t cudaStreamEndCapture(cudaStream_t, cudaGraph_t* g) { *g = nullptr; return cudaSuccess; }
+cudaError_t cudaGraphInstantiate(cudaGraphExec_t* e, cudaGraph_t, unsigned long long) { *e = nullptr; return cudaSuccess; }
+cudaError_t cudaGraphLaunch(cudaGraphExec_t, cudaStream_t) { return cudaSuccess; }
+cudaError_t cudaGraphDestroy(cudaGraph_t) { return cudaSuccess; }
+cudaError_t cudaGraphExecDestroy(cudaGraphExec_t) { return cudaSuccess; }
+cudaError_t cudaEventCreate(cudaEvent_t*) { return cudaSuccess; }
+cudaError_t cudaEventDestroy(cudaEvent_t) { return cudaSuccess; }
+cudaError_t cudaEventRecord(cudaEvent_t, cudaStream_t) { return cudaSuccess; }
+cudaError_t cudaEventSynchronize(cudaEvent_t) { return cudaSuccess; }
+cudaError_t cudaEventElapsedTime(float* ms, cudaEvent_t, cudaEvent_t) { *ms = 1.0f; return cudaSuccess; }
+cudaError_t cudaGetLastError(void) { return cudaSuccess; }
+const char* cudaGetErrorString(cudaError_t) { return "error"; }
+}
+
+// ---- launches
+static int launches = 0;
+namespace gks {
+static cudaError_t launched() { ++launches; return cudaSuccess; }
+template <typename T> cudaError_t Launch<T>::slopes(const DevMesh<T>&, const T*, T*, const Finalize*, cudaStream_t) { return launched(); }
+template <typename T> cudaError_t Launch<T>::recon(const DevMesh<T>&, const HostPhys&, const T*, const T*, T*, T*, int32_t*, const Finalize*, int32_t*, cudaStream_t) { return launched(); }
+template <typename T> cudaError_t Launch<T>::flux(const DevMesh<T>&, const HostPhys&, const T*, const T*, T*, const double*, double, int, cudaStream_t, int) { return launched(); }
+template <typename T> cudaError_t Launch<T>::update1(const DevMesh<T>&, const HostPhys&, const DevState<T>&, cudaStream_t) { return launched(); }
+template <typename T> cudaError_t Launch<T>::update2(const DevMesh<T>&, const HostPhys&, const DevState<T>&, cudaStream_t) { return launched(); }
+template <typename T> cudaError_t Launch<T>::dt_partials(const DevMesh<T>&, const HostPhys&, const T*, double*, cudaStream_t) { return launched(); }
+template <typename T> cudaError_t Launch<T>::pack(const DevMesh<T>&, const HostPhys&, const double*, const double*, T*, double*, unsigned long long*, cudaStream_t, const int32_t*) { return launched(); }
+template <typename T> cudaError_t Launch<T>::unpack(const double*, const T*, double*, double*, int64_t, cudaStream_t, const int32_t*) { return launched(); }
+template <typename T> cudaError_t Launch<T>::to_double(const T*, double*, int64_t, cudaStream_t) { return launched(); }
+template <typename T> cudaError_t Launch<T>::rec_to_double(const T*, const int32_t*, double*, int64_t, int, const DevMesh<T>*, const T*, double, double, cudaStream_t) { return launched(); }
+template <typename T> cudaError_t Launch<T>::poly_to_double(const T*, double*, int64_t, cudaStream_t, const int32_t*) { return launched(); }
+template struct Launch<float>;
+template struct Launch<double>;
+cudaError_t launch_stage(const DevMesh<float>&, const HostPhys&, const DevState<float>&, int, const Launch<float>::Finalize*, unsigned*, cudaStream_t) { return launched(); }
+cudaError_t launch_set_control(double*, double*, double*, unsigned long long*, int32_t, double, double, int, int32_t*, cudaStream_t) { return launched(); }
+cudaError_t launch_rows_gather(const void*, void*, int64_t, int, const int32_t*, cudaStream_t) { return launched(); }
+cudaError_t launch_grid_barrier_probe(unsigned*, int32_t*, int, cudaStream_t) { return launched(); }
+cudaError_t launch_wait_probe(int32_t*, int, cudaStream_t) { return launched(); }
+cudaError_t adjoint_reverse(const DevMesh<double>&, const HostPhys&, double, const AdjBuffers&, const double*, const double*, const double*, const double*, double*, double*, cudaStream_t) { return launched(); }
+int update_blocks(int64_t nc) { return (int)((nc + CELLS_PER_BLOCK - 1) / CELLS_PER_BLOCK); }
+}  // namespace gks
+
+#define REQUIRE(x)                                                                                    \
+    do {                                                                                              \
+        if (!(x)) {                                                                                   \
+            std::printf("%s:%d: %s (last error: %s)\n", __FILE__, __LINE__, #x, gks_last_error());    \
+            std::exit(1);                                                                             \
+        }                                                                                             \
+    } while (0)
+
+struct MeshFile {
+    std::vector<double> xyz, period;
+    std::vector<int64_t> tet;
+    std::vector<int8_t> shift, kind;
+    int64_t nv = 0, nc = 0;
+    explicit MeshFile(const char* path) {
+        std::FILE* f = std::fopen(path, "rb");
+        REQUIRE(f && std::fread(&nv, 8, 1, f) == 1 && std::fread(&nc, 8, 1, f) == 1);
+        xyz.resize(3 * nv);
+        period.resize(3);
+        tet.resize(4 * nc);
+        shift.resize(12 * nc);
+        kind.resize(4 * nc);
+        REQUIRE(std::fread(xyz.data(), 8, xyz.size(), f) == xyz.size());
+        REQUIRE(std::fread(period.data(), 8, 3, f) == 3);
+        REQUIRE(std::fread(tet.data(), 8, tet.size(), f) == tet.size());
+        REQUIRE(std::fread(shift.data(), 1, shift.size(), f) == shift.size());
+        REQUIRE(std::fread(kind.data(), 1, kind.size(), f) == kind.size());
+        std::fclose(f);
+    }
+    gks_mesh* make() const {
+        gks_mesh* m = nullptr;
+        REQUIRE(gks_mesh_create(xyz.data(), nv, tet.data(), shift.data(), nc, period.data(), &m) == GKS_OK);
+        REQUIRE(gks_mesh_set_boundary(m, kind.data()) == GKS_OK);
+        REQUIRE(gks_stencil_build(m, nullptr) == GKS_OK);
+        return m;
+    }
+};
+
+static gks_params parameters(int precision, int weno, int constraint = 0) {
+    gks_params p;
+    gks_params_default(&p);
+    p.precision = precision;
+    p.weno = weno;
+    p.wall_constraint = constraint;
+    return p;
+}
+
+struct Workspace {
+    std::vector<char> raw;
+    char* at;
+    size_t bytes;
+    explicit Workspace(size_t n) : raw(n + 256, 0), bytes(n) {
+        at = raw.data() + (256 - (size_t)((uintptr_t)raw.data() & 255)) % 256;
+    }
+};
+
+// call(): every allocation in turn fails once, until one call has met none;
+// check(status) after each.  Returns the number of refused calls.
+template <typename Call, typename Check>
+static int each_allocation(const Call& call, const Check& check) {
+    int refused = 0;
+    for (long n = 0;; ++n) {
+        gks_status st = GKS_OK;
+        bool escaped = false;
+        fail_in = n;
+        try {
+            st = call();
+        } catch (...) {
+            escaped = true;
+        }
+        const bool met = fail_in.exchange(-1) < 0;
+        REQUIRE(!escaped);
+        REQUIRE(st == GKS_OK || st == GKS_E_NOMEM);
+        REQUIRE(met || st == GKS_OK);
+        check(st);
+        refused += st != GKS_OK;
+        if (!met) return refused;
+    }
+}
+
+// what lies outside the staging buffer
+static std::string outside_stage(const gks_state* s, const Workspace& w) {
+    const size_t a = s->L.stage, b = s->L.cperm ? s->L.cperm : w.bytes;
+    return std::string(w.at, w.at + a) + std::string(w.at + b, w.at + w.bytes);
+}
+
+static int allocations(const MeshFile& file) {
+    int refused = 0;
+    gks_mesh* m = nullptr;
+    refused += each_allocation(
+        [&] { return gks_mesh_create(file.xyz.data(), file.nv, file.tet.data(), file.shift.data(), file.nc, file.period.data(), &m); },
+        [&](gks_status st) {
+            REQUIRE((m != nullptr) == (st == GKS_OK));
+            gks_mesh_destroy(m);
+            m = nullptr;
+        });
+    m = file.make();
+    refused += each_allocation([&] { return gks_mesh_set_boundary(m, file.kind.data()); }, [](gks_status) {});
+    refused += each_allocation([&] { return gks_stencil_build(m, nullptr); }, [](gks_status) {});
+    for (int precision = 0; precision < 3; ++precision) {
+        const gks_params p = parameters(precision, 1, precision == 1);
+        Workspace w(gks_workspace_bytes(m, &p));
+        gks_state* s = nullptr;
+        refused += each_allocation([&] { return gks_state_create(m, &p, w.at, w.bytes, nullptr, &s); },
+                                   [&](gks_status st) {
+                                       REQUIRE((s != nullptr) == (st == GKS_OK));
+                                       gks_state_destroy(s);
+                                       s = nullptr;
+                                   });
+        REQUIRE(gks_state_create(m, &p, w.at, w.bytes, nullptr, &s) == GKS_OK);
+        s->initialised = true;
+        double v[5];
+        refused += each_allocation([&] { return gks_timestep(s, v); }, [](gks_status) {});
+        refused += each_allocation([&] { return gks_residual(s, v); }, [](gks_status) {});
+        // a refused change leaves the device's arrays as they were
+        const std::string first = outside_stage(s, w);
+        REQUIRE(gks_state_set_variant(s, 1, 2, 0) == GKS_OK);
+        const std::string grouped = outside_stage(s, w);
+        REQUIRE(gks_state_set_variant(s, 0, 3, 1) == GKS_OK && outside_stage(s, w) == first && grouped != first);
+        refused += each_allocation([&] { return gks_state_set_variant(s, 1, 2, 0); }, [&](gks_status st) {
+            REQUIRE(outside_stage(s, w) == (st == GKS_OK ? grouped : first));
+            REQUIRE(s->flux_variant == (st == GKS_OK ? 0 : 1) && s->slopes_pass == (st == GKS_OK ? 0 : 1));
+            REQUIRE(gks_state_set_variant(s, 0, 3, 1) == GKS_OK);
+        });
+        for (int order = 1; precision > 0 && order < 3; ++order) {
+            REQUIRE(gks_state_set_cell_order(s, order) == GKS_OK);
+            const std::string there = outside_stage(s, w);
+            refused += each_allocation([&] { return gks_state_set_cell_order(s, 0); }, [&](gks_status st) {
+                REQUIRE(s->cell_order == (st == GKS_OK ? 0 : order) && s->cperm.empty() == (st == GKS_OK));
+                if (st != GKS_OK) REQUIRE(outside_stage(s, w) == there);
+                REQUIRE(gks_state_set_cell_order(s, order) == GKS_OK && outside_stage(s, w) == there);
+            });
+            REQUIRE(gks_state_set_cell_order(s, 0) == GKS_OK);
+            refused += each_allocation([&] { return gks_state_set_cell_order(s, order); }, [&](gks_status st) {
+                REQUIRE(s->cell_order == (st == GKS_OK ? order : 0) && s->cinv.empty() == (st != GKS_OK));
+                REQUIRE(gks_state_set_cell_order(s, 0) == GKS_OK);
+            });
+        }
+        gks_state_destroy(s);
+    }
+    gks_mesh_destroy(m);
+    return refused;
+}
+
+int main(int argc, char** argv) {
+    REQUIRE(argc == 3);
+    const std::string check = argv[1];
+    const MeshFile file(argv[2]);
+    if (check == "allocations") {
+        std::printf("ok %d\n", allocations(file));
+        return 0;
+    }
+    std::printf("unknown check %s\n", argv[1]);
+    return 1;
+}

@@ -1,0 +1,47 @@
+"""The C ABI's host side on the CPU: the library's host sources compiled over
+a stand-in for the CUDA runtime (host_api.cpp), so that what it uploads, and
+what it does when memory runs out, can be looked at without a GPU."""
+import os
+import subprocess
+
+import numpy as np
+import pytest
+
+from paper_2102_01366_gb300 import _build
+from paper_2102_01366_gb300 import inputs as I
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+
+
+@pytest.fixture(scope="module")
+def host_api(tmp_path_factory):
+    """check(name, mesh, kinds): the output of one check of host_api.cpp."""
+    d = tmp_path_factory.mktemp("host_api")
+    exe = str(d / "host_api")
+    src = [os.path.join(HERE, "host_api.cpp")] + [os.path.join(_build.CSRC, f) for f in ("gks_mesh.cpp", "gks_stencil.cpp")]
+    subprocess.run(["g++", "-O1", "-std=c++17", "-pthread", "-I", os.path.join(_build._cuda_home(), "include"),
+                    "-I", _build.INCLUDE, "-I", _build.CSRC] + src + ["-o", exe], check=True)
+
+    def check(name, mesh, kinds):
+        path = str(d / "mesh.bin")
+        with open(path, "wb") as f:
+            np.array([len(mesh["xyz"]), len(mesh["tet"])], np.int64).tofile(f)
+            for a, t in ((mesh["xyz"], np.float64), (mesh["period"], np.float64), (mesh["tet"], np.int64),
+                         (mesh["shift"], np.int8), (kinds, np.int8)):
+                np.ascontiguousarray(a, dtype=t).tofile(f)
+        r = subprocess.run([exe, name, path], capture_output=True, text=True, timeout=600)
+        assert r.returncode == 0 and r.stdout.startswith("ok"), (r.returncode, r.stdout, r.stderr)
+        return [int(x) for x in r.stdout.split()[1:]]
+    return check
+
+
+# 162 cells: one thread; 2,058: several threads in every loop over cells and faces
+@pytest.mark.parametrize("dims", [(3, 3, 3), (7, 7, 7)])
+def test_memory_that_cannot_be_had_is_reported(host_api, dims):
+    """Each allocation of each call fails once: the call returns GKS_E_NOMEM
+    (or succeeds without it), no exception leaves it, and a refused change of
+    the face or cell order leaves the device's arrays as they were."""
+    mesh = I.box_mesh(dims, jitter=0.1, seed=81, periodic=(False, True, True))
+    kinds = I.boundary_kinds(mesh, {(0, "lo"): I.BC_NOSLIP_WALL, (0, "hi"): I.BC_FIXED})
+    refused, = host_api("allocations", mesh, kinds)
+    assert refused > 50
