@@ -51,8 +51,9 @@ bool has_wall_face(const gks_mesh& m, int64_t c);
 
 // threads for a loop over n cells or faces, with at least `grain` of them each
 inline int64_t host_threads(int64_t n, int64_t grain = 16384) {
-    const unsigned hw = std::max(1u, std::thread::hardware_concurrency());
-    return std::min<int64_t>((int64_t)hw, std::max<int64_t>(1, n / grain));
+    // (asked once: it is a system call, 10 us on some hosts)
+    static const int64_t hw = std::max(1u, std::thread::hardware_concurrency());
+    return std::min(hw, std::max<int64_t>(1, n / grain));
 }
 
 // fn(t, lo, hi) over nthr contiguous ranges of [0, n); range 0 on the calling

@@ -221,12 +221,92 @@ static int allocations(const MeshFile& file) {
     return refused;
 }
 
+// the arrays of one state against the mesh, element by element
+template <typename T, typename TO>
+static void compare_arrays(const gks_state* s, const gks_mesh& g) {
+    const Layout& L = s->L;
+    const int64_t nc = g.nc, nf = g.nf, nblk = update_blocks(nc);
+    auto i32 = [&](size_t off) { return reinterpret_cast<const int32_t*>(s->ws + off); };
+    const TO* tile = reinterpret_cast<const TO*>(s->ws + L.tile);
+    const T* fgeo = reinterpret_cast<const T*>(s->ws + L.fgeo);
+    const T* fnw = reinterpret_cast<const T*>(s->ws + L.fnw);
+    const int32_t *perm = i32(L.perm), *flr = i32(L.flr), *cface = i32(L.cface);
+    auto pub = [&](int64_t d) { return s->cperm.empty() ? d : (int64_t)s->cperm[d]; };
+    for (int64_t d = 0; d < nblk * CELLS_PER_BLOCK; ++d) {
+        const TO* blk = tile + d / CELLS_PER_BLOCK * TILE_ROWS * CELLS_PER_BLOCK;
+        auto row = [&](int r) { return blk[tile_at<TO>(r, (int)(d % CELLS_PER_BLOCK))]; };
+        if (d >= nc) {
+            for (int r = 0; r < TILE_ROWS; ++r) REQUIRE(row(r) == TO(0));
+            continue;
+        }
+        const int64_t c = pub(d);
+        double far[3] = {0.0, 0.0, 0.0};
+        for (int k = 0; k < 144; ++k) REQUIRE(row(TILE_M2 + k) == (TO)g.M2[c * 144 + k]);
+        for (int k = 0; k < 12; ++k) REQUIRE(row(TILE_M1 + k) == (TO)g.M1[c * 12 + k]);
+        for (int k = 0; k < 6; ++k) REQUIRE(row(TILE_MOM + k) == (TO)g.mom2[c * 6 + k]);
+        REQUIRE(row(TILE_V23) == (TO)std::pow(g.vol[c], 2.0 / 3.0) && row(TILE_V43) == (TO)std::pow(g.vol[c], 4.0 / 3.0));
+        for (int f = 0; f < 4; ++f) {
+            const int64_t face = g.csr_face[c * 4 + f];
+            const bool left = g.csr_sign[c * 4 + f] > 0;
+            const int32_t e = cface[f * nc + d];
+            REQUIRE(perm[e >> 1] == face && (e & 1) == (left ? 0 : 1));
+            REQUIRE(flr[(left ? 0 : nf) + (e >> 1)] == (int32_t)d);
+            for (int k = 0; k < 9; ++k) {
+                const double x = (left ? g.gp_l : g.gp_r)[face * 9 + k];
+                REQUIRE(row(TILE_G + f * 9 + k) == (TO)x);
+                REQUIRE(fgeo[(e >> 1) * FGEO + (left ? 4 : 13) + k] == (T)x);
+                if (std::abs(x) > far[k % 3]) far[k % 3] = std::abs(x);
+            }
+            if (g.nbr[c * 4 + f] < 0) REQUIRE(flr[(left ? nf : 0) + (e >> 1)] == -1 - (int32_t)g.bkind[face]);
+        }
+        for (int k = 0; k < 3; ++k) REQUIRE(row(TILE_BND + k) == (TO)far[k]);
+    }
+    for (int64_t d = 0; d < nf; ++d) {
+        const int64_t f = perm[d];
+        for (int k = 0; k < 4; ++k) {
+            const T v = k < 3 ? (T)g.fnorm[f * 3 + k] : (T)(g.farea[f] / 3.0);
+            REQUIRE(fgeo[d * FGEO + k] == v && fnw[d * 4 + k] == v);
+        }
+        for (int k = 0; L.fan && k < 3; ++k) {
+            const float* a = reinterpret_cast<const float*>(s->ws + L.fan) + 6 * d + 2 * k;
+            const double v = g.farea[f] * g.fnorm[f * 3 + k];
+            REQUIRE(a[0] == (float)v && a[1] == (float)(v - (double)(float)v));
+        }
+    }
+}
+
+static int arrays(const MeshFile& file) {
+    int states = 0;
+    gks_mesh* m = file.make();
+    for (int precision = 0; precision < 3; ++precision)
+        for (int cells = 0; cells < (precision ? 3 : 1); ++cells)
+            for (int faces = 0; faces < 2; ++faces, ++states) {
+                const gks_params p = parameters(precision, 1);
+                Workspace w(gks_workspace_bytes(m, &p));
+                std::memset(w.at, 0x55, w.bytes);
+                gks_state* s = nullptr;
+                REQUIRE(gks_state_create(m, &p, w.at, w.bytes, nullptr, &s) == GKS_OK);
+                if (cells) REQUIRE(gks_state_set_cell_order(s, cells) == GKS_OK);
+                REQUIRE(gks_state_set_variant(s, faces, 3, 1) == GKS_OK);
+                if (precision == 0) compare_arrays<double, double>(s, *m);
+                if (precision == 1) compare_arrays<float, float>(s, *m);
+                if (precision == 2) compare_arrays<float, double>(s, *m);
+                gks_state_destroy(s);
+            }
+    gks_mesh_destroy(m);
+    return states;
+}
+
 int main(int argc, char** argv) {
     REQUIRE(argc == 3);
     const std::string check = argv[1];
     const MeshFile file(argv[2]);
     if (check == "allocations") {
         std::printf("ok %d\n", allocations(file));
+        return 0;
+    }
+    if (check == "arrays") {
+        std::printf("ok %d\n", arrays(file));
         return 0;
     }
     std::printf("unknown check %s\n", argv[1]);

@@ -45,3 +45,12 @@ def test_memory_that_cannot_be_had_is_reported(host_api, dims):
     kinds = I.boundary_kinds(mesh, {(0, "lo"): I.BC_NOSLIP_WALL, (0, "hi"): I.BC_FIXED})
     refused, = host_api("allocations", mesh, kinds)
     assert refused > 50
+
+
+# a ragged last block of cells; one thread, and several in every loop: from
+# 1,536 cells on for the cells, 16,384 faces and cells for the faces
+@pytest.mark.parametrize("dims", [(1, 1, 1), (5, 3, 1), (8, 8, 4), (17, 13, 13)])
+def test_a_states_mesh_arrays_are_the_meshs(host_api, dims):
+    mesh = I.box_mesh(dims, jitter=0.1, seed=82, periodic=(False,) * 3)
+    kinds = I.boundary_kinds(mesh, {(0, "lo"): I.BC_SLIP_WALL, (1, "hi"): I.BC_FIXED, (2, "lo"): I.BC_MOVING_WALL})
+    assert host_api("arrays", mesh, kinds) == [2 + 6 + 6]
