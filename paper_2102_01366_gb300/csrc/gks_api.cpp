@@ -276,7 +276,7 @@ extern "C" gks_status gks_mesh_wall_stencils(const gks_mesh* m, double* W1, doub
     int64_t n = 0;
     for (int64_t c = 0; c < m->nc; ++c) {
         double w1[15], w2[153];
-        const bool ok = has_wall_face(*m, c) && cell_wall_stencil(*m, c, w2, w1);
+        const bool ok = has_wall_face(*m, m->bkind, c) && cell_wall_stencil(*m, m->bkind, c, w2, w1);
         if (!ok) {
             std::memset(w1, 0, sizeof(w1));
             std::memset(w2, 0, sizeof(w2));
@@ -322,7 +322,7 @@ bool has_fixed(const gks_mesh& m) {
 int64_t wall_cells(const gks_mesh& m, const gks_params& p) {
     if (!p.wall_constraint) return 0;
     int64_t n = 0;
-    for (int64_t c = 0; c < m.nc; ++c) n += has_wall_face(m, c);
+    for (int64_t c = 0; c < m.nc; ++c) n += has_wall_face(m, m.bkind, c);
     return n;
 }
 
@@ -383,6 +383,9 @@ Layout layout_workspace(int64_t nc, int64_t nf, int64_t ncase, bool fp32, bool f
 
 struct gks_state {
     const gks_mesh* mesh = nullptr;
+    // the boundary kinds at the state's creation, by which its workspace and
+    // kernels were chosen (gks_mesh_set_boundary applies to later states)
+    std::vector<int8_t> bkind;
     gks_params params;
     HostPhys phys;
     bool fp32 = false;
@@ -558,7 +561,7 @@ static void make_views(gks_state* s, DevMesh<T>& m, DevState<T>& st) {
     m.wopd = L.wslot && s->ops64 ? at<double>(s, L.wop) : nullptr;
     m.xwalls = 0;
     for (int64_t f = 0; f < s->mesh->nf; ++f)
-        if (s->mesh->bkind[f] == GKS_BC_ISOTHERMAL_WALL || s->mesh->bkind[f] == GKS_BC_MOVING_WALL) m.xwalls = 1;
+        if (s->bkind[f] == GKS_BC_ISOTHERMAL_WALL || s->bkind[f] == GKS_BC_MOVING_WALL) m.xwalls = 1;
     st.Wd = at<double>(s, L.Wd);
     st.X = at<T>(s, L.X);
     st.Xs = at<T>(s, L.Xs);
@@ -625,7 +628,7 @@ static std::vector<char> build_faces(const gks_state* s, int face_order) {
         for (int64_t d = lo; d < hi; ++d) {
             const int64_t f = perm[d];
             // a boundary face's missing side carries its kind: -1 - GKS_BC_*
-            const int32_t miss = -1 - (int32_t)g.bkind[f];
+            const int32_t miss = -1 - (int32_t)s->bkind[f];
             flr[d] = g.face_lr[f * 2] >= 0 ? (int32_t)s->dev(g.face_lr[f * 2]) : miss;
             flr[nf + d] = g.face_lr[f * 2 + 1] >= 0 ? (int32_t)s->dev(g.face_lr[f * 2 + 1]) : miss;
             T* r = &fgeo[d * FGEO];
@@ -683,7 +686,7 @@ static gks_status upload_cells(gks_state* s) {
     for (int64_t d = 0; L.wslot && d < nc; ++d) {
         const int64_t c = s->pub(d);
         double w2[153], w1[15];
-        if (has_wall_face(g, c) && cell_wall_stencil(g, c, w2, w1)) {
+        if (has_wall_face(g, s->bkind, c) && cell_wall_stencil(g, s->bkind, c, w2, w1)) {
             wslot[d] = (int32_t)(nwop++);
             TO* o = &wop[(size_t)wslot[d] * WOP_STRIDE];
             for (int k = 0; k < 153; ++k) o[k] = (TO)w2[k];
@@ -826,6 +829,7 @@ extern "C" gks_status gks_state_create(const gks_mesh* mesh, const gks_params* p
         s->own_stream = true;
     }
     const gks_status st = guarded([&]() -> gks_status {
+        s->bkind = mesh->bkind;
         if (fp32) {
             make_views<float>(s, s->m32, s->s32);
             return upload_mesh<float>(s);
@@ -873,7 +877,7 @@ static gks_status init_impl(gks_state* s, DevMesh<T>& m, DevState<T>& st, const 
 
 extern "C" gks_status gks_set_fixed_state(gks_state* s, const double* d_W, const double* d_dW) {
     if (!s || !d_W || !d_dW) { set_error("gks_set_fixed_state: NULL argument"); return GKS_E_ARG; }
-    if (!has_fixed(*s->mesh)) { set_error("gks_set_fixed_state: the mesh has no fixed boundary faces"); return GKS_E_ARG; }
+    if (!s->L.X0) { set_error("gks_set_fixed_state: the mesh has no fixed boundary faces"); return GKS_E_ARG; }
     order_after_caller(s);
     if (s->fp32)
         GKS_CHECK_CUDA(Launch<float>::pack(s->m32, s->phys, d_W, d_dW, const_cast<float*>(s->m32.fixed), nullptr, nullptr,
@@ -1244,7 +1248,7 @@ static gks_status adjoint_impl(gks_state* s, double dt, const double* d_W, const
         set_error("gks_adjoint_step: scratch smaller than gks_adjoint_workspace_bytes");
         return GKS_E_NOMEM;
     }
-    if (s->fp32 || g.ncase != 1 || (has_fixed(g) && !s->fixed_pinned)) {
+    if (s->fp32 || g.ncase != 1 || (s->L.X0 && !s->fixed_pinned)) {
         set_error("gks_adjoint_step: needs an FP64 state on a single-case mesh, and on a mesh with "
                   "fixed-state faces a fixed state set by gks_set_fixed_state");
         return GKS_E_UNSUPPORTED;

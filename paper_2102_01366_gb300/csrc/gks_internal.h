@@ -46,8 +46,9 @@ gks_status build_stencils(gks_mesh& m);  // M1, M2
 bool cell_linear_fit(const gks_mesh& m, int64_t c, double* M2);  // boundary cells, linear weights
 // Sec. 4.4 constrained operators of a cell with non-slip adiabatic wall
 // faces (see gks_stencil.cpp); false when it has none or they cannot be built
-bool cell_wall_stencil(const gks_mesh& m, int64_t c, double* W2, double* W1);
-bool has_wall_face(const gks_mesh& m, int64_t c);
+// kinds: the boundary kinds (gks_mesh::bkind, or a state's own)
+bool cell_wall_stencil(const gks_mesh& m, const std::vector<int8_t>& kinds, int64_t c, double* W2, double* W1);
+bool has_wall_face(const gks_mesh& m, const std::vector<int8_t>& kinds, int64_t c);
 
 // threads for a loop over n cells or faces, with at least `grain` of them each
 inline int64_t host_threads(int64_t n, int64_t grain = 16384) {

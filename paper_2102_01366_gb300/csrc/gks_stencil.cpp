@@ -352,9 +352,9 @@ bool constrained_ls(int n, int ne, const double* E, int nl, const double* A, dou
 
 }  // namespace
 
-bool has_wall_face(const gks_mesh& m, int64_t c) {
+bool has_wall_face(const gks_mesh& m, const std::vector<int8_t>& kinds, int64_t c) {
     for (int f = 0; f < 4; ++f)
-        if (m.nbr[c * 4 + f] < 0 && m.bkind[m.csr_face[c * 4 + f]] == GKS_BC_NOSLIP_WALL) return true;
+        if (m.nbr[c * 4 + f] < 0 && kinds[m.csr_face[c * 4 + f]] == GKS_BC_NOSLIP_WALL) return true;
     return false;
 }
 
@@ -370,7 +370,7 @@ bool has_wall_face(const gks_mesh& m, int64_t c) {
 // Used when there are at least 3 neighbours + wall faces, at most 3 wall
 // faces, at most 9 equality rows in step 2 (neighbours + 3 per wall face)
 // and at least 9 rows in all.
-bool cell_wall_stencil(const gks_mesh& m, int64_t c, double* W2, double* W1) {
+bool cell_wall_stencil(const gks_mesh& m, const std::vector<int8_t>& kinds, int64_t c, double* W2, double* W1) {
     int fl[4], wl[4], nn = 0, nw = 0;
     double d[4][3];
     for (int f = 0; f < 4; ++f) {
@@ -380,7 +380,7 @@ bool cell_wall_stencil(const gks_mesh& m, int64_t c, double* W2, double* W1) {
                 d[nn][a] = (m.cen[nb * 3 + a] + (double)m.nbr_img[(c * 4 + f) * 3 + a] * m.per(c)[a]) -
                            m.cen[c * 3 + a];
             fl[nn++] = f;
-        } else if (m.bkind[m.csr_face[c * 4 + f]] == GKS_BC_NOSLIP_WALL) {
+        } else if (kinds[m.csr_face[c * 4 + f]] == GKS_BC_NOSLIP_WALL) {
             wl[nw++] = f;
         }
     }

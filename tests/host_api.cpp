@@ -257,7 +257,7 @@ static void compare_arrays(const gks_state* s, const gks_mesh& g) {
                 REQUIRE(fgeo[(e >> 1) * FGEO + (left ? 4 : 13) + k] == (T)x);
                 if (std::abs(x) > far[k % 3]) far[k % 3] = std::abs(x);
             }
-            if (g.nbr[c * 4 + f] < 0) REQUIRE(flr[(left ? nf : 0) + (e >> 1)] == -1 - (int32_t)g.bkind[face]);
+            if (g.nbr[c * 4 + f] < 0) REQUIRE(flr[(left ? nf : 0) + (e >> 1)] == -1 - (int32_t)s->bkind[face]);
         }
         for (int k = 0; k < 3; ++k) REQUIRE(row(TILE_BND + k) == (TO)far[k]);
     }
@@ -297,12 +297,50 @@ static int arrays(const MeshFile& file) {
     return states;
 }
 
+// the mesh's boundary kinds change after a state's creation: the state keeps
+// its own through every re-upload, and takes no fixed state it has no room for
+static int kinds(const MeshFile& file) {
+    int states = 0;
+    for (int precision = 0; precision < 3; ++precision)
+        for (int constraint = 0; constraint < 2; ++constraint)
+            for (int kind = GKS_BC_OPEN; kind <= GKS_BC_MOVING_WALL; ++kind, ++states) {
+                gks_mesh* m = file.make();
+                const gks_params p = parameters(precision, 1, constraint);
+                Workspace w(gks_workspace_bytes(m, &p));
+                gks_state* s = nullptr;
+                REQUIRE(gks_state_create(m, &p, w.at, w.bytes, nullptr, &s) == GKS_OK);
+                const std::string first = outside_stage(s, w);
+                const std::vector<int8_t> later(file.kind.size(), (int8_t)kind);
+                REQUIRE(gks_mesh_set_boundary(m, later.data()) == GKS_OK);
+                REQUIRE(gks_state_set_variant(s, 1, 3, 1) == GKS_OK && gks_state_set_variant(s, 0, 3, 1) == GKS_OK);
+                REQUIRE(outside_stage(s, w) == first);
+                if (precision) {
+                    REQUIRE(gks_state_set_cell_order(s, 2) == GKS_OK && gks_state_set_cell_order(s, 0) == GKS_OK);
+                    // (the order's own two arrays, right after the staging buffer, keep what they held)
+                    const size_t orders = 2 * ((4 * (size_t)m->nc + 255) & ~(size_t)255), at = first.size();
+                    const std::string now = outside_stage(s, w);
+                    const size_t a = s->L.stage, b = a + orders;
+                    REQUIRE(now.substr(0, a) == first.substr(0, a) && now.substr(b, at) == first.substr(b, at));
+                }
+                const int before = launches;
+                std::vector<double> W(20 * (size_t)m->nc, 1.0);
+                REQUIRE(gks_set_fixed_state(s, W.data(), W.data()) == GKS_E_ARG && launches == before);
+                gks_state_destroy(s);
+                gks_mesh_destroy(m);
+            }
+    return states;
+}
+
 int main(int argc, char** argv) {
     REQUIRE(argc == 3);
     const std::string check = argv[1];
     const MeshFile file(argv[2]);
     if (check == "allocations") {
         std::printf("ok %d\n", allocations(file));
+        return 0;
+    }
+    if (check == "kinds") {
+        std::printf("ok %d\n", kinds(file));
         return 0;
     }
     if (check == "arrays") {

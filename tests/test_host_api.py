@@ -54,3 +54,11 @@ def test_a_states_mesh_arrays_are_the_meshs(host_api, dims):
     mesh = I.box_mesh(dims, jitter=0.1, seed=82, periodic=(False,) * 3)
     kinds = I.boundary_kinds(mesh, {(0, "lo"): I.BC_SLIP_WALL, (1, "hi"): I.BC_FIXED, (2, "lo"): I.BC_MOVING_WALL})
     assert host_api("arrays", mesh, kinds) == [2 + 6 + 6]
+
+
+def test_a_state_keeps_its_boundary_kinds(host_api):
+    """Kinds set on the mesh after a state's creation are for later states: a
+    change of order uploads the state's own, with the operators its workspace
+    has room for, and a state without fixed faces refuses a fixed state."""
+    mesh = I.box_mesh((3, 2, 2), jitter=0.1, seed=83, periodic=(False,) * 3)
+    assert host_api("kinds", mesh, I.boundary_kinds(mesh, {(0, "lo"): I.BC_NOSLIP_WALL})) == [3 * 2 * 6]
