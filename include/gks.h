@@ -394,7 +394,7 @@ gks_status gks_residual(gks_state* state, double* out_l2);
  * adjoint of its constant to its own average only; the fallback decision is
  * held fixed (piecewise derivative).  All arrays are
  * device FP64; d_scratch (gks_adjoint_workspace_bytes) is caller-allocated
- * device memory.  On return the state is initialised at (d_W, d_dW) with its
+ * device memory, 16-byte aligned (GKS_E_ARG if not).  On return the state is initialised at (d_W, d_dW) with its
  * time reset.  Synchronises. */
 size_t gks_adjoint_workspace_bytes(const gks_state* state);
 gks_status gks_adjoint_step(gks_state* state, double dt, const double* d_W, const double* d_dW,

@@ -1248,6 +1248,10 @@ static gks_status adjoint_impl(gks_state* s, double dt, const double* d_W, const
         set_error("gks_adjoint_step: scratch smaller than gks_adjoint_workspace_bytes");
         return GKS_E_NOMEM;
     }
+    if (((uintptr_t)d_scratch & 15) != 0) {
+        set_error("gks_adjoint_step: scratch must be 16-byte aligned");
+        return GKS_E_ARG;
+    }
     if (s->fp32 || g.ncase != 1 || (s->L.X0 && !s->fixed_pinned)) {
         set_error("gks_adjoint_step: needs an FP64 state on a single-case mesh, and on a mesh with "
                   "fixed-state faces a fixed state set by gks_set_fixed_state");

@@ -331,6 +331,31 @@ static int kinds(const MeshFile& file) {
     return states;
 }
 
+// the adjoint's scratch is read and written in 16-byte vectors
+static int scratch(const MeshFile& file) {
+    gks_mesh* m = file.make();
+    const gks_params p = parameters(0, 1);
+    Workspace w(gks_workspace_bytes(m, &p));
+    gks_state* s = nullptr;
+    REQUIRE(gks_state_create(m, &p, w.at, w.bytes, nullptr, &s) == GKS_OK);
+    const size_t bytes = gks_adjoint_workspace_bytes(s);
+    Workspace room(bytes + 256);
+    std::vector<double> v(20 * (size_t)m->nc, 1.0);
+    double* d = v.data();
+    int refused = 0;
+    for (size_t off = 0; off < 32; off += 8) {
+        const int before = launches;
+        const gks_status a = gks_adjoint_step(s, 0.1, d, d, d, d, d, d, room.at + off, bytes);
+        const gks_status b = gks_adjoint_step_staged(s, 0.1, d, d, d, d, d, d, d, d, room.at + off, bytes);
+        REQUIRE(a == (off % 16 ? GKS_E_ARG : GKS_OK) && b == a);
+        REQUIRE((launches == before) == (off % 16 != 0));
+        refused += a != GKS_OK;
+    }
+    gks_state_destroy(s);
+    gks_mesh_destroy(m);
+    return refused;
+}
+
 int main(int argc, char** argv) {
     REQUIRE(argc == 3);
     const std::string check = argv[1];
@@ -341,6 +366,10 @@ int main(int argc, char** argv) {
     }
     if (check == "kinds") {
         std::printf("ok %d\n", kinds(file));
+        return 0;
+    }
+    if (check == "scratch") {
+        std::printf("ok %d\n", scratch(file));
         return 0;
     }
     if (check == "arrays") {

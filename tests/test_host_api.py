@@ -62,3 +62,8 @@ def test_a_state_keeps_its_boundary_kinds(host_api):
     has room for, and a state without fixed faces refuses a fixed state."""
     mesh = I.box_mesh((3, 2, 2), jitter=0.1, seed=83, periodic=(False,) * 3)
     assert host_api("kinds", mesh, I.boundary_kinds(mesh, {(0, "lo"): I.BC_NOSLIP_WALL})) == [3 * 2 * 6]
+
+
+def test_misaligned_adjoint_scratch_is_refused(host_api):
+    mesh = I.box_mesh((3, 2, 2), jitter=0.1, seed=84, periodic=(False,) * 3)
+    assert host_api("scratch", mesh, I.wall_kinds(mesh, (0,))) == [2]
