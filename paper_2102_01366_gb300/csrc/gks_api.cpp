@@ -389,6 +389,7 @@ struct gks_state {
     gks_params params;
     HostPhys phys;
     bool fp32 = false;
+    int sms = 1;  // of the device
     bool ops64 = false;  // precision 2: FP32 bulk with FP64 stencil operators
     cudaStream_t stream = nullptr;
     bool own_stream = false;
@@ -559,6 +560,7 @@ static void make_views(gks_state* s, DevMesh<T>& m, DevState<T>& st) {
     m.wslot = L.wslot ? at<int32_t>(s, L.wslot) : nullptr;
     m.wop = L.wslot && !s->ops64 ? at<T>(s, L.wop) : nullptr;
     m.wopd = L.wslot && s->ops64 ? at<double>(s, L.wop) : nullptr;
+    m.sms = s->sms;
     m.xwalls = 0;
     for (int64_t f = 0; f < s->mesh->nf; ++f)
         if (s->bkind[f] == GKS_BC_ISOTHERMAL_WALL || s->bkind[f] == GKS_BC_MOVING_WALL) m.xwalls = 1;
@@ -829,6 +831,9 @@ extern "C" gks_status gks_state_create(const gks_mesh* mesh, const gks_params* p
         s->own_stream = true;
     }
     const gks_status st = guarded([&]() -> gks_status {
+        int device = 0;
+        GKS_CHECK_CUDA(cudaGetDevice(&device));
+        GKS_CHECK_CUDA(cudaDeviceGetAttribute(&s->sms, cudaDevAttrMultiProcessorCount, device));
         s->bkind = mesh->bkind;
         if (fp32) {
             make_views<float>(s, s->m32, s->s32);

@@ -35,7 +35,6 @@ namespace gks {
 // 837 us.
 // FP64 is bound by its pipe (16 cycles a warp instruction): rotating and
 // weighting per face instead of per point took 484 -> 450 us on 49,280 faces.
-constexpr int FLUX_THREADS = 3 * FLUX_FACES;
 
 // Fh, D, W0, dW of a point (stage 2: D, dW); rows padded to an odd length
 // so that the threads of a warp write to different banks
@@ -385,20 +384,6 @@ __global__ void __launch_bounds__(TH, MINB) k_flux(DevMesh<T> m, Phys<T> ph, con
 // launches.  Inviscid stage 2 fits 96 registers without spills: 6 blocks (3.15
 // M faces 631 -> 595 us; the viscous one would spill, 255 -> 260 us on 1.16 M).
 constexpr int FLUX_BLOCKS_V1 = 5, FLUX_BLOCKS_V1_STAGE2 = 6, FLUX_BLOCKS_V0 = 4;
-// FP64 is bound by its pipe whatever the occupancy (218-238 registers, no
-// spills), so a launch lasts as long as the SM with the most warps: blocks of
-// 96 threads (32 faces, no lane idle) or of 64 (21 faces, one lane idle),
-// whichever leaves the fullest SM with fewer warps.  6,144 faces: 6 warps with
-// blocks of 96, 4 with 64, a whole step 215 and 153 us; 49,280 faces:
-// 33 and 32 warps, 1,242 and 1,188 us; from about 10^6 faces the blocks of 96
-// win by their full lanes.
-constexpr int FLUX_THREADS_FP64 = 64, SMS = 152;
-
-inline int64_t fullest_sm_warps(int64_t nf, int threads) {
-    const int64_t blocks = (nf + threads / 3 - 1) / (threads / 3);
-    return (blocks + SMS - 1) / SMS * (threads / 32);
-}
-
 template <typename T, bool XW>
 static cudaError_t launch_flux(const DevMesh<T>& m, const HostPhys& p, const T* W, const T* poly, T* rec,
                                const double* ctrl, double dt_override, int stage, cudaStream_t s, int variant) {
@@ -415,7 +400,7 @@ static cudaError_t launch_flux(const DevMesh<T>& m, const HostPhys& p, const T* 
     };
     using std::integral_constant;
     if constexpr (sizeof(T) == 8) {
-        if (fullest_sm_warps(m.nf, FLUX_THREADS_FP64) < fullest_sm_warps(m.nf, FLUX_THREADS))
+        if (flux_small_blocks(m.nf, m.sms))
             blocks(integral_constant<int, FLUX_THREADS_FP64>{}, integral_constant<int, 4>{});
         else
             blocks(integral_constant<int, FLUX_THREADS>{}, integral_constant<int, 2>{});

@@ -15,6 +15,8 @@ enum { PART_DTMIN = 0, PART_RES = 1, PART_N = 6 };
 enum { ERR_STATE = 1, ERR_TIMEOUT = 2 };
 
 constexpr int FLUX_FACES = 32;       // faces per flux block (3 threads each)
+constexpr int FLUX_THREADS = 3 * FLUX_FACES;
+constexpr int FLUX_THREADS_FP64 = 64;  // the small blocks of the FP64 flux (21 faces)
 constexpr int CELL_THREADS = 128;    // threads per cell-kernel block
 constexpr int CELLS_PER_BLOCK = 24;  // 4 warps x 6 cells, 5 lanes per cell
 constexpr int FGEO = 24;             // reals per face geometry record
@@ -86,6 +88,21 @@ constexpr int64_t tile_at(int row, int cell) {
 // then W1 [3][5] (P1 slopes from [dQ_f (4); Q0])
 enum { WOP_W1 = 153, WOP_STRIDE = 168 };
 
+// The FP64 flux is bound by its pipe whatever the occupancy (218-238 registers,
+// no spills), so a launch lasts as long as the SM with the most warps: blocks
+// of 96 threads (32 faces, no lane idle) or of 64 (21 faces, one lane idle),
+// whichever leaves the fullest of the device's SMs with fewer warps.  On 152
+// SMs, 6,144 faces: 6 warps with blocks of 96, 4 with 64, a whole step 215 and
+// 153 us; 49,280 faces: 33 and 32 warps, 1,242 and 1,188 us; from about 10^6
+// faces the blocks of 96 win by their full lanes.
+inline int64_t fullest_sm_warps(int64_t nf, int threads, int sms) {
+    const int64_t blocks = (nf + threads / 3 - 1) / (threads / 3);
+    return (blocks + sms - 1) / sms * (threads / 32);
+}
+inline bool flux_small_blocks(int64_t nf, int sms) {
+    return fullest_sm_warps(nf, FLUX_THREADS_FP64, sms) < fullest_sm_warps(nf, FLUX_THREADS, sms);
+}
+
 template <typename T>
 struct DevMesh {
     int64_t nc, nf;
@@ -113,6 +130,7 @@ struct DevMesh {
     const T* wop;
     const double* wopd;
     int32_t xwalls;        // 1: the mesh has isothermal or moving wall faces
+    int32_t sms;           // the device's SMs (flux_small_blocks)
 };
 
 template <typename T>

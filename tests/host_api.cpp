@@ -21,6 +21,7 @@ void operator delete(void* p) noexcept { std::free(p); }
 void operator delete(void* p, std::size_t) noexcept { std::free(p); }
 
 // ---- CUDA runtime
+static int sm_count = 152;
 extern "C" {
 cudaError_t cudaMemcpyAsync(void* d, const void* s, size_t n, cudaMemcpyKind, cudaStream_t) {
     std::memmove(d, s, n);
@@ -48,6 +49,11 @@ cudaError_t cudaEventDestroy(cudaEvent_t) { return cudaSuccess; }
 cudaError_t cudaEventRecord(cudaEvent_t, cudaStream_t) { return cudaSuccess; }
 cudaError_t cudaEventSynchronize(cudaEvent_t) { return cudaSuccess; }
 cudaError_t cudaEventElapsedTime(float* ms, cudaEvent_t, cudaEvent_t) { *ms = 1.0f; return cudaSuccess; }
+cudaError_t cudaGetDevice(int* d) { *d = 3; return cudaSuccess; }
+cudaError_t cudaDeviceGetAttribute(int* v, cudaDeviceAttr a, int d) {
+    *v = d == 3 && a == cudaDevAttrMultiProcessorCount ? sm_count : -1;
+    return cudaSuccess;
+}
 cudaError_t cudaGetLastError(void) { return cudaSuccess; }
 const char* cudaGetErrorString(cudaError_t) { return "error"; }
 }
@@ -356,6 +362,38 @@ static int scratch(const MeshFile& file) {
     return refused;
 }
 
+// the FP64 flux's blocks follow the device's own number of SMs
+static int flux_blocks(const MeshFile& file) {
+    gks_mesh* m = file.make();
+    int small = 0;
+    for (int sms : {1, 2, 76, 132, 148, 152, 160}) {
+        sm_count = sms;
+        for (int precision = 0; precision < 2; ++precision) {
+            const gks_params p = parameters(precision, 1);
+            Workspace w(gks_workspace_bytes(m, &p));
+            gks_state* s = nullptr;
+            REQUIRE(gks_state_create(m, &p, w.at, w.bytes, nullptr, &s) == GKS_OK);
+            REQUIRE((precision ? s->m32.sms : s->m64.sms) == sms);
+            gks_state_destroy(s);
+        }
+        // the blocks of a launch dealt to the SMs in turn
+        for (int64_t nf = 1; nf < 60000; nf = nf * 5 / 4 + 1) {
+            int64_t most[2] = {0, 0};
+            for (int small_blocks = 0; small_blocks < 2; ++small_blocks) {
+                const int faces = small_blocks ? 21 : 32, warps = small_blocks ? 2 : 3;
+                std::vector<int64_t> load((size_t)sms, 0);
+                for (int64_t f = 0, b = 0; f < nf; f += faces, ++b) load[(size_t)(b % sms)] += warps;
+                for (int64_t v : load) most[small_blocks] = std::max(most[small_blocks], v);
+            }
+            REQUIRE(flux_small_blocks(nf, sms) == (most[1] < most[0]));
+            small += most[1] < most[0];
+        }
+    }
+    sm_count = 152;
+    gks_mesh_destroy(m);
+    return small;
+}
+
 int main(int argc, char** argv) {
     REQUIRE(argc == 3);
     const std::string check = argv[1];
@@ -370,6 +408,10 @@ int main(int argc, char** argv) {
     }
     if (check == "scratch") {
         std::printf("ok %d\n", scratch(file));
+        return 0;
+    }
+    if (check == "flux_blocks") {
+        std::printf("ok %d\n", flux_blocks(file));
         return 0;
     }
     if (check == "arrays") {

@@ -67,3 +67,10 @@ def test_a_state_keeps_its_boundary_kinds(host_api):
 def test_misaligned_adjoint_scratch_is_refused(host_api):
     mesh = I.box_mesh((3, 2, 2), jitter=0.1, seed=84, periodic=(False,) * 3)
     assert host_api("scratch", mesh, I.wall_kinds(mesh, (0,))) == [2]
+
+
+def test_fp64_flux_blocks_follow_the_devices_sms(host_api):
+    """Blocks of 21 faces exactly where they leave the fullest SM of this
+    device fewer warps than blocks of 32 do."""
+    small, = host_api("flux_blocks", I.box_mesh((2, 2, 2), jitter=0.1, seed=85), np.zeros((48, 4)))
+    assert small > 20
