@@ -1384,8 +1384,8 @@ static gks_status debug_rec_impl(gks_state* s, DevMesh<T>& m, DevState<T>& st, d
     gks_status r = debug_recon_impl<T>(s, m, st, nullptr, nullptr, nullptr);
     if (r != GKS_OK) return r;
     GKS_CHECK_CUDA(Launch<T>::flux(m, s->phys, st.X, st.poly, st.rec, nullptr, dt, stage, s->stream, s->flux_variant));
-    GKS_CHECK_CUDA(Launch<T>::rec_to_double(st.rec, at<int32_t>(s, s->L.perm), d_rec, m.nf, stage == 1 ? 40 : 20,
-                                            &m, st.X, s->phys.gamma - 1.0, dt, s->stream));
+    GKS_CHECK_CUDA(Launch<T>::rec_to_double(m, st.rec, at<int32_t>(s, s->L.perm), d_rec, stage == 1 ? 40 : 20, st.X,
+                                            s->stream));
     return GKS_OK;
 }
 

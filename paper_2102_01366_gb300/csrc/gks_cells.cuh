@@ -62,7 +62,7 @@ struct CellLane {
 };
 
 // vb: the block of CELLS_PER_BLOCK cells, tid: the thread within its
-// CELL_THREADS (defaults: the launch's own block and thread)
+// CELL_THREADS
 __device__ __forceinline__ CellLane cell_lane(int64_t nc, int64_t vb, int tid) {
     CellLane L;
     const int lane = tid & 31;
@@ -75,9 +75,6 @@ __device__ __forceinline__ CellLane cell_lane(int64_t nc, int64_t vb, int tid) {
     L.c = c < nc ? c : nc - 1;
     return L;
 }
-
-__device__ __forceinline__ CellLane cell_lane(int64_t nc) { return cell_lane(nc, blockIdx.x, threadIdx.x); }
-
 
 static inline unsigned cell_grid(int64_t nc) { return (unsigned)((nc + CELLS_PER_BLOCK - 1) / CELLS_PER_BLOCK); }
 

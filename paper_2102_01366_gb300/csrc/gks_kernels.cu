@@ -150,10 +150,10 @@ __global__ void k_rows_gather(const uint32_t* __restrict__ in, uint32_t* __restr
 }
 
 template <typename T>
-__global__ void k_rec_out(const T* __restrict__ rec, const int32_t* __restrict__ perm, double* __restrict__ out,
-                          int64_t nf, int nr, DevMesh<T> m, const T* __restrict__ X, int addback, double gm1,
-                          double dt) {
+__global__ void k_rec_out(DevMesh<T> m, const T* __restrict__ rec, const int32_t* __restrict__ perm,
+                          double* __restrict__ out, int nr, const T* __restrict__ X) {
     constexpr int XSR = Stride<T>::xs;
+    const int64_t nf = m.nf;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nf * nr; i += (int64_t)gridDim.x * blockDim.x) {
         const int64_t d = i / nr;
         const int j = (int)(i - d * nr);
@@ -170,7 +170,7 @@ __global__ void k_rec_out(const T* __restrict__ rec, const int32_t* __restrict__
             const double ref = (double)r[(j % 5) * J + 4] + (double)r[(j % 5) * J + 5];
             v += j < 5 ? ref : 2.0 * ref;
         }
-        if (sizeof(T) == 4 && addback && j >= 10) {
+        if (sizeof(T) == 4 && nr == 40 && j >= 10) {
             // the mean of the two averages (the interior one on a boundary
             // face) times sum_k w_k n = 3 w n
             const int k = (j - 10) % 15, q = k / 3, dir = k - 3 * q;
@@ -266,22 +266,11 @@ cudaError_t Launch<T>::to_double(const T* in, double* out, int64_t n, cudaStream
 }
 
 template <typename T>
-cudaError_t Launch<T>::from_double(const double* in, T* out, int64_t n, cudaStream_t s) {
-    if (n == 0) return cudaSuccess;
-    k_convert<double, T><<<(unsigned)((n + 255) / 256 < 4096 ? (n + 255) / 256 : 4096), 256, 0, s>>>(in, out, n);
-    return cudaGetLastError();
-}
-
-template <typename T>
-cudaError_t Launch<T>::rec_to_double(const T* rec, const int32_t* perm, double* out, int64_t nf, int nr,
-                                     const DevMesh<T>* m, const T* X, double gm1, double dt, cudaStream_t s) {
-    if (nf == 0) return cudaSuccess;
-    const int64_t n = nf * nr;
-    const int addback = (m && X && nr == 40) ? 1 : 0;
-    DevMesh<T> mv{};
-    if (m) mv = *m;
-    k_rec_out<T><<<(unsigned)((n + 255) / 256 < 4096 ? (n + 255) / 256 : 4096), 256, 0, s>>>(rec, perm, out, nf, nr,
-                                                                                            mv, X, addback, gm1, dt);
+cudaError_t Launch<T>::rec_to_double(const DevMesh<T>& m, const T* rec, const int32_t* perm, double* out, int nr,
+                                     const T* X, cudaStream_t s) {
+    if (m.nf == 0) return cudaSuccess;
+    const int64_t n = m.nf * nr;
+    k_rec_out<T><<<(unsigned)((n + 255) / 256 < 4096 ? (n + 255) / 256 : 4096), 256, 0, s>>>(m, rec, perm, out, nr, X);
     return cudaGetLastError();
 }
 
@@ -315,9 +304,8 @@ cudaError_t launch_set_control(double* ctrl, double* case_t, double* case_dt, un
     template cudaError_t Launch<T>::unpack(const double*, const T*, double*, double*, int64_t, cudaStream_t, \
                                            const int32_t*);                                                 \
     template cudaError_t Launch<T>::to_double(const T*, double*, int64_t, cudaStream_t);                    \
-    template cudaError_t Launch<T>::from_double(const double*, T*, int64_t, cudaStream_t);                  \
-    template cudaError_t Launch<T>::rec_to_double(const T*, const int32_t*, double*, int64_t, int,          \
-                                                  const DevMesh<T>*, const T*, double, double, cudaStream_t); \
+    template cudaError_t Launch<T>::rec_to_double(const DevMesh<T>&, const T*, const int32_t*, double*, int, \
+                                                  const T*, cudaStream_t);                                  \
     template cudaError_t Launch<T>::poly_to_double(const T*, double*, int64_t, cudaStream_t, const int32_t*);
 GKS_CELLS_INST(double)
 GKS_CELLS_INST(float)

@@ -205,15 +205,15 @@ struct Launch {
                               const int32_t* cperm = nullptr);
     // conversions for diagnostics
     static cudaError_t to_double(const T* in, double* out, int64_t n, cudaStream_t s);
-    static cudaError_t from_double(const double* in, T* out, int64_t n, cudaStream_t s);
-    // face records in device order -> FP64 in canonical order (perm: device -> canonical).
+    // face records in device order -> FP64 in canonical order (perm: device -> canonical),
+    // the interface-state entries times the mesh's normals.
     // FP32 stage-1 records hold the interface states and fluxes relative to
-    // the mean W_m of the two cells' averages (Stride comment above); with m
-    // and X given, W_m sum_k w_k n and the flux terms (dt / 2) A F_n(W_m),
-    // dt A F_n(W_m) are added back so that the output is the record of the
-    // definition.
-    static cudaError_t rec_to_double(const T* rec, const int32_t* perm, double* out, int64_t nf, int nr,
-                                     const DevMesh<T>* m, const T* X, double gm1, double dt, cudaStream_t s);
+    // the mean W_m of the two cells' averages (Stride comment above): W_m
+    // sum_k w_k n from the state X, and the records' own flux terms
+    // (dt / 2) A F_n(W_m), dt A F_n(W_m), are added back so that the output is
+    // the record of the definition.
+    static cudaError_t rec_to_double(const DevMesh<T>& m, const T* rec, const int32_t* perm, double* out, int nr,
+                                     const T* X, cudaStream_t s);
     // padded reconstruction records -> compact FP64 [nc][50] in centroid-monomial form
     // (rows in the order of cperm's cells)
     static cudaError_t poly_to_double(const T* in, double* out, int64_t nc, cudaStream_t s,

@@ -71,7 +71,7 @@ template <typename T> cudaError_t Launch<T>::dt_partials(const DevMesh<T>&, cons
 template <typename T> cudaError_t Launch<T>::pack(const DevMesh<T>&, const HostPhys&, const double*, const double*, T*, double*, unsigned long long*, cudaStream_t, const int32_t*) { return launched(); }
 template <typename T> cudaError_t Launch<T>::unpack(const double*, const T*, double*, double*, int64_t, cudaStream_t, const int32_t*) { return launched(); }
 template <typename T> cudaError_t Launch<T>::to_double(const T*, double*, int64_t, cudaStream_t) { return launched(); }
-template <typename T> cudaError_t Launch<T>::rec_to_double(const T*, const int32_t*, double*, int64_t, int, const DevMesh<T>*, const T*, double, double, cudaStream_t) { return launched(); }
+template <typename T> cudaError_t Launch<T>::rec_to_double(const DevMesh<T>& m, const T*, const int32_t*, double*, int, const T* X, cudaStream_t) { return m.nf && m.fnw && m.flr && X ? launched() : cudaErrorInvalidValue; }
 template <typename T> cudaError_t Launch<T>::poly_to_double(const T*, double*, int64_t, cudaStream_t, const int32_t*) { return launched(); }
 template struct Launch<float>;
 template struct Launch<double>;
@@ -294,6 +294,10 @@ static int arrays(const MeshFile& file) {
                 REQUIRE(gks_state_create(m, &p, w.at, w.bytes, nullptr, &s) == GKS_OK);
                 if (cells) REQUIRE(gks_state_set_cell_order(s, cells) == GKS_OK);
                 REQUIRE(gks_state_set_variant(s, faces, 3, 1) == GKS_OK);
+                // the records' conversion has the mesh and the state it reads
+                s->initialised = true;
+                for (int stage = 1; stage < 3; ++stage)
+                    REQUIRE(gks_debug_face_records(s, 0.1, stage, reinterpret_cast<double*>(w.at)) == GKS_OK);
                 if (precision == 0) compare_arrays<double, double>(s, *m);
                 if (precision == 1) compare_arrays<float, float>(s, *m);
                 if (precision == 2) compare_arrays<float, double>(s, *m);
