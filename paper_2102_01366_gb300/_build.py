@@ -7,6 +7,7 @@ installed anywhere else.
 from __future__ import annotations
 
 import concurrent.futures as cf
+import hashlib
 import os
 import shutil
 import subprocess
@@ -43,6 +44,17 @@ def _sources():
     hdr = [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith((".h", ".cuh"))]
     hdr.append(os.path.join(INCLUDE, "gks.h"))
     return cu, cpp, hdr
+
+
+def source_digest():
+    """Short digest of the library's sources and build flags (this file): two
+    builds with the same digest run the same kernels."""
+    h = hashlib.sha256()
+    cu, cpp, hdr = _sources()
+    for p in sorted(cu + cpp + hdr) + [os.path.abspath(__file__)]:
+        with open(p, "rb") as f:
+            h.update(os.path.basename(p).encode() + b"\0" + hashlib.sha256(f.read()).digest())
+    return h.hexdigest()[:16]
 
 
 def _compile(cmd):

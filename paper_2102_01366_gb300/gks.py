@@ -8,10 +8,13 @@ entry point raises.
 from __future__ import annotations
 
 import ctypes as C
+import hashlib
 import os
 import re
 
 import numpy as np
+
+from . import _build
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libgks.so")
@@ -107,6 +110,15 @@ def lib():
         fn.argtypes = args
     _lib = L
     return L
+
+
+def _library_digest():
+    """What tells this library's kernels from another version's: its sources,
+    or where they are not at hand the library itself."""
+    try:
+        return _build.source_digest()
+    except OSError:
+        return hashlib.sha256(open(LIB_PATH, "rb").read()).hexdigest()[:16]
 
 
 def _call(name, *args):
@@ -396,15 +408,16 @@ class State:
     def _tune_key(self):
         p = self.params
         name = self.torch.cuda.get_device_name(self.device)
-        return "%s|nc=%d|nf=%d|ncase=%d|prec=%d|weno=%d|order=%d|smooth=%d|visc=%d" % (
+        return "%s|nc=%d|nf=%d|ncase=%d|prec=%d|weno=%d|order=%d|smooth=%d|visc=%d|lib=%s" % (
             name, self.mesh.nc, self.mesh.nf, self.mesh.ncase, p.precision, p.weno, p.order,
-            p.smooth_flux, p.viscous)
+            p.smooth_flux, p.viscous, _library_digest())
 
     def autotune(self, steps=10, cache=None, orders=False):
         """Choose the fastest execution variant for this mesh and options by
         timing them (gks_autotune; with ``orders`` also over the cell
         orderings, gks_autotune_orders); results are cached in a JSON file
-        keyed by GPU name, mesh size and options (``cache``: path, None for
+        keyed by GPU name, mesh size, options and the library's sources (a
+        choice timed on other kernels is not taken; ``cache``: path, None for
         the default ~/.cache/paper_2102_01366_gb300/autotune.json, False for
         no cache)."""
         import json
