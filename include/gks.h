@@ -370,7 +370,7 @@ gks_status gks_timestep_noalloc(const gks_params* p, const double* d_W, const do
 
 /* Per-component root mean square over cells of (W(t) - W_prev) / dt_last,
  * where W_prev is the state before the last step (host out_l2[5];
- * synchronises). */
+ * synchronises).  Zeros before a state's first step. */
 gks_status gks_residual(gks_state* state, double* out_l2);
 
 /* -------------------------------------------------------------- adjoint -- */

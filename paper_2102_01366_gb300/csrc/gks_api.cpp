@@ -835,6 +835,8 @@ extern "C" gks_status gks_state_create(const gks_mesh* mesh, const gks_params* p
         GKS_CHECK_CUDA(cudaGetDevice(&device));
         GKS_CHECK_CUDA(cudaDeviceGetAttribute(&s->sms, cudaDevAttrMultiProcessorCount, device));
         s->bkind = mesh->bkind;
+        // no step yet, no residual (the updates alone write these sums)
+        GKS_CHECK_CUDA(cudaMemsetAsync(s->ws + s->L.part, 0, 8 * PART_N * (size_t)update_blocks(mesh->nc), s->stream));
         if (fp32) {
             make_views<float>(s, s->m32, s->s32);
             return upload_mesh<float>(s);

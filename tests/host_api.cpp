@@ -366,6 +366,26 @@ static int scratch(const MeshFile& file) {
     return refused;
 }
 
+// a state that made no step has no residual, whatever its workspace held
+static int residual(const MeshFile& file) {
+    gks_mesh* m = file.make();
+    int zeros = 0;
+    for (int precision = 0; precision < 3; ++precision) {
+        const gks_params p = parameters(precision, 1);
+        Workspace w(gks_workspace_bytes(m, &p));
+        std::memset(w.at, 0xff, w.bytes);  // every double a NaN
+        gks_state* s = nullptr;
+        REQUIRE(gks_state_create(m, &p, w.at, w.bytes, nullptr, &s) == GKS_OK);
+        s->initialised = true;
+        double dt, r[5];
+        REQUIRE(gks_timestep(s, &dt) == GKS_OK && gks_residual(s, r) == GKS_OK);
+        for (double v : r) zeros += v == 0.0;
+        gks_state_destroy(s);
+    }
+    gks_mesh_destroy(m);
+    return zeros;
+}
+
 // the FP64 flux's blocks follow the device's own number of SMs
 static int flux_blocks(const MeshFile& file) {
     gks_mesh* m = file.make();
@@ -412,6 +432,10 @@ int main(int argc, char** argv) {
     }
     if (check == "scratch") {
         std::printf("ok %d\n", scratch(file));
+        return 0;
+    }
+    if (check == "residual") {
+        std::printf("ok %d\n", residual(file));
         return 0;
     }
     if (check == "flux_blocks") {

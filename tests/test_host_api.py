@@ -69,6 +69,13 @@ def test_misaligned_adjoint_scratch_is_refused(host_api):
     assert host_api("scratch", mesh, I.wall_kinds(mesh, (0,))) == [2]
 
 
+def test_a_state_without_a_step_has_no_residual(host_api):
+    """Its residual is zero, whatever the workspace held before; the time step
+    query no longer writes the sums."""
+    mesh = I.box_mesh((3, 2, 2), jitter=0.1, seed=86, periodic=(False,) * 3)
+    assert host_api("residual", mesh, I.wall_kinds(mesh, (0,))) == [3 * 5]
+
+
 def test_fp64_flux_blocks_follow_the_devices_sms(host_api):
     """Blocks of 21 faces exactly where they leave the fullest SM of this
     device fewer warps than blocks of 32 do."""
