@@ -122,7 +122,8 @@ __device__ __forceinline__ void rotate_in(const double (*Rm)[3], double* v) {
 }
 
 // The point's inputs in the face frame (per side W, g: 20 values) from the
-// stored reconstruction, as the forward flux forms them, and the output
+// stored reconstruction, with R as the plain sum of its terms where the forward
+// flux takes the nested form (the same to rounding, see below), and the output
 // adjoints of the point (face frame) from the record adjoints (the transposed
 // record formulas of the stage).
 template <int NR>
@@ -171,10 +172,12 @@ __device__ __forceinline__ void adj_point_setup(const DevMesh<double>& m, const 
     rotate_in(Rm, lD);
     rotate_in(Rm, ldWt);
     // R as the plain sum: where the field is uniform to rounding, the derivative
-    // of |p_l - p_r| is the sign of what rounding leaves, and the nested form
-    // leaves something where the plain sum, and its transcriptions in plain FP64
-    // arrays, leave zero (gradients of 48,000 cells 1e-12 apart there, 1e-14 with
-    // this; 5,650 -> 5,781 us a reverse step)
+    // of |p_l - p_r| is the sign of what rounding leaves.  Nothing makes one
+    // evaluation exact there, but the plain sum agrees best with the method in
+    // plain FP64 arrays differentiated by autograd: gradients of the vortex
+    // (48,000 cells, three seeds) within 2e-12, against 5e-10 with the nested form
+    // and 3e-9 with the derivative set to zero within four ulps of a tie (either
+    // form); it takes 2 % more (5,650 -> 5,790 us a reverse step).
 #pragma unroll 1
     for (int side = 0; side < 2; ++side)
         side_state<double, true, true>(m, ph, Xavg, poly + side_cell(L, R, side) * POLY_STRIDE, geo, Rm, L, R, side, k,
@@ -292,9 +295,10 @@ __global__ void __launch_bounds__(ADJ_THREADS) k_adj_face_back(DevMesh<double> m
                 to_local_adj(Rm, ls, lg, lW, lgg);
                 for (int q = 0; q < 5; ++q) lw[q] += lW[q];
             } else if (XW && (other == FLR_ISOTHERMAL_WALL || other == FLR_MOVING_WALL)) {
-                // the interior state at the point, face frame, then the ghost's transpose
+                // the interior state at the point, as adj_point_setup forms it, then the
+                // ghost's transpose there
                 double Wv[5], g[3][5], x[20];
-                eval_poly(poly + cell * POLY_STRIDE, X, Wv, g);
+                eval_poly<true>(poly + cell * POLY_STRIDE, X, Wv, g);
                 to_local(Rm, Wv, g, x, reinterpret_cast<double (*)[5]>(x + 5));
                 double Uw[3];
                 rotate_vec(Rm, ph.uwall, Uw);
