@@ -728,7 +728,7 @@ def main():
         "step_hbm": dict(step_hbm(value, "fp32", peaks), peak_source=peak_src,
                          note="latency-bound size: the 24,576-cell workspace fits in L2"),
         "autotuned_variant": {"fp32": results["fp32"]["variant"], "fp64": results["fp64"]["variant"],
-                              "meaning": "[face_order, flux_blocks_per_SM, slopes_pass]",
+                              "meaning": "[face_order, flux occupancy (3 more warps, 2 more registers), slopes_pass]",
                               "fp32_stage_forms": results["fp32"]["forms"],
                               "fp32_cell_order": results["fp32"]["cell_order"],
                               "cell_orders": "0 caller's, 1 reverse Cuthill-McKee, 2 Morton"},

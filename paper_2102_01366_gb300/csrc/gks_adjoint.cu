@@ -175,9 +175,10 @@ __device__ __forceinline__ void adj_point_setup(const DevMesh<double>& m, const 
     // of |p_l - p_r| is the sign of what rounding leaves.  Nothing makes one
     // evaluation exact there, but the plain sum agrees best with the method in
     // plain FP64 arrays differentiated by autograd: gradients of the vortex
-    // (48,000 cells, three seeds) within 2e-12, against 5e-10 with the nested form
-    // and 3e-9 with the derivative set to zero within four ulps of a tie (either
-    // form); it takes 2 % more (5,650 -> 5,790 us a reverse step).
+    // (48,000 cells) within 1e-11 over four seeds, two of them within 3e-14, against
+    // 1e-10 to 5e-10 with the nested form and 2e-9 to 3e-9 with the derivative set
+    // to zero within four ulps of a tie (either form); it takes 2 % more (5,650 ->
+    // 5,790 us a reverse step).
 #pragma unroll 1
     for (int side = 0; side < 2; ++side)
         side_state<double, true, true>(m, ph, Xavg, poly + side_cell(L, R, side) * POLY_STRIDE, geo, Rm, L, R, side, k,

@@ -404,11 +404,11 @@ struct gks_state {
     bool stage_valid = false;  // the stage buffer holds the last step's W*, grad W*
     bool fixed_pinned = false;  // gks_set_fixed_state was called: initialisations keep the fixed state
     int face_order = 0;    // 0: canonical face order, 1: grouped by left cell
-    int flux_variant = 1;  // 1: 3 blocks/SM, 0: 2 blocks/SM (FP32 flux)
-    // 1: reconstruction step 1 as its own pass (WENO only).  The default, as
-    // the faster one at every size measured, from 1,536 cells (a step 37.2 ->
-    // 33.1 us) over 24,576 (81 -> 76; FP64 1,163 -> 1,140) and 409,644 (996 ->
-    // 869) to 580,320 (1,556 -> 1,284 us); 0 forms each neighbour's slopes anew.
+    int flux_variant = 1;  // occupancy of the FP32 flux (gks_flux.cuh): 1 more warps, 0 more registers
+    // 1: reconstruction step 1 as its own pass (WENO only); 0 forms each
+    // neighbour's slopes anew.  The default, as nowhere slower: a step with 0 / 1,
+    // 1,536 cells 33.0 / 33.0 us, 3,330 35.1 / 33.1, 24,576 72.1 / 67.6 (FP64
+    // 1,099 / 1,078), 409,644 891 / 744, 580,320 1,422 / 1,111.
     int slopes_pass = 1;
     int fused = 0;         // 1: each stage as one persistent launch (precision 1 only)
     // cell ordering of the device arrays (FP32 bulk): 0 the caller's, 1

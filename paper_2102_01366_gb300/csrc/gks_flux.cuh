@@ -25,14 +25,13 @@ namespace gks {
 //
 // FP32 is bound by instruction issue, with the gathers of the two 240-byte
 // reconstruction records behind it; the faster layout is therefore the one
-// with the fewest instructions.  Two threads a point (one a side, in two
-// warps) repeated the frame and met four times at a barrier through 60 KB of
-// shared memory: stage 1 / stage 2 on 3.15 M faces 2,087 / 1,335 us there,
-// 1,071 / 687 us here at first, 907 / 594 us now; on 49,280 faces 40.6 / 28.7
-// us, now 22.5 / 18.4 us.
-// Persistent blocks that fetch the next block's records into shared memory hid
-// the gathers, but a block's three warps then waited for each other: 1,207 /
-// 837 us.
+// with the fewest instructions and barriers.  Stage 1 / stage 2 on 3.15 M
+// faces 905 / 594 us, on 49,280 faces 22.1 / 18.5 us.  Against it: two threads
+// a point (one a side, in two warps), which repeat the frame and meet four
+// times at a barrier through 60 KB of shared memory, 2,087 / 1,335 us and 40.6 /
+// 28.7 us; persistent blocks that fetch the next block's records into shared
+// memory, which hides the gathers but has a block's three warps wait for each
+// other, stage 1 1,207 us (the present layout at that time 1,108).
 // FP64 is bound by its pipe (16 cycles a warp instruction): rotating and
 // weighting per face instead of per point took 484 -> 450 us on 49,280 faces.
 
@@ -378,11 +377,15 @@ __global__ void __launch_bounds__(TH, MINB) k_flux(DevMesh<T> m, Phys<T> ph, con
 }
 
 // Threads a block and resident blocks an SM, hence registers.  FP32 variant
-// 1: 15 warps at 128 registers, no spills (stage 1, 3.15 M faces: 1,161 us,
-// against 1,273 us with 6 blocks and 1,419 us with 8, which spill); variant
-// 0: 12 warps with more registers, the faster one in some viscous and small
-// launches.  Inviscid stage 2 fits 96 registers without spills: 6 blocks (3.15
-// M faces 631 -> 595 us; the viscous one would spill, 255 -> 260 us on 1.16 M).
+// 1: the most blocks that spill nothing, 5 (15 warps, 128 registers), in
+// inviscid stage 2 6 (96 registers).  Variant 0: 4 blocks; the faster one where
+// a launch has too few blocks to use the warps (a step of 1,536 cells 33.0 us
+// with variant 1, 31.0-32.2 with 0; 2,592 viscous cells 35.1 and 33.0; from 3,330
+// cells on the same or slower).  Measured, with 4 / 5 / 6 / 8 blocks an SM:
+//   3.15 M faces, inviscid, stage 1   1,069 / 905 / 948 / 1,020 us
+//                           stage 2     612 / 629 / 594 / 634
+//   1.16 M faces, viscous,  stage 1     436 / 381 / 451 / 486
+//                           stage 2     300 / 252 / 260 / 322
 constexpr int FLUX_BLOCKS_V1 = 5, FLUX_BLOCKS_V1_STAGE2 = 6, FLUX_BLOCKS_V0 = 4;
 template <typename T, bool XW>
 static cudaError_t launch_flux(const DevMesh<T>& m, const HostPhys& p, const T* W, const T* poly, T* rec,

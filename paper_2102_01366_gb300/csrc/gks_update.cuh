@@ -57,13 +57,15 @@ __device__ __forceinline__ bool positive(double x) { return __double_as_longlong
 // --------------------------------------------------------------------------
 // cell updates, five lanes per cell (one per component).  Bound by the
 // latency of two dependent gathers (face list, then face records), so all of
-// a cell's gathers are issued before the first is used; in FP32 bulk next by
-// the FP64 pipe, so FP32 <-> FP64 conversions go through the integer pipe
-// (widen, split_pair).  On 1.57 M cells, FP32, stage 1 / stage 2: 393 / 707 us
-// before, 306 / 303 with warp_case_min and cell-major S and G, 281 / 171 with
-// the integer conversions and the normals apart from the Gauss points, 254 /
-// 171 with a component's record entries together.  One thread per cell with 16-byte gathers took 349 / 236 us (too few warps in
-// flight) and twice the time on 1,536 to 3,072 cells.
+// a cell's gathers are issued before the first is used, the normals lie apart
+// from the Gauss points and a component's record entries together; in FP32
+// bulk next by the FP64 pipe, so FP32 <-> FP64 conversions go through the
+// integer pipe (widen, split_pair).  1.57 M cells, FP32, stage 1 / stage 2: 254 /
+// 171 us; 393 / 707 with dependent loads, a block's serial time-step minimum and
+// component-major S and G; 306 / 303 without the integer conversions and the
+// normals apart.  One thread per cell with 16-byte gathers, when five lanes took
+// 281 / 171, took 349 / 236 (too few warps in flight) and twice the time on 1,536
+// to 3,072 cells.
 // --------------------------------------------------------------------------
 
 // N values of a record (8- or 16-byte aligned) as vectors of two
